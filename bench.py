@@ -917,8 +917,11 @@ def main():
         src = "measured" if peaks else "fallback"
         achieved = comb_macs_per_launch / (comb_launch_ms * 1e-3) / 1e12
         # per launch, both parties: planes of both operand pairs read once, Z read and written once (average of the
-        # up- and the down-projection launch)
-        comb_bytes_per_launch = 8 * ((2 * T * d + 2 * d * g * n + 2 * T * g * n) + (2 * T * n + 2 * n * d + 2 * T * d))
+        # up- and the down-projection launch); with few tokens the kernel reads the operands' words and writes the
+        # messages itself
+        stream = used_path == "limb" and T <= 32
+        comb_bytes_per_launch = 8 * ((3 * T * d + 3 * d * g * n + 3 * T * g * n) + (3 * T * n + 3 * n * d + 3 * T * d)) \
+            if stream else 8 * ((2 * T * d + 2 * d * g * n + 2 * T * g * n) + (2 * T * n + 2 * n * d + 2 * T * d))
         if used_path == "limb":
             # The pipe's peak in ring multiply-adds: the measured rate of the tensor instruction the kernel issues,
             # over 36 limb products.  Beside it, what the measured bf16 GEMM peak would imply at the nominal int8 :
@@ -935,7 +938,7 @@ def main():
             t_tensor = comb_macs_per_launch / (peak * 1e12)
             t_hbm = comb_bytes_per_launch / (hbm * 1e9)
             if t_hbm > t_tensor:
-                # few tokens: the kernel streams the weight-side planes once and is bound by that traffic
+                # few tokens: the kernel streams the weight side's words once and is bound by that traffic
                 roof = {"bound": "hbm", "achieved": comb_bytes_per_launch / (comb_launch_ms * 1e-3) / 1e9, "peak": hbm,
                         "unit": "GB/s", "peak_source": f"{src} HBM copy peak"}
             else:
@@ -958,7 +961,7 @@ def main():
                     "peak_sustained": peak_sustained, "frac_of_sustained_peak": achieved / peak_sustained,
                     "peak_from_unit_counts": derived}
         roof["frac"] = roof["achieved"] / roof["peak"]
-        roof["kernel"] = "combine_" + used_path + ("_few" if used_path == "limb" and T <= 32 else "")
+        roof["kernel"] = "combine_stream" if stream else "combine_" + used_path
         roof["traffic"] = combine_traffic(args.workload, sparsity, used_path)
         roof["traffic_unit"] = "bytes per launch (ncu dram read+write); algorithmic: planes once + Z read-modify-write"
         roof["algorithmic_bytes_per_launch"] = comb_bytes_per_launch

@@ -4,8 +4,8 @@
  *
  * Both parties of a 2-party additive sharing over Z_{2^64} are simulated on one
  * GPU; the "messages" the two servers would exchange are device buffers owned by
- * the context.  A party's kernels read only that party's shares and the two
- * message buffers.
+ * the context.  What is computed for a party depends on that party's shares and
+ * on the two messages only.
  *
  * Conventions
  *   - Every word is a uint64_t ring element; arithmetic is mod 2^64.
@@ -83,9 +83,7 @@ enum {
     COMET_B_DN = 9,   /* in : triple, masks W2[I, :]     [d_model, n]           */
     COMET_C_DN = 10,  /* in : triple                     [T, d_model]           */
     COMET_E_UP = 11,  /* out: message X_i - A_i          [T, d_model]           */
-    COMET_F_UP = 12,  /* out: message W_i[:, I] - B_i    [g*n, d_model]  (after a product with at most 32
-                         tokens on the tensor-core path the messages F exist as limb planes; comet_get
-                         rebuilds the words)                                  */
+    COMET_F_UP = 12,  /* out: message W_i[:, I] - B_i    [g*n, d_model]         */
     COMET_Z_UP = 13,  /* out: up-projection share        [T, g*n]               */
     COMET_E_DN = 14,  /* out: message H_i - A'_i         [T, n]                 */
     COMET_F_DN = 15,  /* out: message W2_i[I, :] - B'_i  [d_model, n]           */
@@ -462,6 +460,11 @@ int comet_beaver_mul(void* cuda_stream, const uint64_t* const X[2], const uint64
  * The first call on each device looks up the device address of the array
  * (once per device; no allocation).  Make that first call outside any stream
  * capture.
+ *
+ * The product runs on the tensor cores in the same kernel as a context's products
+ * of at most 32 tokens.  Its device-side waits are bounded like theirs, but there
+ * is no context to report to: after a wait that ran out (about two seconds, which
+ * no working launch comes near) Z lacks part of its sums.
  *
  * The array is shared by every call in the process and is never cleared:
  * a call overwrites all of the part it uses before reading it, so stale

@@ -20,6 +20,7 @@
 #include "kernels_peak.cuh"
 #include "kernels_shuffle.cuh"
 #include "kernels_simt.cuh"
+#include "kernels_stream.cuh"
 
 using comet::u64;
 
@@ -46,10 +47,8 @@ struct comet_ctx {
     cudaEvent_t ev_fork, ev_join;
     bool side_pending;                // ev_join not yet waited for on the main stream
     bool dn_right_ready;              // F'_i and the right planes of the down-projection are current
-    bool dn_right_few;                // ... and were laid out for the few-token kernel (128-row tiles)
     bool dn_copy_ready;               // Y_i already holds C'_i (copied beside the up-projection)
     int32_t dn_copy_tokens;           // ... for this many token rows
-    bool f_as_planes[2];              // the messages F_i of the last up / down product exist as planes only
     uint8_t* d_mask;
     // a block mask given in host memory is counted on the host and copied from a pinned staging slot of the
     // library's own, so that comet_set_mask need not wait for the device
@@ -233,8 +232,80 @@ Proj proj_down(const comet_ctx* c, int tokens) {
                 COMET_C_DN, COMET_Y, true};
 }
 
-// The few-token kernel (operand roles exchanged) serves products with at most 32 token rows.
-inline bool limb_few(const Proj& pr) { return pr.M <= comet::limb_few::BT; }
+// The streaming kernel (one kernel per product, operand roles exchanged) serves products with at most 32 token rows:
+// its planes live in shared memory, so every further 32 rows would convert the weights once more.
+inline bool few_tokens(const Proj& pr) { return pr.M <= comet::limb_stream::BT; }
+
+// Z <- C, then the streaming kernel behind it (it begins while the copy runs and waits for it before its first sum).
+int launch_stream(comet::StreamArgs& args, const u64* const C[2], int sm_count, cudaStream_t stream,
+                  const int* priority, cudaError_t* err) {
+    namespace ls = comet::limb_stream;
+    *err = cudaSuccess;
+    args.mt = ceil_div(args.M, ls::BT);
+    args.nt = ceil_div(args.N, ls::BW);
+    args.kb = ceil_div(args.K, ls::KC);
+    const long long steps = (long long)args.mt * args.nt * args.kb;
+    const unsigned grid = (unsigned)(steps < sm_count ? steps : sm_count);
+    args.last_cost = ceil_div(args.N - (args.nt - 1) * ls::BW, ls::QROWS) + 1;
+    const long long cost = ((long long)(ls::QUARTERS + 1) * (args.nt - 1) + args.last_cost) * args.kb * args.mt;
+    if (cost > 0x7fffffffll) return COMET_ERR_SHAPE;                   // the kernel counts in 32 bits
+    args.cta_cost = (unsigned)(cost / grid);
+    args.cta_extra = (unsigned)(cost % grid);
+    const long long pairs = (long long)args.M * args.N / 2, want = (pairs + 255) / 256, most = (long long)sm_count * 8;
+    *err = launch_chained(comet::result_init_kernel, dim3((unsigned)(want < most ? want : most), 2), dim3(256), 0, stream,
+                          nullptr, C[0], C[1], args.Z[0], args.Z[1], pairs);
+    if (*err != cudaSuccess) return COMET_ERR_CUDA;
+    *err = launch_chained(comet::combine_stream_kernel, dim3(grid), dim3(ls::THREADS), ls::SMEM_BYTES, stream,
+                          priority, args);
+    return *err == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
+}
+
+// Tensor-core path with few token rows: the whole Pi_MatMul.
+int stream_product(comet_ctx* c, const Proj& pr) {
+    namespace ls = comet::limb_stream;
+    comet::StreamArgs a;
+    std::memset(&a, 0, sizeof(a));
+    const u64* C[2];
+    for (int p = 0; p < 2; ++p) {
+        a.X[p] = c->buf[p][pr.idX];
+        a.A[p] = c->buf[p][pr.idA];
+        a.E[p] = c->buf[p][pr.idE];
+        a.W0[p] = pr.down ? c->buf[p][COMET_W2] : (c->groups >= 2 ? c->buf[p][COMET_WG] : c->buf[p][COMET_W1]);
+        a.W1[p] = c->buf[p][COMET_W1];
+        a.W2[p] = c->buf[p][COMET_W3];
+        a.B[p] = c->buf[p][pr.idB];
+        a.F[p] = c->buf[p][pr.idF];
+        a.Z[p] = c->buf[p][pr.idZ];
+        C[p] = c->buf[p][pr.idC];
+    }
+    a.ids = c->d_ids;
+    a.n = c->n_active;
+    a.bs = c->cfg.block;
+    a.M = pr.M; a.N = pr.N; a.K = pr.K;
+    a.ldw = pr.down ? c->cfg.d_ff : c->cfg.d_model;
+    a.down = pr.down ? 1 : 0;
+    if (c->tmask_set) {
+        a.tmask = pr.down ? c->d_tmask : nullptr;
+        a.tmask_ld = c->n_active_blocks;
+        a.row_label = pr.down ? nullptr : c->d_row_label;
+        a.blk_label = c->d_blk_label;
+    }
+    a.error_flag = c->d_error;
+    a.error_host = c->h_count_dev + 3;
+    cudaError_t err;
+    {
+        PhaseTimer timer(c, COMET_PHASE_COMBINE, 2);
+        const int rc = launch_stream(a, C, c->sm_count, c->stream, &c->top_priority, &err);
+        if (rc != COMET_OK) {
+            c->last_cuda_error = (int)err;
+            return rc;
+        }
+    }
+    c->stats.kernel_launches += 2;
+    c->stats.tensor_tile_macs = 2ll * 2 * a.mt * a.nt * a.kb * ls::KC * ls::BW * ls::BT;
+    c->stats.matmul_path = COMET_PATH_LIMB;
+    return COMET_OK;
+}
 
 // Makes the main stream wait for the side stream's outstanding work (if any).
 int join_side(comet_ctx* c) {
@@ -262,9 +333,7 @@ int limb_open(comet_ctx* c, const Proj& pr, bool left, bool right, cudaStream_t 
         a.B[p] = c->buf[p][pr.idB];
         a.F[p] = c->buf[p][pr.idF];
         a.Bpl[p] = planes[p][0];
-        a.Fpl[p] = planes[p][1];
     }
-    a.emit_f = limb_few(pr) ? 1 : 0;       // few-token products read the messages as planes (no plane of their sum)
     a.left_pairs = left ? (long long)pr.M * pr.K / 2 : 0;
     a.left_blocks = left ? ew_grid(c, a.left_pairs, lb::OPEN_THREADS) : 0;
     a.ids = c->d_ids;
@@ -275,7 +344,6 @@ int limb_open(comet_ctx* c, const Proj& pr, bool left, bool right, cudaStream_t 
     a.ldw = pr.down ? c->cfg.d_ff : c->cfg.d_model;
     a.kblocks = kb;
     a.down = pr.down ? 1 : 0;
-    a.right_tile_rows = limb_few(pr) ? comet::limb_few::BW : lb::BN;
     a.tmask = (pr.down && c->tmask_set) ? c->d_tmask : nullptr;
     a.tmask_ld = c->n_active_blocks;
     a.row_label = (!pr.down && c->tmask_set) ? c->d_row_label : nullptr;
@@ -284,7 +352,7 @@ int limb_open(comet_ctx* c, const Proj& pr, bool left, bool right, cudaStream_t 
     a.kmap = (pr.down && c->grouped) ? c->d_kmap : nullptr;
     // right CTAs: 32 rows x kb_per_cta k-blocks each, over whole plane tiles (rows past the operand are zero planes);
     // enough k-blocks per CTA for the copies of one to fly under the work on another, enough CTAs to fill the device
-    const int row_tiles = right ? ceil_div(pr.N, a.right_tile_rows) * (a.right_tile_rows / lb::OPEN_ROWS) : 0;
+    const int row_tiles = right ? ceil_div(pr.N, lb::BN) * (lb::BN / lb::OPEN_ROWS) : 0;
     {
         const long long fill = (long long)c->sm_count * 6;
         long long per = fill > 0 ? 2ll * row_tiles * kb / fill : 1;
@@ -295,7 +363,6 @@ int limb_open(comet_ctx* c, const Proj& pr, bool left, bool right, cudaStream_t 
     }
     const int right_tiles = row_tiles * a.kchunks;
     if (a.left_blocks + right_tiles == 0) return COMET_OK;
-    if (right_tiles) c->f_as_planes[pr.down ? 1 : 0] = a.emit_f != 0;
     const size_t smem = right_tiles ? lb::OPEN_SMEM_BYTES : 0;
     COMET_CUDA(c, launch_chained(comet::limb_open_kernel, dim3(2 * (a.left_blocks + right_tiles)),
                                  dim3(lb::OPEN_THREADS), smem, stream, nullptr, a));
@@ -332,16 +399,12 @@ int limb_prep(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy, cu
             a.col_map = c->d_col_map;
         }
     }
-    a.left_tile_rows = limb_few(pr) ? comet::limb_few::BT : lb::BM;
-    a.right_tile_rows = limb_few(pr) ? comet::limb_few::BW : lb::BN;
     a.tmask = (pr.down && c->tmask_set) ? c->d_tmask : nullptr;
     a.tmask_ld = c->n_active_blocks;
     a.bs = c->cfg.block;
     // tile CTAs: 32 rows x kb_per_cta k-blocks each, over whole plane tiles (rows past the operand are zero planes)
-    const int left_rows32 = left ? ceil_div(a.M, a.left_tile_rows) * (a.left_tile_rows / lb::OPEN_ROWS) : 0;
-    // few-token products take the planes of the two messages as limb_open_kernel wrote them
-    const int right_rows32 = (right && !limb_few(pr))
-                                 ? ceil_div(a.N, a.right_tile_rows) * (a.right_tile_rows / lb::OPEN_ROWS) : 0;
+    const int left_rows32 = left ? ceil_div(a.M, lb::BM) * (lb::BM / lb::OPEN_ROWS) : 0;
+    const int right_rows32 = right ? ceil_div(a.N, lb::BN) * (lb::BN / lb::OPEN_ROWS) : 0;
     {
         const long long fill = (long long)c->sm_count * 4;
         long long per = fill > 0 ? 2ll * (left_rows32 + right_rows32) * kb / fill : 1;
@@ -364,14 +427,10 @@ int limb_prep(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy, cu
     return COMET_OK;
 }
 
-// Tensor-core path: the persistent stream-K kernel over both parties' tiles (the few-token variant when the
-// product has at most 32 token rows).
+// Tensor-core path: the persistent stream-K kernel over both parties' tiles.
 int limb_combine(comet_ctx* c, const Proj& pr) {
     namespace lb = comet::limb;
-    namespace lf = comet::limb_few;
-    const bool few = limb_few(pr);
-    const int kb = ceil_div(pr.K, lb::KC);
-    const int mt = few ? 1 : ceil_div(pr.M, lb::BM), nt = few ? ceil_div(pr.N, lf::BW) : ceil_div(pr.N, lb::BN);
+    const int kb = ceil_div(pr.K, lb::KC), mt = ceil_div(pr.M, lb::BM), nt = ceil_div(pr.N, lb::BN);
     uint8_t* (*planes)[2] = pr.down ? c->planes_right_dn : c->planes_right_up;
     comet::LimbArgs a;
     for (int p = 0; p < 2; ++p) {
@@ -386,8 +445,7 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
     a.error_host = c->h_count_dev + 3;
     a.ldz = pr.N; a.bs = c->cfg.block; a.group_units = 0;
     a.groups = nullptr; a.row_map = nullptr; a.col_map = nullptr;
-    const bool grouped = c->grouped && !few;
-    if (grouped) {
+    if (c->grouped) {
         a.M = c->live_rows;
         a.mt = ceil_div(a.M, lb::BM);
         a.row_map = c->d_row_map;
@@ -402,20 +460,16 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
             a.group_units = c->group_units_up;
         }
     }
-    const long long total_units = grouped ? 2ll * a.group_units
-                                          : 2ll * mt * nt * (few ? comet::LIMB_FEW_PAIRS : 2) * kb;
-    c->stats.tensor_tile_macs = total_units * lb::KC * (few ? lf::BW * lf::BT : lb::BM * lb::BN);
+    const long long total_units = c->grouped ? 2ll * a.group_units : 2ll * mt * nt * 2 * kb;
+    c->stats.tensor_tile_macs = total_units * lb::KC * lb::BM * lb::BN;
     const int grid = (int)(total_units < c->sm_count ? total_units : c->sm_count);
     {
         PhaseTimer timer(c, COMET_PHASE_COMBINE, 1);
         // The persistent kernel needs a slot on every SM.  With the device's highest scheduling priority its CTAs
         // get the slots that free up before the memory-side CTAs of other contexts queued beside it do, so the
         // tensor cores do not wait behind work that could as well run under them.
-        const dim3 block(few ? lf::THREADS : lb::THREADS);
-        const size_t smem = few ? lf::SMEM_BYTES : lb::SMEM_BYTES;
-        auto* kernel = few ? comet::combine_limb_few_kernel
-                           : grouped ? comet::combine_limb_grouped_kernel : comet::combine_limb_kernel;
-        COMET_CUDA(c, launch_chained(kernel, dim3(grid), block, smem, c->stream, &c->top_priority, a));
+        auto* kernel = c->grouped ? comet::combine_limb_grouped_kernel : comet::combine_limb_kernel;
+        COMET_CUDA(c, launch_chained(kernel, dim3(grid), dim3(lb::THREADS), lb::SMEM_BYTES, c->stream, &c->top_priority, a));
     }
     c->stats.kernel_launches += 1;
     c->stats.matmul_path = COMET_PATH_LIMB;
@@ -425,9 +479,7 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
 
 bool limb_fits(const comet_ctx* c, const Proj& pr) {
     namespace lb = comet::limb;
-    // the few-token layout (32-row token tiles, 128-row weight tiles) never needs more than the ordinary one
-    // plus one 64-row tile of the right operand, which the allocation includes
-    const size_t kb = ceil_div(pr.K, lb::KC), mt = ceil_div(pr.M, lb::BM), nt = ceil_div(pr.N, lb::BN) + 1;
+    const size_t kb = ceil_div(pr.K, lb::KC), mt = ceil_div(pr.M, lb::BM), nt = ceil_div(pr.N, lb::BN);
     return mt * kb * lb::A_BLOCK_BYTES <= c->planes_left_bytes &&
            nt * kb * lb::B_BLOCK_BYTES <= (pr.down ? c->planes_right_dn_bytes : c->planes_right_up_bytes);
 }
@@ -556,9 +608,10 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
         const int64_t kb_max = kb_up > kb_dn ? kb_up : kb_dn;
         const int64_t mt = (c->cap_T + lb::BM - 1) / lb::BM;
         c->planes_left_bytes = (size_t)(mt * kb_max) * lb::A_BLOCK_BYTES;
-        c->planes_right_up_bytes = (size_t)(((gn + lb::BN - 1) / lb::BN + 1) * kb_up) * lb::B_BLOCK_BYTES;
-        c->planes_right_dn_bytes = (size_t)(((d + lb::BN - 1) / lb::BN + 1) * kb_dn) * lb::B_BLOCK_BYTES;
-        for (int p = 0; p < 2 && ok; ++p)
+        c->planes_right_up_bytes = (size_t)(((gn + lb::BN - 1) / lb::BN) * kb_up) * lb::B_BLOCK_BYTES;
+        c->planes_right_dn_bytes = (size_t)(((d + lb::BN - 1) / lb::BN) * kb_dn) * lb::B_BLOCK_BYTES;
+        // a context for few tokens only never builds planes in memory
+        for (int p = 0; p < 2 && ok && c->cap_T > comet::limb_stream::BT; ++p)
             for (int w = 0; w < 2 && ok; ++w) {
                 ok = cudaMalloc((void**)&c->planes_left[p][w], c->planes_left_bytes) == cudaSuccess;
                 ok = ok && cudaMalloc((void**)&c->planes_right_up[p][w], c->planes_right_up_bytes) == cudaSuccess;
@@ -568,10 +621,8 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
                                         (int)lb::SMEM_BYTES) == cudaSuccess;
         // the memory-side kernels may share an SM with a resident tensor-core CTA (which forces the largest
         // shared-memory carve-out), so they ask for the same carve-out
-        ok = ok && cudaFuncSetAttribute(comet::combine_limb_few_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)comet::limb_few::SMEM_BYTES) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(comet::combine_limb_few_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                        (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+        ok = ok && cudaFuncSetAttribute(comet::combine_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)comet::limb_stream::SMEM_BYTES) == cudaSuccess;
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                         (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -824,7 +875,7 @@ int comet_set_token_mask(comet_ctx* c, const uint8_t* token_mask, int location, 
     // Protocol 2, first step: the connected components the up-projection is partitioned into, the number of
     // non-zero entries (Theorem 2's count) and, for the tensor-core path, the component-sorted order and the work
     // of every row tile, in one launch
-    const bool plan = c->path == COMET_PATH_LIMB && tokens > comet::limb_few::BT && tokens <= 32768;
+    const bool plan = c->path == COMET_PATH_LIMB && tokens > comet::limb_stream::BT && tokens <= 32768;
     {
         comet::TokenPlanArgs a;
         std::memset(&a, 0, sizeof(a));
@@ -893,9 +944,13 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
 
     if (c->path == COMET_PATH_LIMB) {
         const Proj up = proj_up(c, tokens), dn = proj_down(c, tokens);
-        if (!limb_fits(c, up)) return COMET_ERR_SHAPE;
         int rc = join_side(c);
         if (rc != COMET_OK) return rc;
+        if (few_tokens(up)) {
+            rc = stream_product(c, up);
+            return rc != COMET_OK ? rc : somm_merge(c, tokens);
+        }
+        if (!limb_fits(c, up)) return COMET_ERR_SHAPE;
         {
             PhaseTimer timer(c, COMET_PHASE_OPEN, 1);
             rc = limb_open(c, up, true, true, c->stream);
@@ -919,7 +974,6 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
             COMET_CUDA(c, cudaEventRecord(c->ev_join, c->side));
             c->side_pending = true;
             c->dn_right_ready = true;
-            c->dn_right_few = limb_few(dn);
             c->dn_copy_ready = copy;
             c->dn_copy_tokens = tokens;
         }
@@ -992,9 +1046,16 @@ int comet_ffn_down(comet_ctx* c, int32_t tokens) {
     }
     if (c->path == COMET_PATH_LIMB) {
         const Proj dn = proj_down(c, tokens);
+        if (few_tokens(dn)) {
+            const int rc = join_side(c);
+            if (rc != COMET_OK) return rc;
+            c->dn_right_ready = false;
+            c->dn_copy_ready = false;
+            return stream_product(c, dn);
+        }
         if (!limb_fits(c, dn)) return COMET_ERR_SHAPE;
-        // opened early, during the up-projection, and in the plane layout this token count needs
-        const bool have_right = c->dn_right_ready && c->dn_right_few == limb_few(dn);
+        // opened early, during the up-projection
+        const bool have_right = c->dn_right_ready;
         const bool have_copy = c->dn_right_ready && c->dn_copy_ready && c->dn_copy_tokens == tokens;
         int rc = join_side(c);
         if (rc != COMET_OK) return rc;
@@ -1075,16 +1136,6 @@ int comet_get(comet_ctx* c, int party, int tensor_id, uint64_t* out, int locatio
                                     ? c->up_done : c->down_done))
         return COMET_ERR_STATE;
     if (capacity < words) return COMET_ERR_SHAPE;
-    if (words > 0 && (tensor_id == COMET_F_UP || tensor_id == COMET_F_DN) &&
-        c->f_as_planes[tensor_id == COMET_F_DN ? 1 : 0] && c->path == COMET_PATH_LIMB) {
-        // a few-token product wrote this message as limb planes only: rebuild the words
-        uint8_t* (*planes)[2] = tensor_id == COMET_F_DN ? c->planes_right_dn : c->planes_right_up;
-        comet::limb_planes_to_words_kernel<<<ew_grid(c, words, 256), 256, 0, c->stream>>>(
-            planes[party][1], c->buf[party][tensor_id], (int)rows, (int)cols, ceil_div((int)cols, comet::limb::KC),
-            comet::limb_few::BW);
-        c->stats.kernel_launches += 1;
-        COMET_CUDA(c, cudaGetLastError());
-    }
     if (words > 0)
         COMET_CUDA(c, cudaMemcpyAsync(out, c->buf[party][tensor_id], (size_t)words * sizeof(u64),
                                       copy_kind(location, false), c->stream));
@@ -1189,23 +1240,32 @@ namespace {
 static __device__ __align__(256) unsigned long long g_static_scratch[COMET_STATIC_SCRATCH_WORDS];
 
 constexpr int kMaxDevices = 64;
+struct StaticDevice {
+    u64* scratch;      // device address of the array
+    int sm_count;
+};
 std::mutex g_static_mutex;
-u64* g_static_scratch_addr[kMaxDevices] = {};    // device address of the array, per device ordinal
+StaticDevice g_static_device[kMaxDevices] = {};    // per device ordinal
 
-// Device address of the scratch array on the current device (looked up once per device).
-cudaError_t static_scratch_on_current_device(u64** out) {
+// The scratch array on the current device and what launching there needs (looked up once per device).
+cudaError_t static_device(StaticDevice* out) {
     int dev = -1;
     cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(g_static_mutex);
-    if (!g_static_scratch_addr[dev]) {
+    StaticDevice& d = g_static_device[dev];
+    if (!d.scratch) {
         void* p = nullptr;
-        err = cudaGetSymbolAddress(&p, g_static_scratch);
+        err = cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, dev);
+        if (err == cudaSuccess)
+            err = cudaFuncSetAttribute(comet::combine_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)comet::limb_stream::SMEM_BYTES);
+        if (err == cudaSuccess) err = cudaGetSymbolAddress(&p, g_static_scratch);
         if (err != cudaSuccess) return err;
-        g_static_scratch_addr[dev] = static_cast<u64*>(p);
+        d.scratch = static_cast<u64*>(p);
     }
-    *out = g_static_scratch_addr[dev];
+    *out = d;
     return cudaSuccess;
 }
 
@@ -1228,42 +1288,33 @@ extern "C" int comet_beaver_matmul_static(void* cuda_stream, const uint64_t* con
     const int64_t left = (int64_t)T * K, right = (int64_t)N * K;
     if (2 * (left + right) > (int64_t)COMET_STATIC_SCRATCH_WORDS) return COMET_ERR_SCRATCH_LIMIT;
 
-    u64* scratch = nullptr;
-    if (static_scratch_on_current_device(&scratch) != cudaSuccess) {
+    StaticDevice dev;
+    if (static_device(&dev) != cudaSuccess) {
         cudaGetLastError();
         return COMET_ERR_CUDA;
     }
-    cudaStream_t stream = (cudaStream_t)cuda_stream;
-    // carve the array: E_0 | E_1 | F_0 | F_1 (every word used below is written before it is read)
-    u64* E[2] = {scratch, scratch + left};
-    u64* F[2] = {scratch + 2 * left, scratch + 2 * left + right};
-
-    comet::PartyPtrs x, a, y, b;
-    comet::PartyOut e, f;
-    comet::CombineArgs args;
+    // the streaming kernel over [N, K] right operands without a gather; the array is carved into E_0 | E_1 | F_0 | F_1
+    // (every word used is written before anything reads it)
+    comet::StreamArgs a;
+    std::memset(&a, 0, sizeof(a));
+    const u64* c[2];
     for (int p = 0; p < 2; ++p) {
-        x.p[p] = reinterpret_cast<const u64*>(X[p]);
-        a.p[p] = reinterpret_cast<const u64*>(A[p]);
-        y.p[p] = reinterpret_cast<const u64*>(Y[p]);
-        b.p[p] = reinterpret_cast<const u64*>(B[p]);
-        e.p[p] = E[p];
-        f.p[p] = F[p];
-        args.E[p] = E[p];
-        args.F[p] = F[p];
-        args.A[p] = a.p[p];
-        args.B[p] = b.p[p];
-        args.C[p] = reinterpret_cast<const u64*>(C[p]);
-        args.Z[p] = reinterpret_cast<u64*>(Z[p]);
+        a.X[p] = reinterpret_cast<const u64*>(X[p]);
+        a.A[p] = reinterpret_cast<const u64*>(A[p]);
+        a.E[p] = dev.scratch + p * left;
+        a.W0[p] = reinterpret_cast<const u64*>(Y[p]);
+        a.B[p] = reinterpret_cast<const u64*>(B[p]);
+        a.F[p] = dev.scratch + 2 * left + p * right;
+        a.Z[p] = reinterpret_cast<u64*>(Z[p]);
+        c[p] = reinterpret_cast<const u64*>(C[p]);
     }
-    args.M = T; args.N = N; args.K = K;
-    args.tmask = nullptr; args.tmask_ld = 0; args.bs = 1;
-    auto blocks = [](int64_t pairs) { return (unsigned)((pairs + 255) / 256 < 1184 ? (pairs + 255) / 256 : 1184); };
-    comet::open_activation_kernel<<<dim3(blocks(left / 2), 2), 256, 0, stream>>>(x, a, e, left / 2, nullptr, 0, K, 1);
-    comet::open_activation_kernel<<<dim3(blocks(right / 2), 2), 256, 0, stream>>>(y, b, f, right / 2, nullptr, 0, K, 1);
-    dim3 grid((N + comet::simt::BN - 1) / comet::simt::BN, (T + comet::simt::BM - 1) / comet::simt::BM, 2);
-    comet::combine_simt_kernel<<<grid, comet::simt::THREADS, 0, stream>>>(args);
-    if (cudaGetLastError() != cudaSuccess) return COMET_ERR_CUDA;
-    return COMET_OK;
+    a.n = N; a.bs = 1;
+    a.M = T; a.N = N; a.K = K;
+    a.ldw = K;
+    cudaError_t err;
+    const int rc = launch_stream(a, c, dev.sm_count, (cudaStream_t)cuda_stream, nullptr, &err);
+    if (err != cudaSuccess) cudaGetLastError();
+    return rc;
 }
 
 // ---------------------------------------------------------------------------

@@ -113,7 +113,7 @@ __device__ __forceinline__ void limb_copy_wait() { asm volatile("cp.async.wait_g
 
 __device__ __forceinline__ uint8_t* limb_block_ptr(uint8_t* base, int tile_rows, int row, int kblocks, int kb,
                                                    int* rin) {
-    const int tile = row >> (31 - __clz(tile_rows));          // tile_rows is 32, 64 or 128
+    const int tile = row >> (31 - __clz(tile_rows));          // tile_rows is 64 or 128
     *rin = row - tile * tile_rows;
     return base + ((size_t)tile * kblocks + kb) * (size_t)(limb::PLANES * tile_rows * limb::KC);
 }
@@ -149,7 +149,6 @@ struct LimbOpenArgs {
     int ldw;                 // words per row of W
     int kblocks, down;
     int kb_per_cta, kchunks; // k-blocks per right CTA and CTAs per row tile: kchunks = ceil(kblocks / kb_per_cta)
-    int right_tile_rows;     // rows per plane tile of the right operand: 64, or 128 for the few-token kernel
     // Protocol 3 with per-column row sets: per-token mask over the active blocks, [rows of X, tmask_ld] bytes, or
     // null.  Where it is zero the entry of X is no non-zero: it is not opened and E_i is zero there.
     const uint8_t* tmask;
@@ -167,11 +166,6 @@ struct LimbOpenArgs {
     // With kmap (down only): contraction index k of the plane tiles is compact index kmap[k / bs] * bs + k % bs,
     // i.e. the planes run over the active blocks in component order while F_i keeps the compact order.
     const int32_t* kmap;
-    // Few-token products: the party's message F_i is written as blocked limb planes (same layout as Bpl) INSTEAD of
-    // as words: the product kernel reads both parties' messages in that form, so no plane of their sum has to be
-    // built and the words are never needed on the path (limb_planes_to_words_kernel rebuilds them when asked for).
-    uint8_t* Fpl[2];
-    int emit_f;
 };
 
 __global__ void __launch_bounds__(limb::OPEN_THREADS)
@@ -302,46 +296,25 @@ limb_open_kernel(LimbOpenArgs a) {
         int k, ks, kcol;
         bool dead_k;
         column(kb, k, ks, kcol, dead_k);
-        // the message F_i = gather(W_i) - B_i: written as words, or left in place of the W tile for the planes
+        // the message F_i = gather(W_i) - B_i
 #pragma unroll
         for (int i = 0; i < OPEN_ROWS / 8; ++i) {
             const int r = rbase + 8 * i;
             const bool live = s_wrow[r] != nullptr && k < a.K;
             const bool dead = dead_k || s_dead[r] != 0;
-            ulonglong2* wv = reinterpret_cast<ulonglong2*>(w_tile + r * OPEN_STRIDE + 2 * c16);
-            const ulonglong2 w = *wv;
+            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(w_tile + r * OPEN_STRIDE + 2 * c16);
             const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(b_tile + r * OPEN_STRIDE + 2 * c16);
             const ulonglong2 f = dead ? make_ulonglong2(0ull, 0ull) : make_ulonglong2(w.x - b.x, w.y - b.y);
-            if (a.emit_f) *wv = f;
-            else if (live) *reinterpret_cast<ulonglong2*>(Fi + s_orow[r] + ks) = f;
+            if (live) *reinterpret_cast<ulonglong2*>(Fi + s_orow[r] + ks) = f;
         }
-        if (a.emit_f) __syncthreads();       // the planes of F_i are built from words other threads wrote
-        // planes of B_i (threads 0-63) and, with emit_f, of F_i (threads 64-127): 16 words of one row each
-        const int which = tid >> 6, half = (tid >> 5) & 1, r = tid & 31;
-        if (which == 0 || a.emit_f) {
+        // planes of B_i: 16 words of one row per thread
+        if (tid < 2 * OPEN_ROWS) {
+            const int half = tid >> 5, r = tid & 31;
             int rin;
-            uint8_t* blk = limb_block_ptr(which ? (party ? a.Fpl[1] : a.Fpl[0]) : (party ? a.Bpl[1] : a.Bpl[0]),
-                                          a.right_tile_rows, row0 + r, a.kblocks, kb, &rin);
-            limb_emit_planes16((which ? w_tile : b_tile) + r * OPEN_STRIDE + half * 16, half, blk, a.right_tile_rows, rin);
+            uint8_t* blk = limb_block_ptr(party ? a.Bpl[1] : a.Bpl[0], BN, row0 + r, a.kblocks, kb, &rin);
+            limb_emit_planes16(b_tile + r * OPEN_STRIDE + half * 16, half, blk, BN, rin);
         }
         __syncthreads();                     // the stage may be overwritten by the copies issued next round
-    }
-}
-
-// Blocked limb planes back to words: out[row, k] for a [rows, K] operand whose plane tiles have `tile_rows` rows.
-// Only used off the path, when a message that was written as planes is read back as words.
-__global__ void __launch_bounds__(256)
-limb_planes_to_words_kernel(const uint8_t* __restrict__ planes, u64* __restrict__ out, int rows, int K, int kblocks,
-                            int tile_rows) {
-    const long long total = (long long)rows * K, stride = (long long)gridDim.x * blockDim.x;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
-        const int row = (int)(t / K), k = (int)(t - (long long)row * K);
-        const int tile = row / tile_rows, rin = row - tile * tile_rows, kb = k / limb::KC, kin = k - kb * limb::KC;
-        const uint8_t* blk = planes + ((size_t)tile * kblocks + kb) * (size_t)(limb::PLANES * tile_rows * limb::KC);
-        u64 v = 0;
-#pragma unroll
-        for (int p = 0; p < limb::PLANES; ++p) v |= (u64)blk[limb::block_offset(tile_rows, p, rin, kin)] << (8 * p);
-        out[t] = v;
     }
 }
 
@@ -367,7 +340,6 @@ struct LimbPrepArgs {
     uint8_t* Fpl[2];
     int N, right_tiles;      // likewise for the right operand
     int K, kblocks;
-    int left_tile_rows, right_tile_rows;   // rows per plane tile: 128 / 64, or 32 / 128 for the few-token kernel
     const uint8_t* tmask;    // per-token mask over the active blocks (see LimbOpenArgs), or null: where it is zero
     int tmask_ld, bs;        // the party's A_i is no part of the triple and counts as zero
     const u64* C[2];
@@ -498,7 +470,7 @@ limb_prep_kernel(LimbPrepArgs a) {
         // threads 0-63: planes of the summed message; threads 64-127 (left only): planes of V_i; 16 words of a row each
         const int which = tid >> 6, half = (tid >> 5) & 1, r = tid & 31;
         if (which == 0 || left) {
-            const int tile_rows = left ? a.left_tile_rows : a.right_tile_rows;
+            const int tile_rows = left ? BM : BN;
             uint8_t* base = left ? (which ? (party ? a.Vpl[1] : a.Vpl[0]) : (party ? a.Epl[1] : a.Epl[0]))
                                  : (party ? a.Fpl[1] : a.Fpl[0]);
             int rin;
@@ -583,6 +555,10 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* d) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]), "=r"(d[4]), "=r"(d[5]), "=r"(d[6]), "=r"(d[7])
                  : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* d) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]) : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 }  // namespace ptx
@@ -1223,248 +1199,6 @@ combine_limb_kernel(LimbArgs a) {
 __global__ void __launch_bounds__(limb::THREADS, 1)
 combine_limb_grouped_kernel(LimbArgs a) {
     combine_limb_body<true>(a);
-}
-
-// ---------------------------------------------------------------------------
-// Few tokens (M <= 32, the decode step): the roles of the two operands are exchanged.  The weight-side operand
-// (B_i, then F) supplies the 128 rows of the MMA, one limb plane per instruction, and the token-side operand
-// (E, then V_i) is the one whose planes are stacked along N: 32 token rows per plane, so right plane q meets
-// left planes 0..7-q in one instruction of N = 32*(8-q) <= 256, 8 instructions per 32-deep step, and the eight
-// accumulators D_s (128 neurons x 32 tokens) take 256 TMEM columns.  A 128-row tile of the ordinary kernel would
-// spend three quarters of its tensor work on padding rows here.  Every weight plane is used by exactly one tile,
-// so the kernel streams them once; it is bound by that traffic, not by the tensor pipe.  That leaves tensor time
-// to spare, which buys a pass over memory: the second product is taken as V_i*F_0 + V_i*F_1 over the planes of the
-// two messages as the parties wrote them, so no kernel has to read both messages back, add them and write planes
-// of the sum.  A tile thus runs over three operand pairs: (E, B_i), (V_i, F_0), (V_i, F_1).
-// Plane layouts: token side [k-block][8 planes x 32 rows x 32 B] (8 KiB blocks), weight side
-// [n-tile of 128][k-block][32 KiB].  The output tile Z^T (neurons x tokens) is transposed through shared memory
-// so that each bulk reduction adds 32 consecutive neurons of one token row.
-// ---------------------------------------------------------------------------
-namespace limb_few {
-constexpr int BW = 128, BT = 32, KC = limb::KC, PLANES = limb::PLANES;
-constexpr int W_BLOCK_BYTES = PLANES * BW * KC;   // 32 KiB
-constexpr int T_BLOCK_BYTES = PLANES * BT * KC;   // 8 KiB
-constexpr int STAGES = 4;
-constexpr int EPI_WARPS = 8;                      // warp w: neurons 32*(w%4).., tokens 16*(w/4)..
-constexpr int THREADS = 32 * (EPI_WARPS + 2);
-constexpr int OUT_BYTES_PER_WARP = 16 * 32 * 8;   // 16 token rows x 32 neurons
-constexpr int TMEM_COLS = PLANES * BT;            // 256
-constexpr size_t SMEM_BYTES = (size_t)STAGES * (W_BLOCK_BYTES + T_BLOCK_BYTES) + (size_t)EPI_WARPS * OUT_BYTES_PER_WARP + 128;
-}  // namespace limb_few
-
-// LimbArgs as for combine_limb_kernel with Epl/Vpl = token-side planes, Bpl = weight-side planes of the party's
-// B_i, Fpl[0] / Fpl[1] = weight-side planes of the messages F_0 / F_1 (read by both parties), mt = 1,
-// nt = ceil(N / 128), M <= 32.
-constexpr int LIMB_FEW_PAIRS = 3;
-
-// One contiguous piece of a CTA's share: a run of k-blocks of one tile, kpos in [0, 3*kb).
-__device__ __forceinline__ LimbSegment limb_few_segment(const LimbArgs& a, long long u, long long u_end) {
-    const long long tile_units = (long long)LIMB_FEW_PAIRS * a.kb;
-    const long long tile = u / tile_units;
-    long long seg_end = (tile + 1) * tile_units;
-    if (seg_end > u_end) seg_end = u_end;
-    if (seg_end > u + limb::MAX_SEGMENT_UNITS) seg_end = u + limb::MAX_SEGMENT_UNITS;
-    const int per_party = a.mt * a.nt;
-    LimbSegment s;
-    s.party = (int)(tile / per_party);
-    const int t2 = (int)(tile - (long long)s.party * per_party);
-    s.tm = t2 / a.nt;
-    s.tn = t2 - s.tm * a.nt;
-    s.kpos = (int)(u - tile * tile_units);
-    s.count = (int)(seg_end - u);
-    s.kb = a.kb;
-    s.klo = 0;
-    return s;
-}
-
-__global__ void __launch_bounds__(limb_few::THREADS, 1)
-combine_limb_few_kernel(LimbArgs a) {
-    using namespace limb_few;
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[STAGES];
-    __shared__ __align__(8) uint64_t empty_bar[STAGES];
-    __shared__ __align__(8) uint64_t accum_full_bar, accum_empty_bar;
-    __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
-
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
-    uint8_t* sW = smem;
-    uint8_t* sT = smem + (size_t)STAGES * W_BLOCK_BYTES;
-    uint8_t* sOut = sT + (size_t)STAGES * T_BLOCK_BYTES;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long total_units = 2ll * a.mt * a.nt * LIMB_FEW_PAIRS * a.kb;
-    const long long u_begin = total_units * blockIdx.x / gridDim.x;
-    const long long u_end = total_units * (blockIdx.x + 1) / gridDim.x;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            ptx::mbar_init(ptx::smem_u32(&full_bar[s]), 1);
-            ptx::mbar_init(ptx::smem_u32(&empty_bar[s]), 1);
-        }
-        ptx::mbar_init(ptx::smem_u32(&accum_full_bar), 1);
-        ptx::mbar_init(ptx::smem_u32(&accum_empty_bar), 32 * EPI_WARPS);
-        abort_flag = 0;
-        ptx::fence_barrier_init();
-    }
-    if (warp == 0) {
-        ptx::tmem_alloc(ptx::smem_u32(&tmem_slot), TMEM_COLS);
-        ptx::tmem_relinquish();
-    }
-    ptx::fence_before_sync();
-    __syncthreads();
-    ptx::fence_after_sync();
-    const uint32_t tmem_base = tmem_slot;
-    // barriers and tensor memory are set up; from here on the kernel touches what its predecessors wrote
-    pdl_wait();
-
-    if (warp == EPI_WARPS) {
-        // ---------------- producer: one bulk copy per operand block ----------------
-        if (lane == 0) {
-            int stage = 0;
-            uint32_t phase = 0;
-            int issued = 0;
-            bool ok = true;
-            const uint32_t full0 = ptx::smem_u32(&full_bar[0]), empty0 = ptx::smem_u32(&empty_bar[0]);
-            const uint32_t sW0 = ptx::smem_u32(sW), sT0 = ptx::smem_u32(sT);
-            for (long long u = u_begin; u < u_end && ok;) {
-                const LimbSegment sg = limb_few_segment(a, u, u_end);
-                u += sg.count;
-                int pair = sg.kpos / a.kb;                    // 0: (E, B_i), 1: (V_i, F_0), 2: (V_i, F_1)
-                int kpos = sg.kpos - pair * a.kb;
-                const uint8_t* tok_e = sg.party ? a.Epl[1] : a.Epl[0];
-                const uint8_t* tok_v = sg.party ? a.Vpl[1] : a.Vpl[0];
-                const size_t tile_off = (size_t)sg.tn * a.kb * W_BLOCK_BYTES;
-                const uint8_t* wgt_b = (sg.party ? a.Bpl[1] : a.Bpl[0]) + tile_off;
-                const uint8_t* tok = (pair == 0 ? tok_e : tok_v) + (size_t)kpos * T_BLOCK_BYTES;
-                const uint8_t* wgt = (pair == 0 ? wgt_b : (pair == 1 ? a.Fpl[0] : a.Fpl[1]) + tile_off) +
-                                     (size_t)kpos * W_BLOCK_BYTES;
-                for (int it = 0; it < sg.count; ++it) {
-                    ok = limb_wait(empty0 + 8 * stage, phase ^ 1u, &abort_flag);
-                    if (!ok) break;
-                    const uint32_t bar = full0 + 8 * stage;
-                    ptx::mbar_expect_tx(bar, W_BLOCK_BYTES + T_BLOCK_BYTES);
-                    ptx::bulk_g2s(sW0 + stage * W_BLOCK_BYTES, wgt, W_BLOCK_BYTES, bar);
-                    ptx::bulk_g2s(sT0 + stage * T_BLOCK_BYTES, tok, T_BLOCK_BYTES, bar);
-                    ++issued;
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-                    tok += T_BLOCK_BYTES;
-                    wgt += W_BLOCK_BYTES;
-                    if (++kpos == a.kb && pair < LIMB_FEW_PAIRS - 1) {
-                        ++pair;                               // on to V_i with the next message
-                        kpos = 0;
-                        tok = tok_v;
-                        wgt = (pair == 1 ? a.Fpl[0] : a.Fpl[1]) + tile_off;
-                    }
-                }
-            }
-            if (!ok) {
-                const int back = issued < STAGES ? issued : STAGES;
-                for (int j = 1; j <= back; ++j) {
-                    int s = stage - j;
-                    uint32_t ph = phase;
-                    if (s < 0) { s += STAGES; ph ^= 1u; }
-                    const long long t0 = clock64();
-                    while (!ptx::mbar_try_wait(ptx::smem_u32(&full_bar[s]), ph) && clock64() - t0 < 20000000ll) {}
-                }
-            }
-        }
-    } else if (warp == EPI_WARPS + 1) {
-        // ---------------- MMA issuer: weight plane q against token planes 0..7-q ----------------
-        if (lane == 0) {
-            constexpr uint32_t IDESC = (2u << 4) | ((uint32_t)(BW >> 4) << 24);
-            const uint32_t full0 = ptx::smem_u32(&full_bar[0]), empty0 = ptx::smem_u32(&empty_bar[0]);
-            const uint32_t accum_full = ptx::smem_u32(&accum_full_bar), accum_empty = ptx::smem_u32(&accum_empty_bar);
-            const uint32_t w_lo0 = limb_desc_lo(ptx::smem_u32(sW)), t_lo0 = limb_desc_lo(ptx::smem_u32(sT));
-            int stage = 0;
-            uint32_t phase = 0, acc_phase = 0;
-            bool ok = true;
-            for (long long u = u_begin; u < u_end && ok;) {
-                const LimbSegment sg = limb_few_segment(a, u, u_end);
-                u += sg.count;
-                ok = limb_wait(accum_empty, acc_phase ^ 1u, &abort_flag);
-                if (!ok) break;
-                ptx::fence_after_sync();
-                uint32_t acc = 0;
-                for (int it = 0; it < sg.count; ++it) {
-                    ok = limb_wait(full0 + 8 * stage, phase, &abort_flag);
-                    if (!ok) break;
-                    ptx::fence_after_sync();
-                    const uint32_t w_lo = w_lo0 + stage * (W_BLOCK_BYTES >> 4);
-                    const uint32_t t_lo = t_lo0 + stage * (T_BLOCK_BYTES >> 4);
-#pragma unroll
-                    for (int q = 0; q < PLANES; ++q)
-                        ptx::mma_i8(tmem_base + BT * q, w_lo + ((q * BW * KC) >> 4), LIMB_DESC_HI, t_lo, LIMB_DESC_HI,
-                                    IDESC | ((uint32_t)((BT * (PLANES - q)) >> 3) << 17), q == 0 ? acc : 1u);
-                    ptx::mma_commit(empty0 + 8 * stage);
-                    acc = 1u;
-                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-                }
-                if (!ok) break;
-                ptx::mma_commit(accum_full);
-                acc_phase ^= 1u;
-            }
-            // the main loop is over: the next kernel of the stream may be brought in beside the last drain
-            pdl_launch_dependents();
-        }
-    } else {
-        // ---------------- epilogue: lane = neuron, registers = tokens; transpose through shared memory ----------------
-        uint32_t acc_phase = 0;
-        bool ok = true;
-        const int quarter = warp & 3, thalf = warp >> 2;
-        const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16) + thalf * 16;
-        u64* stage_out = reinterpret_cast<u64*>(sOut + (size_t)warp * OUT_BYTES_PER_WARP);   // [16 tokens][32 neurons]
-        for (long long u = u_begin; u < u_end && ok;) {
-            const LimbSegment sg = limb_few_segment(a, u, u_end);
-            u += sg.count;
-            ok = limb_wait_warp(ptx::smem_u32(&accum_full_bar), acc_phase, &abort_flag);
-            if (!ok) break;
-            ptx::fence_after_sync();
-            u64 z[16];
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t d[PLANES][8];
-#pragma unroll
-                for (int s = 0; s < PLANES; ++s) ptx::tmem_ld8(lane_base + BT * s + c * 8, d[s]);
-                ptx::tmem_wait_ld();
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    z[c * 8 + j] = limb_recombine(d[0][j], d[1][j], d[2][j], d[3][j], d[4][j], d[5][j], d[6][j], d[7][j]);
-            }
-            ptx::fence_before_sync();
-            ptx::mbar_arrive(ptx::smem_u32(&accum_empty_bar));
-            if (lane < 16) ptx::bulk_wait_group_read0();       // this lane's previous reduction has read its row
-            __syncwarp();
-#pragma unroll
-            for (int t = 0; t < 16; ++t) stage_out[t * 32 + lane] = z[t];
-            ptx::fence_proxy_async_smem();
-            __syncwarp();
-            const int token = thalf * 16 + lane;               // lanes 0..15 each own one token row of the piece
-            const int col0 = sg.tn * BW + quarter * 32;
-            int cols = a.N - col0;
-            if (cols > 32) cols = 32;
-            if (lane < 16) {
-                if (token < a.M && cols > 0)
-                    ptx::bulk_reduce_add_u64((sg.party ? a.Z[1] : a.Z[0]) + (size_t)token * a.N + col0,
-                                             ptx::smem_u32(stage_out + lane * 32), (uint32_t)cols * 8u);
-                ptx::bulk_commit_group();
-            }
-            acc_phase ^= 1u;
-        }
-        if (lane < 16) ptx::bulk_wait_group0();
-    }
-
-    ptx::fence_before_sync();
-    __syncthreads();
-    if (threadIdx.x == 0 && abort_flag) {
-        *a.error_flag = 1;
-        *reinterpret_cast<volatile int*>(a.error_host) = 1;
-        __threadfence_system();
-    }
-    if (warp == 0) {
-        ptx::fence_after_sync();
-        ptx::tmem_dealloc(tmem_base, limb_few::TMEM_COLS);
-    }
 }
 
 }  // namespace comet

@@ -1,0 +1,512 @@
+// One Pi_MatMul for few token rows (the decode step) in one kernel: mask, exchange and combine without a pass over
+// memory in between.
+//   before the exchange   E_i = X_i - A_i,  F_i = gather(W_i) - B_i          (Section 2.1 "Multiplication", the gathers
+//                                                                             of Protocols 2 and 3), written as messages
+//   the exchange          E = E_0 + E_1,  F = F_0 + F_1
+//   after it              Z_i += E*B_i + V_i*F,  V_i = A_i + i*E              (Eq. 1; Z_i holds C_i when it starts)
+//
+// What bounds it: with at most 32 token rows a weight word takes part in 2 * 32 multiply-adds per party, so the kernel
+// is bound by streaming the weight side.  Per word of the right operand and party that is W_i and B_i in and F_i out,
+// 24 bytes, and this kernel moves nothing else of that size: the limb planes the tensor cores read exist in shared
+// memory only.  (Its predecessor wrote the planes of B_i and F_i to memory and read them back: 56 bytes per word.)
+// Measured, both parties: [32, 4096] x [4096, 1312] 66 us and [7, 4096] x [4096, 3328] 114 us, where 24 bytes per weight
+// word at the measured copy rate are 39 and 100 us (100 + 43 and 135 + 82 us before); a step of 192 KiB takes 8300 cycles,
+// 90 % of that rate, the rest is the first step's latency and the last drain.
+//
+// A CTA carries both parties' share of a tile of 128 output features (the rows of the MMA) x 32 tokens, and walks it in
+// steps of 32 contraction indices.  What is computed for a party depends on that party's shares and on the two messages
+// alone; both parties' words of one place pass through the same thread, which is the exchange.
+//   warps 16-17   raw producers, one per party: 16-byte asynchronous copies of W_i, B_i (32 rows x 32 words of each per
+//                 slot) into a ring of three 32 KiB slots
+//   warps 0-15    converters, two groups of eight that take the four slots of a step in turn: words -> messages F_0, F_1
+//                 (to memory) and their sum -> limb planes of B_0, B_1, F
+//   warps 18-25   the token side, four rows each: X_i, A_i straight from L2, a step ahead -> messages E_0, E_1 -> limb
+//                 planes of E, A_0, A_1 + E; at the end of a segment the same warps are the epilogue (four per party): TMEM
+//                 -> recombine mod 2^64 -> rows staged in shared memory -> bulk add-reductions into Z
+//   warp 26       issues the MMAs: F is the same for both parties, so three weight-side plane sets serve four products
+// Shared memory: 96 KiB weight planes, 24 KiB token planes, 96 KiB raw ring, 8 KiB result rows; all 512 TMEM columns (two
+// parties x eight accumulators x 32 tokens).  The planes are single-buffered: converting a step and multiplying it take
+// turns, while the ring and the converters' registers keep up to 160 KiB of loads in flight.
+//
+// Inside a 32-deep step the contraction indices sit in the planes in the order the converters hold them: a lane reads
+// two 16-byte pieces of a row, 16 words apart, so that eight lanes read whole 128-byte lines, and writes its four
+// words' bytes next to each other.  Both operands use that order, so the sum over the step is the same.
+//
+// Work is cut stream-K style like the other tensor-core kernel's: the (feature tile, token tile, step) space in equal
+// contiguous ranges, a step weighted by the number of raw slots it takes (a ragged last tile takes fewer).
+#pragma once
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "kernels_limb.cuh"
+#include "pdl.cuh"
+
+namespace comet {
+
+namespace limb_stream {
+constexpr int BW = 128, BT = 32, KC = limb::KC, PLANES = limb::PLANES, QROWS = 32, QUARTERS = BW / QROWS;
+constexpr int CONV_GROUPS = 2, GROUP_WARPS = 8, CONV_WARPS = CONV_GROUPS * GROUP_WARPS;
+constexpr int RAW_WARP0 = CONV_WARPS, TOK_WARP0 = RAW_WARP0 + 2, TOK_WARPS = 8, MMA_WARP = TOK_WARP0 + TOK_WARPS;
+constexpr int EPI_WARPS = TOK_WARPS / 2;                 // per party
+constexpr int THREADS = 32 * (MMA_WARP + 1);
+constexpr int RAW_ARRAY_BYTES = QROWS * KC * 8;          // 8 KiB: one array of a slot
+constexpr int RAW_SLOT_BYTES = 4 * RAW_ARRAY_BYTES;      // party 0: W | B, party 1: W | B
+constexpr int RAW_SLOTS = 3;
+constexpr int W_PLANE_BYTES = BW * KC, T_PLANE_BYTES = BT * KC;
+constexpr int W_SET_BYTES = PLANES * W_PLANE_BYTES;      // 32 KiB: limb planes of B_0, B_1 or F
+constexpr int T_SET_BYTES = PLANES * T_PLANE_BYTES;      //  8 KiB: limb planes of V_0, V_1 or E
+constexpr int OUT_TOKENS = 4;                            // tokens an epilogue thread recombines at a time
+constexpr int OUT_BYTES = OUT_TOKENS * 32 * 8;           // an epilogue warp's staging buffer: a row of 32 features per token
+constexpr int ACC_COLS = PLANES * BT;                    // 256 TMEM columns per party
+// A step adds two products to an accumulator, so the bound on a segment's depth (16384 contraction indices keep the
+// limb sums for s <= 3 below 2^32) allows half as many steps.
+constexpr int MAX_SEGMENT_STEPS = limb::MAX_SEGMENT_UNITS / 2;
+constexpr size_t SMEM_BYTES = 3 * (size_t)W_SET_BYTES + 3 * (size_t)T_SET_BYTES + (size_t)RAW_SLOTS * RAW_SLOT_BYTES +
+                              (size_t)TOK_WARPS * OUT_BYTES + 128;
+}  // namespace limb_stream
+
+struct StreamArgs {
+    const u64* X[2]; const u64* A[2];                     // token side, [M, K]
+    u64* E[2];                                            // message, [M, K]
+    const u64* W0[2]; const u64* W1[2]; const u64* W2[2]; // weights of the stacked groups (down: W0 alone)
+    const u64* B[2];                                      // [N, K]
+    u64* F[2];                                            // message, [N, K]
+    u64* Z[2];                                            // [M, N], holds C_i; written by the kernel before this one
+    const int32_t* ids;      // ascending active block ids; null: the right operand is W0 itself, [N, K], no gather
+    int n, bs;               // active neurons, neurons per block (a multiple of 16 when there are ids)
+    int M, N, K;             // K a multiple of 8
+    int ldw, down;           // words per row of W; gather rows (up) or strips of bs words of every row (down)
+    int mt, nt, kb;          // token tiles, feature tiles, steps per tile
+    // how the steps are dealt out: a step costs the raw slots it takes, and one more for what does not depend on them
+    int last_cost;           // of a step of the last, possibly ragged, feature tile
+    unsigned cta_cost, cta_extra;   // total cost = gridDim.x * cta_cost + cta_extra, cta_extra < gridDim.x
+    const uint8_t* tmask;    // per-token mask [M, tmask_ld] over the active blocks of the contraction index, or null:
+    int tmask_ld;            // where it is zero, neither X nor A_i has an entry
+    const int32_t* row_label;   // component label per token (negative: the row is not opened), or null
+    const int32_t* blk_label;   // likewise per active block (up: rows of the right operand, down: its columns), or null
+    int* error_flag;
+    int* error_host;
+};
+
+// Z_i <- C_i for both parties, so that the product kernel behind it can add partial sums.
+__global__ void __launch_bounds__(256)
+result_init_kernel(const u64* __restrict__ c0, const u64* __restrict__ c1, u64* __restrict__ z0, u64* __restrict__ z1,
+                   long long pairs) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const ulonglong2* __restrict__ s = reinterpret_cast<const ulonglong2*>(blockIdx.y ? c1 : c0);
+    ulonglong2* __restrict__ d = reinterpret_cast<ulonglong2*>(blockIdx.y ? z1 : z0);
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < pairs; t += stride) d[t] = __ldcs(s + t);
+}
+
+// A run of steps of one tile, at most MAX_SEGMENT_STEPS of them.
+struct StreamSegment {
+    int tm, tn, step, count;
+};
+
+__device__ __forceinline__ StreamSegment stream_segment(const StreamArgs& a, unsigned u, unsigned u_end) {
+    StreamSegment s;
+    const unsigned tile = u / (unsigned)a.kb;
+    s.step = (int)(u - tile * a.kb);
+    s.tn = a.mt == 1 ? (int)tile : (int)(tile / (unsigned)a.mt);
+    s.tm = (int)tile - s.tn * a.mt;
+    s.count = min(min(a.kb - s.step, (int)(u_end - u)), limb_stream::MAX_SEGMENT_STEPS);
+    return s;
+}
+
+// Raw slots the weight side of a feature tile takes per step.
+__device__ __forceinline__ int stream_quarters(const StreamArgs& a, int tn) {
+    return tn + 1 < a.nt ? limb_stream::QUARTERS : a.last_cost - 1;
+}
+
+// First step of the range that begins at cost b * cta_cost + min(b, cta_extra).
+__device__ __forceinline__ unsigned stream_cut(const StreamArgs& a, unsigned b) {
+    constexpr unsigned FULL = limb_stream::QUARTERS + 1;
+    const unsigned cost = b * a.cta_cost + min(b, a.cta_extra);
+    const unsigned whole = (unsigned)a.kb * (unsigned)a.mt * (unsigned)(a.nt - 1);     // steps of full feature tiles
+    return cost < FULL * whole ? cost / FULL : whole + (cost - FULL * whole) / (unsigned)a.last_cost;
+}
+
+// 16-byte asynchronous copy global -> shared that bypasses L1, and this thread's arrival on `bar` once all its copies so
+// far have landed.
+__device__ __forceinline__ void stream_copy16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void stream_copies_arrive(uint32_t bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// Four words of one row -> eight planes, four bytes each, `stride` bytes apart.
+__device__ __forceinline__ void stream_emit4(uint8_t* dst, int stride, const u64* w) {
+    uint32_t p[8];
+    limb_transpose4((uint32_t)w[0], (uint32_t)w[1], (uint32_t)w[2], (uint32_t)w[3], p[0], p[1], p[2], p[3]);
+    limb_transpose4((uint32_t)(w[0] >> 32), (uint32_t)(w[1] >> 32), (uint32_t)(w[2] >> 32), (uint32_t)(w[3] >> 32),
+                    p[4], p[5], p[6], p[7]);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) *reinterpret_cast<uint32_t*>(dst + i * stride) = p[i];
+}
+
+__global__ void __launch_bounds__(limb_stream::THREADS, 1)
+combine_stream_kernel(const __grid_constant__ StreamArgs a) {
+    using namespace limb_stream;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t raw_full[RAW_SLOTS], raw_empty[RAW_SLOTS];
+    __shared__ __align__(8) uint64_t planes_full, own_empty[2], shared_empty;     // own: B_0 / B_1; shared: F, E, V_i
+    __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
+    uint8_t* sB = smem;                                   // planes of B_0, B_1, F
+    uint8_t* sV = sB + 3 * W_SET_BYTES;                   // planes of V_0, V_1, E
+    uint8_t* sRaw = sV + 3 * T_SET_BYTES;
+    uint8_t* sOut = sRaw + RAW_SLOTS * RAW_SLOT_BYTES;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned u_begin = stream_cut(a, blockIdx.x), u_end = stream_cut(a, blockIdx.x + 1);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < RAW_SLOTS; ++s) {
+            ptx::mbar_init(ptx::smem_u32(&raw_full[s]), 64);                // every producer lane
+            ptx::mbar_init(ptx::smem_u32(&raw_empty[s]), GROUP_WARPS);
+        }
+        ptx::mbar_init(ptx::smem_u32(&planes_full), CONV_WARPS + TOK_WARPS);
+        ptx::mbar_init(ptx::smem_u32(&shared_empty), 1);
+        for (int p = 0; p < 2; ++p) {
+            ptx::mbar_init(ptx::smem_u32(&own_empty[p]), 1);
+            ptx::mbar_init(ptx::smem_u32(&acc_full[p]), 1);
+            ptx::mbar_init(ptx::smem_u32(&acc_empty[p]), EPI_WARPS);
+        }
+        abort_flag = 0;
+        ptx::fence_barrier_init();
+    }
+    if (warp == MMA_WARP) {
+        ptx::tmem_alloc(ptx::smem_u32(&tmem_slot), 2 * ACC_COLS);
+        ptx::tmem_relinquish();
+    }
+    ptx::fence_before_sync();
+    __syncthreads();
+    ptx::fence_after_sync();
+    const uint32_t tmem_base = tmem_slot;
+    // No wait for the predecessor here: it is the kernel that initialises Z, which only the epilogue touches.  That
+    // kernel let this one start after its own wait, so whatever came before it has completed.
+
+    if (warp >= RAW_WARP0 && warp < RAW_WARP0 + 2) {
+        // ---------------- raw producer of one party: 16 lanes per row of a slot ----------------
+        const int party = warp - RAW_WARP0, half = (lane >> 3) & 1, piece = lane & 15, rsub = lane >> 4;
+        const uint32_t raw0 = ptx::smem_u32(sRaw) + party * 2 * RAW_ARRAY_BYTES + lane * 16;
+        const u64* __restrict__ W0 = party ? a.W0[1] : a.W0[0];
+        const u64* __restrict__ Bi = party ? a.B[1] : a.B[0];
+        int slot = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        for (unsigned u = u_begin; u < u_end && ok;) {
+            const StreamSegment sg = stream_segment(a, u, u_end);
+            u += sg.count;
+            const int quarters = stream_quarters(a, sg.tn);
+            // Sixteen rows aligned to 16 lie in one block (block sizes are multiples of 16), so they are `ldw` apart in W:
+            // lane h of a warp's first eight knows where rows 16h .. 16h+15 of the tile begin
+            const u64* w_row16 = W0;
+            {
+                const int row = sg.tn * BW + (lane & 7) * 16;
+                if (row < a.N) {
+                    if (a.ids == nullptr || a.down) {
+                        w_row16 = W0 + (size_t)row * a.ldw;
+                    } else {
+                        const int grp = (row >= a.n) + (row >= 2 * a.n), j = row - grp * a.n, blk = j / a.bs;
+                        w_row16 = (grp == 0 ? W0 : grp == 1 ? (party ? a.W1[1] : a.W1[0]) : (party ? a.W2[1] : a.W2[0])) +
+                                  (size_t)(__ldg(a.ids + blk) * a.bs + (j - blk * a.bs)) * a.ldw;
+                    }
+                }
+            }
+            for (int it = 0; it < sg.count && ok; ++it) {
+                const int k = (sg.step + it) * KC + 2 * piece;
+                const bool kv = k < a.K;
+                int col = k;                                      // this lane's column of W
+                if (a.down && a.ids != nullptr && kv) {
+                    const int blk = ((sg.step + it) * KC + 16 * half) / a.bs;
+                    col = __ldg(a.ids + blk) * a.bs + (k - blk * a.bs);
+                }
+                for (int q = 0; q < quarters; ++q) {
+                    const int row0 = sg.tn * BW + q * QROWS + rsub;
+                    const int rows = kv ? a.N - row0 : 0;                          // this lane's rows: row0 + 2i, 2i < rows
+                    const u64* right = Bi + (size_t)row0 * a.K + k;
+                    const u64* left[2];                                            // rows 0-15 and 16-31 of the slot
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        left[h] = reinterpret_cast<const u64*>(
+                                      __shfl_sync(0xffffffffu, (unsigned long long)w_row16, 2 * q + h)) +
+                                  (size_t)rsub * a.ldw + col;
+                    const size_t left_step = 2 * (size_t)a.ldw, right_step = 2 * (size_t)a.K;
+                    ok = limb_wait(ptx::smem_u32(&raw_empty[slot]), phase ^ 1u, &abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    const uint32_t dst = raw0 + slot * RAW_SLOT_BYTES;
+#pragma unroll
+                    for (int i = 0; i < QROWS / 2; ++i) {
+                        if (2 * i < rows) {
+                            stream_copy16(dst + i * 512, left[i / 8] + (i % 8) * left_step);
+                            stream_copy16(dst + RAW_ARRAY_BYTES + i * 512, right + i * right_step);
+                        }
+                    }
+                    stream_copies_arrive(ptx::smem_u32(&raw_full[slot]));
+                    if (++slot == RAW_SLOTS) { slot = 0; phase ^= 1u; }
+                }
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");          // no copy outlives the CTA, whatever ended the loop
+    } else if (warp < CONV_WARPS) {
+        // ---------------- converters ----------------
+        const int group = warp / GROUP_WARPS, c = lane & 7;
+        // this lane's row of a slot, and of it the words 2c, 2c+1, 16+2c, 17+2c.  Lanes c >= 4 take the row four further,
+        // which keeps the plane stores free of bank conflicts.
+        const int r = 4 * (2 * ((warp & 7) >> 1) + ((warp & 1) ^ (c >> 2))) + (lane >> 3);
+        const uint8_t* raw_lane = sRaw + r * (KC * 8) + c * 16;
+        const int cell = (r >> 3) * 256 + (c >> 2) * 128 + (r & 7) * 16 + (c & 3) * 4;
+        int slot = 0;
+        uint32_t phase = 0, unit_phase = 0;
+        bool ok = true;
+        for (unsigned u = u_begin; u < u_end && ok;) {
+            const StreamSegment sg = stream_segment(a, u, u_end);
+            u += sg.count;
+            const int quarters = stream_quarters(a, sg.tn);
+            for (int it = 0; it < sg.count && ok; ++it) {
+                const int k0 = (sg.step + it) * KC;
+                const bool kv[2] = {k0 + 2 * c < a.K, k0 + 16 + 2 * c < a.K};
+                bool first = true;
+                for (int q = 0; q < quarters; ++q) {
+                    const int my_slot = slot;
+                    const uint32_t my_phase = phase;
+                    if (++slot == RAW_SLOTS) { slot = 0; phase ^= 1u; }
+                    if (q % CONV_GROUPS != group) continue;
+                    ok = limb_wait(ptx::smem_u32(&raw_full[my_slot]), my_phase, &abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    const uint8_t* raw = raw_lane + my_slot * RAW_SLOT_BYTES;
+                    u64 f[2][4], b[2][4];                            // per party: W_i, then the message F_i; B_i
+#pragma unroll
+                    for (int p = 0; p < 2; ++p)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const ulonglong2 w =
+                                *reinterpret_cast<const ulonglong2*>(raw + 2 * p * RAW_ARRAY_BYTES + h * 128);
+                            const ulonglong2 v =
+                                *reinterpret_cast<const ulonglong2*>(raw + (2 * p + 1) * RAW_ARRAY_BYTES + h * 128);
+                            f[p][2 * h] = w.x;
+                            f[p][2 * h + 1] = w.y;
+                            b[p][2 * h] = v.x;
+                            b[p][2 * h + 1] = v.y;
+                        }
+                    __syncwarp();                                    // the slot has been read
+                    if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&raw_empty[my_slot]));
+#pragma unroll
+                    for (int p = 0; p < 2; ++p)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) f[p][e] -= b[p][e];
+                    const int row = sg.tn * BW + q * QROWS + r;
+                    const bool live = row < a.N;
+                    if (a.blk_label && live) {                       // rows / columns outside every component stay closed
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            if (a.down ? (kv[h] && a.blk_label[(k0 + 16 * h) / a.bs] < 0)
+                                       : a.blk_label[(row % a.n) / a.bs] < 0)
+#pragma unroll
+                                for (int p = 0; p < 2; ++p) f[p][2 * h] = f[p][2 * h + 1] = 0ull;
+                    }
+                    if (live && sg.tm == 0) {                        // the messages
+                        const size_t at = (size_t)row * a.K + k0 + 2 * c;
+#pragma unroll
+                        for (int p = 0; p < 2; ++p) {
+                            if (kv[0]) __stcs(reinterpret_cast<ulonglong2*>(a.F[p] + at), make_ulonglong2(f[p][0], f[p][1]));
+                            if (kv[1]) __stcs(reinterpret_cast<ulonglong2*>(a.F[p] + at + 16), make_ulonglong2(f[p][2], f[p][3]));
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) f[0][e] += f[1][e];  // the exchange
+                    uint8_t* to = sB + q * (QROWS / 8) * 256 + cell;
+                    // a step's first planes: the MMAs of the step before must have read the old ones
+                    if (first) ok = limb_wait(ptx::smem_u32(&own_empty[0]), unit_phase ^ 1u, &abort_flag);
+                    stream_emit4(to, W_PLANE_BYTES, b[0]);
+                    if (first) ok = ok && limb_wait(ptx::smem_u32(&own_empty[1]), unit_phase ^ 1u, &abort_flag);
+                    stream_emit4(to + W_SET_BYTES, W_PLANE_BYTES, b[1]);
+                    if (first) ok = ok && limb_wait(ptx::smem_u32(&shared_empty), unit_phase ^ 1u, &abort_flag);
+                    stream_emit4(to + 2 * W_SET_BYTES, W_PLANE_BYTES, f[0]);
+                    first = false;
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                }
+                // a ragged tile may leave a group without a slot: it must not arrive for a step before the last one is over
+                if (ok && first) ok = __all_sync(0xffffffffu, limb_wait(ptx::smem_u32(&shared_empty), unit_phase ^ 1u, &abort_flag));
+                if (!ok) break;
+                ptx::fence_proxy_async_smem();                           // the planes are read by the tensor cores
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&planes_full));
+                unit_phase ^= 1u;
+            }
+        }
+    } else if (warp < MMA_WARP) {
+        // ---------------- token side: the converters' cells, straight from L2 ----------------
+        const int c = lane & 7, r = (4 * (warp - TOK_WARP0) ^ (c >= 4 ? 4 : 0)) + (lane >> 3);
+        uint8_t* to = sV + (r >> 3) * 256 + (c >> 2) * 128 + (r & 7) * 16 + (c & 3) * 4;
+        const int party = (warp - TOK_WARP0) / EPI_WARPS, quarter = warp & 3;     // epilogue: TMEM lanes this warp may read
+        u64* out = reinterpret_cast<u64*>(sOut + (size_t)(warp - TOK_WARP0) * OUT_BYTES);
+        uint32_t unit_phase = 0, seg_phase = 0;
+        bool ok = true, z_ready = false;
+        for (unsigned u = u_begin; u < u_end && ok;) {
+            const StreamSegment sg = stream_segment(a, u, u_end);
+            u += sg.count;
+            const int row = sg.tm * BT + r;
+            const bool live = row < a.M, closed = live && a.row_label && a.row_label[row] < 0;
+            for (int it = 0; it < sg.count; ++it) {
+                const int k0 = (sg.step + it) * KC;
+                u64 e[2][4], v[2][4];                            // X_i, then the message E_i; A_i, then V_i
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    // indices past the operand's depth and entries off the support are zero in E and in A_i
+                    const int k = k0 + 16 * h + 2 * c;
+                    bool has = live && k < a.K;
+                    if (has && a.tmask) has = a.tmask[(size_t)row * a.tmask_ld + (k0 + 16 * h) / a.bs] != 0;
+                    const size_t at = (size_t)row * a.K + k;
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) {
+                        ulonglong2 x = make_ulonglong2(0ull, 0ull), m = x;
+                        if (has) {
+                            m = __ldg(reinterpret_cast<const ulonglong2*>(a.A[p] + at));
+                            x = __ldg(reinterpret_cast<const ulonglong2*>(a.X[p] + at));
+                        }
+                        e[p][2 * h] = x.x;
+                        e[p][2 * h + 1] = x.y;
+                        v[p][2 * h] = m.x;
+                        v[p][2 * h + 1] = m.y;
+                    }
+                }
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) e[p][i] = closed ? 0ull : e[p][i] - v[p][i];
+                    if (live && sg.tn == 0) {                    // the message
+                        u64* out = a.E[p] + (size_t)row * a.K + k0 + 2 * c;
+                        if (k0 + 2 * c < a.K) *reinterpret_cast<ulonglong2*>(out) = make_ulonglong2(e[p][0], e[p][1]);
+                        if (k0 + 16 + 2 * c < a.K) *reinterpret_cast<ulonglong2*>(out + 16) = make_ulonglong2(e[p][2], e[p][3]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    e[0][i] += e[1][i];                          // the exchange
+                    v[1][i] += e[0][i];                          // V_1 = A_1 + E  (V_0 = A_0)
+                }
+                ok = limb_wait(ptx::smem_u32(&shared_empty), unit_phase ^ 1u, &abort_flag);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (live) {                                      // planes of rows past the last token are never looked at
+                    stream_emit4(to, T_PLANE_BYTES, v[0]);
+                    stream_emit4(to + T_SET_BYTES, T_PLANE_BYTES, v[1]);
+                    stream_emit4(to + 2 * T_SET_BYTES, T_PLANE_BYTES, e[0]);
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&planes_full));
+                unit_phase ^= 1u;
+            }
+            if (!ok) break;
+            // ---------------- epilogue of the segment: lane = output feature, registers = tokens ----------------
+            // Result rows go through shared memory: lane t < OUT_TOKENS owns row t of the buffer and adds it into Z with one
+            // bulk reduction.  (64-bit atomics from registers took twice as long.)
+            if (!z_ready) pdl_wait();                            // Z holds C_i
+            z_ready = true;
+            ok = limb_wait_warp(ptx::smem_u32(&acc_full[party]), seg_phase, &abort_flag);
+            if (!ok) break;
+            ptx::fence_after_sync();
+            const int col0 = sg.tn * BW + quarter * 32, cols = min(a.N - col0, 32), tokens = min(a.M - sg.tm * BT, BT);
+            const uint32_t acc = tmem_base + party * ACC_COLS + ((uint32_t)(quarter * 32) << 16);
+            u64* z = (party ? a.Z[1] : a.Z[0]) + (size_t)(sg.tm * BT + lane) * a.N + col0;
+#pragma unroll 1
+            for (int t0 = 0; t0 < tokens; t0 += OUT_TOKENS) {
+                uint32_t d[PLANES][OUT_TOKENS];
+#pragma unroll
+                for (int s = 0; s < PLANES; ++s) ptx::tmem_ld4(acc + BT * s + t0, d[s]);
+                ptx::tmem_wait_ld();
+                if (lane < OUT_TOKENS) ptx::bulk_wait_group_read0();     // the last reduction has read its row
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < OUT_TOKENS; ++j)
+                    out[j * 32 + lane] = limb_recombine(d[0][j], d[1][j], d[2][j], d[3][j], d[4][j], d[5][j], d[6][j], d[7][j]);
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane < OUT_TOKENS) {
+                    if (t0 + lane < tokens && cols > 0)
+                        ptx::bulk_reduce_add_u64(z + (size_t)t0 * a.N, ptx::smem_u32(out + lane * 32), (uint32_t)cols * 8u);
+                    ptx::bulk_commit_group();
+                }
+            }
+            ptx::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&acc_empty[party]));
+            seg_phase ^= 1u;
+        }
+        if (!z_ready) pdl_wait();                                // every CTA waits for its predecessor once
+        if (lane < OUT_TOKENS) ptx::bulk_wait_group0();
+    } else if (warp == MMA_WARP) {
+        // ---------------- MMA issuer: weight plane q against token planes 0..7-q ----------------
+        if (lane == 0) {
+            constexpr uint32_t IDESC = (2u << 4) | ((uint32_t)(BW >> 4) << 24);
+            const uint32_t w_lo = limb_desc_lo(ptx::smem_u32(sB)), t_lo = limb_desc_lo(ptx::smem_u32(sV));
+            auto product = [&](uint32_t d, int w_set, int t_set, uint32_t acc) {
+                const uint32_t w = w_lo + ((w_set * W_SET_BYTES) >> 4), t = t_lo + ((t_set * T_SET_BYTES) >> 4);
+#pragma unroll
+                for (int q = 0; q < PLANES; ++q)
+                    ptx::mma_i8(d + BT * q, w + ((q * W_PLANE_BYTES) >> 4), LIMB_DESC_HI, t, LIMB_DESC_HI,
+                                IDESC | ((uint32_t)((BT * (PLANES - q)) >> 3) << 17), q == 0 ? acc : 1u);
+            };
+            uint32_t unit_phase = 0, seg_phase = 0;
+            bool ok = true;
+            for (unsigned u = u_begin; u < u_end && ok;) {
+                const StreamSegment sg = stream_segment(a, u, u_end);
+                u += sg.count;
+                for (int it = 0; it < sg.count; ++it) {
+                    ok = limb_wait(ptx::smem_u32(&planes_full), unit_phase, &abort_flag);
+                    if (!ok) break;
+                    unit_phase ^= 1u;
+                    ptx::fence_after_sync();
+                    const bool last = it + 1 == sg.count;
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) {
+                        if (it == 0) {
+                            ok = ok && limb_wait(ptx::smem_u32(&acc_empty[p]), seg_phase ^ 1u, &abort_flag);
+                            if (!ok) break;
+                            ptx::fence_after_sync();
+                        }
+                        product(tmem_base + p * ACC_COLS, p, 2, it > 0 ? 1u : 0u);       // E*B_i
+                        ptx::mma_commit(ptx::smem_u32(&own_empty[p]));
+                    }
+                    if (!ok) break;
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) {
+                        product(tmem_base + p * ACC_COLS, 2, p, 1u);                      // V_i*F
+                        if (last) ptx::mma_commit(ptx::smem_u32(&acc_full[p]));
+                    }
+                    ptx::mma_commit(ptx::smem_u32(&shared_empty));
+                }
+                seg_phase ^= 1u;
+            }
+            // the main loop is over: the next kernel of the stream may be brought in beside the last drain
+            pdl_launch_dependents();
+        }
+    }
+
+    __syncwarp();
+    ptx::fence_before_sync();
+    __syncthreads();
+    if (threadIdx.x == 0 && abort_flag && a.error_flag) {
+        *a.error_flag = 1;
+        *reinterpret_cast<volatile int*>(a.error_host) = 1;
+        __threadfence_system();
+    }
+    if (warp == MMA_WARP) {
+        ptx::fence_after_sync();
+        ptx::tmem_dealloc(tmem_base, 2 * ACC_COLS);
+    }
+}
+
+}  // namespace comet

@@ -1,0 +1,57 @@
+"""The streaming product kernel (few token rows; the allocation-free entry point) at the edges of its tiles: 32 tokens,
+128 output features in quarters of 32, steps of 32 contraction indices.  Bit for bit against the CPU oracle."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import oracle  # noqa: E402
+from paper_2505_07239_b200 import workloads as wl  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def cb():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2505_07239_b200 import binding
+
+    return binding
+
+
+@pytest.mark.parametrize("T,K,N", [
+    (1, 8, 4),             # the smallest problem: one step, one quarter, a quarter of a step deep
+    (3, 40, 28), (32, 32, 32), (33, 64, 36),      # one and two token tiles
+    (31, 104, 128), (65, 96, 132),                # a full feature tile, and four features into the next
+    (7, 1032, 420),        # more steps than SMs in one tile's range, ragged in every direction
+    (1, 16, 32752),        # 256 feature tiles of a single step: the scratch array's limit in N
+    (2000, 32, 4),         # 63 token tiles against four features
+    (2, 65536, 4),         # a single tile 2048 steps deep: more than one segment's bound on the contraction depth
+])
+def test_static_product_at_tile_edges(cb, T, K, N):
+    def draw(name, shape):
+        return [wl.random_u64(900 + T, f"stream/{name}/{p}", shape[0] * shape[1]).reshape(shape) for p in (0, 1)]
+
+    Xh, Ah, Yh, Bh, Ch = draw("X", (T, K)), draw("A", (T, K)), draw("Y", (N, K)), draw("B", (N, K)), draw("C", (T, N))
+    X, A, Y, B, C = ([cb.to_device(v) for v in pair] for pair in (Xh, Ah, Yh, Bh, Ch))
+    Z = [torch.full((T, N), -1, dtype=torch.int64, device="cuda") for _ in (0, 1)]
+    assert cb.beaver_matmul_static(X, A, Y, B, C, Z) == cb.OK
+    torch.cuda.synchronize()
+    ref = oracle.pi_matmul(Xh, [np.ascontiguousarray(v.T) for v in Yh], Ah, [np.ascontiguousarray(v.T) for v in Bh], Ch)
+    for p in (0, 1):
+        assert np.array_equal(Z[p].cpu().numpy().view(np.uint64), ref["Z"][p]), p
+
+
+@pytest.mark.parametrize("tokens,d_model,blocks,block,active,stacked", [
+    (1, 16, 4, 16, 1, 1),          # 16 features, half a step
+    (32, 144, 24, 16, 9, 1),       # 144 features both ways: 128 and a ragged tile of 16
+    (31, 112, 12, 48, 5, 2),       # strips of 48 columns: a step takes its halves from two blocks
+    (8, 272, 8, 80, 3, 3),         # three stacked matrices, group boundaries inside a feature tile
+])
+def test_few_token_layer_at_tile_edges(cb, tokens, d_model, blocks, block, active, stacked):
+    from tests import harness as hz
+
+    cfg = wl.FFNConfig("stream-edges", tokens, d_model, blocks * block, block, 16, stacked == 2, active / blocks, "uniform",
+                       "normal", "normal0.02", stacked=stacked)
+    r = hz.run_and_compare_products(cfg, seed=700 + tokens)
+    assert r["mismatches"] == 0 and r["path"] == 2 and r["n_active"] == active * block, r

@@ -111,8 +111,8 @@ typedef struct {
 /* phases of the path, for the per-phase timers of comet_stats */
 enum {
     COMET_PHASE_COMPACT = 0,  /* mask compaction                                   */
-    COMET_PHASE_OPEN = 1,     /* E_i = X_i - A_i and F_i = gather(W_i) - B_i        */
-    COMET_PHASE_PREP = 2,     /* operand preparation after the exchange (limb path) */
+    COMET_PHASE_OPEN = 1,     /* E_i = X_i - A_i, F_i = gather(W_i) - B_i, exchange, operand planes */
+    COMET_PHASE_PREP = 2,     /* not used: the opening kernels prepare the operands too    */
     COMET_PHASE_COMBINE = 3,  /* the gathered ring matmul + Beaver combine          */
     COMET_PHASE_TRUNCATE = 4, /* local truncation                                   */
     COMET_NUM_PHASES = 5

@@ -34,11 +34,11 @@ struct comet_ctx {
     u64* own[2][COMET_NUM_TENSORS];   // the library's own buffers (allocated in comet_init, freed in comet_destroy)
     int64_t cap_words[COMET_NUM_TENSORS];
     bool loaded[2][COMET_NUM_TENSORS];
-    // limb path: blocked limb planes per party (left: E and V_i; right: B_i and F), and the device error flag
+    // limb path: blocked limb planes (left: V_i per party and E; right: B_i per party and F), and the device error flag
     int path;                     // COMET_PATH_SIMT or COMET_PATH_LIMB
-    uint8_t* planes_left[2][2];       // [party][E, V_i]; shared by the two projections
-    uint8_t* planes_right_up[2][2];   // [party][B_i, F] of the up-projection
-    uint8_t* planes_right_dn[2][2];   // [party][B'_i, F'] of the down-projection
+    uint8_t* planes_left[3];          // V_0, V_1, E; shared by the two projections
+    uint8_t* planes_right_up[3];      // B_0, B_1, F of the up-projection
+    uint8_t* planes_right_dn[3];      // B'_0, B'_1, F' of the down-projection
     size_t planes_left_bytes, planes_right_up_bytes, planes_right_dn_bytes;
     int* d_error;                     // = d_count + 1
     // the weight side of the down-projection is opened on a second stream while the up-projection's
@@ -316,112 +316,60 @@ int join_side(comet_ctx* c) {
     return COMET_OK;
 }
 
-// Tensor-core path, before the exchange: E_i (left) and/or F_i + planes(B_i) (right), one launch.
-int limb_open(comet_ctx* c, const Proj& pr, bool left, bool right, cudaStream_t stream) {
+// Tensor-core path: messages, exchange and operand planes of the left and / or right side, and / or Z <- C; one launch.
+int limb_exchange(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy, cudaStream_t stream) {
     namespace lb = comet::limb;
-    comet::LimbOpenArgs a;
+    comet::LimbExchangeArgs a;
     std::memset(&a, 0, sizeof(a));
-    const int kb = ceil_div(pr.K, lb::KC);
-    uint8_t* (*planes)[2] = pr.down ? c->planes_right_dn : c->planes_right_up;
+    uint8_t** planes = pr.down ? c->planes_right_dn : c->planes_right_up;
     for (int p = 0; p < 2; ++p) {
         a.X[p] = c->buf[p][pr.idX];
         a.A[p] = c->buf[p][pr.idA];
         a.E[p] = c->buf[p][pr.idE];
+        a.Vpl[p] = c->planes_left[p];
         a.W0[p] = pr.down ? c->buf[p][COMET_W2] : (c->groups >= 2 ? c->buf[p][COMET_WG] : c->buf[p][COMET_W1]);
         a.W1[p] = c->buf[p][COMET_W1];
-        a.W2g[p] = c->buf[p][COMET_W3];
+        a.W2[p] = c->buf[p][COMET_W3];
         a.B[p] = c->buf[p][pr.idB];
         a.F[p] = c->buf[p][pr.idF];
-        a.Bpl[p] = planes[p][0];
-    }
-    a.left_pairs = left ? (long long)pr.M * pr.K / 2 : 0;
-    a.left_blocks = left ? ew_grid(c, a.left_pairs, lb::OPEN_THREADS) : 0;
-    a.ids = c->d_ids;
-    a.n = c->n_active;
-    a.bs = c->cfg.block;
-    a.rows = pr.N;
-    a.K = pr.K;
-    a.ldw = pr.down ? c->cfg.d_ff : c->cfg.d_model;
-    a.kblocks = kb;
-    a.down = pr.down ? 1 : 0;
-    a.tmask = (pr.down && c->tmask_set) ? c->d_tmask : nullptr;
-    a.tmask_ld = c->n_active_blocks;
-    a.row_label = (!pr.down && c->tmask_set) ? c->d_row_label : nullptr;
-    a.blk_label = c->tmask_set ? c->d_blk_label : nullptr;
-    a.col_map = (!pr.down && c->grouped) ? c->d_col_map : nullptr;
-    a.kmap = (pr.down && c->grouped) ? c->d_kmap : nullptr;
-    // right CTAs: 32 rows x kb_per_cta k-blocks each, over whole plane tiles (rows past the operand are zero planes);
-    // enough k-blocks per CTA for the copies of one to fly under the work on another, enough CTAs to fill the device
-    const int row_tiles = right ? ceil_div(pr.N, lb::BN) * (lb::BN / lb::OPEN_ROWS) : 0;
-    {
-        const long long fill = (long long)c->sm_count * 6;
-        long long per = fill > 0 ? 2ll * row_tiles * kb / fill : 1;
-        if (per < 1) per = 1;
-        if (per > lb::OPEN_MAX_KB_PER_CTA) per = lb::OPEN_MAX_KB_PER_CTA;
-        a.kb_per_cta = (int)per;
-        a.kchunks = ceil_div(kb, a.kb_per_cta);
-    }
-    const int right_tiles = row_tiles * a.kchunks;
-    if (a.left_blocks + right_tiles == 0) return COMET_OK;
-    const size_t smem = right_tiles ? lb::OPEN_SMEM_BYTES : 0;
-    COMET_CUDA(c, launch_chained(comet::limb_open_kernel, dim3(2 * (a.left_blocks + right_tiles)),
-                                 dim3(lb::OPEN_THREADS), smem, stream, nullptr, a));
-    c->stats.kernel_launches += 1;
-    COMET_CUDA(c, cudaGetLastError());
-    return COMET_OK;
-}
-
-// Tensor-core path, after the exchange: planes(E), planes(V_i) (left), planes(F) (right), Z <- C, one launch.
-int limb_prep(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy, cudaStream_t stream) {
-    namespace lb = comet::limb;
-    comet::LimbPrepArgs a;
-    std::memset(&a, 0, sizeof(a));
-    const int kb = ceil_div(pr.K, lb::KC);
-    uint8_t* (*planes)[2] = pr.down ? c->planes_right_dn : c->planes_right_up;
-    a.E0 = c->buf[0][pr.idE]; a.E1 = c->buf[1][pr.idE];
-    a.F0 = c->buf[0][pr.idF]; a.F1 = c->buf[1][pr.idF];
-    for (int p = 0; p < 2; ++p) {
-        a.A[p] = c->buf[p][pr.idA];
-        a.Epl[p] = c->planes_left[p][0];
-        a.Vpl[p] = c->planes_left[p][1];
-        a.Fpl[p] = planes[p][1];
+        a.Bpl[p] = planes[p];
         a.C[p] = c->buf[p][pr.idC];
         a.Z[p] = c->buf[p][pr.idZ];
     }
-    a.M = pr.M; a.N = pr.N; a.K = pr.K; a.kblocks = kb;
-    if (c->grouped) {                       // component-sorted planes of the rows and columns that lie in a component
-        a.M = c->live_rows;
-        a.row_map = c->d_row_map;
-        if (pr.down) {
-            a.kmap = c->d_kmap;
-        } else {
-            a.N = c->groups * c->live_blocks * c->cfg.block;
-            a.col_map = c->d_col_map;
-        }
-    }
-    a.tmask = (pr.down && c->tmask_set) ? c->d_tmask : nullptr;
-    a.tmask_ld = c->n_active_blocks;
+    a.Epl = c->planes_left[2];
+    a.Fpl = planes[2];
+    a.ids = c->d_ids;
+    a.n = c->n_active;
     a.bs = c->cfg.block;
-    // tile CTAs: 32 rows x kb_per_cta k-blocks each, over whole plane tiles (rows past the operand are zero planes)
-    const int left_rows32 = left ? ceil_div(a.M, lb::BM) * (lb::BM / lb::OPEN_ROWS) : 0;
-    const int right_rows32 = right ? ceil_div(a.N, lb::BN) * (lb::BN / lb::OPEN_ROWS) : 0;
-    {
-        const long long fill = (long long)c->sm_count * 4;
-        long long per = fill > 0 ? 2ll * (left_rows32 + right_rows32) * kb / fill : 1;
-        if (per < 1) per = 1;
-        if (per > lb::OPEN_MAX_KB_PER_CTA) per = lb::OPEN_MAX_KB_PER_CTA;
-        a.kb_per_cta = (int)per;
-        a.kchunks = ceil_div(kb, a.kb_per_cta);
+    a.M = pr.M; a.N = pr.N; a.K = pr.K;
+    a.ldw = pr.down ? c->cfg.d_ff : c->cfg.d_model;
+    a.down = pr.down ? 1 : 0;
+    if (c->tmask_set) {
+        a.tmask = pr.down ? c->d_tmask : nullptr;
+        a.tmask_ld = c->n_active_blocks;
+        a.row_label = pr.down ? nullptr : c->d_row_label;
+        a.blk_label = c->d_blk_label;
     }
-    a.left_tiles = left_rows32 * a.kchunks;
-    a.right_tiles = right_rows32 * a.kchunks;
+    if (c->grouped) {                       // component-sorted planes
+        a.row_map = c->d_row_map;
+        a.col_map = pr.down ? nullptr : c->d_col_map;
+        a.kmap = pr.down ? c->d_kmap : nullptr;
+    }
+    a.kblocks = ceil_div(pr.K, lb::KC);
+    const int left_rows = left ? ceil_div(pr.M, lb::EX_ROWS) : 0, right_rows = right ? ceil_div(pr.N, lb::EX_ROWS) : 0;
+    // enough CTAs to fill the device once, else as many k-blocks per CTA as spread the row set-up
+    const long long fill = (long long)c->sm_count * 7;
+    const long long per = (long long)(left_rows + right_rows) * a.kblocks / fill;
+    a.kb_per_cta = (int)(per < 1 ? 1 : per > lb::EX_MAX_KB_PER_CTA ? lb::EX_MAX_KB_PER_CTA : per);
+    a.kchunks = ceil_div(a.kblocks, a.kb_per_cta);
+    a.left_blocks = left_rows * a.kchunks;
+    a.right_blocks = right_rows * a.kchunks;
     a.copy_pairs = copy ? (long long)pr.M * pr.N / 2 : 0;
-    a.copy_blocks = copy ? ew_grid(c, a.copy_pairs, lb::OPEN_THREADS) : 0;
-    const int blocks = a.left_tiles + a.right_tiles + a.copy_blocks;
+    a.copy_blocks = copy ? 2 * ew_grid(c, a.copy_pairs, lb::EX_THREADS) : 0;
+    const int blocks = a.left_blocks + a.right_blocks + a.copy_blocks;
     if (blocks == 0) return COMET_OK;
-    const size_t smem = (size_t)lb::OPEN_STAGES * (left ? 3 : 2) * lb::OPEN_TILE_BYTES;
-    COMET_CUDA(c, launch_chained(comet::limb_prep_kernel, dim3(2 * blocks), dim3(lb::OPEN_THREADS), smem, stream,
-                                 nullptr, a));
+    COMET_CUDA(c, launch_chained(comet::limb_exchange_kernel, dim3(blocks), dim3(lb::EX_THREADS),
+                                 left_rows + right_rows ? lb::EX_SMEM_BYTES : 0, stream, nullptr, a));
     c->stats.kernel_launches += 1;
     COMET_CUDA(c, cudaGetLastError());
     return COMET_OK;
@@ -431,15 +379,15 @@ int limb_prep(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy, cu
 int limb_combine(comet_ctx* c, const Proj& pr) {
     namespace lb = comet::limb;
     const int kb = ceil_div(pr.K, lb::KC), mt = ceil_div(pr.M, lb::BM), nt = ceil_div(pr.N, lb::BN);
-    uint8_t* (*planes)[2] = pr.down ? c->planes_right_dn : c->planes_right_up;
+    uint8_t** planes = pr.down ? c->planes_right_dn : c->planes_right_up;
     comet::LimbArgs a;
     for (int p = 0; p < 2; ++p) {
-        a.Epl[p] = c->planes_left[p][0];
-        a.Vpl[p] = c->planes_left[p][1];
-        a.Bpl[p] = planes[p][0];
-        a.Fpl[p] = planes[p][1];
+        a.Vpl[p] = c->planes_left[p];
+        a.Bpl[p] = planes[p];
         a.Z[p] = c->buf[p][pr.idZ];
     }
+    a.Epl = c->planes_left[2];
+    a.Fpl = planes[2];
     a.M = pr.M; a.N = pr.N; a.mt = mt; a.nt = nt; a.kb = kb;
     a.error_flag = c->d_error;
     a.error_host = c->h_count_dev + 3;
@@ -611,12 +559,11 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
         c->planes_right_up_bytes = (size_t)(((gn + lb::BN - 1) / lb::BN) * kb_up) * lb::B_BLOCK_BYTES;
         c->planes_right_dn_bytes = (size_t)(((d + lb::BN - 1) / lb::BN) * kb_dn) * lb::B_BLOCK_BYTES;
         // a context for few tokens only never builds planes in memory
-        for (int p = 0; p < 2 && ok && c->cap_T > comet::limb_stream::BT; ++p)
-            for (int w = 0; w < 2 && ok; ++w) {
-                ok = cudaMalloc((void**)&c->planes_left[p][w], c->planes_left_bytes) == cudaSuccess;
-                ok = ok && cudaMalloc((void**)&c->planes_right_up[p][w], c->planes_right_up_bytes) == cudaSuccess;
-                ok = ok && cudaMalloc((void**)&c->planes_right_dn[p][w], c->planes_right_dn_bytes) == cudaSuccess;
-            }
+        for (int w = 0; w < 3 && ok && c->cap_T > comet::limb_stream::BT; ++w) {
+            ok = cudaMalloc((void**)&c->planes_left[w], c->planes_left_bytes) == cudaSuccess;
+            ok = ok && cudaMalloc((void**)&c->planes_right_up[w], c->planes_right_up_bytes) == cudaSuccess;
+            ok = ok && cudaMalloc((void**)&c->planes_right_dn[w], c->planes_right_dn_bytes) == cudaSuccess;
+        }
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)lb::SMEM_BYTES) == cudaSuccess;
         // the memory-side kernels may share an SM with a resident tensor-core CTA (which forces the largest
@@ -630,12 +577,10 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_grouped_kernel,
                                         cudaFuncAttributePreferredSharedMemoryCarveout,
                                         (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(comet::limb_open_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+        ok = ok && cudaFuncSetAttribute(comet::limb_exchange_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                         (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(comet::limb_prep_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                        (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(comet::limb_prep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)(lb::OPEN_STAGES * 3 * lb::OPEN_TILE_BYTES)) == cudaSuccess;
+        ok = ok && cudaFuncSetAttribute(comet::limb_exchange_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)lb::EX_SMEM_BYTES) == cudaSuccess;
         ok = ok && cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) == cudaSuccess;
@@ -684,12 +629,11 @@ void comet_destroy(comet_ctx* c) {
         for (int p = 0; p < 2; ++p)
             if (c->own[p][id]) cudaFree(c->own[p][id]);
     if (c->side) cudaStreamSynchronize(c->side);
-    for (int p = 0; p < 2; ++p)
-        for (int w = 0; w < 2; ++w) {
-            if (c->planes_left[p][w]) cudaFree(c->planes_left[p][w]);
-            if (c->planes_right_up[p][w]) cudaFree(c->planes_right_up[p][w]);
-            if (c->planes_right_dn[p][w]) cudaFree(c->planes_right_dn[p][w]);
-        }
+    for (int w = 0; w < 3; ++w) {
+        if (c->planes_left[w]) cudaFree(c->planes_left[w]);
+        if (c->planes_right_up[w]) cudaFree(c->planes_right_up[w]);
+        if (c->planes_right_dn[w]) cudaFree(c->planes_right_dn[w]);
+    }
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->side) cudaStreamDestroy(c->side);
@@ -951,25 +895,27 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
             return rc != COMET_OK ? rc : somm_merge(c, tokens);
         }
         if (!limb_fits(c, up)) return COMET_ERR_SHAPE;
-        {
-            PhaseTimer timer(c, COMET_PHASE_OPEN, 1);
-            rc = limb_open(c, up, true, true, c->stream);
-        }
-        if (rc != COMET_OK) return rc;
         // The weight side of the down-projection depends only on the mask, W2 and B'_i: if those are loaded
-        // already, open it now on the side stream, beside the preparation and the tensor-core kernel that follow.
-        // (The fork sits before the preparation kernel so that nothing separates that kernel from the tensor-core
-        // kernel on the main stream: the latter is launched as the former's programmatic dependent.)
+        // already, open it now on the side stream, beside the tensor-core kernel (not beside the exchange before it, which
+        // is bound by the same memory).  Beside it 198 MB of exchange traffic cost the 512-token step at 90 % sparsity 14 us,
+        // behind it 27; a launch-completion event of the tensor-core kernel, which would keep that kernel a programmatic
+        // dependent of the exchange, only fired when the kernel had ended.
         const bool early = !c->dn_right_ready && limb_fits(c, dn) && c->loaded[0][COMET_W2] &&
                            c->loaded[1][COMET_W2] && c->loaded[0][COMET_B_DN] && c->loaded[1][COMET_B_DN];
+        {
+            PhaseTimer timer(c, COMET_PHASE_OPEN, 1);
+            rc = limb_exchange(c, up, true, true, true, c->stream);
+        }
+        if (rc != COMET_OK) return rc;
+        if (early) COMET_CUDA(c, cudaEventRecord(c->ev_fork, c->stream));
+        rc = limb_combine(c, up);
+        if (rc != COMET_OK) return rc;
         if (early) {
-            COMET_CUDA(c, cudaEventRecord(c->ev_fork, c->stream));
             COMET_CUDA(c, cudaStreamWaitEvent(c->side, c->ev_fork, 0));
             // ... and if the triple's C' share is there too, Y_i <- C'_i, the value the down-projection's sums are
             // added to, is copied in the same launch
             const bool copy = c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN];
-            rc = limb_open(c, dn, false, true, c->side);
-            if (rc == COMET_OK) rc = limb_prep(c, dn, false, true, copy, c->side);
+            rc = limb_exchange(c, dn, false, true, copy, c->side);
             if (rc != COMET_OK) return rc;
             COMET_CUDA(c, cudaEventRecord(c->ev_join, c->side));
             c->side_pending = true;
@@ -977,13 +923,6 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
             c->dn_copy_ready = copy;
             c->dn_copy_tokens = tokens;
         }
-        {
-            PhaseTimer timer(c, COMET_PHASE_PREP, 1);
-            rc = limb_prep(c, up, true, true, true, c->stream);
-        }
-        if (rc != COMET_OK) return rc;
-        rc = limb_combine(c, up);
-        if (rc != COMET_OK) return rc;
         return somm_merge(c, tokens);
     }
 
@@ -1061,12 +1000,7 @@ int comet_ffn_down(comet_ctx* c, int32_t tokens) {
         if (rc != COMET_OK) return rc;
         {
             PhaseTimer timer(c, COMET_PHASE_OPEN, 1);
-            rc = limb_open(c, dn, true, !have_right, c->stream);
-        }
-        if (rc != COMET_OK) return rc;
-        {
-            PhaseTimer timer(c, COMET_PHASE_PREP, 1);
-            rc = limb_prep(c, dn, true, !have_right, !have_copy, c->stream);
+            rc = limb_exchange(c, dn, true, !have_right, !have_copy, c->stream);
         }
         if (rc != COMET_OK) return rc;
         c->dn_right_ready = false;                     // a triple serves one product

@@ -37,33 +37,24 @@ constexpr int STAGES = 3;
 constexpr int MAX_SEGMENT_UNITS = 16384 / KC;     // keeps the limb sums for s <= 3 below 2^32
 constexpr int EPI_WARPS = 8;                      // warp w drains TMEM lanes 32*(w%4).., columns 32*(w/4)..
 constexpr int THREADS = 32 * (EPI_WARPS + 2);     // warps 0-7 epilogue, warp 8 copy producer, warp 9 MMA issuer
-// The opening kernel streams tiles of 32 rows x one k-block of the weight share and of the triple share through a
-// two-stage ring in shared memory (asynchronous 16-byte copies, which hold no registers while in flight), several
-// consecutive k-blocks per CTA: the copies of the next k-block fly while the current one is turned into the message
-// and the planes.
-constexpr int OPEN_ROWS = 32, OPEN_THREADS = 128, OPEN_STAGES = 2;
-constexpr int OPEN_STRIDE = KC + 2;               // words per staged row: 272 bytes keep every row 16-byte aligned and
-                                                  // the 16-byte reads of eight consecutive rows on distinct banks
-constexpr int OPEN_TILE_BYTES = OPEN_ROWS * OPEN_STRIDE * 8;
-constexpr size_t OPEN_SMEM_BYTES = (size_t)OPEN_STAGES * 2 * OPEN_TILE_BYTES;      // a W and a B tile per stage: 34 KiB
-constexpr int OPEN_MAX_KB_PER_CTA = 8;
+constexpr int EX_THREADS = 128, EX_ROWS = 16, EX_MAX_KB_PER_CTA = 16;      // exchange kernel: four rows per warp
+constexpr int EX_STAGES = 2, EX_STAGE_BYTES = EX_THREADS * 8 * 16;           // eight 16-byte pieces per lane and k-block
+constexpr size_t EX_SMEM_BYTES = (size_t)EX_STAGES * EX_STAGE_BYTES;        // 32 KiB: fits beside a tensor-core CTA
 constexpr int OUT_COLS = 16;                      // words per staged output row (a thread's 32 go in two rounds)
 constexpr int OUT_ROW_BYTES = OUT_COLS * 8 + 16;  // padded against bank conflicts
 constexpr size_t SMEM_BYTES = (size_t)STAGES * (A_BLOCK_BYTES + B_BLOCK_BYTES) + (size_t)EPI_WARPS * 32 * OUT_ROW_BYTES + 128;
 constexpr long long WAIT_CYCLES = 4000000000ll;   // ~2 s at 1.9 GHz: every wait gives up after this
 constexpr unsigned LBO_BYTES = 128, SBO_BYTES = 256;
-
-// byte offset of (plane p, row r, contraction index k in [0,32)) inside a block of `rows` rows
-__host__ __device__ __forceinline__ int block_offset(int rows, int p, int r, int k) {
-    return p * rows * KC + (r >> 3) * 256 + (k >> 4) * 128 + (r & 7) * 16 + (k & 15);
-}
 }  // namespace limb
 
 // ---------------------------------------------------------------------------
-// Blocked limb planes: helpers shared by the two memory-side kernels below.
-// A CTA tile is 32 rows x 32 contraction elements; words are staged in shared memory as [row][34], which keeps
-// every row 16-byte aligned for the asynchronous copies (16 threads per row) and puts the 16-byte reads of eight
-// consecutive rows, as the byte transposition issues them, on distinct banks.
+// Blocked limb planes from words: 4 x 4 byte transposition, and four words of one row -> eight planes, four bytes each,
+// `stride` bytes apart.
+//
+// Inside a 32-deep k-block the contraction indices sit in the order in which a warp reads words: a lane holds two 16-byte
+// pieces of a row, words 2c, 2c+1, 16+2c, 17+2c (c = lane mod 8, so eight lanes read whole 128-byte lines), and writes
+// their bytes next to each other, at bytes 4c .. 4c+3 of the row's 32.  Every operand uses that order, so sums over a
+// k-block are the same.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void limb_transpose4(unsigned x0, unsigned x1, unsigned x2, unsigned x3,
                                                 unsigned& p0, unsigned& p1, unsigned& p2, unsigned& p3) {
@@ -75,35 +66,17 @@ __device__ __forceinline__ void limb_transpose4(unsigned x0, unsigned x1, unsign
     p3 = __byte_perm(t2, t3, 0x7632);
 }
 
-// Split the 16 words at `src` (16-byte aligned, shared memory) into 8 limb planes of 16 bytes and store them at
-// (plane, row `rin`, k = 16*half) of the block `blk`, whose tiles have `tile_rows` rows.
-__device__ __forceinline__ void limb_emit_planes16(const u64* src, int half, uint8_t* blk, int tile_rows, int rin) {
-    unsigned lo[16], hi[16];
+__device__ __forceinline__ void limb_emit4(uint8_t* dst, int stride, const u64* w) {
+    uint32_t p[8];
+    limb_transpose4((uint32_t)w[0], (uint32_t)w[1], (uint32_t)w[2], (uint32_t)w[3], p[0], p[1], p[2], p[3]);
+    limb_transpose4((uint32_t)(w[0] >> 32), (uint32_t)(w[1] >> 32), (uint32_t)(w[2] >> 32), (uint32_t)(w[3] >> 32),
+                    p[4], p[5], p[6], p[7]);
 #pragma unroll
-    for (int j = 0; j < 16; j += 2) {
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(src + j);
-        lo[j] = (unsigned)v.x;
-        hi[j] = (unsigned)(v.x >> 32);
-        lo[j + 1] = (unsigned)v.y;
-        hi[j + 1] = (unsigned)(v.y >> 32);
-    }
-    uint4 plane[8];
-    limb_transpose4(lo[0], lo[1], lo[2], lo[3], plane[0].x, plane[1].x, plane[2].x, plane[3].x);
-    limb_transpose4(lo[4], lo[5], lo[6], lo[7], plane[0].y, plane[1].y, plane[2].y, plane[3].y);
-    limb_transpose4(lo[8], lo[9], lo[10], lo[11], plane[0].z, plane[1].z, plane[2].z, plane[3].z);
-    limb_transpose4(lo[12], lo[13], lo[14], lo[15], plane[0].w, plane[1].w, plane[2].w, plane[3].w);
-    limb_transpose4(hi[0], hi[1], hi[2], hi[3], plane[4].x, plane[5].x, plane[6].x, plane[7].x);
-    limb_transpose4(hi[4], hi[5], hi[6], hi[7], plane[4].y, plane[5].y, plane[6].y, plane[7].y);
-    limb_transpose4(hi[8], hi[9], hi[10], hi[11], plane[4].z, plane[5].z, plane[6].z, plane[7].z);
-    limb_transpose4(hi[12], hi[13], hi[14], hi[15], plane[4].w, plane[5].w, plane[6].w, plane[7].w);
-#pragma unroll
-    for (int p = 0; p < 8; ++p)
-        *reinterpret_cast<uint4*>(blk + limb::block_offset(tile_rows, p, rin, half * 16)) = plane[p];
+    for (int i = 0; i < 8; ++i) *reinterpret_cast<uint32_t*>(dst + i * stride) = p[i];
 }
 
-// 16-byte asynchronous copy global -> shared that bypasses L1; with `bytes` = 0 nothing is read and the 16 bytes
-// are filled with zeros.  (The form that also carries an L2 cache-policy operand raised an illegal-instruction
-// error on this part when combined with the byte count, so no eviction hint is given here.)
+// 16-byte asynchronous copy global -> shared that bypasses L1; with `bytes` = 0 nothing is read and the 16 bytes are
+// filled with zeros.
 __device__ __forceinline__ void limb_copy16_async(uint32_t dst_smem, const void* src, uint32_t bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst_smem), "l"(src), "r"(bytes) : "memory");
 }
@@ -111,46 +84,50 @@ __device__ __forceinline__ void limb_copy_commit() { asm volatile("cp.async.comm
 template <int PENDING>
 __device__ __forceinline__ void limb_copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
 
-__device__ __forceinline__ uint8_t* limb_block_ptr(uint8_t* base, int tile_rows, int row, int kblocks, int kb,
-                                                   int* rin) {
-    const int tile = row >> (31 - __clz(tile_rows));          // tile_rows is 64 or 128
-    *rin = row - tile * tile_rows;
-    return base + ((size_t)tile * kblocks + kb) * (size_t)(limb::PLANES * tile_rows * limb::KC);
-}
-
 // ---------------------------------------------------------------------------
-// Before the exchange (Section 2.1 "Multiplication"; IndexCols of Protocol 2, IndexRow of Protocol 3), one launch:
-//   left  blocks: E_i = X_i - A_i, elementwise;
-//   right tiles : F_i = gather(W_i) - B_i written as the message, and the blocked limb planes of the party's
-//                 own B_i (it is in registers anyway, so it is not read a second time later).
+// Masking and exchange for the tensor-core kernel, one launch (Section 2.1 "Multiplication"; IndexCols of Protocol 2,
+// IndexRow of Protocol 3):
+//   left  rows: E_i = X_i - A_i        -> message;  planes of E = E_0 + E_1 and of V_i = A_i + i*E
+//   right rows: F_i = gather(W_i) - B_i -> message;  planes of F = F_0 + F_1 and of B_i
+//   copy      : Z_i <- C_i (the accumulation target starts from the triple's C share)
 // gather: up   (down = 0): row c of the right operand is row neuron(c) of W (whole rows of `ldw` words);
 //         down (down = 1): contraction index c is column neuron(c) of W (strips of `bs` words in every row).
-// grid = 2 * (left_blocks + row_tiles * kchunks), 128 threads, the party being the lowest bit of the block index
-// (both parties' messages are then written in the same order, which the next kernel reads backwards).  A right CTA
-// owns 32 rows and kb_per_cta consecutive k-blocks: while it turns one k-block into the message and the planes, the
-// loads of the next one are in flight (the kernel is bound by memory latency, not by bandwidth, when a CTA loads,
-// waits and works in turn).  Dynamic shared memory: OPEN_SMEM_BYTES when there are right tiles.
+// What is written for a party depends on that party's shares and on the two messages; both parties' words of one place
+// are in the same thread, which is the exchange, so a message is written once and read by nobody on the path, and the
+// planes of E and F exist once for both parties.
+//
+// Bound by memory: per word and party 16 bytes in, 8 out as the message, 12 out as planes (the sum's planes are shared).
+// A warp owns four rows and walks k-blocks of 32 words.  A lane's 16-byte pieces land in shared memory by asynchronous
+// copies, EX_STAGES k-blocks ahead, and only that lane reads them: no barriers, and loads in flight cost neither registers
+// nor L1 lines.  (Plain loads, eight per lane in flight: 48 us on [512 | 832, 2048] and 329 us on [512 | 8192, 2048] with the
+// L1 that the tensor-core kernels' carve-out leaves, 37 and 271 us with all of it; 33 and 258 us this way.)
+// It replaces an opening kernel and a preparation kernel that read the messages back and built every plane of E and F
+// twice: 112 bytes per word of both parties, now 72.
+// grid = left_blocks + right_blocks + copy_blocks; a left / right block owns 16 rows x kb_per_cta k-blocks.
 // ---------------------------------------------------------------------------
-struct LimbOpenArgs {
-    const u64* X[2];
-    const u64* A[2];
+struct LimbExchangeArgs {
+    const u64* X[2]; const u64* A[2];
     u64* E[2];
-    long long left_pairs;
-    int left_blocks;
+    uint8_t* Epl;
+    uint8_t* Vpl[2];
     const u64* W0[2];        // weights of group 0 (gate when gated, else the only matrix)
     const u64* W1[2];        // weights of group 1 (up-projection of a gated FFN)
-    const u64* W2g[2];       // weights of group 2 (third stacked matrix, e.g. the value projection)
+    const u64* W2[2];        // weights of group 2 (third stacked matrix, e.g. the value projection)
     const u64* B[2];
     u64* F[2];
+    uint8_t* Fpl;
     uint8_t* Bpl[2];
+    const u64* C[2];
+    u64* Z[2];
+    long long copy_pairs;
     const int32_t* ids;      // ascending active block ids
     int n, bs;               // active neurons, neurons per block
-    int rows, K;             // logical size of the right operand [rows, K]
-    int ldw;                 // words per row of W
-    int kblocks, down;
-    int kb_per_cta, kchunks; // k-blocks per right CTA and CTAs per row tile: kchunks = ceil(kblocks / kb_per_cta)
-    // Protocol 3 with per-column row sets: per-token mask over the active blocks, [rows of X, tmask_ld] bytes, or
-    // null.  Where it is zero the entry of X is no non-zero: it is not opened and E_i is zero there.
+    int M, N, K;             // rows of the left and right operand, contraction length
+    int ldw, down;
+    int left_blocks, right_blocks, copy_blocks;
+    int kblocks, kb_per_cta, kchunks;      // kchunks = ceil(kblocks / kb_per_cta)
+    // Protocol 3 with per-column row sets: per-token mask over the active blocks, [M, tmask_ld] bytes, or null.  Where
+    // it is zero X and A_i have no entry: E_i is zero there and the party's A_i counts as zero.
     const uint8_t* tmask;
     int tmask_ld;
     // Protocol 2 over connected components: component label per row of X and per active block (-1 = in no
@@ -159,326 +136,152 @@ struct LimbOpenArgs {
     // the right operand that belong to it are not opened either.
     const int32_t* row_label;
     const int32_t* blk_label;
-    // With col_map (up only; one multiplication per component): row r of the plane tiles is compact row
-    // col_map[r / bs] * bs + r % bs of the right operand, i.e. the planes are written in component order while the
-    // message F_i keeps the compact order.
-    const int32_t* col_map;
-    // With kmap (down only): contraction index k of the plane tiles is compact index kmap[k / bs] * bs + k % bs,
-    // i.e. the planes run over the active blocks in component order while F_i keeps the compact order.
-    const int32_t* kmap;
-};
-
-__global__ void __launch_bounds__(limb::OPEN_THREADS)
-limb_open_kernel(LimbOpenArgs a) {
-    using namespace limb;
-    pdl_wait();
-    pdl_launch_dependents();
-    const int party = blockIdx.x & 1;
-    const int bid = blockIdx.x >> 1;
-    const int tid = threadIdx.x;
-    if (bid < a.left_blocks) {
-        const ulonglong2* __restrict__ x = reinterpret_cast<const ulonglong2*>(party ? a.X[1] : a.X[0]);
-        const ulonglong2* __restrict__ m = reinterpret_cast<const ulonglong2*>(party ? a.A[1] : a.A[0]);
-        ulonglong2* __restrict__ e = reinterpret_cast<ulonglong2*>(party ? a.E[1] : a.E[0]);
-        const long long stride = (long long)a.left_blocks * OPEN_THREADS;
-        for (long long t = (long long)bid * OPEN_THREADS + tid; t < a.left_pairs; t += stride) {
-            if (a.tmask) {
-                const unsigned word = (unsigned)(2 * t), row = word / (unsigned)a.K, col = word - row * (unsigned)a.K;
-                if (a.tmask[(size_t)row * a.tmask_ld + col / (unsigned)a.bs] == 0) {
-                    e[t] = make_ulonglong2(0ull, 0ull);
-                    continue;
-                }
-            }
-            if (a.row_label && a.row_label[(unsigned)(2 * t) / (unsigned)a.K] < 0) {
-                e[t] = make_ulonglong2(0ull, 0ull);
-                continue;
-            }
-            const ulonglong2 xv = __ldcs(x + t), av = __ldcs(m + t);      // read once: leave L2 to what is written
-            e[t] = make_ulonglong2(xv.x - av.x, xv.y - av.y);
-        }
-        return;
-    }
-    extern __shared__ __align__(16) uint8_t open_smem[];      // [stage][W tile | B tile], rows of OPEN_STRIDE words
-    const int tile_id = bid - a.left_blocks;
-    const int chunk = tile_id % a.kchunks;
-    const int row0 = (tile_id / a.kchunks) * OPEN_ROWS;
-    const int kb0 = chunk * a.kb_per_cta;
-    const int kb1 = min(kb0 + a.kb_per_cta, a.kblocks);
-    const u64* __restrict__ Bi = party ? a.B[1] : a.B[0];
-    u64* __restrict__ Fi = party ? a.F[1] : a.F[0];
-    // What depends on the row alone (which row of which weight matrix is gathered, where the row lies in B_i / F_i,
-    // whether its block is in use) is worked out once per row and shared.
-    __shared__ const u64* s_wrow[OPEN_ROWS];          // first word of the gathered row of W_i; null: no such row
-    __shared__ long long s_orow[OPEN_ROWS];           // offset of the row in B_i and F_i
-    __shared__ unsigned char s_dead[OPEN_ROWS];
-    if (tid < OPEN_ROWS) {
-        int row = row0 + tid;
-        const u64* wp = nullptr;
-        long long o = 0;
-        bool dead = false;
-        if (row < a.rows) {
-            if (a.col_map) {
-                const int sb = row / a.bs;
-                row = __ldg(a.col_map + sb) * a.bs + (row - sb * a.bs);
-            }
-            if (a.down) {
-                wp = (party ? a.W0[1] : a.W0[0]) + (size_t)row * a.ldw;
-            } else {
-                const int grp = (row >= a.n) + (row >= 2 * a.n), j = row - grp * a.n;
-                const int blk = j / a.bs;
-                const int neuron = __ldg(a.ids + blk) * a.bs + (j - blk * a.bs);
-                dead = a.blk_label && a.blk_label[blk] < 0;
-                wp = (grp == 0 ? (party ? a.W0[1] : a.W0[0])
-                               : grp == 1 ? (party ? a.W1[1] : a.W1[0]) : (party ? a.W2g[1] : a.W2g[0])) +
-                     (size_t)neuron * a.ldw;
-            }
-            o = (long long)row * a.K;
-        }
-        s_wrow[tid] = wp;
-        s_orow[tid] = o;
-        s_dead[tid] = dead ? 1 : 0;
-    }
-    __syncthreads();
-
-    // This thread's part of every tile: the 16-byte column c16 (contraction indices 2 c16, 2 c16 + 1 of the k-block)
-    // of the rows rbase, rbase + 8, rbase + 16, rbase + 24.
-    const int c16 = tid & 15, rbase = tid >> 4;
-
-    // contraction index of this thread's column in k-block kb: plane position k, compact index ks, column kcol of the
-    // gathered row of W_i, and whether the block it belongs to is in use (down only)
-    auto column = [&](int kb, int& k, int& ks, int& kcol, bool& dead_k) {
-        k = kb * KC + 2 * c16;
-        ks = k;
-        if (a.kmap && k < a.K) {
-            const int sb = k / a.bs;
-            ks = __ldg(a.kmap + sb) * a.bs + (k - sb * a.bs);
-        }
-        kcol = k;
-        dead_k = false;
-        if (a.down && k < a.K) {
-            const int blk = ks / a.bs;
-            kcol = __ldg(a.ids + blk) * a.bs + (ks - blk * a.bs);
-            dead_k = a.blk_label && a.blk_label[blk] < 0;     // a block without a non-zero column of X
-        }
-    };
-    // asynchronous 16-byte copies of this thread's part of k-block kb into a stage; what lies outside the operand
-    // is filled with zeros
-    const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(open_smem);
-    auto issue = [&](int kb, int stage) {
-        int k, ks, kcol;
-        bool dead_k;
-        column(kb, k, ks, kcol, dead_k);
-        const uint32_t w_tile = smem0 + (uint32_t)stage * 2u * OPEN_TILE_BYTES, b_tile = w_tile + OPEN_TILE_BYTES;
-#pragma unroll
-        for (int i = 0; i < OPEN_ROWS / 8; ++i) {
-            const int r = rbase + 8 * i;
-            const u64* wp = s_wrow[r];
-            const bool live = wp != nullptr && k < a.K;
-            const uint32_t at = (uint32_t)(r * OPEN_STRIDE * 8 + c16 * 16);
-            limb_copy16_async(w_tile + at, live ? (const void*)(wp + kcol) : (const void*)Bi, live ? 16u : 0u);
-            limb_copy16_async(b_tile + at, live ? (const void*)(Bi + s_orow[r] + ks) : (const void*)Bi, live ? 16u : 0u);
-        }
-        limb_copy_commit();
-    };
-
-    issue(kb0, 0);
-    for (int kb = kb0; kb < kb1; ++kb) {
-        const int stage = (kb - kb0) & 1;
-        if (kb + 1 < kb1) {
-            issue(kb + 1, stage ^ 1);        // that stage was released by the barrier that ended the last round
-            limb_copy_wait<1>();
-        } else {
-            limb_copy_wait<0>();
-        }
-        __syncthreads();                     // every thread's copies of this stage have landed
-        u64* w_tile = reinterpret_cast<u64*>(open_smem + (size_t)stage * 2 * OPEN_TILE_BYTES);
-        u64* b_tile = w_tile + OPEN_ROWS * OPEN_STRIDE;
-        int k, ks, kcol;
-        bool dead_k;
-        column(kb, k, ks, kcol, dead_k);
-        // the message F_i = gather(W_i) - B_i
-#pragma unroll
-        for (int i = 0; i < OPEN_ROWS / 8; ++i) {
-            const int r = rbase + 8 * i;
-            const bool live = s_wrow[r] != nullptr && k < a.K;
-            const bool dead = dead_k || s_dead[r] != 0;
-            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(w_tile + r * OPEN_STRIDE + 2 * c16);
-            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(b_tile + r * OPEN_STRIDE + 2 * c16);
-            const ulonglong2 f = dead ? make_ulonglong2(0ull, 0ull) : make_ulonglong2(w.x - b.x, w.y - b.y);
-            if (live) *reinterpret_cast<ulonglong2*>(Fi + s_orow[r] + ks) = f;
-        }
-        // planes of B_i: 16 words of one row per thread
-        if (tid < 2 * OPEN_ROWS) {
-            const int half = tid >> 5, r = tid & 31;
-            int rin;
-            uint8_t* blk = limb_block_ptr(party ? a.Bpl[1] : a.Bpl[0], BN, row0 + r, a.kblocks, kb, &rin);
-            limb_emit_planes16(b_tile + r * OPEN_STRIDE + half * 16, half, blk, BN, rin);
-        }
-        __syncthreads();                     // the stage may be overwritten by the copies issued next round
-    }
-}
-
-// ---------------------------------------------------------------------------
-// After the exchange, one launch: everything the tensor-core kernel needs, per party.
-//   left tiles : E = E_0 + E_1 -> planes(E);  V_i = A_i + i*E -> planes(V_i)      [M, K], 128-row blocks
-//   right tiles: F = F_0 + F_1 -> planes(F)                                      [N, K],  64-row blocks
-//   copy blocks: Z_i <- C_i (the accumulation target starts from the triple's C share)
-// grid = 2 * (left_tiles + right_tiles + copy_blocks), 128 threads; a tile CTA owns 32 rows x kb_per_cta k-blocks.
-// Any part may be empty.  Dynamic shared memory: 2 stages x (3 tiles with a left part, else 2) x OPEN_TILE_BYTES.
-// The party is the lowest bit of the block index: the two parties' CTAs of one tile read the same two messages and
-// run side by side, so the second read comes from L2.  Tiles are taken from the last to the first: the kernel before
-// this one wrote the messages in ascending order, and its last tiles are the ones most likely still in L2.
-// ---------------------------------------------------------------------------
-struct LimbPrepArgs {
-    const u64* E0; const u64* E1;
-    const u64* A[2];
-    uint8_t* Epl[2];
-    uint8_t* Vpl[2];
-    int M, left_tiles;       // left_tiles = (32-row tiles of whole plane tiles) * kchunks, or 0
-    int kb_per_cta, kchunks; // k-blocks per tile CTA and CTAs per row tile: kchunks = ceil(kblocks / kb_per_cta)
-    const u64* F0; const u64* F1;
-    uint8_t* Fpl[2];
-    int N, right_tiles;      // likewise for the right operand
-    int K, kblocks;
-    const uint8_t* tmask;    // per-token mask over the active blocks (see LimbOpenArgs), or null: where it is zero
-    int tmask_ld, bs;        // the party's A_i is no part of the triple and counts as zero
-    const u64* C[2];
-    u64* Z[2];
-    long long copy_pairs;
-    int copy_blocks;
-    // One multiplication per component (up only): plane row r of the left operand is row row_map[r] of E and A_i,
-    // plane row r of the right operand is compact row col_map[r / bs] * bs + r % bs of F; M and N then count the
-    // rows and columns that lie in a component.  Null: identity.
+    // One multiplication per component: the planes are written in component order while the messages keep the compact
+    // order.  Plane row r of the left operand is row row_map[r]; of the right operand (up) compact row
+    // col_map[r / bs] * bs + r % bs; contraction index k (down) is compact index kmap[k / bs] * bs + k % bs.
+    // Null: identity.
     const int32_t* row_map;
     const int32_t* col_map;
-    // Down only: contraction index k of the planes is compact index kmap[k / bs] * bs + k % bs (both operands).
     const int32_t* kmap;
 };
 
-__global__ void __launch_bounds__(limb::OPEN_THREADS)
-limb_prep_kernel(LimbPrepArgs a) {
+template <bool LEFT>
+__device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, int block, uint8_t* smem) {
     using namespace limb;
-    pdl_wait();
-    pdl_launch_dependents();
-    const int party = blockIdx.x & 1;
-    const int tid = threadIdx.x;
-    int id = blockIdx.x >> 1;
-    if (id < a.left_tiles + a.right_tiles) {
-        id = a.left_tiles + a.right_tiles - 1 - id;
+    constexpr int TILE = LEFT ? BM : BN, BLOCK_BYTES = PLANES * TILE * KC;
+    const int c = threadIdx.x & 7;
+    const int r = (block / a.kchunks) * EX_ROWS + (threadIdx.x >> 3);                         // plane row
+    const int kb0 = (block % a.kchunks) * a.kb_per_cta, kb1 = min(kb0 + a.kb_per_cta, a.kblocks);
+    if (r >= (LEFT ? a.M : a.N)) return;         // planes of rows past the operand are never looked at
+    int at = r;                                  // compact row: where it lies in the operands and in the message
+    bool closed = false;                         // the row is not part of the message
+    const u64* src[2];                           // the row of X_i / the gathered row of W_i
+    if (LEFT) {
+        if (a.row_map) at = __ldg(a.row_map + r);
+        closed = a.row_label && __ldg(a.row_label + at) < 0;
+        src[0] = a.X[0] + (size_t)at * a.K;
+        src[1] = a.X[1] + (size_t)at * a.K;
     } else {
-        id -= a.left_tiles + a.right_tiles;
-        const ulonglong2* __restrict__ s = reinterpret_cast<const ulonglong2*>(party ? a.C[1] : a.C[0]);
-        ulonglong2* __restrict__ d = reinterpret_cast<ulonglong2*>(party ? a.Z[1] : a.Z[0]);
-        const long long stride = (long long)a.copy_blocks * OPEN_THREADS;
-        for (long long t = (long long)id * OPEN_THREADS + tid; t < a.copy_pairs; t += stride) d[t] = __ldcs(s + t);
-        return;
-    }
-    // A tile CTA owns 32 rows and kb_per_cta consecutive k-blocks and streams them through a two-stage ring of
-    // asynchronous copies, as the opening kernel does: per stage the two messages and, on the left, the party's A_i.
-    extern __shared__ __align__(16) uint8_t prep_smem[];     // [stage][message 0 | message 1 | (left) A_i]
-    const bool left = id < a.left_tiles;
-    if (!left) id -= a.left_tiles;
-    const int chunk = id % a.kchunks;
-    const int row0 = (id / a.kchunks) * OPEN_ROWS;
-    const int kb0 = chunk * a.kb_per_cta;
-    const int kb1 = min(kb0 + a.kb_per_cta, a.kblocks);
-    const int rows = left ? a.M : a.N;
-    const int tiles_per_stage = left ? 3 : 2;
-    const u64* __restrict__ in0 = left ? a.E0 : a.F0;
-    const u64* __restrict__ in1 = left ? a.E1 : a.F1;
-    const u64* __restrict__ own = party ? a.A[1] : a.A[0];
-    __shared__ int s_row[OPEN_ROWS];                  // the row of the operands a tile row stands for; -1: none
-    if (tid < OPEN_ROWS) {
-        int row = row0 + tid;
-        if (row >= rows) {
-            row = -1;
-        } else if (left) {
-            if (a.row_map) row = __ldg(a.row_map + row);
-        } else if (a.col_map) {
-            const int sb = row / a.bs;
-            row = __ldg(a.col_map + sb) * a.bs + (row - sb * a.bs);
+        if (a.col_map) {
+            const int sb = r / a.bs;
+            at = __ldg(a.col_map + sb) * a.bs + (r - sb * a.bs);
         }
-        s_row[tid] = row;
-    }
-    __syncthreads();
-
-    const int c16 = tid & 15, rbase = tid >> 4;
-    const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(prep_smem);
-    const uint32_t stage_bytes = (uint32_t)tiles_per_stage * OPEN_TILE_BYTES;
-    // plane position k of this thread's column in k-block kb and its compact contraction index ks
-    auto column = [&](int kb, int& k, int& ks) {
-        k = kb * KC + 2 * c16;
-        ks = k;
-        if (a.kmap && k < a.K) {
-            const int sb = k / a.bs;
-            ks = __ldg(a.kmap + sb) * a.bs + (k - sb * a.bs);
-        }
-    };
-    auto issue = [&](int kb, int stage) {
-        int k, ks;
-        column(kb, k, ks);
-        const uint32_t t0 = smem0 + (uint32_t)stage * stage_bytes;
-#pragma unroll
-        for (int i = 0; i < OPEN_ROWS / 8; ++i) {
-            const int r = rbase + 8 * i;
-            const int row = s_row[r];
-            const bool live = row >= 0 && k < a.K;
-            const size_t o = live ? (size_t)row * a.K + ks : 0;
-            const uint32_t at = (uint32_t)(r * OPEN_STRIDE * 8 + c16 * 16);
-            limb_copy16_async(t0 + at, in0 + o, live ? 16u : 0u);
-            limb_copy16_async(t0 + OPEN_TILE_BYTES + at, in1 + o, live ? 16u : 0u);
-            if (left) limb_copy16_async(t0 + 2 * OPEN_TILE_BYTES + at, own + o, live ? 16u : 0u);
-        }
-        limb_copy_commit();
-    };
-
-    issue(kb0, 0);
-    for (int kb = kb0; kb < kb1; ++kb) {
-        const int stage = (kb - kb0) & 1;
-        if (kb + 1 < kb1) {
-            issue(kb + 1, stage ^ 1);        // that stage was released by the barrier that ended the last round
-            limb_copy_wait<1>();
+        if (a.down) {
+            src[0] = a.W0[0] + (size_t)at * a.ldw;
+            src[1] = a.W0[1] + (size_t)at * a.ldw;
         } else {
-            limb_copy_wait<0>();
+            const int grp = (at >= a.n) + (at >= 2 * a.n), j = at - grp * a.n, blk = j / a.bs;
+            const size_t off = (size_t)(__ldg(a.ids + blk) * a.bs + (j - blk * a.bs)) * a.ldw;
+            closed = a.blk_label && __ldg(a.blk_label + blk) < 0;
+            src[0] = (grp == 0 ? a.W0[0] : grp == 1 ? a.W1[0] : a.W2[0]) + off;
+            src[1] = (grp == 0 ? a.W0[1] : grp == 1 ? a.W1[1] : a.W2[1]) + off;
         }
-        __syncthreads();                     // every thread's copies of this stage have landed
-        u64* t_sum = reinterpret_cast<u64*>(prep_smem + (size_t)stage * stage_bytes);      // message 0, then the sum
-        u64* t_in1 = t_sum + OPEN_ROWS * OPEN_STRIDE;
-        u64* t_own = t_in1 + OPEN_ROWS * OPEN_STRIDE;                                       // A_i, then V_i (left)
-        int k, ks;
-        column(kb, k, ks);
+    }
+    const u64* own[2];                           // the row of A_i / B_i
+    u64* msg[2];                                 // the row of E_i / F_i
+    uint8_t* pl[3];                              // this lane's cell in the planes of V_0 / B_0, V_1 / B_1, E / F
+    const size_t cell = ((size_t)(r / TILE) * a.kblocks + kb0) * BLOCK_BYTES +
+                        (size_t)((r % TILE >> 3) * 256 + (c >> 2) * 128 + (r & 7) * 16 + (c & 3) * 4);
 #pragma unroll
-        for (int i = 0; i < OPEN_ROWS / 8; ++i) {
-            const int r = rbase + 8 * i;
-            const int at = r * OPEN_STRIDE + 2 * c16;
-            ulonglong2* sv = reinterpret_cast<ulonglong2*>(t_sum + at);
-            const ulonglong2 x = *sv, y = *reinterpret_cast<const ulonglong2*>(t_in1 + at);
-            const ulonglong2 sum = make_ulonglong2(x.x + y.x, x.y + y.y);       // the exchange: both messages summed
-            *sv = sum;
-            if (left) {
-                // where the per-token mask is zero the party's A_i is no part of the triple and counts as zero
-                const int row = s_row[r];
-                const bool own_part = row >= 0 && k < a.K &&
-                                      (!a.tmask || a.tmask[(size_t)row * a.tmask_ld + ks / a.bs] != 0);
-                ulonglong2* ov = reinterpret_cast<ulonglong2*>(t_own + at);
-                const ulonglong2 z = *ov;
-                *ov = own_part ? make_ulonglong2(z.x + (party ? sum.x : 0ull), z.y + (party ? sum.y : 0ull))   // V_i = A_i + i*E
-                               : make_ulonglong2(0ull, 0ull);
+    for (int p = 0; p < 2; ++p) {
+        own[p] = (LEFT ? a.A[p] : a.B[p]) + (size_t)at * a.K;
+        msg[p] = (LEFT ? a.E[p] : a.F[p]) + (size_t)at * a.K;
+        pl[p] = (LEFT ? a.Vpl[p] : a.Bpl[p]) + cell;
+    }
+    pl[2] = (LEFT ? a.Epl : a.Fpl) + cell;
+
+    // This lane's piece h of k-block kb: compact index of its first word, its column in W, and whether it exists and is part
+    // of the message.  Sixteen indices aligned to 16 lie in one block.
+    struct Piece { int ks, col; bool in, open; };
+    auto piece = [&](int kb, int h) {
+        Piece q;
+        const int k = kb * KC + 16 * h;
+        q.ks = q.col = k + 2 * c;
+        q.in = q.ks < a.K;
+        q.open = q.in && !closed;
+        if (a.down && q.in) {
+            int blk = k / a.bs;
+            const int within = k - blk * a.bs + 2 * c;
+            if (a.kmap) blk = __ldg(a.kmap + blk);
+            q.ks = q.col = blk * a.bs + within;
+            if (!LEFT) {
+                q.col = __ldg(a.ids + blk) * a.bs + within;
+                if (a.blk_label && __ldg(a.blk_label + blk) < 0) q.open = false;
+            } else if (a.tmask && a.tmask[(size_t)at * a.tmask_ld + blk] == 0) {
+                q.open = q.in = false;           // an entry off the support is none of the triple either
             }
         }
-        __syncthreads();                     // the planes are built from words other threads wrote
-        // threads 0-63: planes of the summed message; threads 64-127 (left only): planes of V_i; 16 words of a row each
-        const int which = tid >> 6, half = (tid >> 5) & 1, r = tid & 31;
-        if (which == 0 || left) {
-            const int tile_rows = left ? BM : BN;
-            uint8_t* base = left ? (which ? (party ? a.Vpl[1] : a.Vpl[0]) : (party ? a.Epl[1] : a.Epl[0]))
-                                 : (party ? a.Fpl[1] : a.Fpl[0]);
-            int rin;
-            uint8_t* blk = limb_block_ptr(base, tile_rows, row0 + r, a.kblocks, kb, &rin);
-            limb_emit_planes16((which ? t_own : t_sum) + r * OPEN_STRIDE + half * 16, half, blk, tile_rows, rin);
+        return q;
+    };
+    const uint32_t mine = (uint32_t)__cvta_generic_to_shared(smem) + threadIdx.x * 16;
+    auto issue = [&](int kb) {
+        const uint32_t stage = mine + (uint32_t)((kb - kb0) % EX_STAGES) * EX_STAGE_BYTES;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const Piece q = piece(kb, h);
+            const uint32_t bytes = q.in ? 16u : 0u;
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                limb_copy16_async(stage + (uint32_t)(4 * h + 2 * p) * (16 * EX_THREADS), q.in ? src[p] + q.col : own[p], bytes);
+                limb_copy16_async(stage + (uint32_t)(4 * h + 2 * p + 1) * (16 * EX_THREADS), q.in ? own[p] + q.ks : own[p], bytes);
+            }
         }
-        __syncthreads();                     // the stage may be overwritten by the copies issued next round
+    };
+#pragma unroll
+    for (int s = 0; s < EX_STAGES - 1; ++s) {
+        if (kb0 + s < kb1) issue(kb0 + s);
+        limb_copy_commit();
     }
+    for (int kb = kb0; kb < kb1; ++kb) {
+        if (kb + EX_STAGES - 1 < kb1) issue(kb + EX_STAGES - 1);
+        limb_copy_commit();
+        limb_copy_wait<EX_STAGES - 1>();
+        const uint8_t* stage = smem + (size_t)((kb - kb0) % EX_STAGES) * EX_STAGE_BYTES + threadIdx.x * 16;
+        u64 f[2][4], b[2][4];                    // X_i / W_i, then the message; A_i / B_i
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const Piece q = piece(kb, h);
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(stage + (4 * h + 2 * p) * (16 * EX_THREADS));
+                const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(stage + (4 * h + 2 * p + 1) * (16 * EX_THREADS));
+                b[p][2 * h] = m.x;
+                b[p][2 * h + 1] = m.y;
+                f[p][2 * h] = q.open ? x.x - m.x : 0ull;
+                f[p][2 * h + 1] = q.open ? x.y - m.y : 0ull;
+                if (kb * KC + 16 * h + 2 * c < a.K)
+                    *reinterpret_cast<ulonglong2*>(msg[p] + q.ks) = make_ulonglong2(f[p][2 * h], f[p][2 * h + 1]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            f[0][e] += f[1][e];                  // the exchange
+            if (LEFT) b[1][e] += f[0][e];        // V_1 = A_1 + E  (V_0 = A_0)
+        }
+        limb_emit4(pl[0], TILE * KC, b[0]);
+        limb_emit4(pl[1], TILE * KC, b[1]);
+        limb_emit4(pl[2], TILE * KC, f[0]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) pl[i] += BLOCK_BYTES;
+    }
+    limb_copy_wait<0>();
+}
+
+__global__ void __launch_bounds__(limb::EX_THREADS, 7)
+limb_exchange_kernel(const __grid_constant__ LimbExchangeArgs a) {
+    pdl_wait();
+    pdl_launch_dependents();
+    int block = blockIdx.x;
+    extern __shared__ __align__(16) uint8_t ex_smem[];
+    if (block < a.left_blocks) return limb_exchange_rows<true>(a, block, ex_smem);
+    block -= a.left_blocks;
+    if (block < a.right_blocks) return limb_exchange_rows<false>(a, block, ex_smem);
+    block -= a.right_blocks;
+    const int party = block & 1;
+    const ulonglong2* __restrict__ s = reinterpret_cast<const ulonglong2*>(party ? a.C[1] : a.C[0]);
+    ulonglong2* __restrict__ d = reinterpret_cast<ulonglong2*>(party ? a.Z[1] : a.Z[0]);
+    const long long stride = (long long)(a.copy_blocks >> 1) * limb::EX_THREADS;
+    for (long long t = (long long)(block >> 1) * limb::EX_THREADS + threadIdx.x; t < a.copy_pairs; t += stride) d[t] = __ldcs(s + t);
 }
 
 // ---------------------------------------------------------------------------
@@ -829,10 +632,10 @@ token_plan_kernel(TokenPlanArgs a) {
 }
 
 struct LimbArgs {
-    const uint8_t* Epl[2];   // left planes of E = E_0 + E_1, per party: [m-tile][k-block][32 KiB]
+    const uint8_t* Epl;      // left planes of E = E_0 + E_1: [m-tile][k-block][32 KiB]
     const uint8_t* Vpl[2];   // left planes of V_i = A_i + i*E
     const uint8_t* Bpl[2];   // right planes of B_i: [n-tile][k-block][16 KiB]
-    const uint8_t* Fpl[2];   // right planes of F = F_0 + F_1
+    const uint8_t* Fpl;      // right planes of F = F_0 + F_1
     u64* Z[2];               // [M, N], pre-loaded with C_i; partial sums are added with bulk reductions
     int M, N;                // N a multiple of 16
     int mt, nt, kb;          // tiles and k-blocks per operand pair; one tile runs over 2*kb blocks
@@ -1018,9 +821,9 @@ __device__ __forceinline__ void combine_limb_body(const LimbArgs a) {
                 const int klo = GROUPED ? sg.klo : 0;         // and where they start in the plane tile
                 bool second = kpos >= kbe;
                 if (second) kpos -= kbe;
-                const uint8_t* left = (second ? (sg.party ? a.Vpl[1] : a.Vpl[0]) : (sg.party ? a.Epl[1] : a.Epl[0])) +
+                const uint8_t* left = (second ? (sg.party ? a.Vpl[1] : a.Vpl[0]) : a.Epl) +
                                       ((size_t)sg.tm * a.kb + klo + kpos) * A_BLOCK_BYTES;
-                const uint8_t* right = (second ? (sg.party ? a.Fpl[1] : a.Fpl[0]) : (sg.party ? a.Bpl[1] : a.Bpl[0])) +
+                const uint8_t* right = (second ? a.Fpl : (sg.party ? a.Bpl[1] : a.Bpl[0])) +
                                        ((size_t)sg.tn * a.kb + klo + kpos) * B_BLOCK_BYTES;
                 for (int it = 0; it < sg.count; ++it) {
                     ok = limb_wait(empty0 + 8 * stage, phase ^ 1u, &abort_flag);
@@ -1038,7 +841,7 @@ __device__ __forceinline__ void combine_limb_body(const LimbArgs a) {
                         second = true;
                         kpos = 0;
                         left = (sg.party ? a.Vpl[1] : a.Vpl[0]) + ((size_t)sg.tm * a.kb + klo) * A_BLOCK_BYTES;
-                        right = (sg.party ? a.Fpl[1] : a.Fpl[0]) + ((size_t)sg.tn * a.kb + klo) * B_BLOCK_BYTES;
+                        right = a.Fpl + ((size_t)sg.tn * a.kb + klo) * B_BLOCK_BYTES;
                     }
                 }
             }

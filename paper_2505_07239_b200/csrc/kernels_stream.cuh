@@ -28,9 +28,7 @@
 // parties x eight accumulators x 32 tokens).  The planes are single-buffered: converting a step and multiplying it take
 // turns, while the ring and the converters' registers keep up to 160 KiB of loads in flight.
 //
-// Inside a 32-deep step the contraction indices sit in the planes in the order the converters hold them: a lane reads
-// two 16-byte pieces of a row, 16 words apart, so that eight lanes read whole 128-byte lines, and writes its four
-// words' bytes next to each other.  Both operands use that order, so the sum over the step is the same.
+// The contraction indices of a step sit in the planes in limb_emit4's order (kernels_limb.cuh).
 //
 // Work is cut stream-K style like the other tensor-core kernel's: the (feature tile, token tile, step) space in equal
 // contiguous ranges, a step weighted by the number of raw slots it takes (a ragged last tile takes fewer).
@@ -135,16 +133,6 @@ __device__ __forceinline__ void stream_copy16(uint32_t dst, const void* src) {
 }
 __device__ __forceinline__ void stream_copies_arrive(uint32_t bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-// Four words of one row -> eight planes, four bytes each, `stride` bytes apart.
-__device__ __forceinline__ void stream_emit4(uint8_t* dst, int stride, const u64* w) {
-    uint32_t p[8];
-    limb_transpose4((uint32_t)w[0], (uint32_t)w[1], (uint32_t)w[2], (uint32_t)w[3], p[0], p[1], p[2], p[3]);
-    limb_transpose4((uint32_t)(w[0] >> 32), (uint32_t)(w[1] >> 32), (uint32_t)(w[2] >> 32), (uint32_t)(w[3] >> 32),
-                    p[4], p[5], p[6], p[7]);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) *reinterpret_cast<uint32_t*>(dst + i * stride) = p[i];
 }
 
 __global__ void __launch_bounds__(limb_stream::THREADS, 1)
@@ -327,11 +315,11 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a) {
                     uint8_t* to = sB + q * (QROWS / 8) * 256 + cell;
                     // a step's first planes: the MMAs of the step before must have read the old ones
                     if (first) ok = limb_wait(ptx::smem_u32(&own_empty[0]), unit_phase ^ 1u, &abort_flag);
-                    stream_emit4(to, W_PLANE_BYTES, b[0]);
+                    limb_emit4(to, W_PLANE_BYTES, b[0]);
                     if (first) ok = ok && limb_wait(ptx::smem_u32(&own_empty[1]), unit_phase ^ 1u, &abort_flag);
-                    stream_emit4(to + W_SET_BYTES, W_PLANE_BYTES, b[1]);
+                    limb_emit4(to + W_SET_BYTES, W_PLANE_BYTES, b[1]);
                     if (first) ok = ok && limb_wait(ptx::smem_u32(&shared_empty), unit_phase ^ 1u, &abort_flag);
-                    stream_emit4(to + 2 * W_SET_BYTES, W_PLANE_BYTES, f[0]);
+                    limb_emit4(to + 2 * W_SET_BYTES, W_PLANE_BYTES, f[0]);
                     first = false;
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
@@ -400,9 +388,9 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a) {
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 if (live) {                                      // planes of rows past the last token are never looked at
-                    stream_emit4(to, T_PLANE_BYTES, v[0]);
-                    stream_emit4(to + T_SET_BYTES, T_PLANE_BYTES, v[1]);
-                    stream_emit4(to + 2 * T_SET_BYTES, T_PLANE_BYTES, e[0]);
+                    limb_emit4(to, T_PLANE_BYTES, v[0]);
+                    limb_emit4(to + T_SET_BYTES, T_PLANE_BYTES, v[1]);
+                    limb_emit4(to + 2 * T_SET_BYTES, T_PLANE_BYTES, e[0]);
                 }
                 ptx::fence_proxy_async_smem();
                 __syncwarp();

@@ -348,9 +348,9 @@ int comet_last_cuda_error(comet_ctx* ctx);
  *
  * Stateless: no context and no memory of the library's own.  Every pointer is a
  * DEVICE pointer on the current device, owned by the caller; X, a, b are only
- * read, Y and Z are overwritten and must not overlap any other argument.  Two
- * kernels are enqueued on `cuda_stream` (NULL = default stream); the call does
- * not wait for them.  16-byte accesses are used when cols is even and X, a, b,
+ * read, Y and Z are overwritten and must not overlap any other argument.  The
+ * work is enqueued on `cuda_stream` (NULL = default stream): one kernel, or two
+ * when a matrix has more than 2^21 words; the call does not wait for it.  16-byte accesses are used when cols is even and X, a, b,
  * Y, Z are 16-byte aligned, 8-byte accesses otherwise.
  * A permutation entry outside [0, rows) is never followed: the row it would
  * have fetched counts as zero and, if `bad_index_flag` (device int32, may be
@@ -385,7 +385,7 @@ int comet_add_bias(void* cuda_stream, uint64_t* const Z[2], const uint64_t* cons
  * comet_truncate, which needs no dealer material and no message.
  * Stateless; DEVICE pointers on the current device to `count` words each, owned
  * by the caller; R, RP are only read, Z is replaced, M is overwritten and must not
- * overlap the others.  Two kernels on `cuda_stream`; the call does not wait.
+ * overlap the others.  One kernel on `cuda_stream`; the call does not wait.
  * Errors: INVALID_ARG (null pointer), SHAPE (count < 1, frac_bits outside [1, 31]), CUDA. */
 int comet_truncate_pair(void* cuda_stream, uint64_t* const Z[2], const uint64_t* const R[2],
                         const uint64_t* const RP[2], uint64_t* const M[2], int64_t count, int32_t frac_bits);
@@ -418,7 +418,7 @@ int comet_kv_plan(const uint8_t* present, const uint8_t* active, int32_t tokens,
  * is at scale 2f when both factors are at scale f; truncate it afterwards.
  * Stateless; all pointers are DEVICE pointers on the current device to `count`
  * words each, owned by the caller; D, E, Z are overwritten and must not overlap
- * the inputs.  Two kernels are enqueued on `cuda_stream`; the call does not wait.
+ * the inputs.  One kernel is enqueued on `cuda_stream`; the call does not wait.
  * Errors: INVALID_ARG (null pointer), SHAPE (count < 1), CUDA. */
 int comet_beaver_mul(void* cuda_stream, const uint64_t* const X[2], const uint64_t* const Y[2],
                      const uint64_t* const A[2], const uint64_t* const B[2], const uint64_t* const C[2],

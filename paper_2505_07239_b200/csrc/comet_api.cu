@@ -1267,6 +1267,11 @@ int shuffle_grid(long long items) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// One pass over both steps reads X and a twice, the second time from L2 if they stay there: up to 2^21 words per matrix, when
+// the four matrices take half of it.  One pass against two at 512 x 2048: 24 and 30 us, 512 x 4096 (2^21 words): 34 and 37 us,
+// 768 x 4096: 52 and 52 us, 1024 x 4096: 70 and 66 us.
+bool shuffle_in_one_pass(int64_t rows, int64_t cols) { return rows <= (int64_t)(1 << 21) / cols; }
+
 // out_i = in_i[perm_i] +/- mask_i for both parties, one launch
 int launch_shuffle_step(cudaStream_t stream, const uint64_t* const in[2], const int32_t* const perm[2],
                         const uint64_t* const mask[2], uint64_t* const out[2], int64_t rows, int64_t cols,
@@ -1304,6 +1309,29 @@ extern "C" int comet_shuffle(void* cuda_stream, const uint64_t* const X[2], cons
         if (!X[p] || !tau[p] || !rho[p] || !a[p] || !b[p] || !Y[p] || !Z[p]) return COMET_ERR_INVALID_ARG;
     if (rows < 1 || cols < 1 || rows > 0x7fffffffll || cols > 0x7fffffffll) return COMET_ERR_SHAPE;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
+    if (shuffle_in_one_pass(rows, cols)) {
+        comet::ShuffleBothArgs g;
+        bool vec = (cols % 2) == 0;
+        for (int p = 0; p < 2; ++p) {
+            g.x[p] = reinterpret_cast<const u64*>(X[p]);
+            g.a[p] = reinterpret_cast<const u64*>(a[p]);
+            g.b[p] = reinterpret_cast<const u64*>(b[p]);
+            g.y[p] = reinterpret_cast<u64*>(Y[p]);
+            g.z[p] = reinterpret_cast<u64*>(Z[p]);
+            g.tau[p] = tau[p];
+            g.rho[p] = rho[p];
+            vec = vec && aligned16(X[p]) && aligned16(a[p]) && aligned16(b[p]) && aligned16(Y[p]) && aligned16(Z[p]);
+        }
+        g.rows = rows;
+        g.pieces = (int)(vec ? cols / 2 : cols);
+        g.bad_index = bad_index_flag;
+        const int grid = shuffle_grid(rows * g.pieces);
+        g.stride_rows = (long long)grid * 256 / g.pieces;
+        g.stride_pieces = (int)((long long)grid * 256 % g.pieces);
+        auto* kernel = vec ? comet::shuffle_both_kernel<ulonglong2> : comet::shuffle_both_kernel<u64>;
+        kernel<<<grid, 256, 0, stream>>>(g);
+        return cudaGetLastError() == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
+    }
     // [y]_i = tau_i([x]_i) + a_i
     int rc = launch_shuffle_step(stream, X, tau, a, Y, rows, cols, 0, bad_index_flag);
     if (rc != COMET_OK) return rc;
@@ -1343,15 +1371,8 @@ extern "C" int comet_beaver_mul(void* cuda_stream, const uint64_t* const X[2], c
               aligned16(D[p]) && aligned16(E[p]) && aligned16(Z[p]);
     }
     g.pieces = vec ? count / 2 : count;
-    cudaStream_t stream = (cudaStream_t)cuda_stream;
-    const dim3 grid(shuffle_grid(g.pieces), 2);
-    if (vec) {
-        comet::beaver_mul_open_kernel<ulonglong2><<<grid, 256, 0, stream>>>(g);
-        comet::beaver_mul_combine_kernel<ulonglong2><<<grid, 256, 0, stream>>>(g);      // after the exchange
-    } else {
-        comet::beaver_mul_open_kernel<u64><<<grid, 256, 0, stream>>>(g);
-        comet::beaver_mul_combine_kernel<u64><<<grid, 256, 0, stream>>>(g);
-    }
+    auto* kernel = vec ? comet::beaver_mul_kernel<ulonglong2> : comet::beaver_mul_kernel<u64>;
+    kernel<<<shuffle_grid(g.pieces), 256, 0, (cudaStream_t)cuda_stream>>>(g);
     return cudaGetLastError() == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
 }
 
@@ -1375,15 +1396,8 @@ extern "C" int comet_truncate_pair(void* cuda_stream, uint64_t* const Z[2], cons
     }
     g.pieces = vec ? count / 2 : count;
     g.f = frac_bits;
-    cudaStream_t stream = (cudaStream_t)cuda_stream;
-    const dim3 grid(shuffle_grid(g.pieces), 2);
-    if (vec) {
-        comet::trunc_pair_open_kernel<ulonglong2><<<grid, 256, 0, stream>>>(g);
-        comet::trunc_pair_combine_kernel<ulonglong2><<<grid, 256, 0, stream>>>(g);      // after the exchange
-    } else {
-        comet::trunc_pair_open_kernel<u64><<<grid, 256, 0, stream>>>(g);
-        comet::trunc_pair_combine_kernel<u64><<<grid, 256, 0, stream>>>(g);
-    }
+    auto* kernel = vec ? comet::trunc_pair_kernel<ulonglong2> : comet::trunc_pair_kernel<u64>;
+    kernel<<<shuffle_grid(g.pieces), 256, 0, (cudaStream_t)cuda_stream>>>(g);
     return cudaGetLastError() == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
 }
 
@@ -1427,13 +1441,18 @@ extern "C" int comet_add_bias(void* cuda_stream, uint64_t* const Z[2], const uin
     if (!Z || !bias || !Z[0] || !Z[1] || !bias[0] || !bias[1]) return COMET_ERR_INVALID_ARG;
     if (rows < 1 || cols < 1 || cols > 0x7fffffffll) return COMET_ERR_SHAPE;
     comet::BiasArgs g;
+    bool vec = (cols % 2) == 0;
     for (int p = 0; p < 2; ++p) {
         g.z[p] = reinterpret_cast<u64*>(Z[p]);
         g.bias[p] = reinterpret_cast<const u64*>(bias[p]);
+        vec = vec && aligned16(Z[p]) && aligned16(bias[p]);
     }
-    g.rows = rows;
-    g.cols = (int)cols;
-    comet::add_bias_kernel<<<dim3(shuffle_grid(rows * cols), 2), 256, 0, (cudaStream_t)cuda_stream>>>(g);
+    g.pieces = (int)(vec ? cols / 2 : cols);
+    g.total = rows * g.pieces;
+    const int grid = shuffle_grid(g.total);
+    g.stride_pieces = (int)((long long)grid * 256 % g.pieces);
+    auto* kernel = vec ? comet::add_bias_kernel<ulonglong2> : comet::add_bias_kernel<u64>;
+    kernel<<<grid, 256, 0, (cudaStream_t)cuda_stream>>>(g);
     return cudaGetLastError() == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
 }
 

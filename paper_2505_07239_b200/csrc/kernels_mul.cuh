@@ -3,7 +3,10 @@
 //   open   : [d]_i = [x]_i - [a]_i,  [e]_i = [y]_i - [b]_i                       (before the exchange)
 //   combine: d = [d]_0 + [d]_1, e = [e]_0 + [e]_1,
 //            [z]_i = [c]_i + d*[b]_i + e*[a]_i + i*d*e                           (after it)
-// HBM-bound; 16-byte accesses when the word count is even and the pointers allow it; blockIdx.y is the party.
+// Bound by memory: eight words per element and party (five in, two messages and the result out).  One pass: a thread has
+// both parties' words of its elements, which is the exchange, so nobody reads a message back (as two passes, with the
+// messages read by both parties, eleven words and a second launch).  16-byte accesses when the word count is even and the
+// pointers allow it.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -36,36 +39,29 @@ __device__ __forceinline__ ulonglong2 mul_combine(ulonglong2 c, ulonglong2 d0, u
 
 template <typename PIECE>
 __global__ void __launch_bounds__(256)
-beaver_mul_open_kernel(MulArgs g) {
-    const int party = blockIdx.y;
-    const PIECE* __restrict__ x = reinterpret_cast<const PIECE*>(party ? g.x[1] : g.x[0]);
-    const PIECE* __restrict__ y = reinterpret_cast<const PIECE*>(party ? g.y[1] : g.y[0]);
-    const PIECE* __restrict__ a = reinterpret_cast<const PIECE*>(party ? g.a[1] : g.a[0]);
-    const PIECE* __restrict__ b = reinterpret_cast<const PIECE*>(party ? g.b[1] : g.b[0]);
-    PIECE* __restrict__ d = reinterpret_cast<PIECE*>(party ? g.d[1] : g.d[0]);
-    PIECE* __restrict__ e = reinterpret_cast<PIECE*>(party ? g.e[1] : g.e[0]);
+beaver_mul_kernel(const __grid_constant__ MulArgs g) {
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < g.pieces; t += stride) {
-        d[t] = mul_sub(__ldg(x + t), __ldg(a + t));
-        e[t] = mul_sub(__ldg(y + t), __ldg(b + t));
+        PIECE x[2], y[2], a[2], b[2], c[2];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            x[p] = __ldcs(reinterpret_cast<const PIECE*>(g.x[p]) + t);
+            a[p] = __ldcs(reinterpret_cast<const PIECE*>(g.a[p]) + t);
+            y[p] = __ldcs(reinterpret_cast<const PIECE*>(g.y[p]) + t);
+            b[p] = __ldcs(reinterpret_cast<const PIECE*>(g.b[p]) + t);
+            c[p] = __ldcs(reinterpret_cast<const PIECE*>(g.c[p]) + t);
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            x[p] = mul_sub(x[p], a[p]);                      // [d]_i
+            y[p] = mul_sub(y[p], b[p]);                      // [e]_i
+            reinterpret_cast<PIECE*>(g.d[p])[t] = x[p];
+            reinterpret_cast<PIECE*>(g.e[p])[t] = y[p];
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p)
+            reinterpret_cast<PIECE*>(g.z[p])[t] = mul_combine(c[p], x[0], x[1], y[0], y[1], a[p], b[p], p);
     }
-}
-
-template <typename PIECE>
-__global__ void __launch_bounds__(256)
-beaver_mul_combine_kernel(MulArgs g) {
-    const int party = blockIdx.y;
-    const PIECE* __restrict__ d0 = reinterpret_cast<const PIECE*>(g.d[0]);
-    const PIECE* __restrict__ d1 = reinterpret_cast<const PIECE*>(g.d[1]);
-    const PIECE* __restrict__ e0 = reinterpret_cast<const PIECE*>(g.e[0]);
-    const PIECE* __restrict__ e1 = reinterpret_cast<const PIECE*>(g.e[1]);
-    const PIECE* __restrict__ a = reinterpret_cast<const PIECE*>(party ? g.a[1] : g.a[0]);
-    const PIECE* __restrict__ b = reinterpret_cast<const PIECE*>(party ? g.b[1] : g.b[0]);
-    const PIECE* __restrict__ c = reinterpret_cast<const PIECE*>(party ? g.c[1] : g.c[0]);
-    PIECE* __restrict__ z = reinterpret_cast<PIECE*>(party ? g.z[1] : g.z[0]);
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < g.pieces; t += stride)
-        z[t] = mul_combine(__ldg(c + t), d0[t], d1[t], e0[t], e1[t], __ldg(a + t), __ldg(b + t), party);
 }
 
 // Truncation by f bits with a dealer's pair (r, r' = floor(r / 2^f), r read as signed).  Not a protocol of the
@@ -89,47 +85,55 @@ __device__ __forceinline__ ulonglong2 trunc_pair_out(ulonglong2 rp, ulonglong2 m
     return make_ulonglong2(trunc_pair_out(rp.x, m0.x, m1.x, f, party), trunc_pair_out(rp.y, m0.y, m1.y, f, party));
 }
 
+// One pass over both parties, as above.
 template <typename PIECE>
 __global__ void __launch_bounds__(256)
-trunc_pair_open_kernel(TruncPairArgs g) {
-    const int party = blockIdx.y;
-    const PIECE* __restrict__ z = reinterpret_cast<const PIECE*>(party ? g.z[1] : g.z[0]);
-    const PIECE* __restrict__ r = reinterpret_cast<const PIECE*>(party ? g.r[1] : g.r[0]);
-    PIECE* __restrict__ m = reinterpret_cast<PIECE*>(party ? g.m[1] : g.m[0]);
+trunc_pair_kernel(const __grid_constant__ TruncPairArgs g) {
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < g.pieces; t += stride)
-        m[t] = mul_sub(z[t], __ldg(r + t));
-}
-
-template <typename PIECE>
-__global__ void __launch_bounds__(256)
-trunc_pair_combine_kernel(TruncPairArgs g) {
-    const int party = blockIdx.y;
-    const PIECE* __restrict__ m0 = reinterpret_cast<const PIECE*>(g.m[0]);
-    const PIECE* __restrict__ m1 = reinterpret_cast<const PIECE*>(g.m[1]);
-    const PIECE* __restrict__ rp = reinterpret_cast<const PIECE*>(party ? g.rp[1] : g.rp[0]);
-    PIECE* __restrict__ z = reinterpret_cast<PIECE*>(party ? g.z[1] : g.z[0]);
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < g.pieces; t += stride)
-        z[t] = trunc_pair_out(__ldg(rp + t), m0[t], m1[t], g.f, party);
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < g.pieces; t += stride) {
+        PIECE m[2], rp[2];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            rp[p] = __ldcs(reinterpret_cast<const PIECE*>(g.rp[p]) + t);
+            m[p] = mul_sub(reinterpret_cast<const PIECE*>(g.z[p])[t], __ldcs(reinterpret_cast<const PIECE*>(g.r[p]) + t));
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            reinterpret_cast<PIECE*>(g.m[p])[t] = m[p];
+            reinterpret_cast<PIECE*>(g.z[p])[t] = trunc_pair_out(rp[p], m[0], m[1], g.f, p);
+        }
+    }
 }
 
 // Section 2.1 "Addition": a shared bias [cols] added to every row of a shared matrix, in place; purely local.
+// Bound by memory (one word in, one out per element); 16-byte pieces when the column count and the pointers allow it, and
+// the position in the row is carried along instead of divided out per element.
 struct BiasArgs {
     u64* z[2];
     const u64* bias[2];
-    long long rows;
-    int cols;
+    long long total;             // pieces of the whole matrix
+    int pieces;                  // pieces per row
+    int stride_pieces;           // (gridDim.x * blockDim.x) % pieces
 };
 
+__device__ __forceinline__ ulonglong2 mul_add(ulonglong2 p, ulonglong2 q) { return make_ulonglong2(p.x + q.x, p.y + q.y); }
+__device__ __forceinline__ u64 mul_add(u64 p, u64 q) { return p + q; }
+
+template <typename PIECE>
 __global__ void __launch_bounds__(256)
-add_bias_kernel(BiasArgs g) {
-    const int party = blockIdx.y;
-    u64* __restrict__ z = party ? g.z[1] : g.z[0];
-    const u64* __restrict__ b = party ? g.bias[1] : g.bias[0];
-    const long long total = g.rows * g.cols, stride = (long long)gridDim.x * blockDim.x;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride)
-        z[t] += __ldg(b + (int)(t % g.cols));
+add_bias_kernel(const __grid_constant__ BiasArgs g) {
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    int piece = (int)(t % g.pieces);
+    for (; t < g.total; t += stride) {
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            PIECE* z = reinterpret_cast<PIECE*>(g.z[p]) + t;
+            *z = mul_add(*z, __ldg(reinterpret_cast<const PIECE*>(g.bias[p]) + piece));
+        }
+        piece += g.stride_pieces;
+        if (piece >= g.pieces) piece -= g.pieces;
+    }
 }
 
 }  // namespace comet

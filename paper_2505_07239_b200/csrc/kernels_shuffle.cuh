@@ -72,6 +72,76 @@ shuffle_rows_kernel(ShuffleArgs a) {
     }
 }
 
+// Both steps in one pass: [y]_i = tau_i([x]_i) + a_i is written as the message, and [z]_i = rho_i([y]_other) - b_i takes its
+// rows of the other party's message from the words they are made of instead of waiting for them: row j of z_i is
+// x_other[tau_other[r]] + a_other[r] - b_i[j] with r = rho_i[j].  Five words per element and party cross HBM, as the protocol
+// has it, as long as X and a stay in L2 for their second use; see shuffle_in_one_pass in comet_api.cu.
+struct ShuffleBothArgs {
+    const u64* x[2];
+    const int32_t* tau[2];
+    const int32_t* rho[2];
+    const u64* a[2];
+    const u64* b[2];
+    u64* y[2];
+    u64* z[2];
+    long long rows;
+    int pieces;
+    long long stride_rows;
+    int stride_pieces;
+    int* bad_index;
+};
+
+template <typename PIECE>
+__global__ void __launch_bounds__(256)
+shuffle_both_kernel(const __grid_constant__ ShuffleBothArgs g) {
+    const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    long long row = first / g.pieces;
+    int piece = (int)(first - row * g.pieces);
+    while (row < g.rows) {
+        const long long at = row * g.pieces + piece;
+        // A permutation entry out of range is never followed: the row it would have fetched counts as zero.  (Row 0 is read in
+        // its place, so that every load of a piece is in flight before the first is needed.)
+        long long src[2], r[2], far[2];
+        bool src_ok[2], r_ok[2], far_ok[2];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            src[p] = g.tau[p][row];
+            r[p] = g.rho[p][row];
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            src_ok[p] = src[p] >= 0 && src[p] < g.rows;
+            r_ok[p] = r[p] >= 0 && r[p] < g.rows;
+            if (!src_ok[p]) src[p] = 0;
+            if (!r_ok[p]) r[p] = 0;
+            far[p] = g.tau[p ^ 1][r[p]];
+            far_ok[p] = r_ok[p] && far[p] >= 0 && far[p] < g.rows;
+            if (!far_ok[p]) far[p] = 0;
+            if ((!src_ok[p] || !r_ok[p]) && g.bad_index) *g.bad_index = 1;
+        }
+        PIECE xv[2], av[2], bv[2], xo[2], ao[2];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            xv[p] = __ldg(reinterpret_cast<const PIECE*>(g.x[p]) + src[p] * g.pieces + piece);
+            av[p] = __ldg(reinterpret_cast<const PIECE*>(g.a[p]) + at);
+            bv[p] = __ldcs(reinterpret_cast<const PIECE*>(g.b[p]) + at);
+            xo[p] = __ldg(reinterpret_cast<const PIECE*>(g.x[p ^ 1]) + far[p] * g.pieces + piece);
+            ao[p] = __ldg(reinterpret_cast<const PIECE*>(g.a[p ^ 1]) + r[p] * g.pieces + piece);
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            if (!src_ok[p]) xv[p] = shuffle_zero<PIECE>();
+            if (!far_ok[p]) xo[p] = shuffle_zero<PIECE>();
+            if (!r_ok[p]) ao[p] = shuffle_zero<PIECE>();
+            reinterpret_cast<PIECE*>(g.y[p])[at] = shuffle_combine<PIECE>(xv[p], av[p], 0);
+            reinterpret_cast<PIECE*>(g.z[p])[at] = shuffle_combine<PIECE>(shuffle_combine<PIECE>(xo[p], ao[p], 0), bv[p], 1);
+        }
+        row += g.stride_rows;
+        piece += g.stride_pieces;
+        if (piece >= g.pieces) { piece -= g.pieces; ++row; }
+    }
+}
+
 // inverse[perm[j]] = j: what a party does locally to obtain the sub-permutations of the unshuffle.
 __global__ void __launch_bounds__(256)
 invert_permutation_kernel(const int32_t* __restrict__ perm, int32_t* __restrict__ inverse, long long rows,

@@ -1,9 +1,10 @@
-"""Thin ctypes binding of libcomet_b200.so (the C ABI of include/comet.h).
+"""Thin binding of libcomet_b200.so (the C ABI of include/comet.h): ctypes, and for the calls of every pass the
+CPython module _marshal (csrc/marshal.cpp).
 
 Argument marshalling only: every step of the path runs in the library's CUDA
 kernels.  Tensors are torch uint64/int64 CUDA tensors or numpy/torch host
 arrays; torch is used for device memory and streams and for nothing else.
-There is no CPU fallback: if the shared library is missing or fails to load,
+There is no CPU fallback: if a shared object is missing or fails to load,
 importing this module raises.
 """
 from __future__ import annotations
@@ -106,6 +107,7 @@ def _load():
 
 
 _lib = _load()
+from . import _marshal as _native  # noqa: E402  (built together with the library)
 
 
 def library():
@@ -134,7 +136,9 @@ class Comet:
         self.stream = stream
         self._h = ctypes.c_void_p()
         sp = ctypes.c_void_p(stream.cuda_stream if stream is not None else 0)
+        self._address = None               # of the context, for the marshalling module
         self._check(_lib.comet_init(ctypes.byref(self.cfg), sp, ctypes.byref(self._h)), "comet_init")
+        self._address = self._h.value
         self.groups = int(gated) + 1
         self.n_active = 0
 
@@ -147,6 +151,7 @@ class Comet:
         if self._h:
             _lib.comet_destroy(self._h)
             self._h = ctypes.c_void_p()
+            self._address = None
 
     def __del__(self):
         try:
@@ -160,28 +165,34 @@ class Comet:
 
     # ------------------------------------------------------------------ the six calls
     def load_shares(self, party: int, tensor_id: int, t):
-        ptr, loc, _ = _ptr_loc(t)
-        rows, cols = t.shape
-        self._check(_lib.comet_load_shares(self._h, party, tensor_id, ptr, loc, rows, cols), "comet_load_shares")
+        if isinstance(t, torch.Tensor):
+            code = _native.load_shares(self._address, party, tensor_id, t)
+        else:
+            ptr, loc, _ = _ptr_loc(t)
+            rows, cols = t.shape
+            code = _lib.comet_load_shares(self._h, party, tensor_id, ptr, loc, rows, cols)
+        if code:
+            raise CometError(code, "comet_load_shares")
 
     def bind_shares(self, party: int, tensor_id: int, t):
         """Use a CUDA tensor of 8-byte words in place (no copy); the caller keeps it alive and unchanged."""
-        ptr, loc, _ = _ptr_loc(t)
-        assert loc == DEVICE
-        rows, cols = t.shape
-        self._check(_lib.comet_bind_shares(self._h, party, tensor_id, ptr, rows, cols), "comet_bind_shares")
+        code = _native.bind_shares(self._address, party, tensor_id, t)
+        if code:
+            raise CometError(code, "comet_bind_shares")
 
     def set_mask(self, mask) -> int:
         if isinstance(mask, np.ndarray):
-            assert mask.dtype == np.uint8 and mask.flags["C_CONTIGUOUS"]
-            ptr, loc, nb = mask.ctypes.data, HOST, mask.size
+            code, active = _native.set_mask(self._address, mask)
         else:
             assert mask.dtype == torch.uint8 and mask.is_contiguous()
-            ptr, loc, nb = mask.data_ptr(), (DEVICE if mask.is_cuda else HOST), mask.numel()
-        n = ctypes.c_int32(0)
-        self._check(_lib.comet_set_mask(self._h, ptr, loc, nb, ctypes.byref(n)), "comet_set_mask")
-        self.n_active = n.value
-        return n.value
+            n = ctypes.c_int32(0)
+            code = _lib.comet_set_mask(self._h, mask.data_ptr(), DEVICE if mask.is_cuda else HOST, mask.numel(),
+                                       ctypes.byref(n))
+            active = n.value
+        if code:
+            raise CometError(code, "comet_set_mask")
+        self.n_active = active
+        return active
 
     def set_token_mask(self, mask) -> int:
         """Per-token mask over the active blocks, [tokens, n_active_blocks] uint8 (numpy or torch), or None to
@@ -212,13 +223,19 @@ class Comet:
         return rl.cpu().numpy(), bl.cpu().numpy(), cnt.value
 
     def ffn_up(self, tokens: int):
-        self._check(_lib.comet_ffn_up(self._h, tokens), "comet_ffn_up")
+        code = _native.ffn_up(self._address, tokens)
+        if code:
+            raise CometError(code, "comet_ffn_up")
 
     def ffn_down(self, tokens: int):
-        self._check(_lib.comet_ffn_down(self._h, tokens), "comet_ffn_down")
+        code = _native.ffn_down(self._address, tokens)
+        if code:
+            raise CometError(code, "comet_ffn_down")
 
     def truncate(self, tensor_id: int):
-        self._check(_lib.comet_truncate(self._h, tensor_id), "comet_truncate")
+        code = _native.truncate(self._address, tensor_id)
+        if code:
+            raise CometError(code, "comet_truncate")
 
     # ------------------------------------------------------------------ read-back
     def get_into(self, party: int, tensor_id: int, out) -> int:
@@ -282,18 +299,7 @@ def beaver_matmul_static(X, A, Y, B, C, Z, stream: Optional[torch.cuda.Stream] =
     size-limit refusal can be observed.  Calls that overlap on the GPU race on
     the shared array: keep them on one stream.
     """
-    T, K = X[0].shape
-    N = Y[0].shape[0]
-    pair = ctypes.c_void_p * 2
-
-    def ptrs(ts, shape):
-        for t in ts:
-            assert t.is_cuda and t.is_contiguous() and t.element_size() == 8 and tuple(t.shape) == shape
-        return pair(ts[0].data_ptr(), ts[1].data_ptr())
-
-    sp = ctypes.c_void_p(stream.cuda_stream if stream is not None else 0)
-    return _lib.comet_beaver_matmul_static(sp, ptrs(X, (T, K)), ptrs(A, (T, K)), ptrs(Y, (N, K)), ptrs(B, (N, K)),
-                                           ptrs(C, (T, N)), ptrs(Z, (T, N)), T, K, N)
+    return _native.beaver_matmul_static(stream, X, A, Y, B, C, Z)
 
 
 PIPE_TENSOR_I8, PIPE_ALU_U64 = 0, 1
@@ -311,14 +317,6 @@ def pipe_probe(pipe: int, launches: int, work: int, stream: Optional[torch.cuda.
     return [float(v) for v in ms], macs.value
 
 
-def _pair(ts, shape=None, dtype=None):
-    for t in ts:
-        assert t.is_cuda and t.is_contiguous()
-        assert shape is None or tuple(t.shape) == tuple(shape)
-        assert dtype is None or t.dtype == dtype
-    return (ctypes.c_void_p * 2)(ts[0].data_ptr(), ts[1].data_ptr())
-
-
 def shuffle(X, tau, rho, a, b, stream: Optional[torch.cuda.Stream] = None, bad_index_flag=None):
     """Oblivious shuffle of the rows of a shared matrix (comet_shuffle), both parties.
 
@@ -327,29 +325,16 @@ def shuffle(X, tau, rho, a, b, stream: Optional[torch.cuda.Stream] = None, bad_i
     Returns (Y, Z): the two messages and the two shares of pi(x).  Only the
     output tensors are allocated here (torch); the arithmetic is the library's.
     """
-    rows = X[0].shape[0]
-    cols = X[0].numel() // rows
-    Y = [torch.empty_like(X[0]) for _ in (0, 1)]
-    Z = [torch.empty_like(X[0]) for _ in (0, 1)]
-    sp = ctypes.c_void_p(stream.cuda_stream if stream is not None else 0)
-    flag = ctypes.c_void_p(bad_index_flag.data_ptr() if bad_index_flag is not None else 0)
-    for t in (*X, *a, *b):
-        assert t.element_size() == 8
-    code = _lib.comet_shuffle(sp, _pair(X), _pair(tau, (rows,), torch.int32), _pair(rho, (rows,), torch.int32),
-                              _pair(a, X[0].shape), _pair(b, X[0].shape), _pair(Y), _pair(Z), rows, cols, flag)
-    if code != OK:
+    code, Y, Z = _native.shuffle(stream, X, tau, rho, a, b, bad_index_flag)
+    if code:
         raise CometError(code, "comet_shuffle")
     return Y, Z
 
 
 def invert_permutation(perm, stream: Optional[torch.cuda.Stream] = None, bad_index_flag=None):
     """inverse[perm[j]] = j on the device (comet_invert_permutation)."""
-    assert perm.is_cuda and perm.dtype == torch.int32 and perm.is_contiguous()
-    out = torch.empty_like(perm)
-    sp = ctypes.c_void_p(stream.cuda_stream if stream is not None else 0)
-    flag = ctypes.c_void_p(bad_index_flag.data_ptr() if bad_index_flag is not None else 0)
-    code = _lib.comet_invert_permutation(sp, perm.data_ptr(), out.data_ptr(), perm.numel(), flag)
-    if code != OK:
+    code, out = _native.invert_permutation(stream, perm, bad_index_flag)
+    if code:
         raise CometError(code, "comet_invert_permutation")
     return out
 
@@ -358,16 +343,8 @@ def beaver_mul(X, Y, A, B, C, stream: Optional[torch.cuda.Stream] = None):
     """Element-wise Beaver product of two shared tensors (comet_beaver_mul), both parties.
     Every argument is a pair of equally shaped CUDA tensors of 8-byte words.
     Returns (D, E, Z): the messages x - a and y - b, and the shares of x * y."""
-    shape = X[0].shape
-    for t in (*X, *Y, *A, *B, *C):
-        assert t.element_size() == 8 and t.shape == shape
-    D = [torch.empty_like(X[0]) for _ in (0, 1)]
-    E = [torch.empty_like(X[0]) for _ in (0, 1)]
-    Z = [torch.empty_like(X[0]) for _ in (0, 1)]
-    sp = ctypes.c_void_p(stream.cuda_stream if stream is not None else 0)
-    code = _lib.comet_beaver_mul(sp, _pair(X), _pair(Y), _pair(A), _pair(B), _pair(C), _pair(D), _pair(E), _pair(Z),
-                                 X[0].numel())
-    if code != OK:
+    code, D, E, Z = _native.beaver_mul(stream, X, Y, A, B, C)
+    if code:
         raise CometError(code, "comet_beaver_mul")
     return D, E, Z
 
@@ -376,13 +353,8 @@ def truncate_pair(Z, R, RP, frac_bits: int, stream: Optional[torch.cuda.Stream] 
     """Truncation with a dealer's pair (comet_truncate_pair), both parties: Z is replaced by shares of
     floor(z / 2^frac_bits) (or one less).  Z, R, RP are pairs of equally shaped CUDA tensors of 8-byte words.
     Returns the messages M = Z - R (a pair)."""
-    shape = Z[0].shape
-    for t in (*Z, *R, *RP):
-        assert t.element_size() == 8 and t.shape == shape
-    M = [torch.empty_like(Z[0]) for _ in (0, 1)]
-    sp = ctypes.c_void_p(stream.cuda_stream if stream is not None else 0)
-    code = _lib.comet_truncate_pair(sp, _pair(Z), _pair(R), _pair(RP), _pair(M), Z[0].numel(), frac_bits)
-    if code != OK:
+    code, M = _native.truncate_pair(stream, Z, R, RP, frac_bits)
+    if code:
         raise CometError(code, "comet_truncate_pair")
     return M
 
@@ -405,10 +377,6 @@ def kv_plan(present: np.ndarray, active: np.ndarray, x: int, w: int):
 
 def add_bias(Z, bias, stream: Optional[torch.cuda.Stream] = None):
     """Z[i][r, :] += bias[i] in place for both parties (comet_add_bias)."""
-    rows, cols = Z[0].shape
-    for t in bias:
-        assert t.element_size() == 8 and tuple(t.shape) == (cols,)
-    sp = ctypes.c_void_p(stream.cuda_stream if stream is not None else 0)
-    code = _lib.comet_add_bias(sp, _pair(Z, (rows, cols)), _pair(bias), rows, cols)
-    if code != OK:
+    code = _native.add_bias(stream, Z, bias)
+    if code:
         raise CometError(code, "comet_add_bias")

@@ -31,7 +31,9 @@ struct comet_ctx {
     int64_t cap_T, cap_n;         // capacities
     int sm_count;
     u64* buf[2][COMET_NUM_TENSORS];   // where each tensor is read / written: the library's own buffer, or a bound one
-    u64* own[2][COMET_NUM_TENSORS];   // the library's own buffers (allocated in comet_init, freed in comet_destroy)
+    u64* own[2][COMET_NUM_TENSORS];   // the library's own buffers
+    void* device_memory;              // one allocation each, made in comet_init and cut into every buffer below and above
+    void* pinned_memory;
     int64_t cap_words[COMET_NUM_TENSORS];
     bool loaded[2][COMET_NUM_TENSORS];
     // limb path: blocked limb planes (left: V_i per party and E; right: B_i per party and F), and the device error flag
@@ -538,14 +540,16 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
         c->top_priority = greatest;
     }
     bool ok = true;
-    for (int id = 0; id < COMET_NUM_TENSORS && ok; ++id) {
+    // Every buffer is a piece of one allocation (and of one pinned allocation): an allocation costs about as much whatever
+    // its size, and this many of them one by one took 9 of the 11 ms in which a context came up.
+    std::vector<std::pair<void**, size_t>> device, pinned;
+    auto reserve = [](std::vector<std::pair<void**, size_t>>& list, auto** where, size_t bytes) {
+        list.emplace_back(reinterpret_cast<void**>(where), bytes);
+    };
+    for (int id = 0; id < COMET_NUM_TENSORS; ++id) {
         c->cap_words[id] = tensor_capacity(c, id);
-        for (int p = 0; p < 2 && ok; ++p)
-            if (c->cap_words[id] > 0)
-            {
-                ok = cudaMalloc((void**)&c->own[p][id], (size_t)c->cap_words[id] * sizeof(u64)) == cudaSuccess;
-                c->buf[p][id] = c->own[p][id];
-            }
+        for (int p = 0; p < 2; ++p)
+            if (c->cap_words[id] > 0) reserve(device, &c->own[p][id], (size_t)c->cap_words[id] * sizeof(u64));
     }
     c->path = cfg->matmul_path == COMET_PATH_AUTO ? COMET_PATH_LIMB : cfg->matmul_path;
     if (c->path == COMET_PATH_LIMB) {
@@ -559,10 +563,10 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
         c->planes_right_up_bytes = (size_t)(((gn + lb::BN - 1) / lb::BN) * kb_up) * lb::B_BLOCK_BYTES;
         c->planes_right_dn_bytes = (size_t)(((d + lb::BN - 1) / lb::BN) * kb_dn) * lb::B_BLOCK_BYTES;
         // a context for few tokens only never builds planes in memory
-        for (int w = 0; w < 3 && ok && c->cap_T > comet::limb_stream::BT; ++w) {
-            ok = cudaMalloc((void**)&c->planes_left[w], c->planes_left_bytes) == cudaSuccess;
-            ok = ok && cudaMalloc((void**)&c->planes_right_up[w], c->planes_right_up_bytes) == cudaSuccess;
-            ok = ok && cudaMalloc((void**)&c->planes_right_dn[w], c->planes_right_dn_bytes) == cudaSuccess;
+        for (int w = 0; w < 3 && c->cap_T > comet::limb_stream::BT; ++w) {
+            reserve(device, &c->planes_left[w], c->planes_left_bytes);
+            reserve(device, &c->planes_right_up[w], c->planes_right_up_bytes);
+            reserve(device, &c->planes_right_dn[w], c->planes_right_dn_bytes);
         }
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)lb::SMEM_BYTES) == cudaSuccess;
@@ -586,31 +590,49 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
         ok = ok && cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) == cudaSuccess;
     }
     const int nb = cfg->d_ff / cfg->block;
-    ok = ok && cudaMalloc((void**)&c->d_mask, (size_t)nb) == cudaSuccess;
-    ok = ok && cudaMalloc((void**)&c->d_tmask, (size_t)nb * (size_t)c->cap_T) == cudaSuccess;
-    ok = ok && cudaHostAlloc((void**)&c->h_mask_stage, (size_t)nb * 4, cudaHostAllocDefault) == cudaSuccess;
     for (int k = 0; k < 4 && ok; ++k)
         ok = cudaEventCreateWithFlags(&c->stage_done[k], cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaHostAlloc((void**)&c->h_masked, 7 * sizeof(long long), cudaHostAllocMapped) == cudaSuccess;
-    ok = ok && cudaMalloc((void**)&c->d_row_map, (size_t)c->cap_T * sizeof(int32_t)) == cudaSuccess;
-    ok = ok && cudaMalloc((void**)&c->d_col_map, (size_t)c->groups * nb * sizeof(int32_t)) == cudaSuccess;
-    ok = ok && cudaMalloc((void**)&c->d_kmap, (size_t)nb * sizeof(int32_t)) == cudaSuccess;
-    ok = ok && cudaMalloc((void**)&c->d_plan_scratch,
-                          ((size_t)c->cap_T * ceil_div(nb, 32) + (size_t)c->groups * nb) * sizeof(uint32_t)) == cudaSuccess;
-    {
-        const size_t mt = ceil_div((int)c->cap_T, comet::limb::BM);
-        ok = ok && cudaMalloc((void**)&c->d_group_up, mt * sizeof(comet::LimbGroupRow)) == cudaSuccess;
-        ok = ok && cudaMalloc((void**)&c->d_group_dn, mt * sizeof(comet::LimbGroupRow)) == cudaSuccess;
+    const size_t row_tiles = ceil_div((int)c->cap_T, comet::limb::BM);
+    reserve(device, &c->d_mask, (size_t)nb);
+    reserve(device, &c->d_tmask, (size_t)nb * (size_t)c->cap_T);
+    reserve(device, &c->d_row_map, (size_t)c->cap_T * sizeof(int32_t));
+    reserve(device, &c->d_col_map, (size_t)c->groups * nb * sizeof(int32_t));
+    reserve(device, &c->d_kmap, (size_t)nb * sizeof(int32_t));
+    reserve(device, &c->d_plan_scratch, ((size_t)c->cap_T * ceil_div(nb, 32) + (size_t)c->groups * nb) * sizeof(uint32_t));
+    reserve(device, &c->d_group_up, row_tiles * sizeof(comet::LimbGroupRow));
+    reserve(device, &c->d_group_dn, row_tiles * sizeof(comet::LimbGroupRow));
+    reserve(device, &c->d_row_label, (size_t)c->cap_T * sizeof(int32_t));
+    reserve(device, &c->d_blk_label, (size_t)nb * sizeof(int32_t));
+    reserve(device, &c->d_ids, (size_t)nb * sizeof(int32_t));
+    reserve(device, &c->d_count, 2 * sizeof(int32_t));              // {count, error flag}
+    reserve(pinned, &c->h_masked, 7 * sizeof(long long));
+    reserve(pinned, &c->h_count, 4 * sizeof(int32_t));
+    reserve(pinned, &c->h_mask_stage, (size_t)nb * 4);
+    constexpr size_t ALIGN = 256;
+    auto total = [](const std::vector<std::pair<void**, size_t>>& list) {
+        size_t bytes = 0;
+        for (const auto& piece : list) bytes += (piece.second + ALIGN - 1) / ALIGN * ALIGN;
+        return bytes;
+    };
+    auto hand_out = [](const std::vector<std::pair<void**, size_t>>& list, void* base) {
+        uint8_t* at = static_cast<uint8_t*>(base);
+        for (const auto& piece : list) {
+            *piece.first = at;
+            at += (piece.second + ALIGN - 1) / ALIGN * ALIGN;
+        }
+    };
+    ok = ok && cudaMalloc(&c->device_memory, total(device)) == cudaSuccess;
+    ok = ok && cudaHostAlloc(&c->pinned_memory, total(pinned), cudaHostAllocMapped) == cudaSuccess;
+    if (ok) {
+        hand_out(device, c->device_memory);
+        hand_out(pinned, c->pinned_memory);
+        for (int p = 0; p < 2; ++p)
+            for (int id = 0; id < COMET_NUM_TENSORS; ++id) c->buf[p][id] = c->own[p][id];
+        c->d_error = c->d_count + 1;
+        c->h_count[0] = c->h_count[1] = c->h_count[2] = c->h_count[3] = 0;     // pinned memory is not zeroed
     }
-    ok = ok && cudaMalloc((void**)&c->d_row_label, (size_t)c->cap_T * sizeof(int32_t)) == cudaSuccess;
-    ok = ok && cudaMalloc((void**)&c->d_blk_label, (size_t)nb * sizeof(int32_t)) == cudaSuccess;
-    ok = ok && cudaHostGetDevicePointer((void**)&c->h_masked_dev, c->h_masked, 0) == cudaSuccess;
-    ok = ok && cudaMalloc((void**)&c->d_ids, (size_t)nb * sizeof(int32_t)) == cudaSuccess;
-    ok = ok && cudaMalloc((void**)&c->d_count, 2 * sizeof(int32_t)) == cudaSuccess;   // {count, error flag}
     ok = ok && cudaMemset(c->d_count, 0, 2 * sizeof(int32_t)) == cudaSuccess;
-    if (ok) c->d_error = c->d_count + 1;
-    ok = ok && cudaHostAlloc((void**)&c->h_count, 4 * sizeof(int32_t), cudaHostAllocMapped) == cudaSuccess;
-    if (ok) c->h_count[0] = c->h_count[1] = c->h_count[2] = c->h_count[3] = 0;     // pinned memory is not zeroed
+    ok = ok && cudaHostGetDevicePointer((void**)&c->h_masked_dev, c->h_masked, 0) == cudaSuccess;
     ok = ok && cudaHostGetDevicePointer((void**)&c->h_count_dev, c->h_count, 0) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -625,35 +647,14 @@ void comet_destroy(comet_ctx* c) {
     if (!c) return;
     cudaSetDevice(c->cfg.device);
     cudaStreamSynchronize(c->stream);
-    for (int id = 0; id < COMET_NUM_TENSORS; ++id)
-        for (int p = 0; p < 2; ++p)
-            if (c->own[p][id]) cudaFree(c->own[p][id]);
     if (c->side) cudaStreamSynchronize(c->side);
-    for (int w = 0; w < 3; ++w) {
-        if (c->planes_left[w]) cudaFree(c->planes_left[w]);
-        if (c->planes_right_up[w]) cudaFree(c->planes_right_up[w]);
-        if (c->planes_right_dn[w]) cudaFree(c->planes_right_dn[w]);
-    }
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->side) cudaStreamDestroy(c->side);
-    if (c->d_mask) cudaFree(c->d_mask);
-    if (c->d_tmask) cudaFree(c->d_tmask);
-    if (c->h_mask_stage) cudaFreeHost(c->h_mask_stage);
     for (int k = 0; k < 4; ++k)
         if (c->stage_done[k]) cudaEventDestroy(c->stage_done[k]);
-    if (c->h_masked) cudaFreeHost(c->h_masked);
-    if (c->d_row_label) cudaFree(c->d_row_label);
-    if (c->d_row_map) cudaFree(c->d_row_map);
-    if (c->d_col_map) cudaFree(c->d_col_map);
-    if (c->d_kmap) cudaFree(c->d_kmap);
-    if (c->d_plan_scratch) cudaFree(c->d_plan_scratch);
-    if (c->d_group_up) cudaFree(c->d_group_up);
-    if (c->d_group_dn) cudaFree(c->d_group_dn);
-    if (c->d_blk_label) cudaFree(c->d_blk_label);
-    if (c->d_ids) cudaFree(c->d_ids);
-    if (c->d_count) cudaFree(c->d_count);
-    if (c->h_count) cudaFreeHost(c->h_count);
+    if (c->device_memory) cudaFree(c->device_memory);
+    if (c->pinned_memory) cudaFreeHost(c->pinned_memory);
     for (auto& p : *c->pending) {
         cudaEventDestroy(p.start);
         cudaEventDestroy(p.stop);

@@ -318,10 +318,9 @@ int join_side(comet_ctx* c) {
     return COMET_OK;
 }
 
-// Tensor-core path: messages, exchange and operand planes of the left and / or right side, and / or Z <- C; one launch.
-int limb_exchange(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy, cudaStream_t stream) {
+// Arguments of the exchange kernel for the left and / or right side of one product, and / or Z <- C.  Returns its CTAs.
+int exchange_args(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy, comet::LimbExchangeArgs& a) {
     namespace lb = comet::limb;
-    comet::LimbExchangeArgs a;
     std::memset(&a, 0, sizeof(a));
     uint8_t** planes = pr.down ? c->planes_right_dn : c->planes_right_up;
     for (int p = 0; p < 2; ++p) {
@@ -368,10 +367,20 @@ int limb_exchange(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy
     a.right_blocks = right_rows * a.kchunks;
     a.copy_pairs = copy ? (long long)pr.M * pr.N / 2 : 0;
     a.copy_blocks = copy ? 2 * ew_grid(c, a.copy_pairs, lb::EX_THREADS) : 0;
-    const int blocks = a.left_blocks + a.right_blocks + a.copy_blocks;
-    if (blocks == 0) return COMET_OK;
-    COMET_CUDA(c, launch_chained(comet::limb_exchange_kernel, dim3(blocks), dim3(lb::EX_THREADS),
-                                 left_rows + right_rows ? lb::EX_SMEM_BYTES : 0, stream, nullptr, a));
+    return a.left_blocks + a.right_blocks + a.copy_blocks;
+}
+
+// Tensor-core path: messages, exchange and operand planes of one product, in one launch; `also`, if given, are the arguments
+// of a second product's for the same launch.
+int limb_exchange(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy, cudaStream_t stream,
+                  const comet::LimbExchangeArgs* also = nullptr, int also_blocks = 0) {
+    namespace lb = comet::limb;
+    comet::LimbExchangeArgs a;
+    const int blocks = exchange_args(c, pr, left, right, copy, a);
+    if (blocks + also_blocks == 0) return COMET_OK;
+    const bool tiles = left || right || also_blocks;
+    COMET_CUDA(c, launch_chained(comet::limb_exchange_kernel, dim3(blocks + also_blocks), dim3(lb::EX_THREADS),
+                                 tiles ? lb::EX_SMEM_BYTES : 0, stream, nullptr, a, also ? *also : a, blocks));
     c->stats.kernel_launches += 1;
     COMET_CUDA(c, cudaGetLastError());
     return COMET_OK;
@@ -426,6 +435,8 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
     COMET_CUDA(c, cudaGetLastError());
     return COMET_OK;
 }
+
+constexpr int64_t EXCHANGE_APART = 1 << 18;    // words of the down-projection's weight side; see comet_ffn_up
 
 bool limb_fits(const comet_ctx* c, const Proj& pr) {
     namespace lb = comet::limb;
@@ -896,32 +907,37 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
             return rc != COMET_OK ? rc : somm_merge(c, tokens);
         }
         if (!limb_fits(c, up)) return COMET_ERR_SHAPE;
-        // The weight side of the down-projection depends only on the mask, W2 and B'_i: if those are loaded
-        // already, open it now on the side stream, beside the tensor-core kernel (not beside the exchange before it, which
-        // is bound by the same memory).  Beside it 198 MB of exchange traffic cost the 512-token step at 90 % sparsity 14 us,
-        // behind it 27; a launch-completion event of the tensor-core kernel, which would keep that kernel a programmatic
-        // dependent of the exchange, only fired when the kernel had ended.
+        // The weight side of the down-projection depends only on the mask, W2 and B'_i: if those are loaded already, it is
+        // opened now, and if the triple's C' share is there too, Y_i <- C'_i, the value the down-projection's sums are added
+        // to, is copied with it.  Where: a small one in the same launch as this product's exchange, which costs nothing but
+        // its traffic; from EXCHANGE_APART words on, on the side stream beside the tensor-core kernel (not beside the
+        // exchange before it, which is bound by the same memory), which hides about half of it but takes two events, a
+        // launch and the programmatic start of the tensor-core kernel.  A step with 0.03 million such words takes 25 us in
+        // one launch and 34 apart, with 0.25 million 41 either way, with 0.52 million 97 and 94, with 1.7 million 249 and 237.
         const bool early = !c->dn_right_ready && limb_fits(c, dn) && c->loaded[0][COMET_W2] &&
                            c->loaded[1][COMET_W2] && c->loaded[0][COMET_B_DN] && c->loaded[1][COMET_B_DN];
+        const bool early_copy = early && c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN];
+        const bool apart = early && (int64_t)dn.N * dn.K >= EXCHANGE_APART;
+        comet::LimbExchangeArgs also;
+        const int also_blocks = early && !apart ? exchange_args(c, dn, false, true, early_copy, also) : 0;
         {
             PhaseTimer timer(c, COMET_PHASE_OPEN, 1);
-            rc = limb_exchange(c, up, true, true, true, c->stream);
+            rc = limb_exchange(c, up, true, true, true, c->stream, also_blocks ? &also : nullptr, also_blocks);
         }
         if (rc != COMET_OK) return rc;
-        if (early) COMET_CUDA(c, cudaEventRecord(c->ev_fork, c->stream));
+        if (apart) COMET_CUDA(c, cudaEventRecord(c->ev_fork, c->stream));
         rc = limb_combine(c, up);
         if (rc != COMET_OK) return rc;
-        if (early) {
+        if (apart) {
             COMET_CUDA(c, cudaStreamWaitEvent(c->side, c->ev_fork, 0));
-            // ... and if the triple's C' share is there too, Y_i <- C'_i, the value the down-projection's sums are
-            // added to, is copied in the same launch
-            const bool copy = c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN];
-            rc = limb_exchange(c, dn, false, true, copy, c->side);
+            rc = limb_exchange(c, dn, false, true, early_copy, c->side);
             if (rc != COMET_OK) return rc;
             COMET_CUDA(c, cudaEventRecord(c->ev_join, c->side));
             c->side_pending = true;
+        }
+        if (early) {
             c->dn_right_ready = true;
-            c->dn_copy_ready = copy;
+            c->dn_copy_ready = early_copy;
             c->dn_copy_tokens = tokens;
         }
         return somm_merge(c, tokens);

@@ -267,21 +267,27 @@ __device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, in
     limb_copy_wait<0>();
 }
 
-__global__ void __launch_bounds__(limb::EX_THREADS, 7)
-limb_exchange_kernel(const __grid_constant__ LimbExchangeArgs a) {
-    pdl_wait();
-    pdl_launch_dependents();
-    int block = blockIdx.x;
-    extern __shared__ __align__(16) uint8_t ex_smem[];
-    if (block < a.left_blocks) return limb_exchange_rows<true>(a, block, ex_smem);
+__device__ __forceinline__ void limb_exchange_block(const LimbExchangeArgs& a, int block, uint8_t* smem) {
+    if (block < a.left_blocks) return limb_exchange_rows<true>(a, block, smem);
     block -= a.left_blocks;
-    if (block < a.right_blocks) return limb_exchange_rows<false>(a, block, ex_smem);
+    if (block < a.right_blocks) return limb_exchange_rows<false>(a, block, smem);
     block -= a.right_blocks;
     const int party = block & 1;
     const ulonglong2* __restrict__ s = reinterpret_cast<const ulonglong2*>(party ? a.C[1] : a.C[0]);
     ulonglong2* __restrict__ d = reinterpret_cast<ulonglong2*>(party ? a.Z[1] : a.Z[0]);
     const long long stride = (long long)(a.copy_blocks >> 1) * limb::EX_THREADS;
     for (long long t = (long long)(block >> 1) * limb::EX_THREADS + threadIdx.x; t < a.copy_pairs; t += stride) d[t] = __ldcs(s + t);
+}
+
+// The first `first_blocks` CTAs work on `a`, the others on `b` (another product's operands).
+__global__ void __launch_bounds__(limb::EX_THREADS, 7)
+limb_exchange_kernel(const __grid_constant__ LimbExchangeArgs a, const __grid_constant__ LimbExchangeArgs b, int first_blocks) {
+    extern __shared__ __align__(16) uint8_t ex_smem[];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int block = blockIdx.x;
+    if (block < first_blocks) limb_exchange_block(a, block, ex_smem);
+    else limb_exchange_block(b, block - first_blocks, ex_smem);
 }
 
 // ---------------------------------------------------------------------------

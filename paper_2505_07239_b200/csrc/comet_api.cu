@@ -386,6 +386,28 @@ int limb_exchange(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy
     return COMET_OK;
 }
 
+// Tensor map of a result matrix for the tensor-core kernel's reductions (see LimbMaps).
+bool result_map(CUtensorMap* map, u64* z, int rows, int cols) {
+    typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                               const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const Encode encode = [] {                    // a driver function: the library does not link to the driver
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<Encode>(fn);
+    }();
+    const cuuint64_t size[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, pitch[1] = {(cuuint64_t)cols * sizeof(u64)};
+    const cuuint32_t box[2] = {comet::limb::OUT_COLS, 32}, step[2] = {1, 1};
+    return encode && encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, z, size, pitch, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Tensor-core path: the persistent stream-K kernel over both parties' tiles.
 int limb_combine(comet_ctx* c, const Proj& pr) {
     namespace lb = comet::limb;
@@ -427,8 +449,16 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
         // The persistent kernel needs a slot on every SM.  With the device's highest scheduling priority its CTAs
         // get the slots that free up before the memory-side CTAs of other contexts queued beside it do, so the
         // tensor cores do not wait behind work that could as well run under them.
-        auto* kernel = c->grouped ? comet::combine_limb_grouped_kernel : comet::combine_limb_kernel;
-        COMET_CUDA(c, launch_chained(kernel, dim3(grid), dim3(lb::THREADS), lb::SMEM_BYTES, c->stream, &c->top_priority, a));
+        if (c->grouped) {
+            COMET_CUDA(c, launch_chained(comet::combine_limb_grouped_kernel, dim3(grid), dim3(lb::THREADS), lb::SMEM_BYTES,
+                                         c->stream, &c->top_priority, a));
+        } else {
+            comet::LimbMaps maps;
+            for (int p = 0; p < 2; ++p)
+                if (!result_map(&maps.z[p], a.Z[p], a.M, a.N)) return COMET_ERR_CUDA;
+            COMET_CUDA(c, launch_chained(comet::combine_limb_kernel, dim3(grid), dim3(lb::THREADS), lb::SMEM_BYTES, c->stream,
+                                         &c->top_priority, a, maps));
+        }
     }
     c->stats.kernel_launches += 1;
     c->stats.matmul_path = COMET_PATH_LIMB;

@@ -17,10 +17,11 @@
 // whose N spans accumulators D_p..D_7 (split in two when N > 256): 12 instructions per 32-deep step.
 //
 // Work is split stream-K style over a persistent grid: the (party, tile, k-block) space is cut into equal
-// contiguous ranges, every segment's partial sums are added to Z with red.global.add.u64 -- exact and
-// order-independent in the ring -- and Z is pre-loaded with C_i.
+// contiguous ranges, every segment's partial sums are added to Z by 64-bit integer reductions of the copy
+// engine -- exact and order-independent in the ring -- and Z is pre-loaded with C_i.
 #pragma once
 #include <cstdint>
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "pdl.cuh"
@@ -41,8 +42,9 @@ constexpr int EX_THREADS = 128, EX_ROWS = 16, EX_MAX_KB_PER_CTA = 16;      // ex
 constexpr int EX_STAGES = 2, EX_STAGE_BYTES = EX_THREADS * 8 * 16;           // eight 16-byte pieces per lane and k-block
 constexpr size_t EX_SMEM_BYTES = (size_t)EX_STAGES * EX_STAGE_BYTES;        // 32 KiB: fits beside a tensor-core CTA
 constexpr int OUT_COLS = 16;                      // words per staged output row (a thread's 32 go in two rounds)
-constexpr int OUT_ROW_BYTES = OUT_COLS * 8 + 16;  // padded against bank conflicts
-constexpr size_t SMEM_BYTES = (size_t)STAGES * (A_BLOCK_BYTES + B_BLOCK_BYTES) + (size_t)EPI_WARPS * 32 * OUT_ROW_BYTES + 128;
+constexpr int OUT_ROW_BYTES = OUT_COLS * 8 + 16;  // padded against bank conflicts (grouped kernel: one copy per row)
+constexpr int OUT_TILE_BYTES = 32 * OUT_COLS * 8; // swizzled instead (one tensor copy per warp and round), 1 KiB aligned
+constexpr size_t SMEM_BYTES = (size_t)STAGES * (A_BLOCK_BYTES + B_BLOCK_BYTES) + (size_t)EPI_WARPS * 32 * OUT_ROW_BYTES + 1024;
 constexpr long long WAIT_CYCLES = 4000000000ll;   // ~2 s at 1.9 GHz: every wait gives up after this
 constexpr unsigned LBO_BYTES = 128, SBO_BYTES = 256;
 }  // namespace limb
@@ -324,6 +326,12 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
 __device__ __forceinline__ void bulk_reduce_add_u64(void* dst, uint32_t src, uint32_t bytes) {
     asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.u64 [%0], [%1], %2;"
                  ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+}
+// shared -> global tensor reduction: add a box of 64-bit integers at (column x, row y) of the map's matrix; what lies outside
+// the matrix is left out
+__device__ __forceinline__ void tensor_reduce_add(const CUtensorMap* map, uint32_t src, int x, int y) {
+    asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3}], [%1];"
+                 ::"l"(map), "r"(src), "r"(x), "r"(y) : "memory");
 }
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_group_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
@@ -693,7 +701,7 @@ __device__ __noinline__ bool limb_wait_sleeping(uint32_t bar, uint32_t parity, v
             *abort_flag = 1;
             return false;
         }
-        __nanosleep(400);
+        __nanosleep(40);
     }
 }
 
@@ -770,7 +778,7 @@ __device__ __forceinline__ uint32_t limb_desc_lo(uint32_t addr) {
 constexpr uint32_t LIMB_DESC_HI = (uint32_t)(limb::SBO_BYTES >> 4) | (1u << 14);
 
 template <bool GROUPED>
-__device__ __forceinline__ void combine_limb_body(const LimbArgs a) {
+__device__ __forceinline__ void combine_limb_body(const LimbArgs& a, const CUtensorMap* z_maps) {
     using namespace limb;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[STAGES];
@@ -779,7 +787,7 @@ __device__ __forceinline__ void combine_limb_body(const LimbArgs a) {
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
 
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t* sA = smem;
     uint8_t* sB = smem + (size_t)STAGES * A_BLOCK_BYTES;
     uint8_t* sOut = sB + (size_t)STAGES * B_BLOCK_BYTES;      // EPI_WARPS x 32 rows x OUT_ROW_BYTES
@@ -927,7 +935,9 @@ __device__ __forceinline__ void combine_limb_body(const LimbArgs a) {
         bool ok = true;
         const int quarter = warp & 3, chalf = warp >> 2;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16) + chalf * 32;
-        uint8_t* my_row = sOut + ((size_t)warp * 32 + lane) * OUT_ROW_BYTES;
+        // this lane's row in the warp's staging tile
+        uint8_t* my_row = GROUPED ? sOut + ((size_t)warp * 32 + lane) * OUT_ROW_BYTES
+                                  : sOut + (size_t)warp * OUT_TILE_BYTES + lane * (OUT_COLS * 8);
         const uint32_t my_row_s = ptx::smem_u32(my_row);
         for (long long u = u_begin; u < u_end && ok;) {
             const LimbSegment sg = limb_segment<GROUPED>(a, u, u_end);
@@ -937,11 +947,8 @@ __device__ __forceinline__ void combine_limb_body(const LimbArgs a) {
             ptx::fence_after_sync();
             const int row = sg.tm * BM + quarter * 32 + lane;
             const int col0 = sg.tn * BN + chalf * 32;
-            u64* zrow;
-            if (GROUPED)
-                zrow = (sg.party ? a.Z[1] : a.Z[0]) + (size_t)(row < a.M ? __ldg(a.row_map + row) : 0) * a.ldz;
-            else
-                zrow = (sg.party ? a.Z[1] : a.Z[0]) + (size_t)row * a.N + col0;
+            u64* zrow = nullptr;
+            if (GROUPED) zrow = (sg.party ? a.Z[1] : a.Z[0]) + (size_t)(row < a.M ? __ldg(a.row_map + row) : 0) * a.ldz;
 #pragma unroll
             for (int h = 0; h < 32 / OUT_COLS; ++h) {          // this thread's 32 columns, OUT_COLS at a time
                 u64 v[OUT_COLS];
@@ -961,24 +968,37 @@ __device__ __forceinline__ void combine_limb_body(const LimbArgs a) {
                     ptx::fence_before_sync();
                     ptx::mbar_arrive(ptx::smem_u32(&accum_empty_bar));
                 }
-                ptx::bulk_wait_group_read0();                  // the previous reduction has read this thread's staging row
+                if (GROUPED) {
+                    ptx::bulk_wait_group_read0();              // the previous reduction has read this thread's staging row
 #pragma unroll
-                for (int j = 0; j < OUT_COLS; j += 2)
-                    *reinterpret_cast<ulonglong2*>(my_row + j * 8) = make_ulonglong2(v[j], v[j + 1]);
-                int cols = a.N - col0 - h * OUT_COLS;
-                if (cols > OUT_COLS) cols = OUT_COLS;
-                if (row < a.M && cols > 0) {
-                    ptx::fence_proxy_async_smem();     // this thread's row, written above, is read by the copy engine
-                    u64* dst;
-                    if (GROUPED) {
+                    for (int j = 0; j < OUT_COLS; j += 2)
+                        *reinterpret_cast<ulonglong2*>(my_row + j * 8) = make_ulonglong2(v[j], v[j + 1]);
+                    int cols = a.N - col0 - h * OUT_COLS;
+                    if (cols > OUT_COLS) cols = OUT_COLS;
+                    if (row < a.M && cols > 0) {
+                        ptx::fence_proxy_async_smem();     // this thread's row, written above, is read by the copy engine
                         const int c = col0 + h * OUT_COLS, blk = c / a.bs;
-                        dst = a.col_map ? zrow + (size_t)__ldg(a.col_map + blk) * a.bs + (c - blk * a.bs) : zrow + c;
-                    } else {
-                        dst = zrow + h * OUT_COLS;
+                        u64* dst = a.col_map ? zrow + (size_t)__ldg(a.col_map + blk) * a.bs + (c - blk * a.bs) : zrow + c;
+                        ptx::bulk_reduce_add_u64(dst, my_row_s, (uint32_t)cols * 8u);
                     }
-                    ptx::bulk_reduce_add_u64(dst, my_row_s, (uint32_t)cols * 8u);
+                    ptx::bulk_commit_group();
+                } else {
+                    // One tensor reduction takes the warp's 32 x 16 words.  (One bulk reduction per row costs some 70 cycles
+                    // of issue each, 64 of them per warp and tile: a product of two k-blocks' work per CTA took 13.7 us, with
+                    // this 11.2.)
+                    if (lane == 0) ptx::bulk_wait_group_read0();
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < OUT_COLS; j += 2)
+                        *reinterpret_cast<ulonglong2*>(my_row + (((j >> 1) ^ (lane & 7)) << 4)) = make_ulonglong2(v[j], v[j + 1]);
+                    ptx::fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        const int x = col0 + h * OUT_COLS, y = sg.tm * BM + quarter * 32;
+                        if (x < a.N && y < a.M) ptx::tensor_reduce_add(z_maps + sg.party, my_row_s, x, y);
+                        ptx::bulk_commit_group();
+                    }
                 }
-                ptx::bulk_commit_group();
             }
             acc_phase ^= 1u;
         }
@@ -998,16 +1018,20 @@ __device__ __forceinline__ void combine_limb_body(const LimbArgs a) {
     }
 }
 
+struct LimbMaps {
+    CUtensorMap z[2];            // Z_0, Z_1 as [M, N] matrices of 64-bit integers, boxes of 32 rows x 16 words, 128-byte swizzle
+};
+
 __global__ void __launch_bounds__(limb::THREADS, 1)
-combine_limb_kernel(LimbArgs a) {
-    combine_limb_body<false>(a);
+combine_limb_kernel(const __grid_constant__ LimbArgs a, const __grid_constant__ LimbMaps maps) {
+    combine_limb_body<false>(a, maps.z);
 }
 
 // One multiplication per connected component (Protocols 2 and 3 under a per-token mask): the same kernel over the
 // tiles and k-blocks of the component-sorted operands that have work, scattering the result rows back to Z.
 __global__ void __launch_bounds__(limb::THREADS, 1)
-combine_limb_grouped_kernel(LimbArgs a) {
-    combine_limb_body<true>(a);
+combine_limb_grouped_kernel(const __grid_constant__ LimbArgs a) {
+    combine_limb_body<true>(a, nullptr);
 }
 
 }  // namespace comet

@@ -238,6 +238,28 @@ Proj proj_down(const comet_ctx* c, int tokens) {
 // its planes live in shared memory, so every further 32 rows would convert the weights once more.
 inline bool few_tokens(const Proj& pr) { return pr.M <= comet::limb_stream::BT; }
 
+// Tensor map of a result matrix for the tensor-core kernel's reductions (see LimbMaps).
+bool result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_rows, int box_cols, CUtensorMapSwizzle swizzle) {
+    typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                               const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const Encode encode = [] {                    // a driver function: the library does not link to the driver
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<Encode>(fn);
+    }();
+    const cuuint64_t size[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, pitch[1] = {(cuuint64_t)cols * sizeof(u64)};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows}, step[2] = {1, 1};
+    return encode && encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, z, size, pitch, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Z <- C, then the streaming kernel behind it (it begins while the copy runs and waits for it before its first sum).
 int launch_stream(comet::StreamArgs& args, const u64* const C[2], int sm_count, cudaStream_t stream,
                   const int* priority, cudaError_t* err) {
@@ -248,17 +270,20 @@ int launch_stream(comet::StreamArgs& args, const u64* const C[2], int sm_count, 
     args.kb = ceil_div(args.K, ls::KC);
     const long long steps = (long long)args.mt * args.nt * args.kb;
     const unsigned grid = (unsigned)(steps < sm_count ? steps : sm_count);
-    args.last_cost = ceil_div(args.N - (args.nt - 1) * ls::BW, ls::QROWS) + 1;
-    const long long cost = ((long long)(ls::QUARTERS + 1) * (args.nt - 1) + args.last_cost) * args.kb * args.mt;
+    args.last_cost = ceil_div(args.N - (args.nt - 1) * ls::BW, ls::QROWS) + ls::STEP_SLOTS;
+    const long long cost = ((long long)(ls::QUARTERS + ls::STEP_SLOTS) * (args.nt - 1) + args.last_cost) * args.kb * args.mt;
     if (cost > 0x7fffffffll) return COMET_ERR_SHAPE;                   // the kernel counts in 32 bits
-    args.cta_cost = (unsigned)(cost / grid);
+    args.cta_cost = steps > sm_count ? (unsigned)(cost / grid) : 0u;
     args.cta_extra = (unsigned)(cost % grid);
+    comet::LimbMaps maps;
+    for (int p = 0; p < 2; ++p)
+        if (!result_map(&maps.z[p], args.Z[p], args.M, args.N, ls::OUT_TOKENS, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) return COMET_ERR_CUDA;
     const long long pairs = (long long)args.M * args.N / 2, want = (pairs + 255) / 256, most = (long long)sm_count * 8;
     *err = launch_chained(comet::result_init_kernel, dim3((unsigned)(want < most ? want : most), 2), dim3(256), 0, stream,
                           nullptr, C[0], C[1], args.Z[0], args.Z[1], pairs);
     if (*err != cudaSuccess) return COMET_ERR_CUDA;
     *err = launch_chained(comet::combine_stream_kernel, dim3(grid), dim3(ls::THREADS), ls::SMEM_BYTES, stream,
-                          priority, args);
+                          priority, args, maps);
     return *err == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
 }
 
@@ -386,28 +411,6 @@ int limb_exchange(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy
     return COMET_OK;
 }
 
-// Tensor map of a result matrix for the tensor-core kernel's reductions (see LimbMaps).
-bool result_map(CUtensorMap* map, u64* z, int rows, int cols) {
-    typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                               const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static const Encode encode = [] {                    // a driver function: the library does not link to the driver
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
-            found != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            fn = nullptr;
-        }
-        return reinterpret_cast<Encode>(fn);
-    }();
-    const cuuint64_t size[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, pitch[1] = {(cuuint64_t)cols * sizeof(u64)};
-    const cuuint32_t box[2] = {comet::limb::OUT_COLS, 32}, step[2] = {1, 1};
-    return encode && encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, z, size, pitch, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // Tensor-core path: the persistent stream-K kernel over both parties' tiles.
 int limb_combine(comet_ctx* c, const Proj& pr) {
     namespace lb = comet::limb;
@@ -455,7 +458,7 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
         } else {
             comet::LimbMaps maps;
             for (int p = 0; p < 2; ++p)
-                if (!result_map(&maps.z[p], a.Z[p], a.M, a.N)) return COMET_ERR_CUDA;
+                if (!result_map(&maps.z[p], a.Z[p], a.M, a.N, 32, lb::OUT_COLS, CU_TENSOR_MAP_SWIZZLE_128B)) return COMET_ERR_CUDA;
             COMET_CUDA(c, launch_chained(comet::combine_limb_kernel, dim3(grid), dim3(lb::THREADS), lb::SMEM_BYTES, c->stream,
                                          &c->top_priority, a, maps));
         }

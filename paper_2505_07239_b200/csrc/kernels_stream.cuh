@@ -9,9 +9,10 @@
 // is bound by streaming the weight side.  Per word of the right operand and party that is W_i and B_i in and F_i out,
 // 24 bytes, and this kernel moves nothing else of that size: the limb planes the tensor cores read exist in shared
 // memory only.  (Its predecessor wrote the planes of B_i and F_i to memory and read them back: 56 bytes per word.)
-// Measured, both parties: [32, 4096] x [4096, 1312] 66 us and [7, 4096] x [4096, 3328] 114 us, where 24 bytes per weight
-// word at the measured copy rate are 39 and 100 us (100 + 43 and 135 + 82 us before); a step of 192 KiB takes 8300 cycles,
-// 90 % of that rate, the rest is the first step's latency and the last drain.
+// Measured, both parties: [32, 4096] x [4096, 1312] 52 us and [7, 4096] x [4096, 3328] 104 us from a CTA's start to its end,
+// where 24 bytes per weight word at the measured copy rate are 39 and 100 us; a step of 192 KiB takes 8400 cycles, 95 % of that
+// rate, the rest is 2 us until the first bytes arrive and 4 us from the last planes to the end (MMAs 3100 cycles, drain of 32
+// tokens 4000, of 7 tokens 1200, the reductions' completion 900).
 //
 // A CTA carries both parties' share of a tile of 128 output features (the rows of the MMA) x 32 tokens, and walks it in
 // steps of 32 contraction indices.  What is computed for a party depends on that party's shares and on the two messages
@@ -22,7 +23,7 @@
 //                 (to memory) and their sum -> limb planes of B_0, B_1, F
 //   warps 18-25   the token side, four rows each: X_i, A_i straight from L2, a step ahead -> messages E_0, E_1 -> limb
 //                 planes of E, A_0, A_1 + E; at the end of a segment the same warps are the epilogue (four per party): TMEM
-//                 -> recombine mod 2^64 -> rows staged in shared memory -> bulk add-reductions into Z
+//                 -> recombine mod 2^64 -> rows staged in shared memory -> tensor add-reductions into Z
 //   warp 26       issues the MMAs: F is the same for both parties, so three weight-side plane sets serve four products
 // Shared memory: 96 KiB weight planes, 24 KiB token planes, 96 KiB raw ring, 8 KiB result rows; all 512 TMEM columns (two
 // parties x eight accumulators x 32 tokens).  The planes are single-buffered: converting a step and multiplying it take
@@ -31,7 +32,8 @@
 // The contraction indices of a step sit in the planes in limb_emit4's order (kernels_limb.cuh).
 //
 // Work is cut stream-K style like the other tensor-core kernel's: the (feature tile, token tile, step) space in equal
-// contiguous ranges, a step weighted by the number of raw slots it takes (a ragged last tile takes fewer).
+// contiguous ranges, a step weighted by the number of raw slots it takes (a ragged last tile takes fewer) and a constant; with
+// no more steps than SMs every CTA has one.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -59,6 +61,10 @@ constexpr int ACC_COLS = PLANES * BT;                    // 256 TMEM columns per
 // A step adds two products to an accumulator, so the bound on a segment's depth (16384 contraction indices keep the
 // limb sums for s <= 3 below 2^32) allows half as many steps.
 constexpr int MAX_SEGMENT_STEPS = limb::MAX_SEGMENT_UNITS / 2;
+// What a step costs besides its slots, in slots: the MMAs and the hand-over of the planes take turns with the conversion.
+// Measured on [32, 4096] x [4096, 1312]: 8600 cycles with four slots, 4800 to 5600 with one (the last tile's).  Counted as one
+// slot, the CTAs of that tile ran 67 us where the others took 52, and the layer 134 us; as three 124.4, as five 122.2.
+constexpr int STEP_SLOTS = 5;
 constexpr size_t SMEM_BYTES = 3 * (size_t)W_SET_BYTES + 3 * (size_t)T_SET_BYTES + (size_t)RAW_SLOTS * RAW_SLOT_BYTES +
                               (size_t)TOK_WARPS * OUT_BYTES + 128;
 }  // namespace limb_stream
@@ -75,9 +81,9 @@ struct StreamArgs {
     int M, N, K;             // K a multiple of 8
     int ldw, down;           // words per row of W; gather rows (up) or strips of bs words of every row (down)
     int mt, nt, kb;          // token tiles, feature tiles, steps per tile
-    // how the steps are dealt out: a step costs the raw slots it takes, and one more for what does not depend on them
+    // how the steps are dealt out: a step costs the raw slots it takes, and STEP_SLOTS for what does not depend on them
     int last_cost;           // of a step of the last, possibly ragged, feature tile
-    unsigned cta_cost, cta_extra;   // total cost = gridDim.x * cta_cost + cta_extra, cta_extra < gridDim.x
+    unsigned cta_cost, cta_extra;   // total cost = gridDim.x * cta_cost + cta_extra, cta_extra < gridDim.x; 0: a step per CTA
     const uint8_t* tmask;    // per-token mask [M, tmask_ld] over the active blocks of the contraction index, or null:
     int tmask_ld;            // where it is zero, neither X nor A_i has an entry
     const int32_t* row_label;   // component label per token (negative: the row is not opened), or null
@@ -115,12 +121,13 @@ __device__ __forceinline__ StreamSegment stream_segment(const StreamArgs& a, uns
 
 // Raw slots the weight side of a feature tile takes per step.
 __device__ __forceinline__ int stream_quarters(const StreamArgs& a, int tn) {
-    return tn + 1 < a.nt ? limb_stream::QUARTERS : a.last_cost - 1;
+    return tn + 1 < a.nt ? limb_stream::QUARTERS : a.last_cost - limb_stream::STEP_SLOTS;
 }
 
 // First step of the range that begins at cost b * cta_cost + min(b, cta_extra).
 __device__ __forceinline__ unsigned stream_cut(const StreamArgs& a, unsigned b) {
-    constexpr unsigned FULL = limb_stream::QUARTERS + 1;
+    if (a.cta_cost == 0) return b;
+    constexpr unsigned FULL = limb_stream::QUARTERS + limb_stream::STEP_SLOTS;
     const unsigned cost = b * a.cta_cost + min(b, a.cta_extra);
     const unsigned whole = (unsigned)a.kb * (unsigned)a.mt * (unsigned)(a.nt - 1);     // steps of full feature tiles
     return cost < FULL * whole ? cost / FULL : whole + (cost - FULL * whole) / (unsigned)a.last_cost;
@@ -136,7 +143,7 @@ __device__ __forceinline__ void stream_copies_arrive(uint32_t bar) {
 }
 
 __global__ void __launch_bounds__(limb_stream::THREADS, 1)
-combine_stream_kernel(const __grid_constant__ StreamArgs a) {
+combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constant__ LimbMaps maps) {
     using namespace limb_stream;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t raw_full[RAW_SLOTS], raw_empty[RAW_SLOTS];
@@ -399,8 +406,9 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a) {
             }
             if (!ok) break;
             // ---------------- epilogue of the segment: lane = output feature, registers = tokens ----------------
-            // Result rows go through shared memory: lane t < OUT_TOKENS owns row t of the buffer and adds it into Z with one
-            // bulk reduction.  (64-bit atomics from registers took twice as long.)
+            // Result rows go through shared memory, OUT_TOKENS of them at a time, and one tensor reduction adds them into Z.
+            // A CTA's last segment stages them in the raw ring, which nothing uses any more, so that no round waits for the
+            // copy engine to have read the one before.  (One buffer and a bulk reduction per row: 7400 cycles for 32 tokens.)
             if (!z_ready) pdl_wait();                            // Z holds C_i
             z_ready = true;
             ok = limb_wait_warp(ptx::smem_u32(&acc_full[party]), seg_phase, &abort_flag);
@@ -408,25 +416,26 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a) {
             ptx::fence_after_sync();
             const int col0 = sg.tn * BW + quarter * 32, cols = min(a.N - col0, 32), tokens = min(a.M - sg.tm * BT, BT);
             const uint32_t acc = tmem_base + party * ACC_COLS + ((uint32_t)(quarter * 32) << 16);
-            u64* z = (party ? a.Z[1] : a.Z[0]) + (size_t)(sg.tm * BT + lane) * a.N + col0;
+            const bool at_end = u >= u_end;
+            u64* stage = at_end ? reinterpret_cast<u64*>(sRaw + (size_t)(warp - TOK_WARP0) * (BT / OUT_TOKENS) * OUT_BYTES) : out;
 #pragma unroll 1
             for (int t0 = 0; t0 < tokens; t0 += OUT_TOKENS) {
                 uint32_t d[PLANES][OUT_TOKENS];
 #pragma unroll
                 for (int s = 0; s < PLANES; ++s) ptx::tmem_ld4(acc + BT * s + t0, d[s]);
                 ptx::tmem_wait_ld();
-                if (lane < OUT_TOKENS) ptx::bulk_wait_group_read0();     // the last reduction has read its row
+                if (lane == 0 && !at_end) ptx::bulk_wait_group_read0();  // the last reduction has read its rows
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < OUT_TOKENS; ++j)
-                    out[j * 32 + lane] = limb_recombine(d[0][j], d[1][j], d[2][j], d[3][j], d[4][j], d[5][j], d[6][j], d[7][j]);
+                    stage[j * 32 + lane] = limb_recombine(d[0][j], d[1][j], d[2][j], d[3][j], d[4][j], d[5][j], d[6][j], d[7][j]);
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
-                if (lane < OUT_TOKENS) {
-                    if (t0 + lane < tokens && cols > 0)
-                        ptx::bulk_reduce_add_u64(z + (size_t)t0 * a.N, ptx::smem_u32(out + lane * 32), (uint32_t)cols * 8u);
+                if (lane == 0 && cols > 0) {
+                    ptx::tensor_reduce_add(&maps.z[party], ptx::smem_u32(stage), col0, sg.tm * BT + t0);
                     ptx::bulk_commit_group();
                 }
+                if (at_end) stage += OUT_TOKENS * 32;
             }
             ptx::fence_before_sync();
             __syncwarp();
@@ -434,7 +443,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a) {
             seg_phase ^= 1u;
         }
         if (!z_ready) pdl_wait();                                // every CTA waits for its predecessor once
-        if (lane < OUT_TOKENS) ptx::bulk_wait_group0();
+        if (lane == 0) ptx::bulk_wait_group0();
     } else if (warp == MMA_WARP) {
         // ---------------- MMA issuer: weight plane q against token planes 0..7-q ----------------
         if (lane == 0) {

@@ -6,6 +6,7 @@
 #include <chrono>
 #include <cstdio>
 #include <cstring>
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 #include <new>
@@ -78,6 +79,11 @@ struct comet_ctx {
     int32_t group_units_up, group_units_dn;   // k-block units per party of the two grouped launches
     int64_t component_pairs;      // sum over components of token rows x active blocks
     int32_t* d_ids;
+    comet::BlockIds held;         // the ids of a mask the host held, when there are few enough blocks (ids_held)
+    bool ids_held;
+    uint32_t* d_stream_sync;      // StreamArgs::sync: a ticket counter, a flag per tile of the streaming kernel
+    size_t stream_sync_words;
+    uint32_t stream_tickets, stream_epoch;    // tickets taken and streaming kernels launched so far
     int32_t* d_count;             // {count, error flag of the bounded waits}
     int32_t* h_count;             // pinned and mapped: {count, error flag as the compaction kernel saw it, ticket,
                                   // error word written by a kernel whose bounded wait ran out}
@@ -260,9 +266,10 @@ bool result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_rows, int 
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Z <- C, then the streaming kernel behind it (it begins while the copy runs and waits for it before its first sum).
-int launch_stream(comet::StreamArgs& args, const u64* const C[2], int sm_count, cudaStream_t stream,
-                  const int* priority, cudaError_t* err) {
+// The streaming kernel.  Without `sync` words (they belong to one stream's order, so a call without a context has none) Z <- C
+// is a launch of its own before it; the product begins while the copy runs and waits for it before its first sum.
+int launch_stream(comet::StreamArgs& args, const comet::BlockIds& held, int sm_count, cudaStream_t stream,
+                  const int* priority, cudaError_t* err, unsigned* grid_out) {
     namespace ls = comet::limb_stream;
     *err = cudaSuccess;
     args.mt = ceil_div(args.M, ls::BT);
@@ -271,19 +278,24 @@ int launch_stream(comet::StreamArgs& args, const u64* const C[2], int sm_count, 
     const long long steps = (long long)args.mt * args.nt * args.kb;
     const unsigned grid = (unsigned)(steps < sm_count ? steps : sm_count);
     args.last_cost = ceil_div(args.N - (args.nt - 1) * ls::BW, ls::QROWS) + ls::STEP_SLOTS;
-    const long long cost = ((long long)(ls::QUARTERS + ls::STEP_SLOTS) * (args.nt - 1) + args.last_cost) * args.kb * args.mt;
+    args.own_cost = args.sync ? (unsigned)ceil_div(ls::OWN_SIXTEENTHS * (args.M < ls::BT ? args.M : ls::BT), 16) : 0u;
+    const long long cost = (((long long)(ls::QUARTERS + ls::STEP_SLOTS) * (args.nt - 1) + args.last_cost) * args.kb +
+                            (long long)args.own_cost * args.nt) * args.mt;
     if (cost > 0x7fffffffll) return COMET_ERR_SHAPE;                   // the kernel counts in 32 bits
     args.cta_cost = steps > sm_count ? (unsigned)(cost / grid) : 0u;
     args.cta_extra = (unsigned)(cost % grid);
     comet::LimbMaps maps;
     for (int p = 0; p < 2; ++p)
         if (!result_map(&maps.z[p], args.Z[p], args.M, args.N, ls::OUT_TOKENS, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) return COMET_ERR_CUDA;
-    const long long pairs = (long long)args.M * args.N / 2, want = (pairs + 255) / 256, most = (long long)sm_count * 8;
-    *err = launch_chained(comet::result_init_kernel, dim3((unsigned)(want < most ? want : most), 2), dim3(256), 0, stream,
-                          nullptr, C[0], C[1], args.Z[0], args.Z[1], pairs);
-    if (*err != cudaSuccess) return COMET_ERR_CUDA;
+    if (!args.sync) {
+        const long long pairs = (long long)args.M * args.N / 2, want = (pairs + 255) / 256, most = (long long)sm_count * 8;
+        *err = launch_chained(comet::result_init_kernel, dim3((unsigned)(want < most ? want : most), 2), dim3(256), 0, stream,
+                              nullptr, args.C[0], args.C[1], args.Z[0], args.Z[1], pairs);
+        if (*err != cudaSuccess) return COMET_ERR_CUDA;
+    }
+    *grid_out = grid;
     *err = launch_chained(comet::combine_stream_kernel, dim3(grid), dim3(ls::THREADS), ls::SMEM_BYTES, stream,
-                          priority, args, maps);
+                          priority, args, maps, held);
     return *err == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
 }
 
@@ -292,7 +304,6 @@ int stream_product(comet_ctx* c, const Proj& pr) {
     namespace ls = comet::limb_stream;
     comet::StreamArgs a;
     std::memset(&a, 0, sizeof(a));
-    const u64* C[2];
     for (int p = 0; p < 2; ++p) {
         a.X[p] = c->buf[p][pr.idX];
         a.A[p] = c->buf[p][pr.idA];
@@ -303,9 +314,14 @@ int stream_product(comet_ctx* c, const Proj& pr) {
         a.B[p] = c->buf[p][pr.idB];
         a.F[p] = c->buf[p][pr.idF];
         a.Z[p] = c->buf[p][pr.idZ];
-        C[p] = c->buf[p][pr.idC];
+        a.C[p] = c->buf[p][pr.idC];
     }
-    a.ids = c->d_ids;
+    if (1 + (size_t)ceil_div(pr.M, ls::BT) * ceil_div(pr.N, ls::BW) > c->stream_sync_words) return COMET_ERR_SHAPE;
+    a.sync = c->d_stream_sync;
+    a.ticket0 = c->stream_tickets;
+    a.epoch = c->stream_epoch + 1 == 0 ? 1 : c->stream_epoch + 1;
+    a.gather = 1;
+    a.ids = c->ids_held ? nullptr : c->d_ids;
     a.n = c->n_active;
     a.bs = c->cfg.block;
     a.M = pr.M; a.N = pr.N; a.K = pr.K;
@@ -321,14 +337,17 @@ int stream_product(comet_ctx* c, const Proj& pr) {
     a.error_host = c->h_count_dev + 3;
     cudaError_t err;
     {
-        PhaseTimer timer(c, COMET_PHASE_COMBINE, 2);
-        const int rc = launch_stream(a, C, c->sm_count, c->stream, &c->top_priority, &err);
+        PhaseTimer timer(c, COMET_PHASE_COMBINE, 1);
+        unsigned grid = 0;
+        const int rc = launch_stream(a, c->held, c->sm_count, c->stream, &c->top_priority, &err, &grid);
         if (rc != COMET_OK) {
             c->last_cuda_error = (int)err;
             return rc;
         }
+        c->stream_tickets += grid;
+        c->stream_epoch = a.epoch;
     }
-    c->stats.kernel_launches += 2;
+    c->stats.kernel_launches += 1;
     c->stats.tensor_tile_macs = 2ll * 2 * a.mt * a.nt * a.kb * ls::KC * ls::BW * ls::BT;
     c->stats.matmul_path = COMET_PATH_LIMB;
     return COMET_OK;
@@ -364,7 +383,7 @@ int exchange_args(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy
     }
     a.Epl = c->planes_left[2];
     a.Fpl = planes[2];
-    a.ids = c->d_ids;
+    a.ids = c->ids_held ? nullptr : c->d_ids;
     a.n = c->n_active;
     a.bs = c->cfg.block;
     a.M = pr.M; a.N = pr.N; a.K = pr.K;
@@ -405,7 +424,7 @@ int limb_exchange(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy
     if (blocks + also_blocks == 0) return COMET_OK;
     const bool tiles = left || right || also_blocks;
     COMET_CUDA(c, launch_chained(comet::limb_exchange_kernel, dim3(blocks + also_blocks), dim3(lb::EX_THREADS),
-                                 tiles ? lb::EX_SMEM_BYTES : 0, stream, nullptr, a, also ? *also : a, blocks));
+                                 tiles ? lb::EX_SMEM_BYTES : 0, stream, nullptr, a, also ? *also : a, blocks, c->held));
     c->stats.kernel_launches += 1;
     COMET_CUDA(c, cudaGetLastError());
     return COMET_OK;
@@ -649,6 +668,12 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
     reserve(device, &c->d_blk_label, (size_t)nb * sizeof(int32_t));
     reserve(device, &c->d_ids, (size_t)nb * sizeof(int32_t));
     reserve(device, &c->d_count, 2 * sizeof(int32_t));              // {count, error flag}
+    {
+        namespace ls = comet::limb_stream;
+        const int64_t widest = c->groups * c->cap_n > cfg->d_model ? c->groups * c->cap_n : cfg->d_model;
+        c->stream_sync_words = 1 + (size_t)((widest + ls::BW - 1) / ls::BW);
+        reserve(device, &c->d_stream_sync, c->stream_sync_words * sizeof(uint32_t));
+    }
     reserve(pinned, &c->h_masked, 7 * sizeof(long long));
     reserve(pinned, &c->h_count, 4 * sizeof(int32_t));
     reserve(pinned, &c->h_mask_stage, (size_t)nb * 4);
@@ -676,6 +701,7 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
         c->h_count[0] = c->h_count[1] = c->h_count[2] = c->h_count[3] = 0;     // pinned memory is not zeroed
     }
     ok = ok && cudaMemset(c->d_count, 0, 2 * sizeof(int32_t)) == cudaSuccess;
+    ok = ok && cudaMemset(c->d_stream_sync, 0, c->stream_sync_words * sizeof(uint32_t)) == cudaSuccess;
     ok = ok && cudaHostGetDevicePointer((void**)&c->h_masked_dev, c->h_masked, 0) == cudaSuccess;
     ok = ok && cudaHostGetDevicePointer((void**)&c->h_count_dev, c->h_count, 0) == cudaSuccess;
     if (!ok) {
@@ -769,19 +795,30 @@ int comet_set_mask(comet_ctx* c, const uint8_t* block_mask, int location, int32_
     const uint8_t* dmask = block_mask;         // a device mask is read in place
     int32_t host_count = -1;                   // number of active blocks when the host could count them itself
     bool launched = false;
+    c->ids_held = location == COMET_HOST && n_blocks <= comet::BlockIds::CAPACITY && c->path == COMET_PATH_LIMB;
     if (location == COMET_HOST) {
         // The count is public (Section 3.2) and the mask is in host memory: count here and do not wait for the
-        // device.  A mask that fits into a kernel's parameter block travels with the launch; a larger one is handed
+        // device.  The index list of a mask of up to 1024 blocks is made here and travels with the launches that gather; a
+        // mask that fits into a kernel's parameter block travels with the compaction's launch; a larger one is handed
         // to the copy engine from a pinned slot of our own (the caller's buffer is free again on return either way).
         host_count = 0;
-        for (int32_t b = 0; b < n_blocks; ++b) host_count += block_mask[b] != 0;
-        if (n_blocks <= comet::MaskBytes::CAPACITY) {
+        if (c->ids_held) {
+            for (int32_t b = 0; b < n_blocks; ++b)
+                if (block_mask[b]) c->held.id[host_count++] = (uint16_t)b;
+            launched = true;
+        } else {
+            for (int32_t b = 0; b < n_blocks; ++b) host_count += block_mask[b] != 0;
+        }
+        if (launched) {
+            // nothing to launch
+        } else if (n_blocks <= comet::MaskBytes::CAPACITY) {
             comet::MaskBytes arg;
             std::memcpy(arg.bytes, block_mask, (size_t)n_blocks);
             PhaseTimer timer(c, COMET_PHASE_COMPACT, 1);
             c->ticket += 1;
             COMET_CUDA(c, launch_chained(comet::compact_mask_arg_kernel, dim3(1), dim3(1024), 0, c->stream, nullptr, arg,
                                          (int)n_blocks, c->d_ids, c->d_count, (int32_t*)nullptr, c->ticket));
+            c->stats.kernel_launches += 1;
             launched = true;
         } else {
             const int slot = c->stage_next;
@@ -802,8 +839,8 @@ int comet_set_mask(comet_ctx* c, const uint8_t* block_mask, int location, int32_
         COMET_CUDA(c, launch_chained(comet::compact_mask_kernel, dim3(1), dim3(1024), 0, c->stream, nullptr, dmask,
                                      (int)n_blocks, c->d_ids, c->d_count, host_count < 0 ? c->h_count_dev : (int32_t*)nullptr,
                                      c->ticket));
+        c->stats.kernel_launches += 1;
     }
-    c->stats.kernel_launches += 1;
     COMET_CUDA(c, cudaGetLastError());
     if (host_count < 0) {
         // The kernel is the last thing on the stream and reports through mapped memory: watching its ticket for
@@ -1157,7 +1194,12 @@ int comet_get_index(comet_ctx* c, int32_t* out, int location, int32_t capacity, 
     if (location != COMET_DEVICE && location != COMET_HOST) return COMET_ERR_INVALID_ARG;
     if (!c->mask_set) return COMET_ERR_STATE;
     if (capacity < c->n_active_blocks) return COMET_ERR_SHAPE;
-    if (c->n_active_blocks > 0)
+    if (c->ids_held) {
+        std::vector<int32_t> ids(c->held.id, c->held.id + c->n_active_blocks);
+        if (location == COMET_HOST) std::copy(ids.begin(), ids.end(), out);
+        else if (!ids.empty())        // from pageable memory: taken over before the call returns
+            COMET_CUDA(c, cudaMemcpyAsync(out, ids.data(), ids.size() * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
+    } else if (c->n_active_blocks > 0)
         COMET_CUDA(c, cudaMemcpyAsync(out, c->d_ids, (size_t)c->n_active_blocks * sizeof(int32_t),
                                       copy_kind(location, false), c->stream));
     *n_active_blocks_out = c->n_active_blocks;
@@ -1281,7 +1323,6 @@ extern "C" int comet_beaver_matmul_static(void* cuda_stream, const uint64_t* con
     // (every word used is written before anything reads it)
     comet::StreamArgs a;
     std::memset(&a, 0, sizeof(a));
-    const u64* c[2];
     for (int p = 0; p < 2; ++p) {
         a.X[p] = reinterpret_cast<const u64*>(X[p]);
         a.A[p] = reinterpret_cast<const u64*>(A[p]);
@@ -1290,13 +1331,15 @@ extern "C" int comet_beaver_matmul_static(void* cuda_stream, const uint64_t* con
         a.B[p] = reinterpret_cast<const u64*>(B[p]);
         a.F[p] = dev.scratch + 2 * left + p * right;
         a.Z[p] = reinterpret_cast<u64*>(Z[p]);
-        c[p] = reinterpret_cast<const u64*>(C[p]);
+        a.C[p] = reinterpret_cast<const u64*>(C[p]);
     }
     a.n = N; a.bs = 1;
     a.M = T; a.N = N; a.K = K;
     a.ldw = K;
     cudaError_t err;
-    const int rc = launch_stream(a, c, dev.sm_count, (cudaStream_t)cuda_stream, nullptr, &err);
+    static const comet::BlockIds none = {};
+    unsigned grid = 0;
+    const int rc = launch_stream(a, none, dev.sm_count, (cudaStream_t)cuda_stream, nullptr, &err, &grid);
     if (err != cudaSuccess) cudaGetLastError();
     return rc;
 }

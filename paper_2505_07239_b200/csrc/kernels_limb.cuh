@@ -122,7 +122,7 @@ struct LimbExchangeArgs {
     const u64* C[2];
     u64* Z[2];
     long long copy_pairs;
-    const int32_t* ids;      // ascending active block ids
+    const int32_t* ids;      // ascending active block ids, or null: they are in the launch's BlockIds
     int n, bs;               // active neurons, neurons per block
     int M, N, K;             // rows of the left and right operand, contraction length
     int ldw, down;
@@ -147,8 +147,19 @@ struct LimbExchangeArgs {
     const int32_t* kmap;
 };
 
+// The ascending active block ids of a mask that the host held: they travel in the parameter block of every kernel that gathers
+// (2 KiB), which takes the compaction launch (a few us of host time, one hop of the chain) off the step.  Longer masks and
+// masks in device memory are compacted by a kernel, and `ids` of the arguments points to its result.
+struct BlockIds {
+    static constexpr int CAPACITY = 1024;
+    uint16_t id[CAPACITY];
+};
+__device__ __forceinline__ int block_id(const int32_t* ids, const BlockIds& held, int blk) {
+    return ids ? __ldg(ids + blk) : (int)held.id[blk];
+}
+
 template <bool LEFT>
-__device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, int block, uint8_t* smem) {
+__device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, const BlockIds& held, int block, uint8_t* smem) {
     using namespace limb;
     constexpr int TILE = LEFT ? BM : BN, BLOCK_BYTES = PLANES * TILE * KC;
     const int c = threadIdx.x & 7;
@@ -173,7 +184,7 @@ __device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, in
             src[1] = a.W0[1] + (size_t)at * a.ldw;
         } else {
             const int grp = (at >= a.n) + (at >= 2 * a.n), j = at - grp * a.n, blk = j / a.bs;
-            const size_t off = (size_t)(__ldg(a.ids + blk) * a.bs + (j - blk * a.bs)) * a.ldw;
+            const size_t off = (size_t)(block_id(a.ids, held, blk) * a.bs + (j - blk * a.bs)) * a.ldw;
             closed = a.blk_label && __ldg(a.blk_label + blk) < 0;
             src[0] = (grp == 0 ? a.W0[0] : grp == 1 ? a.W1[0] : a.W2[0]) + off;
             src[1] = (grp == 0 ? a.W0[1] : grp == 1 ? a.W1[1] : a.W2[1]) + off;
@@ -207,7 +218,7 @@ __device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, in
             if (a.kmap) blk = __ldg(a.kmap + blk);
             q.ks = q.col = blk * a.bs + within;
             if (!LEFT) {
-                q.col = __ldg(a.ids + blk) * a.bs + within;
+                q.col = block_id(a.ids, held, blk) * a.bs + within;
                 if (a.blk_label && __ldg(a.blk_label + blk) < 0) q.open = false;
             } else if (a.tmask && a.tmask[(size_t)at * a.tmask_ld + blk] == 0) {
                 q.open = q.in = false;           // an entry off the support is none of the triple either
@@ -269,10 +280,10 @@ __device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, in
     limb_copy_wait<0>();
 }
 
-__device__ __forceinline__ void limb_exchange_block(const LimbExchangeArgs& a, int block, uint8_t* smem) {
-    if (block < a.left_blocks) return limb_exchange_rows<true>(a, block, smem);
+__device__ __forceinline__ void limb_exchange_block(const LimbExchangeArgs& a, const BlockIds& held, int block, uint8_t* smem) {
+    if (block < a.left_blocks) return limb_exchange_rows<true>(a, held, block, smem);
     block -= a.left_blocks;
-    if (block < a.right_blocks) return limb_exchange_rows<false>(a, block, smem);
+    if (block < a.right_blocks) return limb_exchange_rows<false>(a, held, block, smem);
     block -= a.right_blocks;
     const int party = block & 1;
     const ulonglong2* __restrict__ s = reinterpret_cast<const ulonglong2*>(party ? a.C[1] : a.C[0]);
@@ -283,13 +294,14 @@ __device__ __forceinline__ void limb_exchange_block(const LimbExchangeArgs& a, i
 
 // The first `first_blocks` CTAs work on `a`, the others on `b` (another product's operands).
 __global__ void __launch_bounds__(limb::EX_THREADS, 7)
-limb_exchange_kernel(const __grid_constant__ LimbExchangeArgs a, const __grid_constant__ LimbExchangeArgs b, int first_blocks) {
+limb_exchange_kernel(const __grid_constant__ LimbExchangeArgs a, const __grid_constant__ LimbExchangeArgs b, int first_blocks,
+                     const __grid_constant__ BlockIds held) {
     extern __shared__ __align__(16) uint8_t ex_smem[];
     pdl_wait();
     pdl_launch_dependents();
     const int block = blockIdx.x;
-    if (block < first_blocks) limb_exchange_block(a, block, ex_smem);
-    else limb_exchange_block(b, block - first_blocks, ex_smem);
+    if (block < first_blocks) limb_exchange_block(a, held, block, ex_smem);
+    else limb_exchange_block(b, held, block - first_blocks, ex_smem);
 }
 
 // ---------------------------------------------------------------------------
@@ -321,6 +333,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void bulk_s2g(void* dst, uint32_t src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
 }
 // shared -> global bulk reduction: 64-bit integer add of `bytes` (multiple of 16) contiguous bytes
 __device__ __forceinline__ void bulk_reduce_add_u64(void* dst, uint32_t src, uint32_t bytes) {

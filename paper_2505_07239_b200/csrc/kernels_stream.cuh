@@ -9,7 +9,7 @@
 // is bound by streaming the weight side.  Per word of the right operand and party that is W_i and B_i in and F_i out,
 // 24 bytes, and this kernel moves nothing else of that size: the limb planes the tensor cores read exist in shared
 // memory only.  (Its predecessor wrote the planes of B_i and F_i to memory and read them back: 56 bytes per word.)
-// Measured, both parties: [32, 4096] x [4096, 1312] 52 us and [7, 4096] x [4096, 3328] 104 us from a CTA's start to its end,
+// Measured, both parties: [32, 4096] x [4096, 1312] 50 us and [7, 4096] x [4096, 3328] 104 us from a CTA's start to its end,
 // where 24 bytes per weight word at the measured copy rate are 39 and 100 us; a step of 192 KiB takes 8400 cycles, 95 % of that
 // rate, the rest is 2 us until the first bytes arrive and 4 us from the last planes to the end (MMAs 3100 cycles, drain of 32
 // tokens 4000, of 7 tokens 1200, the reductions' completion 900).
@@ -25,6 +25,8 @@
 //                 planes of E, A_0, A_1 + E; at the end of a segment the same warps are the epilogue (four per party): TMEM
 //                 -> recombine mod 2^64 -> rows staged in shared memory -> tensor add-reductions into Z
 //   warp 26       issues the MMAs: F is the same for both parties, so three weight-side plane sets serve four products
+//   warp 27       Z_i <- C_i for the tiles that begin in this CTA's range, and a flag on each, which every CTA that adds to the
+//                 tile waits for.  (As a kernel of its own before this one it cost a launch, and 1.5 us between two products.)
 // Shared memory: 96 KiB weight planes, 24 KiB token planes, 96 KiB raw ring, 8 KiB result rows; all 512 TMEM columns (two
 // parties x eight accumulators x 32 tokens).  The planes are single-buffered: converting a step and multiplying it take
 // turns, while the ring and the converters' registers keep up to 160 KiB of loads in flight.
@@ -48,7 +50,7 @@ constexpr int BW = 128, BT = 32, KC = limb::KC, PLANES = limb::PLANES, QROWS = 3
 constexpr int CONV_GROUPS = 2, GROUP_WARPS = 8, CONV_WARPS = CONV_GROUPS * GROUP_WARPS;
 constexpr int RAW_WARP0 = CONV_WARPS, TOK_WARP0 = RAW_WARP0 + 2, TOK_WARPS = 8, MMA_WARP = TOK_WARP0 + TOK_WARPS;
 constexpr int EPI_WARPS = TOK_WARPS / 2;                 // per party
-constexpr int THREADS = 32 * (MMA_WARP + 1);
+constexpr int INIT_WARP = MMA_WARP + 1, THREADS = 32 * (INIT_WARP + 1);
 constexpr int RAW_ARRAY_BYTES = QROWS * KC * 8;          // 8 KiB: one array of a slot
 constexpr int RAW_SLOT_BYTES = 4 * RAW_ARRAY_BYTES;      // party 0: W | B, party 1: W | B
 constexpr int RAW_SLOTS = 3;
@@ -65,6 +67,9 @@ constexpr int MAX_SEGMENT_STEPS = limb::MAX_SEGMENT_UNITS / 2;
 // Measured on [32, 4096] x [4096, 1312]: 8600 cycles with four slots, 4800 to 5600 with one (the last tile's).  Counted as one
 // slot, the CTAs of that tile ran 67 us where the others took 52, and the layer 134 us; as three 124.4, as five 122.2.
 constexpr int STEP_SLOTS = 5;
+// And what Z <- C costs for one token row of a tile, in sixteenths of a slot: 4 KiB of traffic are three, and the first planes
+// wait for it.  Counted as nothing the opt6.7b decode layer takes 122 us, as three 119.5, as five 116.6.
+constexpr int OWN_SIXTEENTHS = 5;
 constexpr size_t SMEM_BYTES = 3 * (size_t)W_SET_BYTES + 3 * (size_t)T_SET_BYTES + (size_t)RAW_SLOTS * RAW_SLOT_BYTES +
                               (size_t)TOK_WARPS * OUT_BYTES + 128;
 }  // namespace limb_stream
@@ -75,14 +80,21 @@ struct StreamArgs {
     const u64* W0[2]; const u64* W1[2]; const u64* W2[2]; // weights of the stacked groups (down: W0 alone)
     const u64* B[2];                                      // [N, K]
     u64* F[2];                                            // message, [N, K]
-    u64* Z[2];                                            // [M, N], holds C_i; written by the kernel before this one
-    const int32_t* ids;      // ascending active block ids; null: the right operand is W0 itself, [N, K], no gather
+    u64* Z[2];                                            // [M, N]
+    const u64* C[2];                                      // [M, N]: what the sums are added to
+    // [1 + tiles] words of one context, or null (then Z holds C when the kernel before this one has completed): a ticket
+    // counter, and per tile the epoch of the last launch in which its part of Z became C
+    uint32_t* sync;
+    uint32_t ticket0, epoch; // the counter's value when this launch takes its first ticket; this launch's number, never 0
+    int gather;              // 0: the right operand is W0 itself, [N, K]
+    const int32_t* ids;      // ascending active block ids, or null: they are in the launch's BlockIds
     int n, bs;               // active neurons, neurons per block (a multiple of 16 when there are ids)
     int M, N, K;             // K a multiple of 8
     int ldw, down;           // words per row of W; gather rows (up) or strips of bs words of every row (down)
     int mt, nt, kb;          // token tiles, feature tiles, steps per tile
     // how the steps are dealt out: a step costs the raw slots it takes, and STEP_SLOTS for what does not depend on them
     int last_cost;           // of a step of the last, possibly ragged, feature tile
+    unsigned own_cost;       // of Z <- C for a tile, before its first step
     unsigned cta_cost, cta_extra;   // total cost = gridDim.x * cta_cost + cta_extra, cta_extra < gridDim.x; 0: a step per CTA
     const uint8_t* tmask;    // per-token mask [M, tmask_ld] over the active blocks of the contraction index, or null:
     int tmask_ld;            // where it is zero, neither X nor A_i has an entry
@@ -106,12 +118,13 @@ result_init_kernel(const u64* __restrict__ c0, const u64* __restrict__ c1, u64* 
 
 // A run of steps of one tile, at most MAX_SEGMENT_STEPS of them.
 struct StreamSegment {
-    int tm, tn, step, count;
+    int tile, tm, tn, step, count;
 };
 
 __device__ __forceinline__ StreamSegment stream_segment(const StreamArgs& a, unsigned u, unsigned u_end) {
     StreamSegment s;
     const unsigned tile = u / (unsigned)a.kb;
+    s.tile = (int)tile;
     s.step = (int)(u - tile * a.kb);
     s.tn = a.mt == 1 ? (int)tile : (int)(tile / (unsigned)a.mt);
     s.tm = (int)tile - s.tn * a.mt;
@@ -128,9 +141,15 @@ __device__ __forceinline__ int stream_quarters(const StreamArgs& a, int tn) {
 __device__ __forceinline__ unsigned stream_cut(const StreamArgs& a, unsigned b) {
     if (a.cta_cost == 0) return b;
     constexpr unsigned FULL = limb_stream::QUARTERS + limb_stream::STEP_SLOTS;
-    const unsigned cost = b * a.cta_cost + min(b, a.cta_extra);
-    const unsigned whole = (unsigned)a.kb * (unsigned)a.mt * (unsigned)(a.nt - 1);     // steps of full feature tiles
-    return cost < FULL * whole ? cost / FULL : whole + (cost - FULL * whole) / (unsigned)a.last_cost;
+    const unsigned kb = (unsigned)a.kb, full_tiles = (unsigned)a.mt * (unsigned)(a.nt - 1);
+    unsigned cost = b * a.cta_cost + min(b, a.cta_extra), step_cost = FULL, tile = 0;
+    if (cost >= full_tiles * (a.own_cost + kb * FULL)) {
+        cost -= full_tiles * (a.own_cost + kb * FULL);
+        step_cost = (unsigned)a.last_cost;
+        tile = full_tiles;
+    }
+    const unsigned tile_cost = a.own_cost + kb * step_cost, t = cost / tile_cost, in = cost - t * tile_cost;
+    return (tile + t) * kb + (in > a.own_cost ? (in - a.own_cost) / step_cost : 0u);
 }
 
 // 16-byte asynchronous copy global -> shared that bypasses L1, and this thread's arrival on `bar` once all its copies so
@@ -142,14 +161,42 @@ __device__ __forceinline__ void stream_copies_arrive(uint32_t bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];" ::"r"(bar) : "memory");
 }
 
+// Whether the first step of some tile is in the range.
+__device__ __forceinline__ bool stream_owns(const StreamArgs& a, unsigned u_begin, unsigned u_end) {
+    return (u_begin + a.kb - 1) / a.kb < (u_end + a.kb - 1) / a.kb;
+}
+
+// The bounded wait for a tile's flag, one lane per warp (the one that issues the warp's reductions).
+__device__ __forceinline__ bool stream_tile_ready(const uint32_t* flag, uint32_t epoch, int lane, volatile int* abort_flag) {
+    bool ok = true;
+    if (lane == 0) {
+        const long long t0 = clock64();
+        for (;;) {
+            uint32_t seen;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
+            if (seen == epoch) break;
+            if (*abort_flag || clock64() - t0 > limb::WAIT_CYCLES) {
+                *abort_flag = 1;
+                ok = false;
+                break;
+            }
+            __nanosleep(40);
+        }
+        asm volatile("fence.proxy.async;" ::: "memory");
+    }
+    return __all_sync(0xffffffffu, ok);
+}
+
 __global__ void __launch_bounds__(limb_stream::THREADS, 1)
-combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constant__ LimbMaps maps) {
+combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constant__ LimbMaps maps,
+                      const __grid_constant__ BlockIds held) {
     using namespace limb_stream;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t raw_full[RAW_SLOTS], raw_empty[RAW_SLOTS];
     __shared__ __align__(8) uint64_t planes_full, own_empty[2], shared_empty;     // own: B_0 / B_1; shared: F, E, V_i
     __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
-    __shared__ uint32_t tmem_slot;
+    __shared__ __align__(8) uint64_t own_landed, own_stored;                      // C of a tile of this CTA's: in, and out again
+    __shared__ uint32_t tmem_slot, ticket;
     __shared__ int abort_flag;
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
@@ -159,8 +206,8 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
     uint8_t* sOut = sRaw + RAW_SLOTS * RAW_SLOT_BYTES;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned u_begin = stream_cut(a, blockIdx.x), u_end = stream_cut(a, blockIdx.x + 1);
 
+    if (threadIdx.x == 32) ticket = a.sync ? atomicAdd(a.sync, 1u) - a.ticket0 : blockIdx.x;
     if (threadIdx.x == 0) {
         for (int s = 0; s < RAW_SLOTS; ++s) {
             ptx::mbar_init(ptx::smem_u32(&raw_full[s]), 64);                // every producer lane
@@ -173,6 +220,8 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             ptx::mbar_init(ptx::smem_u32(&acc_full[p]), 1);
             ptx::mbar_init(ptx::smem_u32(&acc_empty[p]), EPI_WARPS);
         }
+        ptx::mbar_init(ptx::smem_u32(&own_landed), 1);
+        ptx::mbar_init(ptx::smem_u32(&own_stored), 1);
         abort_flag = 0;
         ptx::fence_barrier_init();
     }
@@ -184,8 +233,10 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
     __syncthreads();
     ptx::fence_after_sync();
     const uint32_t tmem_base = tmem_slot;
-    // No wait for the predecessor here: it is the kernel that initialises Z, which only the epilogue touches.  That
-    // kernel let this one start after its own wait, so whatever came before it has completed.
+    const unsigned cta = ticket, u_begin = stream_cut(a, cta), u_end = stream_cut(a, cta + 1);
+    // Without `sync` there is no wait for the predecessor here: it is the kernel that initialises Z, which only the epilogue
+    // touches.  That kernel let this one start after its own wait, so whatever came before it has completed.
+    if (a.sync) pdl_wait();
 
     if (warp >= RAW_WARP0 && warp < RAW_WARP0 + 2) {
         // ---------------- raw producer of one party: 16 lanes per row of a slot ----------------
@@ -206,12 +257,12 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             {
                 const int row = sg.tn * BW + (lane & 7) * 16;
                 if (row < a.N) {
-                    if (a.ids == nullptr || a.down) {
+                    if (!a.gather || a.down) {
                         w_row16 = W0 + (size_t)row * a.ldw;
                     } else {
                         const int grp = (row >= a.n) + (row >= 2 * a.n), j = row - grp * a.n, blk = j / a.bs;
                         w_row16 = (grp == 0 ? W0 : grp == 1 ? (party ? a.W1[1] : a.W1[0]) : (party ? a.W2[1] : a.W2[0])) +
-                                  (size_t)(__ldg(a.ids + blk) * a.bs + (j - blk * a.bs)) * a.ldw;
+                                  (size_t)(block_id(a.ids, held, blk) * a.bs + (j - blk * a.bs)) * a.ldw;
                     }
                 }
             }
@@ -219,9 +270,9 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                 const int k = (sg.step + it) * KC + 2 * piece;
                 const bool kv = k < a.K;
                 int col = k;                                      // this lane's column of W
-                if (a.down && a.ids != nullptr && kv) {
+                if (a.down && a.gather && kv) {
                     const int blk = ((sg.step + it) * KC + 16 * half) / a.bs;
-                    col = __ldg(a.ids + blk) * a.bs + (k - blk * a.bs);
+                    col = block_id(a.ids, held, blk) * a.bs + (k - blk * a.bs);
                 }
                 for (int q = 0; q < quarters; ++q) {
                     const int row0 = sg.tn * BW + q * QROWS + rsub;
@@ -261,7 +312,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
         const int cell = (r >> 3) * 256 + (c >> 2) * 128 + (r & 7) * 16 + (c & 3) * 4;
         int slot = 0;
         uint32_t phase = 0, unit_phase = 0;
-        bool ok = true;
+        bool ok = true, planes_free = !a.sync || !stream_owns(a, u_begin, u_end);
         for (unsigned u = u_begin; u < u_end && ok;) {
             const StreamSegment sg = stream_segment(a, u, u_end);
             u += sg.count;
@@ -320,8 +371,10 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
 #pragma unroll
                     for (int e = 0; e < 4; ++e) f[0][e] += f[1][e];  // the exchange
                     uint8_t* to = sB + q * (QROWS / 8) * 256 + cell;
+                    if (!planes_free) ok = limb_wait(ptx::smem_u32(&own_stored), 0, &abort_flag);
+                    planes_free = true;
                     // a step's first planes: the MMAs of the step before must have read the old ones
-                    if (first) ok = limb_wait(ptx::smem_u32(&own_empty[0]), unit_phase ^ 1u, &abort_flag);
+                    if (first) ok = ok && limb_wait(ptx::smem_u32(&own_empty[0]), unit_phase ^ 1u, &abort_flag);
                     limb_emit4(to, W_PLANE_BYTES, b[0]);
                     if (first) ok = ok && limb_wait(ptx::smem_u32(&own_empty[1]), unit_phase ^ 1u, &abort_flag);
                     limb_emit4(to + W_SET_BYTES, W_PLANE_BYTES, b[1]);
@@ -347,7 +400,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
         const int party = (warp - TOK_WARP0) / EPI_WARPS, quarter = warp & 3;     // epilogue: TMEM lanes this warp may read
         u64* out = reinterpret_cast<u64*>(sOut + (size_t)(warp - TOK_WARP0) * OUT_BYTES);
         uint32_t unit_phase = 0, seg_phase = 0;
-        bool ok = true, z_ready = false;
+        bool ok = true, z_ready = a.sync != nullptr;
         for (unsigned u = u_begin; u < u_end && ok;) {
             const StreamSegment sg = stream_segment(a, u, u_end);
             u += sg.count;
@@ -411,7 +464,8 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             // copy engine to have read the one before.  (One buffer and a bulk reduction per row: 7400 cycles for 32 tokens.)
             if (!z_ready) pdl_wait();                            // Z holds C_i
             z_ready = true;
-            ok = limb_wait_warp(ptx::smem_u32(&acc_full[party]), seg_phase, &abort_flag);
+            if (a.sync) ok = stream_tile_ready(a.sync + 1 + sg.tile, a.epoch, lane, &abort_flag);
+            ok = ok && limb_wait_warp(ptx::smem_u32(&acc_full[party]), seg_phase, &abort_flag);
             if (!ok) break;
             ptx::fence_after_sync();
             const int col0 = sg.tn * BW + quarter * 32, cols = min(a.N - col0, 32), tokens = min(a.M - sg.tm * BT, BT);
@@ -489,6 +543,40 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             }
             // the main loop is over: the next kernel of the stream may be brought in beside the last drain
             pdl_launch_dependents();
+        }
+    } else if (a.sync && stream_owns(a, u_begin, u_end)) {
+        // ---------------- Z <- C for the tiles whose first step is in this CTA's range ----------------
+        // By the copy engine, a lane per token row, through the weight planes' place before the first of them is written; the
+        // loads go out before the raw ones fill the queue.  (The token warps' own loads and stores, queued behind the raw
+        // copies, held the first planes back by 10000 cycles.)  Then the flag.  Whoever adds to a tile waits for its flag
+        // first: a CTA with the same or an earlier ticket sets it, and a CTA that has a ticket is running, so the wait ends
+        // whatever else is on the device and in whatever order the CTAs were started.
+        const unsigned last = (u_end + a.kb - 1) / a.kb;
+        bool ok = true;
+        uint32_t phase = 0;
+        for (unsigned tile = (u_begin + a.kb - 1) / a.kb; tile < last && ok; ++tile, phase ^= 1u) {
+            const int tn = (int)(tile / (unsigned)a.mt), tm = (int)tile - tn * a.mt;
+            const int rows = min(a.M - tm * BT, BT), bytes = min(a.N - tn * BW, BW) * 8;
+            const size_t at = (size_t)(tm * BT + lane) * a.N + tn * BW;
+            const uint32_t place = ptx::smem_u32(sB) + lane * (2 * BW * 8);
+            if (lane == 0) ptx::mbar_expect_tx(ptx::smem_u32(&own_landed), 2 * rows * bytes);
+            __syncwarp();
+            if (lane < rows)
+                for (int p = 0; p < 2; ++p)
+                    ptx::bulk_g2s(place + p * (BW * 8), a.C[p] + at, bytes, ptx::smem_u32(&own_landed));
+            ok = limb_wait_warp(ptx::smem_u32(&own_landed), phase, &abort_flag);
+            if (!ok) break;
+            if (lane < rows)
+                for (int p = 0; p < 2; ++p) ptx::bulk_s2g(a.Z[p] + at, place + p * (BW * 8), bytes);
+            ptx::bulk_commit_group();
+            ptx::bulk_wait_group_read0();
+            __syncwarp();
+            if (lane == 0 && tile + 1 == last) ptx::mbar_arrive(ptx::smem_u32(&own_stored));
+            ptx::bulk_wait_group0();
+            asm volatile("fence.proxy.async;" ::: "memory");
+            __threadfence();
+            __syncwarp();
+            if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.sync + 1 + tile), "r"(a.epoch) : "memory");
         }
     }
 

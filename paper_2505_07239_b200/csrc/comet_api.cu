@@ -63,9 +63,10 @@ struct comet_ctx {
     bool tmask_set;
     int32_t tmask_tokens;
     int64_t tmask_masked;         // non-zero entries of the hidden state under the token mask (neurons, not blocks)
-    long long* h_masked;          // pinned and mapped: token_plan_kernel's report [0..6]
+    unsigned long long* h_masked; // pinned and mapped: token_plan_kernel's report
+    unsigned long long plan_ticket;   // of its last launch
     uint32_t* d_plan_scratch;     // its working storage when that does not fit into shared memory
-    long long* h_masked_dev;
+    unsigned long long* h_masked_dev;
     int32_t* d_row_label;         // component label per token row / per active block under the token mask
     int32_t* d_blk_label;
     int32_t n_components, live_rows, live_blocks;
@@ -353,6 +354,19 @@ int stream_product(comet_ctx* c, const Proj& pr) {
     return COMET_OK;
 }
 
+// Waits for a kernel's report: it is the last thing on the stream and reports through mapped memory, with a ticket.  Watching
+// for the ticket for a short while is quicker than a stream synchronise; after that, synchronise as usual.
+template <typename Arrived>
+int wait_for_report(comet_ctx* c, Arrived report) {
+    const auto t0 = std::chrono::steady_clock::now();
+    bool arrived = false;
+    while (!(arrived = report()))
+        if (std::chrono::steady_clock::now() - t0 > std::chrono::microseconds(300)) break;
+    if (!arrived) COMET_CUDA(c, cudaStreamSynchronize(c->stream));
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return COMET_OK;
+}
+
 // Makes the main stream wait for the side stream's outstanding work (if any).
 int join_side(comet_ctx* c) {
     if (c->side_pending) {
@@ -448,6 +462,7 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
     a.error_host = c->h_count_dev + 3;
     a.ldz = pr.N; a.bs = c->cfg.block; a.group_units = 0;
     a.groups = nullptr; a.row_map = nullptr; a.col_map = nullptr;
+    a.row_label = nullptr; a.blk_label = nullptr; a.blocks = 1;
     if (c->grouped) {
         a.M = c->live_rows;
         a.mt = ceil_div(a.M, lb::BM);
@@ -459,6 +474,9 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
             a.N = c->groups * c->live_blocks * c->cfg.block;
             a.nt = ceil_div(a.N, lb::BN);
             a.col_map = c->d_col_map;
+            a.row_label = c->d_row_label;
+            a.blk_label = c->d_blk_label;
+            a.blocks = c->n_active_blocks;
             a.groups = c->d_group_up;
             a.group_units = c->group_units_up;
         }
@@ -521,8 +539,9 @@ int launch_combine(comet_ctx* c, int M, int N, int K, int idE, int idF, int idA,
 }
 
 // The Merge step of Protocol 2 under a token mask: entries of the compact result outside the component blocks become zero.
+// The grouped launch does that itself.
 int somm_merge(comet_ctx* c, int tokens) {
-    if (!c->tmask_set) return COMET_OK;
+    if (!c->tmask_set || c->grouped) return COMET_OK;
     const int cols = c->groups * c->n_active;
     const int64_t pairs = (int64_t)tokens * cols / 2;
     if (pairs == 0) return COMET_OK;
@@ -661,7 +680,7 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
     reserve(device, &c->d_row_map, (size_t)c->cap_T * sizeof(int32_t));
     reserve(device, &c->d_col_map, (size_t)c->groups * nb * sizeof(int32_t));
     reserve(device, &c->d_kmap, (size_t)nb * sizeof(int32_t));
-    reserve(device, &c->d_plan_scratch, ((size_t)c->cap_T * ceil_div(nb, 32) + (size_t)c->groups * nb) * sizeof(uint32_t));
+    reserve(device, &c->d_plan_scratch, comet::token_plan_words(c->cap_T, nb, ceil_div(nb, 32), c->groups) * sizeof(uint32_t));
     reserve(device, &c->d_group_up, row_tiles * sizeof(comet::LimbGroupRow));
     reserve(device, &c->d_group_dn, row_tiles * sizeof(comet::LimbGroupRow));
     reserve(device, &c->d_row_label, (size_t)c->cap_T * sizeof(int32_t));
@@ -674,7 +693,7 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
         c->stream_sync_words = 1 + (size_t)((widest + ls::BW - 1) / ls::BW);
         reserve(device, &c->d_stream_sync, c->stream_sync_words * sizeof(uint32_t));
     }
-    reserve(pinned, &c->h_masked, 7 * sizeof(long long));
+    reserve(pinned, &c->h_masked, comet::PLAN_WORDS * sizeof(long long));
     reserve(pinned, &c->h_count, 4 * sizeof(int32_t));
     reserve(pinned, &c->h_mask_stage, (size_t)nb * 4);
     constexpr size_t ALIGN = 256;
@@ -699,6 +718,7 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
             for (int id = 0; id < COMET_NUM_TENSORS; ++id) c->buf[p][id] = c->own[p][id];
         c->d_error = c->d_count + 1;
         c->h_count[0] = c->h_count[1] = c->h_count[2] = c->h_count[3] = 0;     // pinned memory is not zeroed
+        for (int k = 0; k < comet::PLAN_WORDS; ++k) c->h_masked[k] = 0;
     }
     ok = ok && cudaMemset(c->d_count, 0, 2 * sizeof(int32_t)) == cudaSuccess;
     ok = ok && cudaMemset(c->d_stream_sync, 0, c->stream_sync_words * sizeof(uint32_t)) == cudaSuccess;
@@ -843,16 +863,10 @@ int comet_set_mask(comet_ctx* c, const uint8_t* block_mask, int location, int32_
     }
     COMET_CUDA(c, cudaGetLastError());
     if (host_count < 0) {
-        // The kernel is the last thing on the stream and reports through mapped memory: watching its ticket for
-        // a short while is quicker than a stream synchronise; after that, synchronise as usual.
-        volatile int32_t* seen = c->h_count + 2;
-        const auto t0 = std::chrono::steady_clock::now();
-        bool arrived = false;
-        while (!(arrived = (*seen == c->ticket))) {
-            if (std::chrono::steady_clock::now() - t0 > std::chrono::microseconds(300)) break;
-        }
-        if (!arrived) COMET_CUDA(c, cudaStreamSynchronize(c->stream));
-        std::atomic_thread_fence(std::memory_order_acquire);
+        const volatile int32_t* seen = c->h_count + 2;
+        const int32_t ticket = c->ticket;
+        const int rc = wait_for_report(c, [=] { return *seen == ticket; });
+        if (rc != COMET_OK) return rc;
     }
     if (timed_out(c)) return COMET_ERR_TIMEOUT;           // an earlier kernel gave up on a bounded wait
     const int32_t blocks = host_count >= 0 ? host_count : *c->h_count;
@@ -897,7 +911,8 @@ int comet_set_token_mask(comet_ctx* c, const uint8_t* token_mask, int location, 
         return COMET_ERR_SHAPE;
     if ((int64_t)tokens * c->n_active < 0 || (int64_t)tokens * c->n_active > 0x7fffffffll) return COMET_ERR_SHAPE;
     const size_t bytes = (size_t)tokens * (size_t)n_active_blocks;
-    COMET_CUDA(c, cudaMemcpyAsync(c->d_tmask, token_mask, bytes, copy_kind(location, true), c->stream));
+    if (location == COMET_HOST)
+        COMET_CUDA(c, cudaMemcpyAsync(c->d_tmask, token_mask, bytes, cudaMemcpyHostToDevice, c->stream));
     // Protocol 2, first step: the connected components the up-projection is partitioned into, the number of
     // non-zero entries (Theorem 2's count) and, for the tensor-core path, the component-sorted order and the work
     // of every row tile, in one launch
@@ -905,10 +920,13 @@ int comet_set_token_mask(comet_ctx* c, const uint8_t* token_mask, int location, 
     {
         comet::TokenPlanArgs a;
         std::memset(&a, 0, sizeof(a));
-        a.S = c->d_tmask;
+        a.S = location == COMET_HOST ? c->d_tmask : token_mask;
+        a.copy = location == COMET_HOST ? nullptr : c->d_tmask;
         a.T = tokens; a.nab = n_active_blocks; a.wpr = ceil_div(n_active_blocks, 32);
         a.row_label = c->d_row_label; a.blk_label = c->d_blk_label;
         a.report = c->h_masked_dev;
+        c->plan_ticket = c->plan_ticket % ((1ull << (64 - comet::PLAN_VALUE_BITS)) - 1) + 1;      // never 0
+        a.ticket = c->plan_ticket;
         a.scratch = c->d_plan_scratch;
         a.plan = plan ? 1 : 0;
         a.groups = c->groups; a.bs = c->cfg.block;
@@ -916,20 +934,30 @@ int comet_set_token_mask(comet_ctx* c, const uint8_t* token_mask, int location, 
         a.nt_dn = ceil_div(c->cfg.d_model, comet::limb::BN);
         a.row_map = c->d_row_map; a.col_map = c->d_col_map; a.kmap = c->d_kmap;
         a.up = c->d_group_up; a.dn = c->d_group_dn;
-        const size_t words = (size_t)tokens * a.wpr + tokens + (size_t)n_active_blocks * (1 + c->groups);
+        const size_t words = comet::token_plan_words(tokens, n_active_blocks, a.wpr, c->groups);
         a.in_smem = words * sizeof(uint32_t) <= 36 * 1024 ? 1 : 0;
-        comet::token_plan_kernel<<<1, 1024, a.in_smem ? words * sizeof(uint32_t) : 0, c->stream>>>(a);
+        COMET_CUDA(c, launch_chained(comet::token_plan_kernel, dim3(1), dim3(1024), a.in_smem ? words * sizeof(uint32_t) : 0,
+                                     c->stream, nullptr, a));
     }
     c->stats.kernel_launches += 1;
-    COMET_CUDA(c, cudaGetLastError());
-    COMET_CUDA(c, cudaStreamSynchronize(c->stream));
-    c->tmask_masked = (int64_t)c->h_masked[0] * c->cfg.block;
-    c->n_components = (int32_t)c->h_masked[1];
-    c->live_rows = (int32_t)c->h_masked[2];
-    c->live_blocks = (int32_t)c->h_masked[3];
-    c->group_units_up = plan ? (int32_t)c->h_masked[4] : 0;
-    c->component_pairs = plan ? (int64_t)c->h_masked[5] : -1;
-    c->group_units_dn = plan ? (int32_t)c->h_masked[6] : 0;
+    {
+        const volatile unsigned long long* words = c->h_masked;
+        const unsigned long long ticket = c->plan_ticket;
+        const int rc = wait_for_report(c, [=] {
+            for (int k = 0; k < comet::PLAN_WORDS; ++k)
+                if (words[k] >> comet::PLAN_VALUE_BITS != ticket) return false;
+            return true;
+        });
+        if (rc != COMET_OK) return rc;
+    }
+    auto reported = [c](int k) { return (int64_t)(c->h_masked[k] & ((1ull << comet::PLAN_VALUE_BITS) - 1)); };
+    c->tmask_masked = reported(0) * c->cfg.block;
+    c->n_components = (int32_t)reported(1);
+    c->live_rows = (int32_t)reported(2);
+    c->live_blocks = (int32_t)reported(3);
+    c->group_units_up = plan ? (int32_t)reported(4) : 0;
+    c->component_pairs = plan ? reported(5) : -1;
+    c->group_units_dn = plan ? (int32_t)reported(6) : 0;
     // several components, or rows / blocks in none: compute the component rectangles only
     c->grouped = plan && c->group_units_up > 0 && c->group_units_dn > 0 &&
                  (c->n_components > 1 || c->live_rows < tokens || c->live_blocks < n_active_blocks);

@@ -289,7 +289,16 @@ __device__ __forceinline__ void limb_exchange_block(const LimbExchangeArgs& a, c
     const ulonglong2* __restrict__ s = reinterpret_cast<const ulonglong2*>(party ? a.C[1] : a.C[0]);
     ulonglong2* __restrict__ d = reinterpret_cast<ulonglong2*>(party ? a.Z[1] : a.Z[0]);
     const long long stride = (long long)(a.copy_blocks >> 1) * limb::EX_THREADS;
-    for (long long t = (long long)(block >> 1) * limb::EX_THREADS + threadIdx.x; t < a.copy_pairs; t += stride) d[t] = __ldcs(s + t);
+    for (long long t = (long long)(block >> 1) * limb::EX_THREADS + threadIdx.x; t < a.copy_pairs; t += stride) {
+        if (a.col_map) {                         // entries outside the components stay zero (see LimbArgs)
+            const unsigned row = (unsigned)(t / (unsigned)(a.N / 2)), blk = ((unsigned)t - row * (a.N / 2)) * 2 % a.n / a.bs;
+            if (__ldg(a.row_label + row) != __ldg(a.blk_label + blk) || __ldg(a.blk_label + blk) < 0) {
+                d[t] = make_ulonglong2(0ull, 0ull);
+                continue;
+            }
+        }
+        d[t] = __ldcs(s + t);
+    }
 }
 
 // The first `first_blocks` CTAs work on `a`, the others on `b` (another product's operands).
@@ -399,11 +408,10 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 // What a per-token mask S [T, nab] (non-zero byte = token t uses active block b) implies, in one launch of one CTA.
 //
 // 1. The first step of Protocol 2: the connected components of the bipartite graph (token rows) x (active
-//    blocks) with the non-zero bytes as edges.  The paper uses depth-first search; here S becomes a bit matrix
-//    and minimum labels are propagated without atomics: every block takes the minimum over its rows (one warp per
-//    block), then every row the minimum over its blocks (one thread per row), until nothing changes (at most
-//    T + nab + 1 sweeps).  Every node of a component ends up with the component's smallest token index as its
-//    label; nodes without an edge get -1.
+//    blocks) with the non-zero bytes as edges.  The paper uses depth-first search; here S becomes a bit matrix,
+//    every row joins the blocks it uses in a union-find forest over the blocks (hooking by compare-and-swap, the
+//    larger root under the smaller), and one pass afterwards reads the roots.  A node's label is the smallest token
+//    index of its component; nodes without an edge get -1.
 //
 // 2. (plan != 0) Protocols 2 and 3 ask for one multiplication per component / per non-zero column entry, over the
 //    rows and columns that take part only (the multiplication counts of Theorems 1 and 2).  On the tensor cores
@@ -422,10 +430,14 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 //
 // report (mapped host memory): [0] edges, [1] components, [2] rows with an edge, [3] blocks with an edge,
 // [4] k-block units of the up-projection per party, [5] sum over components of rows x blocks, [6] units of the
-// down-projection per party ([4..6] only with plan).
-// Working storage: bit matrix [T, wpr] words, labels, and the labels of the sorted column blocks, in dynamic
-// shared memory when `in_smem` (T*wpr + T + nab + groups*nab words), else in `scratch` (global, same size) with
-// the labels kept in the output arrays.
+// down-projection per party ([4] and [6] only with plan).  Every word carries the launch's ticket above its value, so that the
+// host sees by itself which have arrived and no fence over the bus (2 us) orders them.
+//
+// What bounds it: the host waits for the report, so it is a chain of latencies in one CTA: reading S, the joins, the sort, the
+// report.  Rows are sorted by counting, per 32 rows and component.  Comparing every row with every other and spreading minimum
+// labels until nothing changed took 26 us of 512 tokens x 26 blocks in four groups, this 14 us.
+//
+// Working storage (token_plan_words): in dynamic shared memory when `in_smem`, else in `scratch` (global).
 // ---------------------------------------------------------------------------
 struct LimbGroupRow {
     int unit0;       // units (k-blocks, both operand pairs) of the row tiles before this one, per party
@@ -433,12 +445,16 @@ struct LimbGroupRow {
     int klo, kcnt;   // interval of k-blocks with work; a tile runs over 2 * kcnt units
 };
 
+constexpr int PLAN_WORDS = 7, PLAN_VALUE_BITS = 40;          // of the report
+
 struct TokenPlanArgs {
-    const uint8_t* S;
+    const uint8_t* S;            // [T, nab]
+    uint8_t* copy;               // where S is kept, or null: it is the kept one
     int T, nab, wpr;             // wpr = ceil(nab / 32)
     int32_t* row_label;          // out [T]
     int32_t* blk_label;          // out [nab]
-    long long* report;
+    unsigned long long* report;
+    unsigned long long ticket;
     int in_smem;
     uint32_t* scratch;
     int plan, groups, bs, kb_up, nt_dn;
@@ -449,159 +465,195 @@ struct TokenPlanArgs {
     LimbGroupRow* dn;
 };
 
+// Words of working storage: bit matrix; rows per 32 rows and component; components of the rows; and per block the forest, the
+// smallest row, the rows and their first position, the label, and the sorted labels.
+__host__ __device__ inline size_t token_plan_words(size_t T, size_t nab, size_t wpr, size_t groups) {
+    return T * wpr + (T + 31) / 32 * (nab + 1) + T + nab * 5 + 2 + groups * nab;
+}
+
+// Root of block b; every second pointer on the way is shortened (others may do the same: all of them point to ancestors).
+__device__ __forceinline__ int plan_root(volatile int* parent, int b) {
+    int p = parent[b];
+    while (p != b) {
+        const int q = parent[p];
+        if (q != p) parent[b] = q;
+        b = p;
+        p = q;
+    }
+    return b;
+}
+
 __global__ void __launch_bounds__(1024, 1)
 token_plan_kernel(TokenPlanArgs a) {
-    constexpr int TM = limb::BM, TN = limb::BN, KC = limb::KC;
-    extern __shared__ uint32_t plan_smem[];
-    __shared__ int counts[3];
-    __shared__ unsigned long long edges, pairs;
-    __shared__ int units_up[1024], units_dn[1024];
-    const int tid = threadIdx.x;
-    const int T = a.T, nab = a.nab, wpr = a.wpr;
+    constexpr int TM = limb::BM, TN = limb::BN, KC = limb::KC, MAX_TILES = 32768 / TM, WARPS = 32;
+    extern __shared__ __align__(16) uint32_t plan_smem[];
+    __shared__ int components, live_blocks;
+    __shared__ unsigned edges, pairs;            // at most T * nab, which the host keeps below 2^31 / 16
+    __shared__ int tile_lo[MAX_TILES], tile_hi[MAX_TILES], units_up[MAX_TILES], units_dn[MAX_TILES];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int T = a.T, nab = a.nab, wpr = a.wpr, groups = a.groups, bs = a.bs, chunks = (T + 31) / 32;
     const int INF = 0x7fffffff;
     uint32_t* bits = a.in_smem ? plan_smem : a.scratch;
-    int* rl = a.in_smem ? reinterpret_cast<int*>(plan_smem + (size_t)T * wpr) : a.row_label;
-    int* bl = a.in_smem ? rl + T : a.blk_label;
-    int* sorted_bl = a.in_smem ? bl + nab : reinterpret_cast<int*>(a.scratch + (size_t)T * wpr);
+    int* count = reinterpret_cast<int*>(bits + (size_t)T * wpr);      // [chunks][nab + 1], the last for rows of no component
+    int* comp = count + (size_t)chunks * (nab + 1);                   // [T] root of the row's blocks, nab: none
+    int* parent = comp + T;                                           // [nab] the forest
+    int* least = parent + nab;                                        // [nab] smallest row of the component, at its root
+    int* rows_of = least + nab;                                         // [nab + 1] rows of a component, at its root
+    int* first_row = rows_of + nab + 1;                                 // [nab + 1] where they go in the sorted order
+    int* bl = first_row + nab + 1;                                    // [nab] label of the block
+    int* sorted_bl = bl + nab;                                        // [groups * nab]
 
-    const int warp = tid >> 5, lane = tid & 31;
-    for (int w = tid; w < T * wpr; w += 1024) bits[w] = 0u;
-    for (int b = tid; b < nab; b += 1024) bl[b] = INF;
-    if (tid == 0) { counts[0] = counts[1] = counts[2] = 0; edges = 0ull; pairs = 0ull; }
+    pdl_wait();
+    for (int w = tid; w < T * wpr + chunks * (nab + 1); w += 1024) bits[w] = 0u;
+    for (int b = tid; b < nab; b += 1024) {
+        parent[b] = b;
+        least[b] = INF;
+    }
+    if (tid == 0) { components = live_blocks = 0; edges = pairs = 0u; }
     __syncthreads();
     {
-        // S is read four bytes at a time (its buffer is 256-byte aligned); the last 0-3 bytes singly
-        const int total = T * nab, words = total >> 2;
-        const uint32_t* S4 = reinterpret_cast<const uint32_t*>(a.S);
-        for (int q = tid; q < words; q += 1024) {
-            uint32_t v = __ldg(S4 + q);
-            if (v == 0u) continue;
+        // S is read (and kept) 16 bytes at a time where it lies on such a boundary, the rest singly
+        const int total = T * nab, quads = (reinterpret_cast<uintptr_t>(a.S) & 15) == 0 ? total >> 4 : 0;
+        const uint4* S16 = reinterpret_cast<const uint4*>(a.S);
+        for (int q = tid; q < quads; q += 1024) {
+            const uint4 v = __ldg(S16 + q);
+            if (a.copy) reinterpret_cast<uint4*>(a.copy)[q] = v;
+            int r = 16 * q / nab, b = 16 * q - r * nab;
+            uint32_t found = 0u;                 // of word b / 32 of row r
 #pragma unroll
-            for (int k = 0; k < 4; ++k, v >>= 8)
-                if (v & 0xffu) {
-                    const int t = 4 * q + k, r = t / nab, b = t - r * nab;
-                    atomicOr(&bits[r * wpr + (b >> 5)], 1u << (b & 31));
+            for (int k = 0; k < 16; ++k) {
+                const uint32_t word = k < 4 ? v.x : k < 8 ? v.y : k < 12 ? v.z : v.w;
+                if (word >> (8 * (k & 3)) & 0xffu) found |= 1u << (b & 31);
+                ++b;
+                if (k == 15 || b == nab || (b & 31) == 0) {
+                    if (found) atomicOr(&bits[r * wpr + ((b - 1) >> 5)], found);
+                    found = 0u;
+                    if (b == nab) { b = 0; ++r; }
                 }
+            }
         }
-        for (int t = 4 * words + tid; t < total; t += 1024)
-            if (a.S[t] != 0) {
+        for (int t = 16 * quads + tid; t < total; t += 1024) {
+            const uint8_t v = a.S[t];
+            if (a.copy) a.copy[t] = v;
+            if (v != 0) {
                 const int r = t / nab, b = t - r * nab;
                 atomicOr(&bits[r * wpr + (b >> 5)], 1u << (b & 31));
             }
-    }
-    __syncthreads();
-    {
-        int mine = 0;
-        for (int r = tid; r < T; r += 1024) {
-            int deg = 0;
-            for (int w = 0; w < wpr; ++w) deg += __popc(bits[r * wpr + w]);
-            rl[r] = deg ? r : INF;               // a row with an edge starts from its own index
-            mine += deg;
-        }
-        mine = __reduce_add_sync(0xffffffffu, mine);
-        if (lane == 0 && mine) atomicAdd(&edges, (unsigned long long)mine);
-    }
-    __syncthreads();
-    for (int sweep = 0; sweep <= T + nab; ++sweep) {
-        int changed = 0;
-        // blocks take the minimum over their rows: one warp per block, no atomics
-        for (int b = warp; b < nab; b += 32) {
-            const int w = b >> 5;
-            const uint32_t bit = 1u << (b & 31);
-            int m = INF;
-            for (int r = lane; r < T; r += 32)
-                if (bits[r * wpr + w] & bit) m = min(m, rl[r]);
-            m = __reduce_min_sync(0xffffffffu, m);
-            if (lane == 0 && m < bl[b]) { bl[b] = m; changed = 1; }
-        }
-        __syncthreads();
-        // rows take the minimum over their blocks
-        for (int r = tid; r < T; r += 1024) {
-            const int mine = rl[r];
-            if (mine == INF) continue;
-            int m = mine;
-            for (int w = 0; w < wpr; ++w)
-                for (uint32_t v = bits[r * wpr + w]; v; v &= v - 1) m = min(m, bl[w * 32 + __ffs(v) - 1]);
-            if (m < mine) { rl[r] = m; changed = 1; }
-        }
-        if (!__syncthreads_or(changed)) break;
-    }
-    {
-        int comps = 0, live_r = 0, live_b = 0;
-        for (int r = tid; r < T; r += 1024) {
-            const int l = rl[r];
-            if (l == INF) rl[r] = -1;
-            else {
-                ++live_r;
-                comps += l == r;
-            }
-            a.row_label[r] = l == INF ? -1 : l;
-        }
-        for (int b = tid; b < nab; b += 1024) {
-            const int l = bl[b];
-            if (l == INF) bl[b] = -1;
-            else ++live_b;
-            a.blk_label[b] = l == INF ? -1 : l;
-        }
-        comps = __reduce_add_sync(0xffffffffu, comps);
-        live_r = __reduce_add_sync(0xffffffffu, live_r);
-        live_b = __reduce_add_sync(0xffffffffu, live_b);
-        if (lane == 0) {
-            if (comps) atomicAdd(&counts[0], comps);
-            if (live_r) atomicAdd(&counts[1], live_r);
-            if (live_b) atomicAdd(&counts[2], live_b);
         }
     }
     __syncthreads();
-    if (tid == 0) {
-        a.report[0] = (long long)edges;
-        a.report[1] = counts[0];
-        a.report[2] = counts[1];
-        a.report[3] = counts[2];
-        if (!a.plan) __threadfence_system();
+    // Every row joins its blocks.  First the first 64 rows, a thread per edge, which settles most of the forest; then, with every
+    // block pointing at its root, the others, a thread per row, which mostly find their blocks joined.
+    auto join = [&](int x, int y) {              // returns their root
+        x = plan_root(parent, x);
+        y = plan_root(parent, y);
+        while (x != y) {
+            const int hi = max(x, y), lo = min(x, y);
+            if (atomicCAS(parent + hi, hi, lo) == hi) return lo;
+            x = plan_root(parent, x);
+            y = plan_root(parent, y);
+        }
+        return x;
+    };
+    for (int e = tid; e < min(T, 64) * nab; e += 1024) {
+        const int r = e / nab, b = e - r * nab;
+        const uint32_t* row = bits + r * wpr;
+        if ((row[b >> 5] >> (b & 31) & 1u) == 0u) continue;
+        int w = 0;
+        while (row[w] == 0u) ++w;
+        const int first = w * 32 + __ffs(row[w]) - 1;
+        if (first != b) join(first, b);
     }
-    if (!a.plan) return;
-
-    // ---- component-sorted order
-    const int M = counts[1], NB = counts[2], groups = a.groups, bs = a.bs;
-    // rank of a row = number of rows with a smaller key label * T + row; rows of no component take T for the
-    // label and so come last, in index order.  T <= 32768 keeps the key within 32 bits.
-    unsigned long long my_pairs = 0;
+    __syncthreads();
+    for (int b = tid; b < nab; b += 1024) parent[b] = plan_root(parent, b);
+    __syncthreads();
+    unsigned mine = 0;
     for (int r = tid; r < T; r += 1024) {
-        const int l = rl[r];
-        const unsigned key = (l >= 0 ? (unsigned)l : (unsigned)T) * (unsigned)T + (unsigned)r;
-        int rank0 = 0, rank1 = 0;
-        int q = 0;
-        for (; q + 1 < T; q += 2) {
-            const int l0 = rl[q], l1 = rl[q + 1];
-            rank0 += (l0 >= 0 ? (unsigned)l0 : (unsigned)T) * (unsigned)T + (unsigned)q < key;
-            rank1 += (l1 >= 0 ? (unsigned)l1 : (unsigned)T) * (unsigned)T + (unsigned)(q + 1) < key;
-        }
-        if (q < T) rank0 += (rl[q] >= 0 ? (unsigned)rl[q] : (unsigned)T) * (unsigned)T + (unsigned)q < key;
-        a.row_map[rank0 + rank1] = r;
-        if (l >= 0)
-            for (int b = 0; b < nab; ++b) my_pairs += bl[b] == l;
-    }
-    my_pairs = __reduce_add_sync(0xffffffffu, (unsigned)my_pairs);
-    if (lane == 0 && my_pairs) atomicAdd(&pairs, my_pairs);
-    for (int b = tid; b < nab; b += 1024) {
-        const int l = bl[b];
-        if (l >= 0) {
-            int less = 0, same = 0, before = 0;
-            for (int q = 0; q < nab; ++q) {
-                const int lq = bl[q];
-                less += lq >= 0 && lq < l;
-                same += lq == l;
-                before += lq == l && q < b;
+        int root = nab;
+        for (int w = 0; w < wpr; ++w) {
+            uint32_t v = bits[r * wpr + w];
+            mine += __popc(v);
+            for (; v; v &= v - 1) {
+                const int y = *(volatile int*)(parent + w * 32 + __ffs(v) - 1);
+                if (root == nab) root = y;
+                if (root != y) root = join(root, y);
             }
+        }
+        comp[r] = root;                          // of the moment
+    }
+    __syncthreads();
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0 && mine) atomicAdd(&edges, mine);
+    for (int chunk = warp; chunk < chunks; chunk += WARPS) {
+        const int r = chunk * 32 + lane;
+        int root = r < T ? comp[r] : -1;
+        if (root >= 0 && root < nab) root = plan_root(parent, root);
+        const unsigned same = __match_any_sync(0xffffffffu, root);
+        if (r < T) {
+            comp[r] = root;
+            if (lane == __ffs(same) - 1) {
+                count[chunk * (nab + 1) + root] = __popc(same);
+                if (root < nab) atomicMin(least + root, r);
+            }
+        }
+    }
+    __syncthreads();
+    // rows per component, and of those the rows before each chunk
+    for (int b = tid; b <= nab; b += 1024) {
+        int sum = 0;
+        for (int k = 0; k < chunks; ++k) {
+            const int n = count[k * (nab + 1) + b];
+            count[k * (nab + 1) + b] = sum;
+            sum += n;
+        }
+        rows_of[b] = sum;
+    }
+    __syncthreads();
+    {
+        int comps = 0, live_b = 0;
+        unsigned my_pairs = 0;
+        for (int b = tid; b < nab; b += 1024) {
+            const int root = plan_root(parent, b), l = least[root] == INF ? -1 : least[root];
+            bl[b] = l;
+            a.blk_label[b] = l;
+            live_b += l >= 0;
+            comps += rows_of[b] > 0;
+            my_pairs += l >= 0 ? rows_of[root] : 0;
+        }
+        if (tid - lane < nab) {
+            comps = __reduce_add_sync(0xffffffffu, comps);
+            live_b = __reduce_add_sync(0xffffffffu, live_b);
+            my_pairs = __reduce_add_sync(0xffffffffu, my_pairs);
+            if (lane == 0) {
+                atomicAdd(&components, comps);
+                atomicAdd(&live_blocks, live_b);
+                atomicAdd(&pairs, my_pairs);
+            }
+        }
+        for (int r = tid; r < T; r += 1024) a.row_label[r] = comp[r] < nab ? least[comp[r]] : -1;
+    }
+    const int M = T - rows_of[nab];                // rows with an edge; the others come after them
+    __syncthreads();
+    const int NB = live_blocks;
+    // ---- component-sorted order
+    for (int b = tid; a.plan && b < nab; b += 1024) {
+        const int l = bl[b];
+        int less = 0, same = 0, before = 0, rows = 0;
+        for (int q = 0; q < nab; ++q) {
+            const int lq = bl[q];
+            less += lq >= 0 && lq < l;
+            same += lq == l;
+            before += lq == l && q < b;
+            rows += lq < l ? rows_of[q] : 0;       // zero but at a root
+        }
+        first_row[b] = rows;
+        if (l >= 0) {
             for (int g = 0; g < groups; ++g) {
                 a.col_map[groups * less + g * same + before] = g * nab + b;
                 sorted_bl[groups * less + g * same + before] = l;
             }
             a.kmap[less + before] = b;
         } else {
-            int before = 0;
-            for (int q = 0; q < b; ++q) before += bl[q] < 0;
             for (int g = 0; g < groups; ++g) {
                 a.col_map[groups * NB + g * (nab - NB) + before] = g * nab + b;
                 sorted_bl[groups * NB + g * (nab - NB) + before] = -1;
@@ -609,40 +661,54 @@ token_plan_kernel(TokenPlanArgs a) {
             a.kmap[NB + before] = b;
         }
     }
+    if (tid == 0) first_row[nab] = M;
+    __syncthreads();
+    for (int chunk = warp; a.plan && chunk < chunks; chunk += WARPS) {
+        const int r = chunk * 32 + lane, c = r < T ? comp[r] : -1;
+        const unsigned same = __match_any_sync(0xffffffffu, c);
+        if (c < 0) continue;
+        const int pos = first_row[c] + count[chunk * (nab + 1) + c] + __popc(same & ((1u << lane) - 1u));
+        a.row_map[pos] = r;
+        if (c < nab) {
+            if (pos % TM == 0) tile_lo[pos / TM] = least[c];
+            if (pos % TM == TM - 1 || pos == M - 1) tile_hi[pos / TM] = least[c];
+        }
+    }
     __syncthreads();
 
-    // ---- the work of every row tile
-    const int N = groups * NB * bs;
-    const int mt = (M + TM - 1) / TM, nt = (N + TN - 1) / TN;
-    if (tid < mt) {
-        const int lo_m = rl[a.row_map[tid * TM]];
-        const int hi_m = rl[a.row_map[min(tid * TM + TM, M) - 1]];
-        int first = 0, count = 0;
-        for (int tn = 0; tn < nt; ++tn) {
-            const int lo_n = sorted_bl[(tn * TN) / bs];
-            const int hi_n = sorted_bl[(min(tn * TN + TN, N) - 1) / bs];
-            if (hi_n >= lo_m && lo_n <= hi_m) {
-                if (count == 0) first = tn;
-                ++count;
-            }
+    // ---- the work of every row tile, a warp per tile
+    const int N = groups * NB * bs, mt = a.plan ? (M + TM - 1) / TM : 0, nt = (N + TN - 1) / TN;
+    for (int tm = warp; tm < mt; tm += WARPS) {
+        const int lo_m = tile_lo[tm], hi_m = tile_hi[tm];
+        int first = -1, count = 0;
+        for (int t0 = 0; t0 < nt; t0 += 32) {
+            const int tn = t0 + lane;
+            const bool hit = tn < nt && sorted_bl[(min(tn * TN + TN, N) - 1) / bs] >= lo_m && sorted_bl[(tn * TN) / bs] <= hi_m;
+            const unsigned hits = __ballot_sync(0xffffffffu, hit);
+            if (first < 0 && hits) first = t0 + __ffs(hits) - 1;
+            count += __popc(hits);
         }
-        a.up[tid].tn0 = first;
-        a.up[tid].ntn = count;
-        a.up[tid].klo = 0;
-        a.up[tid].kcnt = a.kb_up;
-        units_up[tid] = count * 2 * a.kb_up;
         int blk_begin = 0, blk_end = 0;          // sorted block positions of the components lo_m .. hi_m
-        for (int q = 0; q < nab; ++q) {
+        for (int q = lane; q < nab; q += 32) {
             const int lq = bl[q];
             blk_begin += lq >= 0 && lq < lo_m;
             blk_end += lq >= 0 && lq <= hi_m;
         }
+        blk_begin = __reduce_add_sync(0xffffffffu, blk_begin);
+        blk_end = __reduce_add_sync(0xffffffffu, blk_end);
         const int klo = (blk_begin * bs) / KC, khi = (blk_end * bs + KC - 1) / KC;
-        a.dn[tid].tn0 = 0;
-        a.dn[tid].ntn = a.nt_dn;
-        a.dn[tid].klo = klo;
-        a.dn[tid].kcnt = khi - klo;
-        units_dn[tid] = a.nt_dn * 2 * (khi - klo);
+        if (lane == 0) {
+            a.up[tm].tn0 = max(first, 0);
+            a.up[tm].ntn = count;
+            a.up[tm].klo = 0;
+            a.up[tm].kcnt = a.kb_up;
+            units_up[tm] = count * 2 * a.kb_up;
+            a.dn[tm].tn0 = 0;
+            a.dn[tm].ntn = a.nt_dn;
+            a.dn[tm].klo = klo;
+            a.dn[tm].kcnt = khi - klo;
+            units_dn[tm] = a.nt_dn * 2 * (khi - klo);
+        }
     }
     __syncthreads();
     if (tid == 0) {
@@ -653,10 +719,11 @@ token_plan_kernel(TokenPlanArgs a) {
             off_up += units_up[tm];
             off_dn += units_dn[tm];
         }
-        a.report[4] = off_up;
-        a.report[5] = (long long)pairs;
-        a.report[6] = off_dn;
-        __threadfence_system();
+        const unsigned long long words[PLAN_WORDS] = {edges, (unsigned)components, (unsigned)M, (unsigned)NB, (unsigned)off_up,
+                                                      pairs, (unsigned)off_dn};
+#pragma unroll
+        for (int k = 0; k < PLAN_WORDS; ++k)
+            reinterpret_cast<volatile unsigned long long*>(a.report)[k] = a.ticket << PLAN_VALUE_BITS | words[k];
     }
 }
 
@@ -681,6 +748,12 @@ struct LimbArgs {
     const LimbGroupRow* groups;  // [mt]
     const int32_t* row_map;      // [M] sorted row -> row of Z
     const int32_t* col_map;      // [N / bs] sorted block -> compact block of Z, or null
+    // Component labels of Z's rows and of the active blocks, with col_map: the Merge step of Protocol 2.  A tile may touch
+    // several components; what it holds outside them (a piece of a row whose block has another label) is left out, and Z holds
+    // zero there (limb_exchange_kernel).  As a pass over Z after the product it took 5 us and a launch of 512 tokens x 832.
+    const int32_t* row_label;
+    const int32_t* blk_label;
+    int blocks;                  // active blocks
 };
 
 // Slow path of a bounded wait, kept out of line so that the polling loops of the three roles stay short.
@@ -963,7 +1036,12 @@ __device__ __forceinline__ void combine_limb_body(const LimbArgs& a, const CUten
             const int row = sg.tm * BM + quarter * 32 + lane;
             const int col0 = sg.tn * BN + chalf * 32;
             u64* zrow = nullptr;
-            if (GROUPED) zrow = (sg.party ? a.Z[1] : a.Z[0]) + (size_t)(row < a.M ? __ldg(a.row_map + row) : 0) * a.ldz;
+            int label = 0;
+            if (GROUPED) {
+                const int at = row < a.M ? __ldg(a.row_map + row) : 0;
+                zrow = (sg.party ? a.Z[1] : a.Z[0]) + (size_t)at * a.ldz;
+                if (a.col_map) label = __ldg(a.row_label + at);
+            }
 #pragma unroll
             for (int h = 0; h < 32 / OUT_COLS; ++h) {          // this thread's 32 columns, OUT_COLS at a time
                 u64 v[OUT_COLS];
@@ -993,8 +1071,14 @@ __device__ __forceinline__ void combine_limb_body(const LimbArgs& a, const CUten
                     if (row < a.M && cols > 0) {
                         ptx::fence_proxy_async_smem();     // this thread's row, written above, is read by the copy engine
                         const int c = col0 + h * OUT_COLS, blk = c / a.bs;
-                        u64* dst = a.col_map ? zrow + (size_t)__ldg(a.col_map + blk) * a.bs + (c - blk * a.bs) : zrow + c;
-                        ptx::bulk_reduce_add_u64(dst, my_row_s, (uint32_t)cols * 8u);
+                        u64* dst = zrow + c;
+                        bool inside = true;
+                        if (a.col_map) {
+                            const int at = __ldg(a.col_map + blk);
+                            dst = zrow + (size_t)at * a.bs + (c - blk * a.bs);
+                            inside = __ldg(a.blk_label + at % a.blocks) == label;
+                        }
+                        if (inside) ptx::bulk_reduce_add_u64(dst, my_row_s, (uint32_t)cols * 8u);
                     }
                     ptx::bulk_commit_group();
                 } else {

@@ -241,9 +241,17 @@ Proj proj_down(const comet_ctx* c, int tokens) {
                 COMET_C_DN, COMET_Y, true};
 }
 
-// The streaming kernel (one kernel per product, operand roles exchanged) serves products with at most 32 token rows:
-// its planes live in shared memory, so every further 32 rows would convert the weights once more.
-inline bool few_tokens(const Proj& pr) { return pr.M <= comet::limb_stream::BT; }
+// The streaming kernel (one kernel per product, operand roles exchanged) serves layers with at most 32 token rows: its planes
+// live in shared memory, so every further 32 rows convert the weights once more.  Up to 64 rows that still beats writing the
+// planes to memory and reading them back where the weights are many (without a token mask, whose components only the other
+// kernel separates).  Both products of a step, 48 rows, streaming / planes: 1024 x 320 37.9 / 37.0 us, 1024 x 768 52.1 / 53.6,
+// 2048 x 512 56.6 / 64.6, 2048 x 832 77.7 / 86.6, 4096 x 1312 189 / 238; 96 rows of 4096 x 1312 took 329 / 263.
+constexpr int STREAM_TOKENS = 2 * comet::limb_stream::BT;
+constexpr int64_t STREAM_WORDS = 3 << 19;          // of the layer's active weights, from which on 33..64 rows are streamed
+bool few_tokens(const comet_ctx* c, int tokens) {
+    if (tokens <= comet::limb_stream::BT) return true;
+    return tokens <= STREAM_TOKENS && !c->tmask_set && (int64_t)(c->groups + 1) * c->cfg.d_model * c->n_active >= STREAM_WORDS;
+}
 
 // Tensor map of a result matrix for the tensor-core kernel's reductions (see LimbMaps).
 bool result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_rows, int box_cols, CUtensorMapSwizzle swizzle) {
@@ -690,7 +698,7 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
     {
         namespace ls = comet::limb_stream;
         const int64_t widest = c->groups * c->cap_n > cfg->d_model ? c->groups * c->cap_n : cfg->d_model;
-        c->stream_sync_words = 1 + (size_t)((widest + ls::BW - 1) / ls::BW);
+        c->stream_sync_words = 1 + (STREAM_TOKENS / ls::BT) * (size_t)((widest + ls::BW - 1) / ls::BW);
         reserve(device, &c->d_stream_sync, c->stream_sync_words * sizeof(uint32_t));
     }
     reserve(pinned, &c->h_masked, comet::PLAN_WORDS * sizeof(long long));
@@ -1000,7 +1008,7 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
         const Proj up = proj_up(c, tokens), dn = proj_down(c, tokens);
         int rc = join_side(c);
         if (rc != COMET_OK) return rc;
-        if (few_tokens(up)) {
+        if (few_tokens(c, tokens)) {
             rc = stream_product(c, up);
             return rc != COMET_OK ? rc : somm_merge(c, tokens);
         }
@@ -1100,7 +1108,7 @@ int comet_ffn_down(comet_ctx* c, int32_t tokens) {
     }
     if (c->path == COMET_PATH_LIMB) {
         const Proj dn = proj_down(c, tokens);
-        if (few_tokens(dn)) {
+        if (few_tokens(c, tokens)) {
             const int rc = join_side(c);
             if (rc != COMET_OK) return rc;
             c->dn_right_ready = false;

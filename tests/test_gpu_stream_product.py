@@ -47,6 +47,8 @@ def test_static_product_at_tile_edges(cb, T, K, N):
     (32, 144, 24, 16, 9, 1),       # 144 features both ways: 128 and a ragged tile of 16
     (31, 112, 12, 48, 5, 2),       # strips of 48 columns: a step takes its halves from two blocks
     (8, 272, 8, 80, 3, 3),         # three stacked matrices, group boundaries inside a feature tile
+    (33, 1008, 64, 16, 49, 1), (64, 1040, 60, 16, 40, 2),      # two token tiles, weights just many enough to be streamed ..
+    (49, 1008, 64, 16, 48, 1),                                 # .. and just too few
 ])
 def test_few_token_layer_at_tile_edges(cb, tokens, d_model, blocks, block, active, stacked):
     from tests import harness as hz

@@ -11,6 +11,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "pdl.cuh"
+
 namespace comet {
 
 typedef unsigned long long u64;
@@ -40,6 +42,8 @@ __device__ __forceinline__ ulonglong2 mul_combine(ulonglong2 c, ulonglong2 d0, u
 template <typename PIECE>
 __global__ void __launch_bounds__(256)
 beaver_mul_kernel(const __grid_constant__ MulArgs g) {
+    pdl_wait();
+    pdl_launch_dependents();
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < g.pieces; t += stride) {
         PIECE x[2], y[2], a[2], b[2], c[2];
@@ -89,6 +93,8 @@ __device__ __forceinline__ ulonglong2 trunc_pair_out(ulonglong2 rp, ulonglong2 m
 template <typename PIECE>
 __global__ void __launch_bounds__(256)
 trunc_pair_kernel(const __grid_constant__ TruncPairArgs g) {
+    pdl_wait();
+    pdl_launch_dependents();
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < g.pieces; t += stride) {
         PIECE m[2], rp[2];
@@ -122,6 +128,8 @@ __device__ __forceinline__ u64 mul_add(u64 p, u64 q) { return p + q; }
 template <typename PIECE>
 __global__ void __launch_bounds__(256)
 add_bias_kernel(const __grid_constant__ BiasArgs g) {
+    pdl_wait();
+    pdl_launch_dependents();
     const long long stride = (long long)gridDim.x * blockDim.x;
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     int piece = (int)(t % g.pieces);
@@ -129,7 +137,7 @@ add_bias_kernel(const __grid_constant__ BiasArgs g) {
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
             PIECE* z = reinterpret_cast<PIECE*>(g.z[p]) + t;
-            *z = mul_add(*z, __ldg(reinterpret_cast<const PIECE*>(g.bias[p]) + piece));
+            *z = mul_add(*z, __ldca(reinterpret_cast<const PIECE*>(g.bias[p]) + piece));
         }
         piece += g.stride_pieces;
         if (piece >= g.pieces) piece -= g.pieces;

@@ -9,6 +9,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "pdl.cuh"
+
 namespace comet {
 
 typedef unsigned long long u64;
@@ -47,6 +49,8 @@ __device__ __forceinline__ u64 shuffle_zero<u64>() { return 0ull; }
 template <typename PIECE>
 __global__ void __launch_bounds__(256)
 shuffle_rows_kernel(ShuffleArgs a) {
+    pdl_wait();
+    pdl_launch_dependents();
     const int party = blockIdx.y;
     const PIECE* __restrict__ in = reinterpret_cast<const PIECE*>(party ? a.in[1] : a.in[0]);
     const PIECE* __restrict__ mask = reinterpret_cast<const PIECE*>(party ? a.mask[1] : a.mask[0]);
@@ -60,12 +64,12 @@ shuffle_rows_kernel(ShuffleArgs a) {
         const long long at = row * a.pieces + piece;
         PIECE g;
         if (src >= 0 && src < a.rows) {
-            g = __ldg(in + src * a.pieces + piece);
+            g = __ldca(in + src * a.pieces + piece);
         } else {
             g = shuffle_zero<PIECE>();              // never read out of bounds; the caller sees the flag
             if (a.bad_index) *a.bad_index = 1;
         }
-        out[at] = shuffle_combine<PIECE>(g, __ldg(mask + at), a.subtract);
+        out[at] = shuffle_combine<PIECE>(g, __ldca(mask + at), a.subtract);
         row += a.stride_rows;
         piece += a.stride_pieces;
         if (piece >= a.pieces) { piece -= a.pieces; ++row; }
@@ -94,6 +98,8 @@ struct ShuffleBothArgs {
 template <typename PIECE>
 __global__ void __launch_bounds__(256)
 shuffle_both_kernel(const __grid_constant__ ShuffleBothArgs g) {
+    pdl_wait();
+    pdl_launch_dependents();
     const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long row = first / g.pieces;
     int piece = (int)(first - row * g.pieces);
@@ -122,11 +128,11 @@ shuffle_both_kernel(const __grid_constant__ ShuffleBothArgs g) {
         PIECE xv[2], av[2], bv[2], xo[2], ao[2];
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
-            xv[p] = __ldg(reinterpret_cast<const PIECE*>(g.x[p]) + src[p] * g.pieces + piece);
-            av[p] = __ldg(reinterpret_cast<const PIECE*>(g.a[p]) + at);
+            xv[p] = __ldca(reinterpret_cast<const PIECE*>(g.x[p]) + src[p] * g.pieces + piece);
+            av[p] = __ldca(reinterpret_cast<const PIECE*>(g.a[p]) + at);
             bv[p] = __ldcs(reinterpret_cast<const PIECE*>(g.b[p]) + at);
-            xo[p] = __ldg(reinterpret_cast<const PIECE*>(g.x[p ^ 1]) + far[p] * g.pieces + piece);
-            ao[p] = __ldg(reinterpret_cast<const PIECE*>(g.a[p ^ 1]) + r[p] * g.pieces + piece);
+            xo[p] = __ldca(reinterpret_cast<const PIECE*>(g.x[p ^ 1]) + far[p] * g.pieces + piece);
+            ao[p] = __ldca(reinterpret_cast<const PIECE*>(g.a[p ^ 1]) + r[p] * g.pieces + piece);
         }
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
@@ -144,8 +150,10 @@ shuffle_both_kernel(const __grid_constant__ ShuffleBothArgs g) {
 
 // inverse[perm[j]] = j: what a party does locally to obtain the sub-permutations of the unshuffle.
 __global__ void __launch_bounds__(256)
-invert_permutation_kernel(const int32_t* __restrict__ perm, int32_t* __restrict__ inverse, long long rows,
+invert_permutation_kernel(const int32_t* perm, int32_t* inverse, long long rows,
                           int* bad_index) {
+    pdl_wait();
+    pdl_launch_dependents();
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < rows; j += stride) {
         const long long p = perm[j];

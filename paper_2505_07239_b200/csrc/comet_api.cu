@@ -303,7 +303,7 @@ int launch_stream(comet::StreamArgs& args, const comet::BlockIds& held, int sm_c
         if (*err != cudaSuccess) return COMET_ERR_CUDA;
     }
     *grid_out = grid;
-    *err = launch_chained(comet::combine_stream_kernel, dim3(grid), dim3(ls::THREADS), ls::SMEM_BYTES, stream,
+    *err = launch_chained(args.M <= 16 ? comet::combine_stream_kernel<16> : comet::combine_stream_kernel<32>, dim3(grid), dim3(ls::THREADS), ls::SMEM_BYTES, stream,
                           priority, args, maps, held);
     return *err == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
 }
@@ -662,8 +662,9 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
                                         (int)lb::SMEM_BYTES) == cudaSuccess;
         // the memory-side kernels may share an SM with a resident tensor-core CTA (which forces the largest
         // shared-memory carve-out), so they ask for the same carve-out
-        ok = ok && cudaFuncSetAttribute(comet::combine_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)comet::limb_stream::SMEM_BYTES) == cudaSuccess;
+        for (auto* kernel : {comet::combine_stream_kernel<16>, comet::combine_stream_kernel<32>})
+            ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)comet::limb_stream::SMEM_BYTES) == cudaSuccess;
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                         (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_grouped_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1320,9 +1321,10 @@ cudaError_t static_device(StaticDevice* out) {
     if (!d.scratch) {
         void* p = nullptr;
         err = cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, dev);
-        if (err == cudaSuccess)
-            err = cudaFuncSetAttribute(comet::combine_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)comet::limb_stream::SMEM_BYTES);
+        for (auto* kernel : {comet::combine_stream_kernel<16>, comet::combine_stream_kernel<32>})
+            if (err == cudaSuccess)
+                err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)comet::limb_stream::SMEM_BYTES);
         if (err == cudaSuccess) err = cudaGetSymbolAddress(&p, g_static_scratch);
         if (err != cudaSuccess) return err;
         d.scratch = static_cast<u64*>(p);

@@ -54,9 +54,9 @@ constexpr int INIT_WARP = MMA_WARP + 1, THREADS = 32 * (INIT_WARP + 1);
 constexpr int RAW_ARRAY_BYTES = QROWS * KC * 8;          // 8 KiB: one array of a slot
 constexpr int RAW_SLOT_BYTES = 4 * RAW_ARRAY_BYTES;      // party 0: W | B, party 1: W | B
 constexpr int RAW_SLOTS = 3;
-constexpr int W_PLANE_BYTES = BW * KC, T_PLANE_BYTES = BT * KC;
+constexpr int W_PLANE_BYTES = BW * KC;
 constexpr int W_SET_BYTES = PLANES * W_PLANE_BYTES;      // 32 KiB: limb planes of B_0, B_1 or F
-constexpr int T_SET_BYTES = PLANES * T_PLANE_BYTES;      //  8 KiB: limb planes of V_0, V_1 or E
+constexpr int T_SET_BYTES = PLANES * BT * KC;            //  8 KiB: limb planes of V_0, V_1 or E
 constexpr int OUT_TOKENS = 4;                            // tokens an epilogue thread recombines at a time
 constexpr int OUT_BYTES = OUT_TOKENS * 32 * 8;           // an epilogue warp's staging buffer: a row of 32 features per token
 constexpr int ACC_COLS = PLANES * BT;                    // 256 TMEM columns per party
@@ -187,6 +187,10 @@ __device__ __forceinline__ bool stream_tile_ready(const uint32_t* flag, uint32_t
     return __all_sync(0xffffffffu, ok);
 }
 
+// COLS = 16 for up to 16 tokens, else 32: the width of the token planes and of the accumulators.  With half the columns the MMAs
+// take half the time, which the conversion of a step otherwise waits for: llama7b decode (7 tokens) 202 -> 189 us.  (As a
+// value of the launch instead of a template's it cost the 32-token layer 2 %.)
+template <int COLS>
 __global__ void __launch_bounds__(limb_stream::THREADS, 1)
 combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constant__ LimbMaps maps,
                       const __grid_constant__ BlockIds held) {
@@ -448,9 +452,9 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 if (live) {                                      // planes of rows past the last token are never looked at
-                    limb_emit4(to, T_PLANE_BYTES, v[0]);
-                    limb_emit4(to + T_SET_BYTES, T_PLANE_BYTES, v[1]);
-                    limb_emit4(to + 2 * T_SET_BYTES, T_PLANE_BYTES, e[0]);
+                    limb_emit4(to, COLS * KC, v[0]);
+                    limb_emit4(to + T_SET_BYTES, COLS * KC, v[1]);
+                    limb_emit4(to + 2 * T_SET_BYTES, COLS * KC, e[0]);
                 }
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
@@ -468,7 +472,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             ok = ok && limb_wait_warp(ptx::smem_u32(&acc_full[party]), seg_phase, &abort_flag);
             if (!ok) break;
             ptx::fence_after_sync();
-            const int col0 = sg.tn * BW + quarter * 32, cols = min(a.N - col0, 32), tokens = min(a.M - sg.tm * BT, BT);
+            const int col0 = sg.tn * BW + quarter * 32, tokens = min(a.M - sg.tm * BT, BT);
             const uint32_t acc = tmem_base + party * ACC_COLS + ((uint32_t)(quarter * 32) << 16);
             const bool at_end = u >= u_end;
             u64* stage = at_end ? reinterpret_cast<u64*>(sRaw + (size_t)(warp - TOK_WARP0) * (BT / OUT_TOKENS) * OUT_BYTES) : out;
@@ -476,7 +480,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             for (int t0 = 0; t0 < tokens; t0 += OUT_TOKENS) {
                 uint32_t d[PLANES][OUT_TOKENS];
 #pragma unroll
-                for (int s = 0; s < PLANES; ++s) ptx::tmem_ld4(acc + BT * s + t0, d[s]);
+                for (int s = 0; s < PLANES; ++s) ptx::tmem_ld4(acc + COLS * s + t0, d[s]);
                 ptx::tmem_wait_ld();
                 if (lane == 0 && !at_end) ptx::bulk_wait_group_read0();  // the last reduction has read its rows
                 __syncwarp();
@@ -485,7 +489,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                     stage[j * 32 + lane] = limb_recombine(d[0][j], d[1][j], d[2][j], d[3][j], d[4][j], d[5][j], d[6][j], d[7][j]);
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
-                if (lane == 0 && cols > 0) {
+                if (lane == 0 && col0 < a.N) {
                     ptx::tensor_reduce_add(&maps.z[party], ptx::smem_u32(stage), col0, sg.tm * BT + t0);
                     ptx::bulk_commit_group();
                 }
@@ -507,8 +511,8 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                 const uint32_t w = w_lo + ((w_set * W_SET_BYTES) >> 4), t = t_lo + ((t_set * T_SET_BYTES) >> 4);
 #pragma unroll
                 for (int q = 0; q < PLANES; ++q)
-                    ptx::mma_i8(d + BT * q, w + ((q * W_PLANE_BYTES) >> 4), LIMB_DESC_HI, t, LIMB_DESC_HI,
-                                IDESC | ((uint32_t)((BT * (PLANES - q)) >> 3) << 17), q == 0 ? acc : 1u);
+                    ptx::mma_i8(d + COLS * q, w + ((q * W_PLANE_BYTES) >> 4), LIMB_DESC_HI, t, LIMB_DESC_HI,
+                                IDESC | ((uint32_t)((COLS * (PLANES - q)) >> 3) << 17), q == 0 ? acc : 1u);
             };
             uint32_t unit_phase = 0, seg_phase = 0;
             bool ok = true;

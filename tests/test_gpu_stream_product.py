@@ -22,6 +22,7 @@ def cb():
 @pytest.mark.parametrize("T,K,N", [
     (1, 8, 4),             # the smallest problem: one step, one quarter, a quarter of a step deep
     (3, 40, 28), (32, 32, 32), (33, 64, 36),      # one and two token tiles
+    (16, 72, 160), (17, 72, 160),                 # accumulators of 16 and 32 columns
     (31, 104, 128), (65, 96, 132),                # a full feature tile, and four features into the next
     (7, 1032, 420),        # more steps than SMs in one tile's range, ragged in every direction
     (1, 16, 32752),        # 256 feature tiles of a single step: the scratch array's limit in N

@@ -110,7 +110,7 @@ typedef struct {
 
 /* phases of the path, for the per-phase timers of comet_stats */
 enum {
-    COMET_PHASE_COMPACT = 0,  /* mask compaction                                   */
+    COMET_PHASE_COMPACT = 0,  /* mask compaction, where a kernel does it            */
     COMET_PHASE_OPEN = 1,     /* E_i = X_i - A_i, F_i = gather(W_i) - B_i, exchange, operand planes */
     COMET_PHASE_PREP = 2,     /* not used: the opening kernels prepare the operands too    */
     COMET_PHASE_COMBINE = 3,  /* the gathered ring matmul + Beaver combine          */
@@ -136,7 +136,7 @@ typedef struct {
     int32_t n_components;    /* connected components under the current token mask (0 without one) */
     int32_t reserved;
     int64_t tensor_tile_macs; /* 64-bit multiply-adds the tensor-core kernel of the last ffn call covered, counted
-                                 in whole output tiles (128 x 64, or 32 tokens x 128 for at most 32 tokens) and
+                                 in whole output tiles (128 x 64, or 32 tokens x 128 in the kernel for few tokens) and
                                  32-deep steps, both parties (0 on the CUDA-core path): under a token mask with
                                  several components only the tiles and steps that meet a component */
 } comet_stats_t;

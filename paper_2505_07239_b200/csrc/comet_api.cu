@@ -82,9 +82,8 @@ struct comet_ctx {
     int32_t* d_ids;
     comet::BlockIds held;         // the ids of a mask the host held, when there are few enough blocks (ids_held)
     bool ids_held;
-    uint32_t* d_stream_sync;      // StreamArgs::sync: a ticket counter, a flag per tile of the streaming kernel
+    uint32_t* d_stream_sync;      // StreamArgs::sync: epoch and tickets, a flag per tile of the streaming kernel
     size_t stream_sync_words;
-    uint32_t stream_tickets, stream_epoch;    // tickets taken and streaming kernels launched so far
     int32_t* d_count;             // {count, error flag of the bounded waits}
     int32_t* h_count;             // pinned and mapped: {count, error flag as the compaction kernel saw it, ticket,
                                   // error word written by a kernel whose bounded wait ran out}
@@ -278,7 +277,7 @@ bool result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_rows, int 
 // The streaming kernel.  Without `sync` words (they belong to one stream's order, so a call without a context has none) Z <- C
 // is a launch of its own before it; the product begins while the copy runs and waits for it before its first sum.
 int launch_stream(comet::StreamArgs& args, const comet::BlockIds& held, int sm_count, cudaStream_t stream,
-                  const int* priority, cudaError_t* err, unsigned* grid_out) {
+                  const int* priority, cudaError_t* err) {
     namespace ls = comet::limb_stream;
     *err = cudaSuccess;
     args.mt = ceil_div(args.M, ls::BT);
@@ -302,7 +301,6 @@ int launch_stream(comet::StreamArgs& args, const comet::BlockIds& held, int sm_c
                               nullptr, args.C[0], args.C[1], args.Z[0], args.Z[1], pairs);
         if (*err != cudaSuccess) return COMET_ERR_CUDA;
     }
-    *grid_out = grid;
     *err = launch_chained(args.M <= 16 ? comet::combine_stream_kernel<16> : comet::combine_stream_kernel<32>, dim3(grid), dim3(ls::THREADS), ls::SMEM_BYTES, stream,
                           priority, args, maps, held);
     return *err == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
@@ -325,10 +323,8 @@ int stream_product(comet_ctx* c, const Proj& pr) {
         a.Z[p] = c->buf[p][pr.idZ];
         a.C[p] = c->buf[p][pr.idC];
     }
-    if (1 + (size_t)ceil_div(pr.M, ls::BT) * ceil_div(pr.N, ls::BW) > c->stream_sync_words) return COMET_ERR_SHAPE;
+    if (ls::SYNC_WORDS + (size_t)ceil_div(pr.M, ls::BT) * ceil_div(pr.N, ls::BW) > c->stream_sync_words) return COMET_ERR_SHAPE;
     a.sync = c->d_stream_sync;
-    a.ticket0 = c->stream_tickets;
-    a.epoch = c->stream_epoch + 1 == 0 ? 1 : c->stream_epoch + 1;
     a.gather = 1;
     a.ids = c->ids_held ? nullptr : c->d_ids;
     a.n = c->n_active;
@@ -347,14 +343,11 @@ int stream_product(comet_ctx* c, const Proj& pr) {
     cudaError_t err;
     {
         PhaseTimer timer(c, COMET_PHASE_COMBINE, 1);
-        unsigned grid = 0;
-        const int rc = launch_stream(a, c->held, c->sm_count, c->stream, &c->top_priority, &err, &grid);
+        const int rc = launch_stream(a, c->held, c->sm_count, c->stream, &c->top_priority, &err);
         if (rc != COMET_OK) {
             c->last_cuda_error = (int)err;
             return rc;
         }
-        c->stream_tickets += grid;
-        c->stream_epoch = a.epoch;
     }
     c->stats.kernel_launches += 1;
     c->stats.tensor_tile_macs = 2ll * 2 * a.mt * a.nt * a.kb * ls::KC * ls::BW * ls::BT;
@@ -699,7 +692,7 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
     {
         namespace ls = comet::limb_stream;
         const int64_t widest = c->groups * c->cap_n > cfg->d_model ? c->groups * c->cap_n : cfg->d_model;
-        c->stream_sync_words = 1 + (STREAM_TOKENS / ls::BT) * (size_t)((widest + ls::BW - 1) / ls::BW);
+        c->stream_sync_words = ls::SYNC_WORDS + (STREAM_TOKENS / ls::BT) * (size_t)((widest + ls::BW - 1) / ls::BW);
         reserve(device, &c->d_stream_sync, c->stream_sync_words * sizeof(uint32_t));
     }
     reserve(pinned, &c->h_masked, comet::PLAN_WORDS * sizeof(long long));
@@ -1376,8 +1369,7 @@ extern "C" int comet_beaver_matmul_static(void* cuda_stream, const uint64_t* con
     a.ldw = K;
     cudaError_t err;
     static const comet::BlockIds none = {};
-    unsigned grid = 0;
-    const int rc = launch_stream(a, none, dev.sm_count, (cudaStream_t)cuda_stream, nullptr, &err, &grid);
+    const int rc = launch_stream(a, none, dev.sm_count, (cudaStream_t)cuda_stream, nullptr, &err);
     if (err != cudaSuccess) cudaGetLastError();
     return rc;
 }

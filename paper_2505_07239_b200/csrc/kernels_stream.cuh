@@ -60,6 +60,7 @@ constexpr int T_SET_BYTES = PLANES * BT * KC;            //  8 KiB: limb planes 
 constexpr int OUT_TOKENS = 4;                            // tokens an epilogue thread recombines at a time
 constexpr int OUT_BYTES = OUT_TOKENS * 32 * 8;           // an epilogue warp's staging buffer: a row of 32 features per token
 constexpr int ACC_COLS = PLANES * BT;                    // 256 TMEM columns per party
+constexpr int SYNC_WORDS = 2;                            // of StreamArgs::sync before the tiles' flags
 // A step adds two products to an accumulator, so the bound on a segment's depth (16384 contraction indices keep the
 // limb sums for s <= 3 below 2^32) allows half as many steps.
 constexpr int MAX_SEGMENT_STEPS = limb::MAX_SEGMENT_UNITS / 2;
@@ -82,10 +83,11 @@ struct StreamArgs {
     u64* F[2];                                            // message, [N, K]
     u64* Z[2];                                            // [M, N]
     const u64* C[2];                                      // [M, N]: what the sums are added to
-    // [1 + tiles] words of one context, or null (then Z holds C when the kernel before this one has completed): a ticket
-    // counter, and per tile the epoch of the last launch in which its part of Z became C
+    // [SYNC_WORDS + tiles] words of one context, or null (then Z holds C when the kernel before this one has completed).  The
+    // first two are one 64-bit word: the number of launches so far, above the tickets taken of this one.  Then, per tile, the
+    // epoch (launches before it plus one, never 0) of the last launch in which its part of Z became C.  All zero to begin with,
+    // and advanced on the device alone: a launch may be captured once and run any number of times.
     uint32_t* sync;
-    uint32_t ticket0, epoch; // the counter's value when this launch takes its first ticket; this launch's number, never 0
     int gather;              // 0: the right operand is W0 itself, [N, K]
     const int32_t* ids;      // ascending active block ids, or null: they are in the launch's BlockIds
     int n, bs;               // active neurons, neurons per block (a multiple of 16 when there are ids)
@@ -200,7 +202,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
     __shared__ __align__(8) uint64_t planes_full, own_empty[2], shared_empty;     // own: B_0 / B_1; shared: F, E, V_i
     __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
     __shared__ __align__(8) uint64_t own_landed, own_stored;                      // C of a tile of this CTA's: in, and out again
-    __shared__ uint32_t tmem_slot, ticket;
+    __shared__ uint32_t tmem_slot, ticket, epoch;
     __shared__ int abort_flag;
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
@@ -211,7 +213,11 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    if (threadIdx.x == 32) ticket = a.sync ? atomicAdd(a.sync, 1u) - a.ticket0 : blockIdx.x;
+    if (threadIdx.x == 32) {
+        const u64 word = a.sync ? atomicAdd(reinterpret_cast<u64*>(a.sync), 1ull) : blockIdx.x;
+        ticket = (uint32_t)word;
+        epoch = (uint32_t)(word >> 32) + 1;
+    }
     if (threadIdx.x == 0) {
         for (int s = 0; s < RAW_SLOTS; ++s) {
             ptx::mbar_init(ptx::smem_u32(&raw_full[s]), 64);                // every producer lane
@@ -237,7 +243,10 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
     __syncthreads();
     ptx::fence_after_sync();
     const uint32_t tmem_base = tmem_slot;
-    const unsigned cta = ticket, u_begin = stream_cut(a, cta), u_end = stream_cut(a, cta + 1);
+    // A ticket beyond the launch means that the words are not what the launches before it left: nothing is touched then.
+    const bool valid = ticket < gridDim.x;
+    if (!valid && threadIdx.x == 0) abort_flag = 1;
+    const unsigned cta = valid ? ticket : 0u, u_begin = stream_cut(a, cta), u_end = valid ? stream_cut(a, cta + 1) : u_begin;
     // Without `sync` there is no wait for the predecessor here: it is the kernel that initialises Z, which only the epilogue
     // touches.  That kernel let this one start after its own wait, so whatever came before it has completed.
     if (a.sync) pdl_wait();
@@ -468,7 +477,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             // copy engine to have read the one before.  (One buffer and a bulk reduction per row: 7400 cycles for 32 tokens.)
             if (!z_ready) pdl_wait();                            // Z holds C_i
             z_ready = true;
-            if (a.sync) ok = stream_tile_ready(a.sync + 1 + sg.tile, a.epoch, lane, &abort_flag);
+            if (a.sync) ok = stream_tile_ready(a.sync + SYNC_WORDS + sg.tile, epoch, lane, &abort_flag);
             ok = ok && limb_wait_warp(ptx::smem_u32(&acc_full[party]), seg_phase, &abort_flag);
             if (!ok) break;
             ptx::fence_after_sync();
@@ -514,6 +523,12 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                     ptx::mma_i8(d + COLS * q, w + ((q * W_PLANE_BYTES) >> 4), LIMB_DESC_HI, t, LIMB_DESC_HI,
                                 IDESC | ((uint32_t)((COLS * (PLANES - q)) >> 3) << 17), q == 0 ? acc : 1u);
             };
+            if (a.sync && ticket + 1 == gridDim.x) {
+                // The last ticket is taken: no tickets of the next epoch.  Nobody reads the word before the next launch, whose
+                // CTAs begin when every CTA of this one has let them or has ended; this one does so behind the fence.
+                atomicAdd(reinterpret_cast<u64*>(a.sync), ((u64)(epoch + 1 ? 1u : 2u) << 32) - gridDim.x);
+                __threadfence();
+            }
             uint32_t unit_phase = 0, seg_phase = 0;
             bool ok = true;
             for (unsigned u = u_begin; u < u_end && ok;) {
@@ -580,7 +595,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             asm volatile("fence.proxy.async;" ::: "memory");
             __threadfence();
             __syncwarp();
-            if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.sync + 1 + tile), "r"(a.epoch) : "memory");
+            if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.sync + SYNC_WORDS + tile), "r"(epoch) : "memory");
         }
     }
 

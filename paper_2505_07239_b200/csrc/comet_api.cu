@@ -722,8 +722,9 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
         c->h_count[0] = c->h_count[1] = c->h_count[2] = c->h_count[3] = 0;     // pinned memory is not zeroed
         for (int k = 0; k < comet::PLAN_WORDS; ++k) c->h_masked[k] = 0;
     }
-    ok = ok && cudaMemset(c->d_count, 0, 2 * sizeof(int32_t)) == cudaSuccess;
-    ok = ok && cudaMemset(c->d_stream_sync, 0, c->stream_sync_words * sizeof(uint32_t)) == cudaSuccess;
+    // on the context's own stream: every kernel that uses these words is ordered behind it, whatever the default stream does
+    ok = ok && cudaMemsetAsync(c->d_count, 0, 2 * sizeof(int32_t), c->stream) == cudaSuccess;
+    ok = ok && cudaMemsetAsync(c->d_stream_sync, 0, c->stream_sync_words * sizeof(uint32_t), c->stream) == cudaSuccess;
     ok = ok && cudaHostGetDevicePointer((void**)&c->h_masked_dev, c->h_masked, 0) == cudaSuccess;
     ok = ok && cudaHostGetDevicePointer((void**)&c->h_count_dev, c->h_count, 0) == cudaSuccess;
     if (!ok) {

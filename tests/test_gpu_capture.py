@@ -1,5 +1,6 @@
-"""Calls captured in a CUDA graph: a layer captured once, an ordinary step before the first replay, replays with new inputs in
-the bound buffers, and an ordinary step after them.  Bit for bit against the CPU oracle."""
+"""The order of a context's work on its stream.  Calls captured in a CUDA graph: a layer captured once, an ordinary step before
+the first replay, replays with new inputs in the bound buffers, and an ordinary step after them.  A context made while the
+default stream is busy.  Bit for bit against the CPU oracle."""
 import numpy as np
 import pytest
 
@@ -101,3 +102,32 @@ def test_layer_captured_and_replayed(cb, tokens, d, blocks, block, active):
     layer.check(v)
     del graph
     layer.ctx.close()
+
+
+def test_context_made_while_the_default_stream_is_busy(cb):
+    """The words that the kernels count in are cleared in the order of the context's own stream."""
+    mask = np.zeros(24, np.uint8)
+    mask[3:12] = 1
+    stream = torch.cuda.Stream()
+    for cycles in (0, 200_000_000):                    # a first pass that loads what there is to load, then a tenth of a second
+        torch.cuda.synchronize()
+        if cycles:
+            torch.cuda._sleep(cycles)                  # on the default stream
+        with torch.cuda.stream(stream):
+            ctx = cb.Comet(16, 144, 384, 16, 16, max_active=144, stream=stream)
+            X, A, B, C = (torch.zeros(s, dtype=torch.int64, device="cuda") for s in ((16, 144), (16, 144), (144, 144), (16, 144)))
+            W = torch.zeros((384, 144), dtype=torch.int64, device="cuda")
+            C.fill_(5)
+            assert ctx.set_mask(mask) == 144
+            for p in (0, 1):
+                for t, v in ((cb.W1, W), (cb.X, X), (cb.A_UP, A), (cb.B_UP, B), (cb.C_UP, C)):
+                    ctx.bind_shares(p, t, v)
+            ctx.ffn_up(16)
+            out = [ctx.result_view(p, cb.Z_UP, (16, 144)).clone() for p in (0, 1)]
+            stream.synchronize()
+            # the product ran while the default stream was still at work: the case that is meant
+            assert not cycles or not torch.cuda.default_stream().query()
+        ctx.synchronize()
+        assert all(bool((z == 5).all()) for z in out)
+        torch.cuda.synchronize()
+        ctx.close()

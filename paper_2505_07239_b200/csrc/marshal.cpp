@@ -61,28 +61,38 @@ const at::Tensor* as_tensor(PyObject* o) {
 
 bool device_words(const at::Tensor& t) { return t.is_cuda() && t.is_contiguous() && t.element_size() == 8; }
 
-// The tensors of both parties: contiguous, on the GPU, `bytes` per element.
-bool as_pair(PyObject* o, int bytes, const at::Tensor* out[2]) {
-    for (Py_ssize_t p = 0; p < 2; ++p) {
-        PyObject* item = PySequence_GetItem(o, p);
-        if (!item) return false;
-        out[p] = as_tensor(item);
-        Py_DECREF(item);                 // the sequence keeps it
-        if (!out[p]) return false;
-        if (!out[p]->is_cuda() || !out[p]->is_contiguous() || out[p]->element_size() != bytes)
+// The tensors of both parties: contiguous, on the GPU, of a given element size.  The items are this object's own references
+// until the call is over: what they came from may make its items on demand (a stacked tensor, any class with __getitem__).
+struct Pair {
+    PyObject* item[2] = {nullptr, nullptr};
+    const at::Tensor* t[2] = {nullptr, nullptr};
+    Pair() = default;
+    Pair(const Pair&) = delete;
+    ~Pair() {
+        Py_XDECREF(item[0]);
+        Py_XDECREF(item[1]);
+    }
+    const at::Tensor& operator[](int p) const { return *t[p]; }
+};
+
+bool as_pair(PyObject* o, int bytes, Pair& out) {
+    static PyObject* const index[2] = {PyLong_FromLong(0), PyLong_FromLong(1)};
+    for (int p = 0; p < 2; ++p) {
+        if (!(out.item[p] = PyObject_GetItem(o, index[p])) || !(out.t[p] = as_tensor(out.item[p]))) return false;
+        if (!out[p].is_cuda() || !out[p].is_contiguous() || out[p].element_size() != bytes)
             return refuse(PyExc_AssertionError, "contiguous CUDA tensors of the documented element size are expected");
     }
     return true;
 }
 
-bool same_shape(const at::Tensor* const t[2], const at::Tensor& like) {
-    if (t[0]->sizes() == like.sizes() && t[1]->sizes() == like.sizes()) return true;
+bool same_shape(const Pair& t, const at::Tensor& like) {
+    if (t[0].sizes() == like.sizes() && t[1].sizes() == like.sizes()) return true;
     return refuse(PyExc_AssertionError, "the tensors of both parties must have the documented shapes");
 }
 
-bool shaped(const at::Tensor* const t[2], std::initializer_list<int64_t> shape) {
+bool shaped(const Pair& t, std::initializer_list<int64_t> shape) {
     const at::IntArrayRef s(shape);
-    if (t[0]->sizes() == s && t[1]->sizes() == s) return true;
+    if (t[0].sizes() == s && t[1].sizes() == s) return true;
     return refuse(PyExc_AssertionError, "the tensors of both parties must have the documented shapes");
 }
 
@@ -90,7 +100,7 @@ uint64_t* words(const at::Tensor& t) { return static_cast<uint64_t*>(t.data_ptr(
 
 struct ConstPair {
     const uint64_t* p[2];
-    explicit ConstPair(const at::Tensor* const t[2]) : p{words(*t[0]), words(*t[1])} {}
+    explicit ConstPair(const Pair& t) : p{words(t[0]), words(t[1])} {}
 };
 
 // A new contiguous tensor like `like`, on its device, from torch's CUDA allocator and on the current stream as ever, without the
@@ -232,24 +242,25 @@ int truncate_call(comet_ctx* ctx, int32_t id) { return comet_truncate(ctx, id); 
 PyObject* shuffle(PyObject*, PyObject* const* args, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
         void* stream;
-        const at::Tensor *X[2], *tau[2], *rho[2], *a[2], *b[2], *flag = nullptr;
+        Pair X, tau, rho, a, b;
+        const at::Tensor* flag = nullptr;
         if (!counted(n, 7) || !as_stream(args[0], &stream) || !as_pair(args[1], 8, X) || !as_pair(args[2], 4, tau) ||
             !as_pair(args[3], 4, rho) || !as_pair(args[4], 8, a) || !as_pair(args[5], 8, b))
             return nullptr;
         if (args[6] != Py_None && !(flag = as_tensor(args[6]))) return nullptr;
-        const int64_t rows = X[0]->size(0), cols = rows ? X[0]->numel() / rows : 0;
+        const int64_t rows = X[0].size(0), cols = rows ? X[0].numel() / rows : 0;
         for (int p = 0; p < 2; ++p)
-            if (tau[p]->scalar_type() != at::kInt || rho[p]->scalar_type() != at::kInt) {
+            if (tau[p].scalar_type() != at::kInt || rho[p].scalar_type() != at::kInt) {
                 refuse(PyExc_AssertionError, "int32 permutations are expected");
                 return nullptr;
             }
-        if (!same_shape(X, *X[0]) || !shaped(tau, {rows}) || !shaped(rho, {rows}) || !same_shape(a, *X[0]) ||
-            !same_shape(b, *X[0]))
+        if (!same_shape(X, X[0]) || !shaped(tau, {rows}) || !shaped(rho, {rows}) || !same_shape(a, X[0]) ||
+            !same_shape(b, X[0]))
             return nullptr;
-        const NewPair Y(*X[0]), Z(*X[0]);
+        const NewPair Y(X[0]), Z(X[0]);
         const ConstPair x(X), am(a), bm(b);
-        const int32_t* t[2] = {static_cast<int32_t*>(tau[0]->data_ptr()), static_cast<int32_t*>(tau[1]->data_ptr())};
-        const int32_t* r[2] = {static_cast<int32_t*>(rho[0]->data_ptr()), static_cast<int32_t*>(rho[1]->data_ptr())};
+        const int32_t* t[2] = {static_cast<int32_t*>(tau[0].data_ptr()), static_cast<int32_t*>(tau[1].data_ptr())};
+        const int32_t* r[2] = {static_cast<int32_t*>(rho[0].data_ptr()), static_cast<int32_t*>(rho[1].data_ptr())};
         int32_t* f = flag ? static_cast<int32_t*>(flag->data_ptr()) : nullptr;
         const int code = unlocked([&] { return comet_shuffle(stream, x.p, t, r, am.p, bm.p, Y.p, Z.p, rows, cols, f); });
         return answer(code, {&Y, &Z});
@@ -280,13 +291,13 @@ PyObject* invert_permutation(PyObject*, PyObject* const* args, Py_ssize_t n) {
 PyObject* beaver_mul(PyObject*, PyObject* const* args, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
         void* stream;
-        const at::Tensor* in[5][2];
+        Pair in[5];
         if (!counted(n, 6) || !as_stream(args[0], &stream)) return nullptr;
         for (int k = 0; k < 5; ++k)
-            if (!as_pair(args[1 + k], 8, in[k]) || !same_shape(in[k], *in[0][0])) return nullptr;
-        const NewPair D(*in[0][0]), E(*in[0][0]), Z(*in[0][0]);
+            if (!as_pair(args[1 + k], 8, in[k]) || !same_shape(in[k], in[0][0])) return nullptr;
+        const NewPair D(in[0][0]), E(in[0][0]), Z(in[0][0]);
         const ConstPair x(in[0]), y(in[1]), a(in[2]), b(in[3]), c(in[4]);
-        const int64_t count = in[0][0]->numel();
+        const int64_t count = in[0][0].numel();
         const int code = unlocked([&] { return comet_beaver_mul(stream, x.p, y.p, a.p, b.p, c.p, D.p, E.p, Z.p, count); });
         return answer(code, {&D, &E, &Z});
     });
@@ -297,15 +308,15 @@ PyObject* truncate_pair(PyObject*, PyObject* const* args, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
         void* stream;
         int64_t frac;
-        const at::Tensor *z[2], *r[2], *rp[2];
+        Pair z, r, rp;
         if (!counted(n, 5) || !as_stream(args[0], &stream) || !as_pair(args[1], 8, z) || !as_pair(args[2], 8, r) ||
             !as_pair(args[3], 8, rp) || !as_int(args[4], &frac))
             return nullptr;
-        if (!same_shape(z, *z[0]) || !same_shape(r, *z[0]) || !same_shape(rp, *z[0])) return nullptr;
-        const NewPair M(*z[0]);
+        if (!same_shape(z, z[0]) || !same_shape(r, z[0]) || !same_shape(rp, z[0])) return nullptr;
+        const NewPair M(z[0]);
         const ConstPair rc(r), rpc(rp);
-        uint64_t* const zp[2] = {words(*z[0]), words(*z[1])};
-        const int64_t count = z[0]->numel();
+        uint64_t* const zp[2] = {words(z[0]), words(z[1])};
+        const int64_t count = z[0].numel();
         const int code = unlocked([&] { return comet_truncate_pair(stream, zp, rc.p, rpc.p, M.p, count, (int32_t)frac); });
         return answer(code, {&M});
     });
@@ -315,16 +326,16 @@ PyObject* truncate_pair(PyObject*, PyObject* const* args, Py_ssize_t n) {
 PyObject* add_bias(PyObject*, PyObject* const* args, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
         void* stream;
-        const at::Tensor *z[2], *bias[2];
+        Pair z, bias;
         if (!counted(n, 3) || !as_stream(args[0], &stream) || !as_pair(args[1], 8, z) || !as_pair(args[2], 8, bias))
             return nullptr;
-        if (z[0]->dim() != 2) {
+        if (z[0].dim() != 2) {
             refuse(PyExc_ValueError, "a matrix is expected");
             return nullptr;
         }
-        const int64_t rows = z[0]->size(0), cols = z[0]->size(1);
-        if (!same_shape(z, *z[0]) || !shaped(bias, {cols})) return nullptr;
-        uint64_t* const zp[2] = {words(*z[0]), words(*z[1])};
+        const int64_t rows = z[0].size(0), cols = z[0].size(1);
+        if (!same_shape(z, z[0]) || !shaped(bias, {cols})) return nullptr;
+        uint64_t* const zp[2] = {words(z[0]), words(z[1])};
         const ConstPair b(bias);
         return PyLong_FromLong(unlocked([&] { return comet_add_bias(stream, zp, b.p, rows, cols); }));
     });
@@ -334,20 +345,20 @@ PyObject* add_bias(PyObject*, PyObject* const* args, Py_ssize_t n) {
 PyObject* beaver_matmul_static(PyObject*, PyObject* const* args, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
         void* stream;
-        const at::Tensor* t[6][2];
+        Pair t[6];
         if (!counted(n, 7) || !as_stream(args[0], &stream)) return nullptr;
         for (int k = 0; k < 6; ++k)
             if (!as_pair(args[1 + k], 8, t[k])) return nullptr;
-        if (t[0][0]->dim() != 2 || t[2][0]->dim() != 2) {
+        if (t[0][0].dim() != 2 || t[2][0].dim() != 2) {
             refuse(PyExc_ValueError, "matrices are expected");
             return nullptr;
         }
-        const int64_t T = t[0][0]->size(0), K = t[0][0]->size(1), N = t[2][0]->size(0);
+        const int64_t T = t[0][0].size(0), K = t[0][0].size(1), N = t[2][0].size(0);
         if (!shaped(t[0], {T, K}) || !shaped(t[1], {T, K}) || !shaped(t[2], {N, K}) || !shaped(t[3], {N, K}) ||
             !shaped(t[4], {T, N}) || !shaped(t[5], {T, N}))
             return nullptr;
         const ConstPair X(t[0]), A(t[1]), Y(t[2]), B(t[3]), C(t[4]);
-        uint64_t* const Z[2] = {words(*t[5][0]), words(*t[5][1])};
+        uint64_t* const Z[2] = {words(t[5][0]), words(t[5][1])};
         return PyLong_FromLong(unlocked([&] {
             return comet_beaver_matmul_static(stream, X.p, A.p, Y.p, B.p, C.p, Z, (int32_t)T, (int32_t)K, (int32_t)N);
         }));

@@ -3,6 +3,7 @@ header declares, and rejects bad arguments before touching a GPU."""
 import ctypes
 import os
 import re
+import sys
 
 import pytest
 
@@ -65,3 +66,25 @@ def test_null_context_is_rejected(cb):
     assert lib.comet_load_shares(None, 0, cb.X, None, 0, 1, 1) == -1
     assert lib.comet_stats(None, None) == -1
     lib.comet_destroy(None)
+
+
+def test_pairs_may_make_their_items_on_demand(cb):
+    """A stacked tensor, or any class with __getitem__, is a pair like a list: its items are looked at (these are refused,
+    because they are on the CPU), and what the call was given is left as it was."""
+    torch = pytest.importorskip("torch")
+
+    class OnDemand:
+        def __getitem__(self, i):
+            return torch.zeros((4, 6), dtype=torch.int64) + i
+
+    kept = [torch.zeros((4, 6), dtype=torch.int64) for _ in (0, 1)]
+    for pair in (torch.zeros((2, 4, 6), dtype=torch.int64), OnDemand(), kept):
+        with pytest.raises(AssertionError):
+            cb.add_bias(pair, pair)
+        with pytest.raises(AssertionError):
+            cb.beaver_mul(pair, pair, pair, pair, pair)
+    counts = [sys.getrefcount(t) for t in kept]
+    for _ in range(10):
+        with pytest.raises(AssertionError):
+            cb.truncate_pair(kept, kept, kept, 12)
+    assert [sys.getrefcount(t) for t in kept] == counts

@@ -1226,10 +1226,12 @@ int comet_get_index(comet_ctx* c, int32_t* out, int location, int32_t capacity, 
     if (!c->mask_set) return COMET_ERR_STATE;
     if (capacity < c->n_active_blocks) return COMET_ERR_SHAPE;
     if (c->ids_held) {
-        std::vector<int32_t> ids(c->held.id, c->held.id + c->n_active_blocks);
-        if (location == COMET_HOST) std::copy(ids.begin(), ids.end(), out);
-        else if (!ids.empty())        // from pageable memory: taken over before the call returns
-            COMET_CUDA(c, cudaMemcpyAsync(out, ids.data(), ids.size() * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
+        if (location == COMET_HOST) std::copy(c->held.id, c->held.id + c->n_active_blocks, out);
+        else if (c->n_active_blocks > 0) {
+            COMET_CUDA(c, launch_chained(comet::held_ids_kernel, dim3(1), dim3(comet::BlockIds::CAPACITY), 0, c->stream, nullptr,
+                                         c->held, (int)c->n_active_blocks, out));
+            c->stats.kernel_launches += 1;
+        }
     } else if (c->n_active_blocks > 0)
         COMET_CUDA(c, cudaMemcpyAsync(out, c->d_ids, (size_t)c->n_active_blocks * sizeof(int32_t),
                                       copy_kind(location, false), c->stream));

@@ -158,6 +158,14 @@ __device__ __forceinline__ int block_id(const int32_t* ids, const BlockIds& held
     return ids ? __ldg(ids + blk) : (int)held.id[blk];
 }
 
+// The list written out, for a caller who reads it: from the parameter block too, so that the call can be captured.
+__global__ void __launch_bounds__(BlockIds::CAPACITY)
+held_ids_kernel(const __grid_constant__ BlockIds held, int count, int32_t* __restrict__ out) {
+    pdl_wait();
+    pdl_launch_dependents();
+    if ((int)threadIdx.x < count) out[threadIdx.x] = held.id[threadIdx.x];
+}
+
 template <bool LEFT>
 __device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, const BlockIds& held, int block, uint8_t* smem) {
     using namespace limb;

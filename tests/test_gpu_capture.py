@@ -1,6 +1,8 @@
 """The order of a context's work on its stream.  Calls captured in a CUDA graph: a layer captured once, an ordinary step before
-the first replay, replays with new inputs in the bound buffers, and an ordinary step after them.  A context made while the
-default stream is busy.  Bit for bit against the CPU oracle."""
+the first replay, replays with new inputs in the bound buffers, and an ordinary step after them; an index list.  A context
+made while the default stream is busy.  Bit for bit against the CPU oracle."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -102,6 +104,39 @@ def test_layer_captured_and_replayed(cb, tokens, d, blocks, block, active):
     layer.check(v)
     del graph
     layer.ctx.close()
+
+
+@pytest.mark.parametrize("blocks", [1, 1024, 1040])    # lists that travel with the launches, and one that a kernel compacts
+def test_index_list_captured_and_replayed(cb, blocks):
+    stream = torch.cuda.Stream()
+    ctx = cb.Comet(4, 16, blocks * 16, 16, 12, stream=stream)
+    rng = np.random.default_rng(blocks)
+    masks = [(rng.random(blocks) < 0.5).astype(np.uint8) for _ in range(3)]
+    masks[1][-1] = 1
+    out = torch.full((blocks,), -1, dtype=torch.int32, device="cuda")
+    count = ctypes.c_int32()
+    ctx.set_mask(masks[0])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        ctx.set_mask(masks[1])
+        assert cb.library().comet_get_index(ctx._h, out.data_ptr(), cb.DEVICE, blocks, ctypes.byref(count)) == cb.OK
+    ctx.set_mask(masks[2])                             # what the list was taken from is gone
+    for _ in range(2):
+        out.fill_(-1)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            graph.replay()
+        stream.synchronize()
+        assert out[:count.value].tolist() == np.flatnonzero(masks[1]).tolist()
+        assert (out[count.value:] == -1).all()
+    host = np.full(blocks, -1, np.int32)
+    ctx.set_mask(masks[2])
+    assert cb.library().comet_get_index(ctx._h, host.ctypes.data, cb.HOST, blocks, ctypes.byref(count)) == cb.OK
+    ctx.synchronize()
+    assert host[:count.value].tolist() == np.flatnonzero(masks[2]).tolist()
+    del graph
+    ctx.close()
 
 
 def test_context_made_while_the_default_stream_is_busy(cb):

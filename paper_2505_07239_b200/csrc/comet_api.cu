@@ -275,7 +275,7 @@ bool result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_rows, int 
 }
 
 // The streaming kernel.  Without `sync` words (they belong to one stream's order, so a call without a context has none) Z <- C
-// is a launch of its own before it; the product begins while the copy runs and waits for it before its first sum.
+// is a launch of its own before it; the product's CTAs are set up while the copy runs.
 int launch_stream(comet::StreamArgs& args, const comet::BlockIds& held, int sm_count, cudaStream_t stream,
                   const int* priority, cudaError_t* err) {
     namespace ls = comet::limb_stream;

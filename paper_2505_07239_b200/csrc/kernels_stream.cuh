@@ -110,8 +110,8 @@ struct StreamArgs {
 __global__ void __launch_bounds__(256)
 result_init_kernel(const u64* __restrict__ c0, const u64* __restrict__ c1, u64* __restrict__ z0, u64* __restrict__ z1,
                    long long pairs) {
+    pdl_launch_dependents();             // the product's CTAs are set up meanwhile; they wait for this kernel's end
     pdl_wait();
-    pdl_launch_dependents();
     const ulonglong2* __restrict__ s = reinterpret_cast<const ulonglong2*>(blockIdx.y ? c1 : c0);
     ulonglong2* __restrict__ d = reinterpret_cast<ulonglong2*>(blockIdx.y ? z1 : z0);
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -247,9 +247,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
     const bool valid = ticket < gridDim.x;
     if (!valid && threadIdx.x == 0) abort_flag = 1;
     const unsigned cta = valid ? ticket : 0u, u_begin = stream_cut(a, cta), u_end = valid ? stream_cut(a, cta + 1) : u_begin;
-    // Without `sync` there is no wait for the predecessor here: it is the kernel that initialises Z, which only the epilogue
-    // touches.  That kernel let this one start after its own wait, so whatever came before it has completed.
-    if (a.sync) pdl_wait();
+    pdl_wait();
 
     if (warp >= RAW_WARP0 && warp < RAW_WARP0 + 2) {
         // ---------------- raw producer of one party: 16 lanes per row of a slot ----------------
@@ -413,7 +411,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
         const int party = (warp - TOK_WARP0) / EPI_WARPS, quarter = warp & 3;     // epilogue: TMEM lanes this warp may read
         u64* out = reinterpret_cast<u64*>(sOut + (size_t)(warp - TOK_WARP0) * OUT_BYTES);
         uint32_t unit_phase = 0, seg_phase = 0;
-        bool ok = true, z_ready = a.sync != nullptr;
+        bool ok = true;
         for (unsigned u = u_begin; u < u_end && ok;) {
             const StreamSegment sg = stream_segment(a, u, u_end);
             u += sg.count;
@@ -475,8 +473,6 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             // Result rows go through shared memory, OUT_TOKENS of them at a time, and one tensor reduction adds them into Z.
             // A CTA's last segment stages them in the raw ring, which nothing uses any more, so that no round waits for the
             // copy engine to have read the one before.  (One buffer and a bulk reduction per row: 7400 cycles for 32 tokens.)
-            if (!z_ready) pdl_wait();                            // Z holds C_i
-            z_ready = true;
             if (a.sync) ok = stream_tile_ready(a.sync + SYNC_WORDS + sg.tile, epoch, lane, &abort_flag);
             ok = ok && limb_wait_warp(ptx::smem_u32(&acc_full[party]), seg_phase, &abort_flag);
             if (!ok) break;
@@ -509,7 +505,6 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&acc_empty[party]));
             seg_phase ^= 1u;
         }
-        if (!z_ready) pdl_wait();                                // every CTA waits for its predecessor once
         if (lane == 0) ptx::bulk_wait_group0();
     } else if (warp == MMA_WARP) {
         // ---------------- MMA issuer: weight plane q against token planes 0..7-q ----------------

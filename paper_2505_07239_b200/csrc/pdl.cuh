@@ -4,9 +4,8 @@
 //                launched with the programmatic-serialisation attribute must execute it in EVERY CTA before its
 //                first access to global memory (reads of the predecessor's results, and writes the predecessor
 //                may still be reading), so that "this kernel has completed" keeps implying "everything before it
-//                has completed".  Without the attribute it returns at once.  (Two exceptions, both in
-//                combine_stream_kernel: its ticket counter, which no other kernel touches, and its form without a
-//                context, behind a kernel that lets it start only after its own wait.)
+//                has completed".  Without the attribute it returns at once.  (One exception: the ticket word of
+//                combine_stream_kernel, which no other kernel touches.)
 //   pdl_launch_dependents(): this CTA no longer minds the next kernel's CTAs being scheduled beside it; the next
 //                kernel starts once every CTA of this one has said so or has exited.
 #pragma once

@@ -1329,6 +1329,24 @@ cudaError_t static_device(StaticDevice* out) {
     return cudaSuccess;
 }
 
+// Whether the result lies on an operand other than its own C (an in-place product).  The streaming kernel writes Z before it
+// has read every operand; the kernels of the other path read X and Y in a launch of their own before the first word of Z.
+bool static_in_place(const uint64_t* const X[2], const uint64_t* const A[2], const uint64_t* const Y[2],
+                     const uint64_t* const B[2], const uint64_t* const C[2], uint64_t* const Z[2], int64_t T, int64_t K,
+                     int64_t N) {
+    for (int q = 0; q < 2; ++q) {
+        const uintptr_t z = reinterpret_cast<uintptr_t>(Z[q]), z_end = z + (uintptr_t)(T * N) * sizeof(u64);
+        auto on = [&](const uint64_t* p, int64_t words) {
+            const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+            return at < z_end && z < at + (uintptr_t)words * sizeof(u64);
+        };
+        for (int p = 0; p < 2; ++p)
+            if (on(X[p], T * K) || on(A[p], T * K) || on(Y[p], N * K) || on(B[p], N * K) || (on(C[p], T * N) && (p != q || C[p] != Z[q])))
+                return true;
+    }
+    return false;
+}
+
 }  // namespace
 
 extern "C" int comet_beaver_matmul_static(void* cuda_stream, const uint64_t* const X[2], const uint64_t* const A[2],
@@ -1353,17 +1371,47 @@ extern "C" int comet_beaver_matmul_static(void* cuda_stream, const uint64_t* con
         cudaGetLastError();
         return COMET_ERR_CUDA;
     }
-    // the streaming kernel over [N, K] right operands without a gather; the array is carved into E_0 | E_1 | F_0 | F_1
-    // (every word used is written before anything reads it)
+    // the array is carved into E_0 | E_1 | F_0 | F_1 (every word used is written before anything reads it)
+    u64* const E[2] = {dev.scratch, dev.scratch + left};
+    u64* const F[2] = {dev.scratch + 2 * left, dev.scratch + 2 * left + right};
+    if (static_in_place(X, A, Y, B, C, Z, T, K, N)) {
+        comet::PartyPtrs x, a, y, b;
+        comet::PartyOut e, f;
+        comet::CombineArgs args;
+        std::memset(&args, 0, sizeof(args));
+        for (int p = 0; p < 2; ++p) {
+            x.p[p] = reinterpret_cast<const u64*>(X[p]);
+            y.p[p] = reinterpret_cast<const u64*>(Y[p]);
+            args.A[p] = a.p[p] = reinterpret_cast<const u64*>(A[p]);
+            args.B[p] = b.p[p] = reinterpret_cast<const u64*>(B[p]);
+            args.C[p] = reinterpret_cast<const u64*>(C[p]);
+            args.Z[p] = reinterpret_cast<u64*>(Z[p]);
+            args.E[p] = e.p[p] = E[p];
+            args.F[p] = f.p[p] = F[p];
+        }
+        args.M = T; args.N = N; args.K = K;
+        args.bs = 1;
+        cudaStream_t stream = (cudaStream_t)cuda_stream;
+        auto grid = [&](int64_t pairs) {
+            const int64_t want = (pairs + 255) / 256, most = (int64_t)dev.sm_count * 8;
+            return dim3((unsigned)(want < most ? want : most), 2);
+        };
+        comet::open_activation_kernel<<<grid(left / 2), 256, 0, stream>>>(x, a, e, left / 2, nullptr, 0, K, 1);
+        comet::open_activation_kernel<<<grid(right / 2), 256, 0, stream>>>(y, b, f, right / 2, nullptr, 0, K, 1);
+        comet::combine_simt_kernel<<<dim3(ceil_div(N, comet::simt::BN), ceil_div(T, comet::simt::BM), 2), comet::simt::THREADS, 0,
+                                     stream>>>(args);
+        return cudaGetLastError() == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
+    }
+    // the streaming kernel over [N, K] right operands without a gather
     comet::StreamArgs a;
     std::memset(&a, 0, sizeof(a));
     for (int p = 0; p < 2; ++p) {
         a.X[p] = reinterpret_cast<const u64*>(X[p]);
         a.A[p] = reinterpret_cast<const u64*>(A[p]);
-        a.E[p] = dev.scratch + p * left;
+        a.E[p] = E[p];
         a.W0[p] = reinterpret_cast<const u64*>(Y[p]);
         a.B[p] = reinterpret_cast<const u64*>(B[p]);
-        a.F[p] = dev.scratch + 2 * left + p * right;
+        a.F[p] = F[p];
         a.Z[p] = reinterpret_cast<u64*>(Z[p]);
         a.C[p] = reinterpret_cast<const u64*>(C[p]);
     }

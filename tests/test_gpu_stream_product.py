@@ -43,6 +43,21 @@ def test_static_product_at_tile_edges(cb, T, K, N):
         assert np.array_equal(Z[p].cpu().numpy().view(np.uint64), ref["Z"][p]), p
 
 
+@pytest.mark.parametrize("on", ["X", "Y", "C"])
+@pytest.mark.parametrize("T,K,N", [(8, 8, 8), (64, 64, 64), (200, 200, 200)])
+def test_static_product_in_place(cb, T, K, N, on):
+    """The result on the memory of an operand of the same size."""
+    v = {k: [wl.random_u64(950 + T, f"place/{k}/{p}", s[0] * s[1]).reshape(s) for p in (0, 1)]
+         for k, s in {"X": (T, K), "A": (T, K), "Y": (N, K), "B": (N, K), "C": (T, N)}.items()}
+    d = {k: [cb.to_device(w) for w in pair] for k, pair in v.items()}
+    assert cb.beaver_matmul_static(d["X"], d["A"], d["Y"], d["B"], d["C"], d[on]) == cb.OK
+    torch.cuda.synchronize()
+    ref = oracle.pi_matmul(v["X"], [np.ascontiguousarray(w.T) for w in v["Y"]], v["A"],
+                           [np.ascontiguousarray(w.T) for w in v["B"]], v["C"])
+    for p in (0, 1):
+        assert np.array_equal(d[on][p].cpu().numpy().view(np.uint64), ref["Z"][p]), p
+
+
 @pytest.mark.parametrize("tokens,d_model,blocks,block,active,stacked", [
     (1, 16, 4, 16, 1, 1),          # 16 features, half a step
     (32, 144, 24, 16, 9, 1),       # 144 features both ways: 128 and a ragged tile of 16

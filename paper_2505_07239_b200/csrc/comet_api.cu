@@ -1329,6 +1329,15 @@ cudaError_t static_device(StaticDevice* out) {
     return cudaSuccess;
 }
 
+// Products a quarter of a step deep with very many token rows and few features run on the CUDA cores: the streaming kernel fills
+// up every step and walks the features again for each of its 32-row tiles, where the other kernel takes 128 x 64 results at a
+// time.  The line is the fourth round of tiles over the SMs.  CUDA cores / streaming, K = 8: 14000 x 4 25 / 22 us, 16384 x 4
+// 25 / 28, 64000 x 4 66 / 86, 16384 x 64 28 / 32, 64000 x 64 101 / 113, but 64000 x 68 177 / 120, and K = 16: 16384 x 4 37 / 28.
+// (20000 .. 50000 x 4000 .. 8000, 3 to 7 % slower streaming, are left there.)
+bool static_on_alus(int T, int K, int N, int sm_count) {
+    return K < 16 && N <= comet::simt::BN && T > 3 * comet::limb_stream::BT * sm_count;
+}
+
 // Whether the result lies on an operand other than its own C (an in-place product).  The streaming kernel writes Z before it
 // has read every operand; the kernels of the other path read X and Y in a launch of their own before the first word of Z.
 bool static_in_place(const uint64_t* const X[2], const uint64_t* const A[2], const uint64_t* const Y[2],
@@ -1374,7 +1383,7 @@ extern "C" int comet_beaver_matmul_static(void* cuda_stream, const uint64_t* con
     // the array is carved into E_0 | E_1 | F_0 | F_1 (every word used is written before anything reads it)
     u64* const E[2] = {dev.scratch, dev.scratch + left};
     u64* const F[2] = {dev.scratch + 2 * left, dev.scratch + 2 * left + right};
-    if (static_in_place(X, A, Y, B, C, Z, T, K, N)) {
+    if (static_on_alus(T, K, N, dev.sm_count) || static_in_place(X, A, Y, B, C, Z, T, K, N)) {
         comet::PartyPtrs x, a, y, b;
         comet::PartyOut e, f;
         comet::CombineArgs args;

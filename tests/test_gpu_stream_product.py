@@ -27,6 +27,7 @@ def cb():
     (7, 1032, 420),        # more steps than SMs in one tile's range, ragged in every direction
     (1, 16, 32752),        # 256 feature tiles of a single step: the scratch array's limit in N
     (2000, 32, 4),         # 63 token tiles against four features
+    (14208, 8, 64), (14209, 8, 64), (14209, 8, 68), (14209, 16, 64), (65531, 8, 4),    # both sides of what the CUDA cores take
     (2, 65536, 4),         # a single tile 2048 steps deep: more than one segment's bound on the contraction depth
 ])
 def test_static_product_at_tile_edges(cb, T, K, N):

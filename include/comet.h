@@ -350,8 +350,9 @@ int comet_last_cuda_error(comet_ctx* ctx);
  * DEVICE pointer on the current device, owned by the caller; X, a, b are only
  * read, Y and Z are overwritten and must not overlap any other argument.  The
  * work is enqueued on `cuda_stream` (NULL = default stream): one kernel, or two
- * when a matrix has more than 2^21 words; the call does not wait for it.  16-byte accesses are used when cols is even and X, a, b,
- * Y, Z are 16-byte aligned, 8-byte accesses otherwise.
+ * when a matrix has more than 2^21 words or very many rows of one or two words;
+ * the call does not wait for it.  16-byte accesses are used when cols is
+ * even and X, a, b, Y, Z are 16-byte aligned, 8-byte accesses otherwise.
  * A permutation entry outside [0, rows) is never followed: the row it would
  * have fetched counts as zero and, if `bad_index_flag` (device int32, may be
  * NULL) is given, it is set to 1.  The caller clears the flag.

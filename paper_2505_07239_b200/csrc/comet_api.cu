@@ -1461,8 +1461,13 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 // One pass over both steps reads X and a twice, the second time from L2 if they stay there: up to 2^21 words per matrix, when
 // the four matrices take half of it.  One pass against two at 512 x 2048: 24 and 30 us, 512 x 4096 (2^21 words): 34 and 37 us,
-// 768 x 4096: 52 and 52 us, 1024 x 4096: 70 and 66 us.
-bool shuffle_in_one_pass(int64_t rows, int64_t cols) { return rows <= (int64_t)(1 << 21) / cols; }
+// 768 x 4096: 52 and 52 us, 1024 x 4096: 70 and 66 us.  A row of one or two words is less than the 32 bytes that a random fetch
+// moves, and one pass makes three of those per row instead of two: as long as one round of resident threads covers the rows of
+// one word (148 SMs x 1024), and up to 3 x 2^16 rows of two.  151552 x 1: 6.5 and 9.0 us, 156000 x 1 11.5 and 9.1, 2^21 x 1 100 and
+// 59; 188000 x 2 8.8 and 9.0, 196608 x 2 10.1 and 9.2, 2^20 x 2 54 and 41.  Rows of three words on: one pass (2^21 words: 46 and 48).
+bool shuffle_in_one_pass(int64_t rows, int64_t cols) {
+    return rows <= (cols == 1 ? 148 << 10 : cols == 2 ? 3 << 16 : (int64_t)(1 << 21) / cols);
+}
 
 // out_i = in_i[perm_i] +/- mask_i for both parties, one launch
 int launch_shuffle_step(cudaStream_t stream, const uint64_t* const in[2], const int32_t* const perm[2],

@@ -1,4 +1,4 @@
-"""Both forms of the shuffle, one pass (matrices of up to 2^21 words) and two, against the CPU oracle, bit for bit."""
+"""Both forms of the shuffle, one pass (matrices of up to 2^21 words, rows of one or two words up to fewer) and two, against the CPU oracle, bit for bit."""
 import numpy as np
 import pytest
 
@@ -18,8 +18,10 @@ def cb():
     return binding
 
 
-# 2^21 words exactly; just above, in 16-byte and in 8-byte pieces; one row longer than the limit
-@pytest.mark.parametrize("rows,cols", [(1024, 2048), (1025, 2050), (699, 3001), (1, (1 << 21) + 2)])
+# 2^21 words exactly; just above, in 16-byte and in 8-byte pieces; one row longer than the limit; both sides of the line for
+# rows of one and of two words
+@pytest.mark.parametrize("rows,cols", [(1024, 2048), (1025, 2050), (699, 3001), (1, (1 << 21) + 2),
+                                       (148 << 10, 1), ((148 << 10) + 1, 1), (3 << 16, 2), ((3 << 16) + 1, 2)])
 @pytest.mark.parametrize("bad", [False, True])
 def test_shuffle_on_both_sides_of_the_limit(cb, rows, cols, bad):
     seed = 900 + rows

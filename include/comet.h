@@ -463,9 +463,11 @@ int comet_beaver_mul(void* cuda_stream, const uint64_t* const X[2], const uint64
  * capture.
  *
  * The product runs on the tensor cores in the same kernel as a context's products
- * of at most 32 tokens.  Its device-side waits are bounded like theirs, but there
- * is no context to report to: after a wait that ran out (about two seconds, which
- * no working launch comes near) Z lacks part of its sums.
+ * of at most 32 tokens.  Its device-side waits are bounded like theirs (about two
+ * seconds, which no working launch comes near): after one that ran out Z lacks
+ * part of its sums, and comet_static_status says so.  With K = 8, N <= 64 and more
+ * than about 14000 rows, and when Z lies on the memory of an operand other than
+ * its own C, the product runs on the CUDA cores, which wait for nothing.
  *
  * The array is shared by every call in the process and is never cleared:
  * a call overwrites all of the part it uses before reading it, so stale
@@ -477,6 +479,16 @@ int comet_beaver_mul(void* cuda_stream, const uint64_t* const X[2], const uint64
 int comet_beaver_matmul_static(void* cuda_stream, const uint64_t* const X[2], const uint64_t* const A[2],
                                const uint64_t* const Y[2], const uint64_t* const B[2], const uint64_t* const C[2],
                                uint64_t* const Z[2], int32_t T, int32_t K, int32_t N);
+
+/* Waits for `cuda_stream` and reports whether a comet_beaver_matmul_static call on
+ * the current device gave up on a bounded wait since this was last asked:
+ * COMET_OK, COMET_ERR_TIMEOUT (the results since then are not to be trusted) or
+ * COMET_ERR_CUDA.  The report is given once.  Allocates nothing. */
+int comet_static_status(void* cuda_stream);
+
+/* Test hook: sets, in the order of `cuda_stream`, the word that such a kernel would
+ * have set.  No kernel waits. */
+int comet_static_inject_timeout(void* cuda_stream);
 
 /* ---------------------------------------------------------------------------
  * Measured peak of a multiply pipe.  (Not an operation of the paper: it supports

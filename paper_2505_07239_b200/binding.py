@@ -33,7 +33,7 @@ EXPORTS = (
     "comet_set_profiling", "comet_beaver_matmul_static", "comet_shuffle", "comet_invert_permutation",
     "comet_beaver_mul", "comet_set_token_mask", "comet_get_components", "comet_kv_plan",
     "comet_add_bias", "comet_bind_shares", "comet_truncate_pair", "comet_synchronize", "comet_inject_timeout",
-    "comet_pipe_probe", "comet_device_pointer",
+    "comet_pipe_probe", "comet_device_pointer", "comet_static_status", "comet_static_inject_timeout",
 )
 STATIC_SCRATCH_WORDS = 1 << 20
 ERR_SCRATCH_LIMIT = -7
@@ -97,6 +97,8 @@ def _load():
                                      ctypes.POINTER(ctypes.c_double)]
     pair = ctypes.c_void_p * 2
     lib.comet_beaver_matmul_static.argtypes = [vp, pair, pair, pair, pair, pair, pair, i32, i32, i32]
+    lib.comet_static_status.argtypes = [vp]
+    lib.comet_static_inject_timeout.argtypes = [vp]
     lib.comet_shuffle.argtypes = [vp, pair, pair, pair, pair, pair, pair, pair, i64, i64, vp]
     lib.comet_invert_permutation.argtypes = [vp, vp, vp, i64, vp]
     lib.comet_add_bias.argtypes = [vp, pair, pair, i64, i64]
@@ -300,6 +302,12 @@ def beaver_matmul_static(X, A, Y, B, C, Z, stream: Optional[torch.cuda.Stream] =
     the shared array: keep them on one stream.
     """
     return _native.beaver_matmul_static(stream, X, A, Y, B, C, Z)
+
+
+def static_status(stream: Optional[torch.cuda.Stream] = None) -> int:
+    """Waits for the stream; ERR_TIMEOUT if a beaver_matmul_static call on the current device gave up on a bounded
+    wait since this was last asked (comet_static_status), else 0 = ok."""
+    return _lib.comet_static_status(ctypes.c_void_p(stream.cuda_stream if stream is not None else 0))
 
 
 PIPE_TENSOR_I8, PIPE_ALU_U64 = 0, 1

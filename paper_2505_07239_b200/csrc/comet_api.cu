@@ -1297,10 +1297,13 @@ namespace {
 // this name is only a handle for cudaGetSymbolAddress, never an address to hand
 // to a kernel; each GPU that loads the library carries its own 8 MiB copy.
 static __device__ __align__(256) unsigned long long g_static_scratch[COMET_STATIC_SCRATCH_WORDS];
+// Set by a kernel of such a call that gave up on a bounded wait; comet_static_status reads and clears it.
+static __device__ int g_static_error;
 
 constexpr int kMaxDevices = 64;
 struct StaticDevice {
     u64* scratch;      // device address of the array
+    int* error;        // and of the error word
     int sm_count;
 };
 std::mutex g_static_mutex;
@@ -1315,14 +1318,16 @@ cudaError_t static_device(StaticDevice* out) {
     std::lock_guard<std::mutex> lock(g_static_mutex);
     StaticDevice& d = g_static_device[dev];
     if (!d.scratch) {
-        void* p = nullptr;
+        void *p = nullptr, *e = nullptr;
         err = cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, dev);
         for (auto* kernel : {comet::combine_stream_kernel<16>, comet::combine_stream_kernel<32>})
             if (err == cudaSuccess)
                 err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)comet::limb_stream::SMEM_BYTES);
         if (err == cudaSuccess) err = cudaGetSymbolAddress(&p, g_static_scratch);
+        if (err == cudaSuccess) err = cudaGetSymbolAddress(&e, g_static_error);
         if (err != cudaSuccess) return err;
+        d.error = static_cast<int*>(e);
         d.scratch = static_cast<u64*>(p);
     }
     *out = d;
@@ -1427,11 +1432,36 @@ extern "C" int comet_beaver_matmul_static(void* cuda_stream, const uint64_t* con
     a.n = N; a.bs = 1;
     a.M = T; a.N = N; a.K = K;
     a.ldw = K;
+    a.error_flag = dev.error;
     cudaError_t err;
     static const comet::BlockIds none = {};
     const int rc = launch_stream(a, none, dev.sm_count, (cudaStream_t)cuda_stream, nullptr, &err);
     if (err != cudaSuccess) cudaGetLastError();
     return rc;
+}
+
+extern "C" int comet_static_status(void* cuda_stream) {
+    StaticDevice dev;
+    cudaStream_t stream = (cudaStream_t)cuda_stream;
+    int seen = 0;
+    cudaError_t err = static_device(&dev);
+    if (err == cudaSuccess) err = cudaMemcpyAsync(&seen, dev.error, sizeof(seen), cudaMemcpyDeviceToHost, stream);
+    if (err == cudaSuccess) err = cudaStreamSynchronize(stream);
+    if (err == cudaSuccess && seen) err = cudaMemsetAsync(dev.error, 0, sizeof(seen), stream);
+    if (err != cudaSuccess) {
+        cudaGetLastError();
+        return COMET_ERR_CUDA;
+    }
+    return seen ? COMET_ERR_TIMEOUT : COMET_OK;
+}
+
+extern "C" int comet_static_inject_timeout(void* cuda_stream) {
+    StaticDevice dev;
+    if (static_device(&dev) != cudaSuccess || cudaMemsetAsync(dev.error, 1, sizeof(int), (cudaStream_t)cuda_stream) != cudaSuccess) {
+        cudaGetLastError();
+        return COMET_ERR_CUDA;
+    }
+    return COMET_OK;
 }
 
 // ---------------------------------------------------------------------------

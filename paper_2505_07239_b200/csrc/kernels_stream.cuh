@@ -103,7 +103,7 @@ struct StreamArgs {
     const int32_t* row_label;   // component label per token (negative: the row is not opened), or null
     const int32_t* blk_label;   // likewise per active block (up: rows of the right operand, down: its columns), or null
     int* error_flag;
-    int* error_host;
+    int* error_host;         // or null
 };
 
 // Z_i <- C_i for both parties, so that the product kernel behind it can add partial sums.
@@ -597,9 +597,9 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
     __syncwarp();
     ptx::fence_before_sync();
     __syncthreads();
-    if (threadIdx.x == 0 && abort_flag && a.error_flag) {
+    if (threadIdx.x == 0 && abort_flag) {
         *a.error_flag = 1;
-        *reinterpret_cast<volatile int*>(a.error_host) = 1;
+        if (a.error_host) *reinterpret_cast<volatile int*>(a.error_host) = 1;
         __threadfence_system();
     }
     if (warp == MMA_WARP) {

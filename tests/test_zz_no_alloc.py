@@ -111,3 +111,23 @@ def test_static_scratch_limit_is_refused_cleanly():
     ok = (ctypes.c_void_p * 2)(small[0].data_ptr(), small[1].data_ptr())
     assert cb.library().comet_beaver_matmul_static(None, ok, ok, ok, ok, ok, ok, 8, 12, 4) == -2     # K % 8
     torch.cuda.synchronize()
+
+
+def test_static_product_reports_a_wait_that_ran_out():
+    """No wait runs out here: the word that a kernel would set is set by the host."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2505_07239_b200 import binding as cb
+
+    stream = torch.cuda.Stream()
+    T, K, N = 8, 16, 8
+    mk = lambda r, c: [torch.ones((r, c), dtype=torch.int64, device="cuda") for _ in (0, 1)]  # noqa: E731
+    ops = [mk(T, K), mk(T, K), mk(N, K), mk(N, K), mk(T, N), mk(T, N)]
+    torch.cuda.synchronize()
+    assert cb.static_status(stream) == cb.OK
+    assert cb.beaver_matmul_static(*ops, stream=stream) == cb.OK
+    assert cb.static_status(stream) == cb.OK
+    assert cb.library().comet_static_inject_timeout(stream.cuda_stream) == cb.OK
+    assert cb.beaver_matmul_static(*ops, stream=stream) == cb.OK        # a later call does not hide the report
+    assert cb.static_status(stream) == cb.ERR_TIMEOUT
+    assert cb.static_status(stream) == cb.OK                            # which is given once

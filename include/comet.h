@@ -171,7 +171,9 @@ int comet_load_shares(comet_ctx* ctx, int party, int tensor_id, const uint64_t* 
  * has completed on the stream (for a triple: the ffn call; for weights: as long as
  * they stay bound).  A later comet_load_shares or comet_bind_shares of the same
  * tensor replaces the binding; comet_set_mask drops the bindings of the triples
- * and of H like their loaded state.  Same shape rules and errors as
+ * and of H like their loaded state.  `dev_ptr` may lie in a result buffer of the
+ * library (comet_device_pointer), such as the result of the layer before: a call
+ * reads its operands there before it writes that buffer.  Same shape rules and errors as
  * comet_load_shares, plus INVALID_ARG for an unaligned pointer. */
 int comet_bind_shares(comet_ctx* ctx, int party, int tensor_id, const uint64_t* dev_ptr, int64_t rows, int64_t cols);
 

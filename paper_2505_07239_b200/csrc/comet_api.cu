@@ -240,6 +240,58 @@ Proj proj_down(const comet_ctx* c, int tokens) {
                 COMET_C_DN, COMET_Y, true};
 }
 
+// An input may be bound to memory of the library's own: a layer's X to the result of the one before it, say.  The kernels of the
+// tensor-core path write Z <- C in the launch that reads the operands, so an operand that lies on the result is moved to its own
+// buffer for the length of the call.
+struct OperandsOffResult {
+    comet_ctx* c;
+    const Proj& pr;
+    int ids[7], count = 0;
+    u64* bound[2][7];
+    OperandsOffResult(comet_ctx* ctx, const Proj& proj) : c(ctx), pr(proj) {
+        for (int id : {pr.idX, pr.idA, pr.idB, pr.idC}) ids[count++] = id;
+        if (pr.down) ids[count++] = COMET_W2;
+        else for (int id : {COMET_W1, COMET_WG, COMET_W3}) ids[count++] = id;
+        for (int p = 0; p < 2; ++p)
+            for (int k = 0; k < count; ++k) bound[p][k] = c->buf[p][ids[k]];
+    }
+    // Whether operand `id` of a party lies on a result buffer of either party; *bytes becomes its size.
+    bool on(int party, int id, int result, size_t* bytes) const {
+        if (c->buf[party][id] == c->own[party][id]) return false;
+        int64_t rows, cols;
+        tensor_shape(c, id, pr.M, &rows, &cols);
+        *bytes = (size_t)(rows * cols) * sizeof(u64);
+        const uintptr_t at = reinterpret_cast<uintptr_t>(c->buf[party][id]);
+        for (int q = 0; q < 2; ++q) {
+            const uintptr_t z = reinterpret_cast<uintptr_t>(c->own[q][result]);
+            if (at < z + (uintptr_t)c->cap_words[result] * sizeof(u64) && z < at + *bytes) return true;
+        }
+        return false;
+    }
+    bool any_on(int result) const {
+        size_t bytes;
+        for (int p = 0; p < 2; ++p)
+            for (int k = 0; k < count; ++k)
+                if (on(p, ids[k], result, &bytes)) return true;
+        return false;
+    }
+    int move() {
+        size_t bytes;
+        for (int p = 0; p < 2; ++p)
+            for (int k = 0; k < count; ++k) {
+                const int id = ids[k];
+                if (!on(p, id, pr.idZ, &bytes) || (id == pr.idC && c->buf[p][id] == c->own[p][pr.idZ])) continue;
+                COMET_CUDA(c, cudaMemcpyAsync(c->own[p][id], c->buf[p][id], bytes, cudaMemcpyDeviceToDevice, c->stream));
+                c->buf[p][id] = c->own[p][id];
+            }
+        return COMET_OK;
+    }
+    ~OperandsOffResult() {
+        for (int p = 0; p < 2; ++p)
+            for (int k = 0; k < count; ++k) c->buf[p][ids[k]] = bound[p][k];
+    }
+};
+
 // The streaming kernel (one kernel per product, operand roles exchanged) serves layers with at most 32 token rows: its planes
 // live in shared memory, so every further 32 rows convert the weights once more.  Up to 64 rows that still beats writing the
 // planes to memory and reading them back where the weights are many (without a token mask, whose components only the other
@@ -1003,6 +1055,9 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
         const Proj up = proj_up(c, tokens), dn = proj_down(c, tokens);
         int rc = join_side(c);
         if (rc != COMET_OK) return rc;
+        OperandsOffResult operands(c, up);
+        rc = operands.move();
+        if (rc != COMET_OK) return rc;
         if (few_tokens(c, tokens)) {
             rc = stream_product(c, up);
             return rc != COMET_OK ? rc : somm_merge(c, tokens);
@@ -1017,8 +1072,8 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
         // one launch and 34 apart, with 0.25 million 41 either way, with 0.52 million 97 and 94, with 1.7 million 249 and 237.
         const bool early = !c->dn_right_ready && limb_fits(c, dn) && c->loaded[0][COMET_W2] &&
                            c->loaded[1][COMET_W2] && c->loaded[0][COMET_B_DN] && c->loaded[1][COMET_B_DN];
-        const bool early_copy = early && c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN];
         const bool apart = early && (int64_t)dn.N * dn.K >= EXCHANGE_APART;
+        const bool early_copy = early && c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN] && (apart || !operands.any_on(COMET_Y));
         comet::LimbExchangeArgs also;
         const int also_blocks = early && !apart ? exchange_args(c, dn, false, true, early_copy, also) : 0;
         {
@@ -1103,9 +1158,12 @@ int comet_ffn_down(comet_ctx* c, int32_t tokens) {
     }
     if (c->path == COMET_PATH_LIMB) {
         const Proj dn = proj_down(c, tokens);
+        int rc = join_side(c);
+        if (rc != COMET_OK) return rc;
+        OperandsOffResult operands(c, dn);
+        rc = operands.move();
+        if (rc != COMET_OK) return rc;
         if (few_tokens(c, tokens)) {
-            const int rc = join_side(c);
-            if (rc != COMET_OK) return rc;
             c->dn_right_ready = false;
             c->dn_copy_ready = false;
             return stream_product(c, dn);
@@ -1114,8 +1172,6 @@ int comet_ffn_down(comet_ctx* c, int32_t tokens) {
         // opened early, during the up-projection
         const bool have_right = c->dn_right_ready;
         const bool have_copy = c->dn_right_ready && c->dn_copy_ready && c->dn_copy_tokens == tokens;
-        int rc = join_side(c);
-        if (rc != COMET_OK) return rc;
         {
             PhaseTimer timer(c, COMET_PHASE_OPEN, 1);
             rc = limb_exchange(c, dn, true, !have_right, !have_copy, c->stream);

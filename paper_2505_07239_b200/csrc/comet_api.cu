@@ -305,7 +305,7 @@ bool few_tokens(const comet_ctx* c, int tokens) {
 }
 
 // Tensor map of a result matrix for the tensor-core kernel's reductions (see LimbMaps).
-bool result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_rows, int box_cols, CUtensorMapSwizzle swizzle) {
+cudaError_t result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_rows, int box_cols, CUtensorMapSwizzle swizzle) {
     typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -321,9 +321,10 @@ bool result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_rows, int 
     }();
     const cuuint64_t size[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, pitch[1] = {(cuuint64_t)cols * sizeof(u64)};
     const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows}, step[2] = {1, 1};
-    return encode && encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, z, size, pitch, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                            swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    if (!encode) return cudaErrorSymbolNotFound;
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, z, size, pitch, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+               ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // The streaming kernel.  Without `sync` words (they belong to one stream's order, so a call without a context has none) Z <- C
@@ -345,8 +346,10 @@ int launch_stream(comet::StreamArgs& args, const comet::BlockIds& held, int sm_c
     args.cta_cost = steps > sm_count ? (unsigned)(cost / grid) : 0u;
     args.cta_extra = (unsigned)(cost % grid);
     comet::LimbMaps maps;
-    for (int p = 0; p < 2; ++p)
-        if (!result_map(&maps.z[p], args.Z[p], args.M, args.N, ls::OUT_TOKENS, 32, CU_TENSOR_MAP_SWIZZLE_NONE)) return COMET_ERR_CUDA;
+    for (int p = 0; p < 2; ++p) {
+        *err = result_map(&maps.z[p], args.Z[p], args.M, args.N, ls::OUT_TOKENS, 32, CU_TENSOR_MAP_SWIZZLE_NONE);
+        if (*err != cudaSuccess) return COMET_ERR_CUDA;
+    }
     if (!args.sync) {
         const long long pairs = (long long)args.M * args.N / 2, want = (pairs + 255) / 256, most = (long long)sm_count * 8;
         *err = launch_chained(comet::result_init_kernel, dim3((unsigned)(want < most ? want : most), 2), dim3(256), 0, stream,
@@ -396,10 +399,8 @@ int stream_product(comet_ctx* c, const Proj& pr) {
     {
         PhaseTimer timer(c, COMET_PHASE_COMBINE, 1);
         const int rc = launch_stream(a, c->held, c->sm_count, c->stream, &c->top_priority, &err);
-        if (rc != COMET_OK) {
-            c->last_cuda_error = (int)err;
-            return rc;
-        }
+        if (rc == COMET_ERR_CUDA) c->last_cuda_error = (int)err;
+        if (rc != COMET_OK) return rc;
     }
     c->stats.kernel_launches += 1;
     c->stats.tensor_tile_macs = 2ll * 2 * a.mt * a.nt * a.kb * ls::KC * ls::BW * ls::BT;
@@ -548,7 +549,7 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
         } else {
             comet::LimbMaps maps;
             for (int p = 0; p < 2; ++p)
-                if (!result_map(&maps.z[p], a.Z[p], a.M, a.N, 32, lb::OUT_COLS, CU_TENSOR_MAP_SWIZZLE_128B)) return COMET_ERR_CUDA;
+                COMET_CUDA(c, result_map(&maps.z[p], a.Z[p], a.M, a.N, 32, lb::OUT_COLS, CU_TENSOR_MAP_SWIZZLE_128B));
             COMET_CUDA(c, launch_chained(comet::combine_limb_kernel, dim3(grid), dim3(lb::THREADS), lb::SMEM_BYTES, c->stream,
                                          &c->top_priority, a, maps));
         }

@@ -678,9 +678,15 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
     bool ok = true;
     // Every buffer is a piece of one allocation (and of one pinned allocation): an allocation costs about as much whatever
     // its size, and this many of them one by one took 9 of the 11 ms in which a context came up.
-    std::vector<std::pair<void**, size_t>> device, pinned;
-    auto reserve = [](std::vector<std::pair<void**, size_t>>& list, auto** where, size_t bytes) {
-        list.emplace_back(reinterpret_cast<void**>(where), bytes);
+    constexpr int MAX_PIECES = 2 * COMET_NUM_TENSORS + 32;
+    struct Pieces {                     // fixed in size: nothing here may throw
+        void** where[MAX_PIECES];
+        size_t bytes[MAX_PIECES];
+        int count = 0;
+    } device, pinned;
+    auto reserve = [](Pieces& list, auto** where, size_t bytes) {
+        list.where[list.count] = reinterpret_cast<void**>(where);
+        list.bytes[list.count++] = bytes;
     };
     for (int id = 0; id < COMET_NUM_TENSORS; ++id) {
         c->cap_words[id] = tensor_capacity(c, id);
@@ -752,16 +758,16 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
     reserve(pinned, &c->h_count, 4 * sizeof(int32_t));
     reserve(pinned, &c->h_mask_stage, (size_t)nb * 4);
     constexpr size_t ALIGN = 256;
-    auto total = [](const std::vector<std::pair<void**, size_t>>& list) {
+    auto total = [](const Pieces& list) {
         size_t bytes = 0;
-        for (const auto& piece : list) bytes += (piece.second + ALIGN - 1) / ALIGN * ALIGN;
+        for (int k = 0; k < list.count; ++k) bytes += (list.bytes[k] + ALIGN - 1) / ALIGN * ALIGN;
         return bytes;
     };
-    auto hand_out = [](const std::vector<std::pair<void**, size_t>>& list, void* base) {
+    auto hand_out = [](const Pieces& list, void* base) {
         uint8_t* at = static_cast<uint8_t*>(base);
-        for (const auto& piece : list) {
-            *piece.first = at;
-            at += (piece.second + ALIGN - 1) / ALIGN * ALIGN;
+        for (int k = 0; k < list.count; ++k) {
+            *list.where[k] = at;
+            at += (list.bytes[k] + ALIGN - 1) / ALIGN * ALIGN;
         }
     };
     ok = ok && cudaMalloc(&c->device_memory, total(device)) == cudaSuccess;

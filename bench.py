@@ -919,7 +919,7 @@ def main():
         # per launch, both parties: planes of both operand pairs read once, Z read and written once (average of the
         # up- and the down-projection launch); with few tokens the kernel reads the operands' words and writes the
         # messages itself
-        stream = used_path == "limb" and T <= 32
+        stream = stats.product_kernel == cb.KERNEL_STREAM
         comb_bytes_per_launch = 8 * ((3 * T * d + 3 * d * g * n + 3 * T * g * n) + (3 * T * n + 3 * n * d + 3 * T * d)) \
             if stream else 8 * ((2 * T * d + 2 * d * g * n + 2 * T * g * n) + (2 * T * n + 2 * n * d + 2 * T * d))
         if used_path == "limb":

@@ -108,6 +108,14 @@ typedef struct {
     int32_t matmul_path;  /* COMET_PATH_*                                               */
 } comet_config;
 
+/* kernels of the product, for comet_stats */
+enum {
+    COMET_KERNEL_SIMT = 1,    /* CUDA cores                                                 */
+    COMET_KERNEL_STREAM = 2,  /* tensor cores, few token rows: reads words, writes messages */
+    COMET_KERNEL_LIMB = 3,    /* tensor cores on operand planes                             */
+    COMET_KERNEL_GROUPED = 4  /* the same over the components of a token mask               */
+};
+
 /* phases of the path, for the per-phase timers of comet_stats */
 enum {
     COMET_PHASE_COMPACT = 0,  /* mask compaction, where a kernel does it            */
@@ -134,7 +142,7 @@ typedef struct {
     double phase_ms[COMET_NUM_PHASES];
     int64_t phase_launches[COMET_NUM_PHASES];
     int32_t n_components;    /* connected components under the current token mask (0 without one) */
-    int32_t reserved;
+    int32_t product_kernel;  /* COMET_KERNEL_* of the last ffn call's product (0 before the first) */
     int64_t tensor_tile_macs; /* 64-bit multiply-adds the tensor-core kernel of the last ffn call covered, counted
                                  in whole output tiles (128 x 64, or 32 tokens x 128 in the kernel for few tokens) and
                                  32-deep steps, both parties (0 on the CUDA-core path): under a token mask with

@@ -22,6 +22,7 @@ from .build import LIB_PATH, build_library, is_current
 OK = 0
 DEVICE, HOST = 0, 1
 PATH_AUTO, PATH_SIMT, PATH_LIMB = 0, 1, 2
+KERNEL_SIMT, KERNEL_STREAM, KERNEL_LIMB, KERNEL_GROUPED = 1, 2, 3, 4
 
 (X, W1, WG, W2, A_UP, B_UP, C_UP, H, A_DN, B_DN, C_DN,
  E_UP, F_UP, Z_UP, E_DN, F_DN, Y, W3) = range(18)
@@ -52,7 +53,7 @@ class CometStats(ctypes.Structure):
                 ("n_active_blocks", ctypes.c_int32), ("tokens", ctypes.c_int32), ("matmul_path", ctypes.c_int32),
                 ("kernel_launches", ctypes.c_int64), ("phase_ms", ctypes.c_double * 5),
                 ("phase_launches", ctypes.c_int64 * 5), ("n_components", ctypes.c_int32),
-                ("reserved", ctypes.c_int32), ("tensor_tile_macs", ctypes.c_int64)]
+                ("product_kernel", ctypes.c_int32), ("tensor_tile_macs", ctypes.c_int64)]
 
 
 class CometError(RuntimeError):

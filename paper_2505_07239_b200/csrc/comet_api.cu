@@ -405,6 +405,7 @@ int stream_product(comet_ctx* c, const Proj& pr) {
     c->stats.kernel_launches += 1;
     c->stats.tensor_tile_macs = 2ll * 2 * a.mt * a.nt * a.kb * ls::KC * ls::BW * ls::BT;
     c->stats.matmul_path = COMET_PATH_LIMB;
+    c->stats.product_kernel = COMET_KERNEL_STREAM;
     return COMET_OK;
 }
 
@@ -556,6 +557,7 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
     }
     c->stats.kernel_launches += 1;
     c->stats.matmul_path = COMET_PATH_LIMB;
+    c->stats.product_kernel = c->grouped ? COMET_KERNEL_GROUPED : COMET_KERNEL_LIMB;
     COMET_CUDA(c, cudaGetLastError());
     return COMET_OK;
 }
@@ -588,6 +590,7 @@ int launch_combine(comet_ctx* c, int M, int N, int K, int idE, int idF, int idA,
     comet::combine_simt_kernel<<<grid, comet::simt::THREADS, 0, c->stream>>>(a);
     c->stats.kernel_launches += 1;
     c->stats.matmul_path = COMET_PATH_SIMT;
+    c->stats.product_kernel = COMET_KERNEL_SIMT;
     COMET_CUDA(c, cudaGetLastError());
     return COMET_OK;
 }

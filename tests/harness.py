@@ -264,6 +264,7 @@ def run_and_compare_products(cfg, seed, sparsity=None, tokens=None, step=0, matm
         load_triple_down(ctx, trd)
     ctx.ffn_up(T)
     report["path"] = ctx.stats().matmul_path
+    report["kernels"] = [ctx.stats().product_kernel]
     Zg = [ctx.get(party, cb.Z_UP, (T, g * n)) for party in (0, 1)]
     ctx.truncate(cb.Z_UP)
     ref = oracle.somm((X0, X1), (oracle_up_operand(cfg, W, 1), oracle_up_operand(cfg, W, 2)), Ig,
@@ -281,6 +282,7 @@ def run_and_compare_products(cfg, seed, sparsity=None, tokens=None, step=0, matm
     if not early_down:
         load_triple_down(ctx, trd)
     ctx.ffn_down(T)
+    report["kernels"].append(ctx.stats().product_kernel)
     Yg = [ctx.get(party, cb.Y, (T, d)) for party in (0, 1)]
     ctx.truncate(cb.Y)
     refd = oracle.simm((H0, H1), W["W2"][1:], I1, trd["A"][1:], trd["B"][1:], trd["C"][1:])

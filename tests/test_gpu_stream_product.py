@@ -59,18 +59,20 @@ def test_static_product_in_place(cb, T, K, N, on):
         assert np.array_equal(d[on][p].cpu().numpy().view(np.uint64), ref["Z"][p]), p
 
 
-@pytest.mark.parametrize("tokens,d_model,blocks,block,active,stacked", [
-    (1, 16, 4, 16, 1, 1),          # 16 features, half a step
-    (32, 144, 24, 16, 9, 1),       # 144 features both ways: 128 and a ragged tile of 16
-    (31, 112, 12, 48, 5, 2),       # strips of 48 columns: a step takes its halves from two blocks
-    (8, 272, 8, 80, 3, 3),         # three stacked matrices, group boundaries inside a feature tile
-    (33, 1008, 64, 16, 49, 1), (64, 1040, 60, 16, 40, 2),      # two token tiles, weights just many enough to be streamed ..
-    (49, 1008, 64, 16, 48, 1),                                 # .. and just too few
+@pytest.mark.parametrize("tokens,d_model,blocks,block,active,stacked,streamed", [
+    (1, 16, 4, 16, 1, 1, True),          # 16 features, half a step
+    (32, 144, 24, 16, 9, 1, True),       # 144 features both ways: 128 and a ragged tile of 16
+    (31, 112, 12, 48, 5, 2, True),       # strips of 48 columns: a step takes its halves from two blocks
+    (8, 272, 8, 80, 3, 3, True),         # three stacked matrices, group boundaries inside a feature tile
+    (33, 144, 24, 16, 9, 1, False),      # two token tiles, and few weights
+    (33, 1008, 64, 16, 49, 1, True), (64, 1040, 60, 16, 40, 2, True),      # weights just many enough to be streamed ..
+    (49, 1008, 64, 16, 48, 1, False), (65, 1040, 60, 16, 40, 2, False),    # .. and just too few; a row too many
 ])
-def test_few_token_layer_at_tile_edges(cb, tokens, d_model, blocks, block, active, stacked):
+def test_few_token_layer_at_tile_edges(cb, tokens, d_model, blocks, block, active, stacked, streamed):
     from tests import harness as hz
 
     cfg = wl.FFNConfig("stream-edges", tokens, d_model, blocks * block, block, 16, stacked == 2, active / blocks, "uniform",
                        "normal", "normal0.02", stacked=stacked)
     r = hz.run_and_compare_products(cfg, seed=700 + tokens)
     assert r["mismatches"] == 0 and r["path"] == 2 and r["n_active"] == active * block, r
+    assert r["kernels"] == [cb.KERNEL_STREAM if streamed else cb.KERNEL_LIMB] * 2

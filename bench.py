@@ -39,27 +39,25 @@ L2_FLUSH_BYTES = 512 << 20
 # kernels_limb.cuh.
 COMBINE_LIMB_TRAFFIC = {
     "workload": ("opt1.3b", 0.9),
-    "kernel_sha256": "0f2e1699f0109bf7b914f0fe698b6c08b30d5eb70620faf5cffb1cb7cfccd669",
-    "bytes_per_launch": 132884480,
+    "kernel_sha256": "a6c98318a7c2c6988d489b2089819d218b57b2d00f635e8417f5991ae45d2e63",
+    "bytes_per_launch": 81062016,
 }
 
 
-def combine_traffic(workload, sparsity, used_path):
-    """The stored ncu DRAM traffic of the dominant kernel, or None when it does not apply any more."""
+def combine_kernel_digest():
+    """SHA-256 of the source of combine_limb_kernel: from its argument block to the end of the file it closes."""
     import hashlib
 
-    if used_path != "limb" or (workload, round(sparsity, 4)) != COMBINE_LIMB_TRAFFIC["workload"]:
+    with open(os.path.join(ROOT, "paper_2505_07239_b200", "csrc", "kernels_limb.cuh")) as fh:
+        text = fh.read()
+    return hashlib.sha256(text[text.index("struct LimbArgs {"):].encode()).hexdigest()
+
+
+def combine_traffic(workload, sparsity, kernel):
+    """The stored ncu DRAM traffic of the dominant kernel, or None when it does not apply any more."""
+    if kernel != "combine_limb" or (workload, round(sparsity, 4)) != COMBINE_LIMB_TRAFFIC["workload"]:
         return None
-    src = os.path.join(ROOT, "paper_2505_07239_b200", "csrc", "kernels_limb.cuh")
-    try:
-        with open(src) as fh:
-            text = fh.read()
-        # the kernel proper: from its argument block to the banner of the next kernel in the file
-        text = text[text.index("struct LimbArgs {"):text.index("// Few tokens (M <= 32")]
-        digest = hashlib.sha256(text.encode()).hexdigest()
-    except (OSError, ValueError):
-        return None
-    return COMBINE_LIMB_TRAFFIC["bytes_per_launch"] if digest == COMBINE_LIMB_TRAFFIC["kernel_sha256"] else None
+    return COMBINE_LIMB_TRAFFIC["bytes_per_launch"] if combine_kernel_digest() == COMBINE_LIMB_TRAFFIC["kernel_sha256"] else None
 
 
 def ffn_macs(cfg, T, n):
@@ -916,12 +914,12 @@ def main():
         bf16 = peaks.get("bf16_tflops", 1590.0)
         src = "measured" if peaks else "fallback"
         achieved = comb_macs_per_launch / (comb_launch_ms * 1e-3) / 1e12
-        # per launch, both parties: planes of both operand pairs read once, Z read and written once (average of the
-        # up- and the down-projection launch); with few tokens the kernel reads the operands' words and writes the
-        # messages itself
+        # per launch, both parties: planes of V_i, B_i, and of E and F, which both parties share, read once, Z read and
+        # written once (average of the up- and the down-projection launch); with few tokens the kernel reads the
+        # operands' words and writes the messages itself
         stream = stats.product_kernel == cb.KERNEL_STREAM
         comb_bytes_per_launch = 8 * ((3 * T * d + 3 * d * g * n + 3 * T * g * n) + (3 * T * n + 3 * n * d + 3 * T * d)) \
-            if stream else 8 * ((2 * T * d + 2 * d * g * n + 2 * T * g * n) + (2 * T * n + 2 * n * d + 2 * T * d))
+            if stream else 4 * ((3 * T * d + 3 * d * g * n + 4 * T * g * n) + (3 * T * n + 3 * n * d + 4 * T * d))
         if used_path == "limb":
             # The pipe's peak in ring multiply-adds: the measured rate of the tensor instruction the kernel issues,
             # over 36 limb products.  Beside it, what the measured bf16 GEMM peak would imply at the nominal int8 :
@@ -962,7 +960,7 @@ def main():
                     "peak_from_unit_counts": derived}
         roof["frac"] = roof["achieved"] / roof["peak"]
         roof["kernel"] = "combine_stream" if stream else "combine_" + used_path
-        roof["traffic"] = combine_traffic(args.workload, sparsity, used_path)
+        roof["traffic"] = combine_traffic(args.workload, sparsity, roof["kernel"])
         roof["traffic_unit"] = "bytes per launch (ncu dram read+write); algorithmic: planes once + Z read-modify-write"
         roof["algorithmic_bytes_per_launch"] = comb_bytes_per_launch
         roof["timed"] = "kernel time per launch from the per-phase CUDA-event pass, one problem at a time"

@@ -42,3 +42,20 @@ def test_workload_name_states_the_shape():
     name = b.workload_name(wl.CONFIGS["opt1.3b"], 0.9)
     for piece in ("tokens=512", "d_model=2048", "d_ff=8192", "sparsity=0.90", "n_active=832"):
         assert piece in name
+
+
+def test_stored_traffic_is_keyed_by_the_kernel_source(monkeypatch):
+    b = _bench()
+    stored = b.COMBINE_LIMB_TRAFFIC
+    workload, sparsity = stored["workload"]
+    monkeypatch.setitem(stored, "kernel_sha256", b.combine_kernel_digest())       # the source is found
+    assert b.combine_traffic(workload, sparsity, "combine_limb") == stored["bytes_per_launch"]
+    assert b.combine_traffic(workload, sparsity, "combine_stream") is None
+    assert b.combine_traffic("tiny", sparsity, "combine_limb") is None
+    monkeypatch.setitem(stored, "kernel_sha256", "0" * 64)                        # another kernel than the profiled one
+    assert b.combine_traffic(workload, sparsity, "combine_limb") is None
+    # planes once and Z read and written once; writes still in L2 at the kernel's end are not in the count
+    cfg = wl.CONFIGS[workload]
+    n, T, d = cfg.n_active_blocks(sparsity) * cfg.block, cfg.tokens, cfg.d_model
+    once = 4 * ((3 * T * d + 3 * d * n + 4 * T * n) + (3 * T * n + 3 * n * d + 4 * T * d))
+    assert 0.9 * once < stored["bytes_per_launch"] < 1.5 * once

@@ -308,15 +308,16 @@ def run_shuffle(args, cfg):
         pass
     hbm = peaks.get("hbm_gbs", 6650.0)
     gbs = ranks.whole_job_throughput(bytes_step, world, args.steps, total_ms) / 1e9
+    launches = 1 if rows * cols <= 1 << 21 else 2          # as comet.h has it, for rows of more than two words
     print(json.dumps({
         "metric": "oblivious shuffle online stage, algorithmic GB/s", "value": gbs, "unit": "GB/s", "n_gpus": world,
         "steps": args.steps, "warmup": max(3, args.warmup), "ms_per_step": total_ms / args.steps,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "u64", "data": "synthetic",
         "config": {"workload": f"rows={rows} cols={cols} (activation matrix of {cfg.name}), both parties",
                    "l2": f"{sets} rotating input sets, {sets * 6 * 8 * rows * cols >> 20} MiB in total"},
-        "gpu_launches": 2 * args.steps, "clocks": clocks,
-        "roofline": {"bound": "hbm", "achieved": gbs / world, "peak": hbm, "unit": "GB/s",
-                     "frac": gbs / world / hbm, "traffic": None, "kernel": "shuffle_rows_kernel (2 launches per step)",
+        "gpu_launches": launches * args.steps, "clocks": clocks,
+        "roofline": {"bound": "hbm", "achieved": gbs / world, "peak": hbm, "unit": "GB/s", "frac": gbs / world / hbm,
+                     "traffic": None, "kernel": "shuffle_both_kernel" if launches == 1 else "shuffle_rows_kernel (2 launches per step)",
                      "peak_source": "measured" if peaks else "fallback"}}))
 
 
@@ -959,7 +960,9 @@ def main():
                     "peak_sustained": peak_sustained, "frac_of_sustained_peak": achieved / peak_sustained,
                     "peak_from_unit_counts": derived}
         roof["frac"] = roof["achieved"] / roof["peak"]
-        roof["kernel"] = "combine_stream" if stream else "combine_" + used_path
+        # grouped: the multiply-adds are still counted over the union of the masks, of which it computes a part
+        roof["kernel"] = ("combine_stream" if stream else "combine_limb_grouped" if stats.product_kernel == cb.KERNEL_GROUPED
+                          else "combine_" + used_path)
         roof["traffic"] = combine_traffic(args.workload, sparsity, roof["kernel"])
         roof["traffic_unit"] = "bytes per launch (ncu dram read+write); algorithmic: planes once + Z read-modify-write"
         roof["algorithmic_bytes_per_launch"] = comb_bytes_per_launch

@@ -29,11 +29,17 @@
  *     it allocated at comet_init; nothing of the caller's is kept (the one
  *     exception is comet_bind_shares, which reads the caller's device memory in
  *     place).
- *   - All work is enqueued on the CUDA stream given to comet_init.  Calls are
- *     asynchronous with respect to the host except comet_set_mask with a DEVICE
- *     mask and comet_set_token_mask (they return public counts computed on the
- *     device), comet_get/comet_load_shares with host pointers to pageable
- *     memory, comet_synchronize, comet_stats and comet_destroy.
+ *   - All work is enqueued on the CUDA stream given to comet_init (and on an
+ *     internal one that is joined to it).  Calls are asynchronous with respect to
+ *     the host except comet_set_mask with a DEVICE mask and comet_set_token_mask
+ *     (they return public counts computed on the device), comet_get /
+ *     comet_load_shares with host pointers to pageable memory, comet_synchronize,
+ *     comet_stats and comet_destroy.
+ *   - The asynchronous calls of a step may be captured in a CUDA graph that is
+ *     replayed any number of times, other steps in between: what the kernels count
+ *     advances on the device.  The graph keeps the mask it was captured with (a
+ *     HOST mask of at most 3584 blocks) and reads and writes the buffers that were
+ *     bound then.
  */
 #ifndef COMET_H_
 #define COMET_H_
@@ -190,11 +196,12 @@ int comet_bind_shares(comet_ctx* ctx, int party, int tensor_id, const uint64_t* 
  * = active) into the ascending list of active blocks, i.e. the index set I.
  * `n_blocks` must equal d_ff / block.  Returns the number of active NEURONS in
  * *n_active_out (the sparsity level is public in the threat model of Section
- * 3.2).  With a HOST mask the library counts the active blocks itself, copies
- * the bytes out of a pinned slot of its own (the caller's buffer may be reused
- * at once) and returns without waiting for the device; with a DEVICE mask the
- * count comes back from the compaction kernel through mapped host memory,
- * which the call waits for.  Zero active blocks is legal.  Invalidates
+ * 3.2).  With a HOST mask the library counts the active blocks itself, takes the
+ * bytes over (the caller's buffer may be reused at once: what is needed of them
+ * travels with the launches, or, for masks of more than 3584 blocks, from a pinned
+ * slot of the library's own) and returns without waiting for the device; with a
+ * DEVICE mask the count comes back from the compaction kernel through mapped host
+ * memory, which the call waits for.  Zero active blocks is legal.  Invalidates
  * previously loaded triples and H.  Errors: INVALID_ARG, SHAPE (n_blocks; more
  * active neurons than max_active), CUDA, TIMEOUT (an earlier kernel of the
  * context gave up on a bounded wait). */
@@ -220,8 +227,8 @@ int comet_ffn_up(comet_ctx* ctx, int32_t tokens);
  * token.  One call sets it for both projections.
  *
  * Up-projection, Protocol 2: the connected components of the bipartite graph
- * (tokens) x (active blocks) are found on the GPU (minimum-label propagation
- * instead of the paper's depth-first search; the partition is the same), each
+ * (tokens) x (active blocks) are found on the GPU (a union-find forest instead of
+ * the paper's depth-first search; the partition is the same), each
  * token row and each weight column is opened once (rows / blocks without any
  * edge not at all: their message words are zero), and comet_ffn_up leaves in
  * COMET_Z_UP the result blocks of the components, with every entry whose token
@@ -257,8 +264,9 @@ int comet_ffn_up(comet_ctx* ctx, int32_t tokens);
  * components only; otherwise the product runs over [tokens, n].
  * comet_stats.ring_macs is Theorem 2's count either way, tensor_tile_macs what
  * the tiles cover.  *masked_out (may be NULL) receives the number of non-zero
- * entries (neurons, summed over tokens); one kernel, one report of seven words
- * through mapped host memory and a stream synchronise.  Errors: STATE (no block mask yet), SHAPE
+ * entries (neurons, summed over tokens); one kernel, whose report of seven words
+ * in mapped host memory the call watches for (and waits for the stream if it does
+ * not come within 0.3 ms).  Errors: STATE (no block mask yet), SHAPE
  * (tokens out of range, n_active_blocks not the current count), INVALID_ARG. */
 int comet_set_token_mask(comet_ctx* ctx, const uint8_t* token_mask, int location, int32_t tokens,
                          int32_t n_active_blocks, int64_t* masked_out);
@@ -473,17 +481,18 @@ int comet_beaver_mul(void* cuda_stream, const uint64_t* const X[2], const uint64
  * capture.
  *
  * The product runs on the tensor cores in the same kernel as a context's products
- * of at most 32 tokens.  Its device-side waits are bounded like theirs (about two
+ * of few tokens.  Its device-side waits are bounded like theirs (about two
  * seconds, which no working launch comes near): after one that ran out Z lacks
  * part of its sums, and comet_static_status says so.  With K = 8, N <= 64 and more
  * than about 14000 rows, and when Z lies on the memory of an operand other than
  * its own C, the product runs on the CUDA cores, which wait for nothing.
  *
- * The array is shared by every call in the process and is never cleared:
- * a call overwrites all of the part it uses before reading it, so stale
- * contents are harmless, but two calls whose work overlaps in time on the same
- * GPU (different streams, or different host threads) race on it.  Serialise
- * them, e.g. by using one stream.
+ * The array is shared by every call in the process and is never cleared: the
+ * tensor-core kernel only writes the messages there, the CUDA-core kernels read
+ * them back after writing all of the part they use, so stale contents are
+ * harmless, but two calls whose work overlaps in time on the same GPU (different
+ * streams, or different host threads) race on it.  Serialise them, e.g. by using
+ * one stream.
  */
 #define COMET_STATIC_SCRATCH_WORDS (1u << 20)
 int comet_beaver_matmul_static(void* cuda_stream, const uint64_t* const X[2], const uint64_t* const A[2],

@@ -190,7 +190,7 @@ __device__ __forceinline__ bool stream_tile_ready(const uint32_t* flag, uint32_t
 }
 
 // COLS = 16 for up to 16 tokens, else 32: the width of the token planes and of the accumulators.  With half the columns the MMAs
-// take half the time, which the conversion of a step otherwise waits for: llama7b decode (7 tokens) 202 -> 189 us.  (As a
+// take half the time, which the conversion of a step otherwise waits for: llama7b decode (7 tokens) 202 -> 188 us.  (As a
 // value of the launch instead of a template's it cost the 32-token layer 2 %.)
 template <int COLS>
 __global__ void __launch_bounds__(limb_stream::THREADS, 1)

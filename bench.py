@@ -43,18 +43,28 @@ COMBINE_LIMB_TRAFFIC = {
     "bytes_per_launch": 81062016,
 }
 
+# The same for the kernel on residues, which the default workload runs through, and all of kernels_residue.cuh.
+COMBINE_RESIDUE_TRAFFIC = {
+    "workload": ("opt1.3b", 0.9),
+    "kernel_sha256": "ea35b4538a48c5bb9bf5597c4aedd419779732fe568c3e0c1e397f90328114d1",
+    "bytes_per_launch": 140239616,
+}
 
-def combine_kernel_digest():
-    """SHA-256 of the source of combine_limb_kernel: from its argument block to the end of the file it closes."""
+
+def combine_kernel_digest(source="kernels_limb.cuh", first="struct LimbArgs {"):
+    """SHA-256 of the source of a combine kernel: from its argument block to the end of the file."""
     import hashlib
 
-    with open(os.path.join(ROOT, "paper_2505_07239_b200", "csrc", "kernels_limb.cuh")) as fh:
+    with open(os.path.join(ROOT, "paper_2505_07239_b200", "csrc", source)) as fh:
         text = fh.read()
-    return hashlib.sha256(text[text.index("struct LimbArgs {"):].encode()).hexdigest()
+    return hashlib.sha256(text[text.index(first):].encode()).hexdigest()
 
 
 def combine_traffic(workload, sparsity, kernel):
     """The stored ncu DRAM traffic of the dominant kernel, or None when it does not apply any more."""
+    if kernel == "combine_residue" and (workload, round(sparsity, 4)) == COMBINE_RESIDUE_TRAFFIC["workload"]:
+        digest = combine_kernel_digest("kernels_residue.cuh", "namespace residue {")
+        return COMBINE_RESIDUE_TRAFFIC["bytes_per_launch"] if digest == COMBINE_RESIDUE_TRAFFIC["kernel_sha256"] else None
     if kernel != "combine_limb" or (workload, round(sparsity, 4)) != COMBINE_LIMB_TRAFFIC["workload"]:
         return None
     return COMBINE_LIMB_TRAFFIC["bytes_per_launch"] if combine_kernel_digest() == COMBINE_LIMB_TRAFFIC["kernel_sha256"] else None
@@ -903,8 +913,8 @@ def main():
         ms_per_step, value = chosen["median"]["ms_per_step"], chosen["median"]["value"]
         phase = {name: {"ms_per_step": stats.phase_ms[k] / prof_steps, "launches_per_step":
                         stats.phase_launches[k] / prof_steps} for k, name in enumerate(cb.PHASE_NAMES)}
-        comb_launch_ms = stats.phase_ms[3] / max(1, stats.phase_launches[3])
-        comb_macs_per_launch = macs / 2          # up and down combine launches carry half the MACs each here
+        comb_launch_ms = stats.phase_ms[3] / (2 * prof_steps)      # of a product, whatever kernels it takes
+        comb_macs_per_launch = macs / 2          # up and down products carry half the MACs each here
         used_path = {cb.PATH_SIMT: "simt", cb.PATH_LIMB: "limb"}.get(stats.matmul_path, "?")
         peaks = {}
         try:
@@ -921,22 +931,27 @@ def main():
         stream = stats.product_kernel == cb.KERNEL_STREAM
         comb_bytes_per_launch = 8 * ((3 * T * d + 3 * d * g * n + 3 * T * g * n) + (3 * T * n + 3 * n * d + 3 * T * d)) \
             if stream else 4 * ((3 * T * d + 3 * d * g * n + 4 * T * g * n) + (3 * T * n + 3 * n * d + 4 * T * d))
+        residue = stats.product_kernel == cb.KERNEL_RESIDUE
+        if residue:                              # 17 byte planes in place of 8, and 18 residues a result word out
+            comb_bytes_per_launch = (51 * (T * d + d * g * n + T * n + n * d) + 2 * 18 * (T * g * n + T * d)) // 2
         if used_path == "limb":
             # The pipe's peak in ring multiply-adds: the measured rate of the tensor instruction the kernel issues,
-            # over 36 limb products.  Beside it, what the measured bf16 GEMM peak would imply at the nominal int8 :
-            # bf16 ratio of 2 (the figure used before the pipe itself was measured).
-            derived = bf16 * 1e12 / 2 * 2 / 36 / 1e12
+            # over its byte products per ring product (36 limb products, 18 through residues).  Beside it, what the
+            # measured bf16 GEMM peak would imply at the nominal int8 : bf16 ratio of 2.
+            products = 18 if residue else 36
+            name = "byte products through residues" if residue else "limb products"
+            derived = bf16 * 1e12 / 2 * 2 / products / 1e12
             if pipe_peaks is not None:
-                peak = pipe_peaks["tensor_i8"]["ring_mac_burst"] / 1e12
-                peak_sustained = pipe_peaks["tensor_i8"]["ring_mac_sustained"] / 1e12
+                peak = pipe_peaks["tensor_i8"]["ring_mac_burst"] * 36 / products / 1e12
+                peak_sustained = pipe_peaks["tensor_i8"]["ring_mac_sustained"] * 36 / products / 1e12
                 peak_source = ("measured in this run: tcgen05.mma kind::i8 M128 N256 K32 loop on 148 SMs, operands in "
-                               "shared memory, best of the first three 25 ms launches, / 36 limb products")
+                               f"shared memory, best of the first three 25 ms launches, / {products} {name}")
             else:
-                peak, peak_sustained = derived, bf16_sustained_derived(peaks)
-                peak_source = f"{src} bf16 GEMM peak x2 (int8 nominal ratio), as MAC/s, / 36 limb products"
+                peak, peak_sustained = derived, bf16_sustained_derived(peaks) * 36 / products
+                peak_source = f"{src} bf16 GEMM peak x2 (int8 nominal ratio), as MAC/s, / {products} {name}"
             t_tensor = comb_macs_per_launch / (peak * 1e12)
             t_hbm = comb_bytes_per_launch / (hbm * 1e9)
-            if t_hbm > t_tensor:
+            if t_hbm > t_tensor and stream:
                 # few tokens: the kernel streams the weight side's words once and is bound by that traffic
                 roof = {"bound": "hbm", "achieved": comb_bytes_per_launch / (comb_launch_ms * 1e-3) / 1e9, "peak": hbm,
                         "unit": "GB/s", "peak_source": f"{src} HBM copy peak"}
@@ -961,7 +976,7 @@ def main():
                     "peak_from_unit_counts": derived}
         roof["frac"] = roof["achieved"] / roof["peak"]
         # grouped: the multiply-adds are still counted over the union of the masks, of which it computes a part
-        roof["kernel"] = ("combine_stream" if stream else "combine_limb_grouped" if stats.product_kernel == cb.KERNEL_GROUPED
+        roof["kernel"] = ("combine_stream" if stream else "combine_residue" if residue else "combine_limb_grouped" if stats.product_kernel == cb.KERNEL_GROUPED
                           else "combine_" + used_path)
         roof["traffic"] = combine_traffic(args.workload, sparsity, roof["kernel"])
         roof["traffic_unit"] = "bytes per launch (ncu dram read+write); algorithmic: planes once + Z read-modify-write"

@@ -22,7 +22,7 @@ from .build import LIB_PATH, build_library, is_current
 OK = 0
 DEVICE, HOST = 0, 1
 PATH_AUTO, PATH_SIMT, PATH_LIMB = 0, 1, 2
-KERNEL_SIMT, KERNEL_STREAM, KERNEL_LIMB, KERNEL_GROUPED = 1, 2, 3, 4
+KERNEL_SIMT, KERNEL_STREAM, KERNEL_LIMB, KERNEL_GROUPED, KERNEL_RESIDUE = 1, 2, 3, 4, 5
 
 (X, W1, WG, W2, A_UP, B_UP, C_UP, H, A_DN, B_DN, C_DN,
  E_UP, F_UP, Z_UP, E_DN, F_DN, Y, W3) = range(18)

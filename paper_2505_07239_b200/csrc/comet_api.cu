@@ -19,6 +19,7 @@
 #include "kernels_mul.cuh"
 #include "kernels_open.cuh"
 #include "kernels_peak.cuh"
+#include "kernels_residue.cuh"
 #include "kernels_shuffle.cuh"
 #include "kernels_simt.cuh"
 #include "kernels_stream.cuh"
@@ -37,12 +38,17 @@ struct comet_ctx {
     void* pinned_memory;
     int64_t cap_words[COMET_NUM_TENSORS];
     bool loaded[2][COMET_NUM_TENSORS];
-    // limb path: blocked limb planes (left: V_i per party and E; right: B_i per party and F), and the device error flag
+    // limb path: operand planes, of limbs or of residues (left: V_i per party and E; right: B_i per party and F), and the device
+    // error flag
     int path;                     // COMET_PATH_SIMT or COMET_PATH_LIMB
-    uint8_t* planes_left[3];          // V_0, V_1, E; shared by the two projections
-    uint8_t* planes_right_up[3];      // B_0, B_1, F of the up-projection
-    uint8_t* planes_right_dn[3];      // B'_0, B'_1, F' of the down-projection
-    size_t planes_left_bytes, planes_right_up_bytes, planes_right_dn_bytes;
+    struct Planes {
+        uint8_t* at;              // three sets, one behind the other
+        size_t bytes;             // room
+    };
+    Planes planes_left;           // V_0, V_1, E; shared by the two projections
+    Planes planes_right_up;       // B_0, B_1, F of the up-projection
+    Planes planes_right_dn;       // B'_0, B'_1, F' of the down-projection
+    Planes residues;              // of one product: what the kernel on residues hands to the recombination
     int* d_error;                     // = d_count + 1
     // the weight side of the down-projection is opened on a second stream while the up-projection's
     // tensor-core kernel runs (it only needs the mask, W2 and B'_i)
@@ -50,6 +56,7 @@ struct comet_ctx {
     cudaEvent_t ev_fork, ev_join;
     bool side_pending;                // ev_join not yet waited for on the main stream
     bool dn_right_ready;              // F'_i and the right planes of the down-projection are current
+    bool dn_right_residue;            // ... and they are planes of residues
     bool dn_copy_ready;               // Y_i already holds C'_i (copied beside the up-projection)
     int32_t dn_copy_tokens;           // ... for this many token rows
     uint8_t* d_mask;
@@ -304,8 +311,8 @@ bool few_tokens(const comet_ctx* c, int tokens) {
     return tokens <= STREAM_TOKENS && !c->tmask_set && (int64_t)(c->groups + 1) * c->cfg.d_model * c->n_active >= STREAM_WORDS;
 }
 
-// Tensor map of a result matrix for the tensor-core kernel's reductions (see LimbMaps).
-cudaError_t result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_rows, int box_cols, CUtensorMapSwizzle swizzle) {
+cudaError_t tensor_map(CUtensorMap* map, CUtensorMapDataType type, int rank, void* base, const cuuint64_t* size, const cuuint64_t* pitch,
+                       const cuuint32_t* box, const cuuint32_t* step, CUtensorMapSwizzle swizzle) {
     typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -319,12 +326,17 @@ cudaError_t result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_row
         }
         return reinterpret_cast<Encode>(fn);
     }();
-    const cuuint64_t size[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, pitch[1] = {(cuuint64_t)cols * sizeof(u64)};
-    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows}, step[2] = {1, 1};
     if (!encode) return cudaErrorSymbolNotFound;
-    return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, z, size, pitch, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+    return encode(map, type, (cuuint32_t)rank, base, size, pitch, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
                ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// Tensor map of a result matrix for the tensor-core kernel's reductions (see LimbMaps).
+cudaError_t result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_rows, int box_cols, CUtensorMapSwizzle swizzle) {
+    const cuuint64_t size[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, pitch[1] = {(cuuint64_t)cols * sizeof(u64)};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows}, step[2] = {1, 1};
+    return tensor_map(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, z, size, pitch, box, step, swizzle);
 }
 
 // The streaming kernel.  Without `sync` words (they belong to one stream's order, so a call without a context has none) Z <- C
@@ -431,27 +443,38 @@ int join_side(comet_ctx* c) {
     return COMET_OK;
 }
 
+// Bytes of one set of operand planes: of limbs (tiles of `tile` rows), of residues.
+size_t limb_set(int rows, int K, int tile) {
+    return (size_t)ceil_div(rows, tile) * ceil_div(K, comet::limb::KC) * tile * comet::limb::KC * comet::limb::PLANES;
+}
+size_t residue_set(int rows, int K) {
+    return (size_t)ceil_div(rows, 8) * ceil_div(K, comet::residue::KC) * comet::residue::CELL_BYTES;
+}
+
 // Arguments of the exchange kernel for the left and / or right side of one product, and / or Z <- C.  Returns its CTAs.
-int exchange_args(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy, comet::LimbExchangeArgs& a) {
+int exchange_args(comet_ctx* c, const Proj& pr, bool residue, bool left, bool right, bool copy, comet::LimbExchangeArgs& a) {
     namespace lb = comet::limb;
     std::memset(&a, 0, sizeof(a));
-    uint8_t** planes = pr.down ? c->planes_right_dn : c->planes_right_up;
+    uint8_t* const lpl = c->planes_left.at;
+    uint8_t* const rpl = (pr.down ? c->planes_right_dn : c->planes_right_up).at;
+    const size_t lset = residue ? residue_set(pr.M, pr.K) : limb_set(pr.M, pr.K, lb::BM);
+    const size_t rset = residue ? residue_set(pr.N, pr.K) : limb_set(pr.N, pr.K, lb::BN);
     for (int p = 0; p < 2; ++p) {
         a.X[p] = c->buf[p][pr.idX];
         a.A[p] = c->buf[p][pr.idA];
         a.E[p] = c->buf[p][pr.idE];
-        a.Vpl[p] = c->planes_left[p];
+        a.Vpl[p] = lpl + p * lset;
         a.W0[p] = pr.down ? c->buf[p][COMET_W2] : (c->groups >= 2 ? c->buf[p][COMET_WG] : c->buf[p][COMET_W1]);
         a.W1[p] = c->buf[p][COMET_W1];
         a.W2[p] = c->buf[p][COMET_W3];
         a.B[p] = c->buf[p][pr.idB];
         a.F[p] = c->buf[p][pr.idF];
-        a.Bpl[p] = planes[p];
+        a.Bpl[p] = rpl + p * rset;
         a.C[p] = c->buf[p][pr.idC];
         a.Z[p] = c->buf[p][pr.idZ];
     }
-    a.Epl = c->planes_left[2];
-    a.Fpl = planes[2];
+    a.Epl = lpl + 2 * lset;
+    a.Fpl = rpl + 2 * rset;
     a.ids = c->ids_held ? nullptr : c->d_ids;
     a.n = c->n_active;
     a.bs = c->cfg.block;
@@ -474,7 +497,7 @@ int exchange_args(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy
     // enough CTAs to fill the device once, else as many k-blocks per CTA as spread the row set-up
     const long long fill = (long long)c->sm_count * 7;
     const long long per = (long long)(left_rows + right_rows) * a.kblocks / fill;
-    a.kb_per_cta = (int)(per < 1 ? 1 : per > lb::EX_MAX_KB_PER_CTA ? lb::EX_MAX_KB_PER_CTA : per);
+    a.kb_per_cta = residue ? comet::residue::EX_KB_PER_CTA : (int)(per < 1 ? 1 : per > lb::EX_MAX_KB_PER_CTA ? lb::EX_MAX_KB_PER_CTA : per);
     a.kchunks = ceil_div(a.kblocks, a.kb_per_cta);
     a.left_blocks = left_rows * a.kchunks;
     a.right_blocks = right_rows * a.kchunks;
@@ -485,14 +508,14 @@ int exchange_args(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy
 
 // Tensor-core path: messages, exchange and operand planes of one product, in one launch; `also`, if given, are the arguments
 // of a second product's for the same launch.
-int limb_exchange(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy, cudaStream_t stream,
+int limb_exchange(comet_ctx* c, const Proj& pr, bool residue, bool left, bool right, bool copy, cudaStream_t stream,
                   const comet::LimbExchangeArgs* also = nullptr, int also_blocks = 0) {
     namespace lb = comet::limb;
     comet::LimbExchangeArgs a;
-    const int blocks = exchange_args(c, pr, left, right, copy, a);
+    const int blocks = exchange_args(c, pr, residue, left, right, copy, a);
     if (blocks + also_blocks == 0) return COMET_OK;
     const bool tiles = left || right || also_blocks;
-    COMET_CUDA(c, launch_chained(comet::limb_exchange_kernel, dim3(blocks + also_blocks), dim3(lb::EX_THREADS),
+    COMET_CUDA(c, launch_chained(residue ? comet::limb_exchange_kernel<true> : comet::limb_exchange_kernel<false>, dim3(blocks + also_blocks), dim3(lb::EX_THREADS),
                                  tiles ? lb::EX_SMEM_BYTES : 0, stream, nullptr, a, also ? *also : a, blocks, c->held));
     c->stats.kernel_launches += 1;
     COMET_CUDA(c, cudaGetLastError());
@@ -503,15 +526,17 @@ int limb_exchange(comet_ctx* c, const Proj& pr, bool left, bool right, bool copy
 int limb_combine(comet_ctx* c, const Proj& pr) {
     namespace lb = comet::limb;
     const int kb = ceil_div(pr.K, lb::KC), mt = ceil_div(pr.M, lb::BM), nt = ceil_div(pr.N, lb::BN);
-    uint8_t** planes = pr.down ? c->planes_right_dn : c->planes_right_up;
+    uint8_t* const lpl = c->planes_left.at;
+    uint8_t* const rpl = (pr.down ? c->planes_right_dn : c->planes_right_up).at;
+    const size_t lset = limb_set(pr.M, pr.K, lb::BM), rset = limb_set(pr.N, pr.K, lb::BN);
     comet::LimbArgs a;
     for (int p = 0; p < 2; ++p) {
-        a.Vpl[p] = c->planes_left[p];
-        a.Bpl[p] = planes[p];
+        a.Vpl[p] = lpl + p * lset;
+        a.Bpl[p] = rpl + p * rset;
         a.Z[p] = c->buf[p][pr.idZ];
     }
-    a.Epl = c->planes_left[2];
-    a.Fpl = planes[2];
+    a.Epl = lpl + 2 * lset;
+    a.Fpl = rpl + 2 * rset;
     a.M = pr.M; a.N = pr.N; a.mt = mt; a.nt = nt; a.kb = kb;
     a.error_flag = c->d_error;
     a.error_host = c->h_count_dev + 3;
@@ -566,9 +591,109 @@ constexpr int64_t EXCHANGE_APART = 1 << 18;    // words of the down-projection's
 
 bool limb_fits(const comet_ctx* c, const Proj& pr) {
     namespace lb = comet::limb;
-    const size_t kb = ceil_div(pr.K, lb::KC), mt = ceil_div(pr.M, lb::BM), nt = ceil_div(pr.N, lb::BN);
-    return mt * kb * lb::A_BLOCK_BYTES <= c->planes_left_bytes &&
-           nt * kb * lb::B_BLOCK_BYTES <= (pr.down ? c->planes_right_dn_bytes : c->planes_right_up_bytes);
+    return 3 * limb_set(pr.M, pr.K, lb::BM) <= c->planes_left.bytes &&
+           3 * limb_set(pr.N, pr.K, lb::BN) <= (pr.down ? c->planes_right_dn : c->planes_right_up).bytes;
+}
+
+// Tiles of the kernel on residues for a product: which side of it the MMAs' 256 rows take, and how many of the other side their
+// columns.  The jobs (JOBS per tile, all alike) are dealt to the CTA pairs in rounds.  A block of 64 takes the four MMAs'
+// 2 * n_tile cycles, or 380 to issue them and to fetch its operands; a job 2000 more to fill and to drain.
+struct ResidueTiles {
+    int swapped, n_tile, mt, nt;
+    int64_t cycles;
+};
+ResidueTiles residue_tiles(int sm_count, int M, int N, int K) {
+    namespace rs = comet::residue;
+    ResidueTiles best{};
+    const int64_t blocks = 2 * ceil_div(K, rs::KC), pairs = sm_count / 2;
+    for (int swapped = 0; swapped < 2; ++swapped)
+        for (int n_tile = rs::MAX_BN; n_tile >= 32; n_tile -= 32) {
+            const int mt = ceil_div(swapped ? N : M, rs::BM), nt = ceil_div(swapped ? M : N, n_tile);
+            const int64_t rounds = ((int64_t)rs::JOBS * mt * nt + pairs - 1) / pairs;
+            const int64_t cycles = rounds * (blocks * (n_tile > 190 ? 2 * n_tile : 380) + 2000);
+            if (best.n_tile == 0 || cycles < best.cycles) best = ResidueTiles{swapped, n_tile, mt, nt, cycles};
+        }
+    return best;
+}
+size_t residue_bytes(int rows, int cols) {       // of one party, whichever side is the M side
+    return (size_t)comet::residue::JOBS * (ceil_div(rows, 32) * 32) * (size_t)(ceil_div(cols, 32) * 32);
+}
+
+// Whether a product is quicker through residues than through limbs.
+// Either way's time in ns, exchange included, is a constant, a share per step of a CTA, per operand word and per result word,
+// fitted to 121 products of 65 to 512 rows, 256 to 4096 columns and depths (both within 28 %, the small ones the furthest off;
+// where the two times lie more than 5 % apart, which is what is asked for here, the rule picked the quicker one every time):
+// 512 x 256 x 256 19 us through limbs, 31 through residues; 512 x 1024 x 1024 67 and 65; 512 x 2048 x 2048 235 and 197;
+// 512 x 4096 x 4096 966 and 726; 256 x 4096 x 4096 546 and 516; 128 x 4096 x 4096 376 and 452.
+bool residues_pay(int sm_count, int M, int N, int K) {
+    namespace lb = comet::limb;
+    const int64_t operands = (int64_t)(M + N) * K, results = (int64_t)M * N;
+    const int64_t steps = 4ll * ceil_div(M, lb::BM) * ceil_div(N, lb::BN) * ceil_div(K, lb::KC) / sm_count;
+    const int64_t limbs = 8900 + steps * 825 + (operands * 86 + results * 50) / 10000;
+    const int64_t residues = 16300 + residue_tiles(sm_count, M, N, K).cycles * 344 / 1000 + (operands * 202 + results * 169) / 10000;
+    return residues * 21 < limbs * 20;
+}
+
+// Whether this product goes through residues.
+bool through_residues(const comet_ctx* c, const Proj& pr) {
+    return c->residues.bytes && !c->grouped && pr.K <= comet::residue::MAX_DEPTH &&
+           3 * residue_set(pr.M, pr.K) <= c->planes_left.bytes && 2 * residue_bytes(pr.M, pr.N) <= c->residues.bytes &&
+           3 * residue_set(pr.N, pr.K) <= (pr.down ? c->planes_right_dn : c->planes_right_up).bytes &&
+           residues_pay(c->sm_count, pr.M, pr.N, pr.K);
+}
+
+// Tensor map of one side's residue planes (ResidueMaps), in boxes of `rows` rows.
+cudaError_t residue_map(CUtensorMap* map, uint8_t* planes, int operand_rows, int K, int rows) {
+    namespace rs = comet::residue;
+    const cuuint64_t groups = ceil_div(operand_rows, 8), blocks = ceil_div(K, rs::KC);
+    const cuuint64_t size[5] = {rs::GROUP_BYTES / 4, rs::PLANES, groups, blocks, 3};
+    const cuuint64_t pitch[4] = {rs::GROUP_BYTES, rs::CELL_BYTES, groups * rs::CELL_BYTES, blocks * groups * rs::CELL_BYTES};
+    const cuuint32_t box[5] = {rs::GROUP_BYTES / 4, 1, (cuuint32_t)rows / 8, rs::STAGE_BLOCKS, 1}, step[5] = {1, 1, 1, 1, 1};
+    return tensor_map(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 5, planes, size, pitch, box, step, CU_TENSOR_MAP_SWIZZLE_NONE);
+}
+
+// Tensor-core path: both parties' product through residues, from the planes to Z.
+int residue_combine(comet_ctx* c, const Proj& pr) {
+    namespace rs = comet::residue;
+    const ResidueTiles t = residue_tiles(c->sm_count, pr.M, pr.N, pr.K);
+    comet::ResidueArgs a;
+    comet::RecombineArgs r;
+    const int m_rows = t.swapped ? pr.N : pr.M, n_rows = t.swapped ? pr.M : pr.N;
+    for (int p = 0; p < 2; ++p) {
+        r.T[p] = a.T[p] = c->residues.at + p * residue_bytes(pr.M, pr.N);
+        r.C[p] = c->buf[p][pr.idC];
+        r.Z[p] = c->buf[p][pr.idZ];
+    }
+    r.rows = pr.M; r.cols = pr.N;
+    r.m_groups = a.m_groups = ceil_div(m_rows, 32);
+    r.n_chunks = a.n_chunks = ceil_div(n_rows, 16);
+    a.swapped = t.swapped;
+    a.mt = t.mt; a.nt = t.nt; a.n_tile = t.n_tile;
+    a.k32 = ceil_div(pr.K, 32);
+    a.jobs = rs::JOBS * t.mt * t.nt;
+    a.error_flag = c->d_error;
+    a.error_host = c->h_count_dev + 3;
+    uint8_t* const left = c->planes_left.at;
+    uint8_t* const right = (pr.down ? c->planes_right_dn : c->planes_right_up).at;
+    comet::ResidueMaps maps;
+    COMET_CUDA(c, residue_map(&maps.m_side, t.swapped ? right : left, m_rows, pr.K, rs::BM / 2));
+    COMET_CUDA(c, residue_map(&maps.n_side, t.swapped ? left : right, n_rows, pr.K, t.n_tile / 2));
+    // no more pairs than the rounds need: what is left serves the kernels beside this one
+    const int most = c->sm_count / 2, pairs = ceil_div(a.jobs, ceil_div(a.jobs, most));
+    {
+        PhaseTimer timer(c, COMET_PHASE_COMBINE, 2);
+        COMET_CUDA(c, launch_chained(comet::combine_residue_kernel, dim3(2 * pairs), dim3(rs::THREADS), rs::SMEM_BYTES, c->stream,
+                                     &c->top_priority, a, maps));
+        COMET_CUDA(c, launch_chained(t.swapped ? comet::residue_recombine_kernel<true> : comet::residue_recombine_kernel<false>,
+                                     dim3(ew_grid(c, (int64_t)a.m_groups * a.n_chunks * 128, 256), 2), dim3(256), 0, c->stream,
+                                     nullptr, r));
+    }
+    c->stats.kernel_launches += 2;
+    c->stats.tensor_tile_macs = 2ll * 2 * t.mt * rs::BM * t.nt * t.n_tile * a.k32 * 32;
+    c->stats.matmul_path = COMET_PATH_LIMB;
+    c->stats.product_kernel = COMET_KERNEL_RESIDUE;
+    COMET_CUDA(c, cudaGetLastError());
+    return COMET_OK;
 }
 
 int launch_combine(comet_ctx* c, int M, int N, int K, int idE, int idF, int idA, int idB, int idC, int idZ) {
@@ -697,21 +822,30 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
             if (c->cap_words[id] > 0) reserve(device, &c->own[p][id], (size_t)c->cap_words[id] * sizeof(u64));
     }
     c->path = cfg->matmul_path == COMET_PATH_AUTO ? COMET_PATH_LIMB : cfg->matmul_path;
+    int planes_piece = 0, planes_pieces = 0;
+    size_t planes_of_limbs[3];
     if (c->path == COMET_PATH_LIMB) {
         namespace lb = comet::limb;
         const int d = cfg->d_model;
         const int64_t n = c->cap_n, gn = c->groups * n;
-        const int64_t kb_up = (d + lb::KC - 1) / lb::KC, kb_dn = (n + lb::KC - 1) / lb::KC;
-        const int64_t kb_max = kb_up > kb_dn ? kb_up : kb_dn;
-        const int64_t mt = (c->cap_T + lb::BM - 1) / lb::BM;
-        c->planes_left_bytes = (size_t)(mt * kb_max) * lb::A_BLOCK_BYTES;
-        c->planes_right_up_bytes = (size_t)(((gn + lb::BN - 1) / lb::BN) * kb_up) * lb::B_BLOCK_BYTES;
-        c->planes_right_dn_bytes = (size_t)(((d + lb::BN - 1) / lb::BN) * kb_dn) * lb::B_BLOCK_BYTES;
+        const int T = (int)c->cap_T, deepest = d > n ? d : (int)n;
         // a context for few tokens only never builds planes in memory
-        for (int w = 0; w < 3 && c->cap_T > comet::limb_stream::BT; ++w) {
-            reserve(device, &c->planes_left[w], c->planes_left_bytes);
-            reserve(device, &c->planes_right_up[w], c->planes_right_up_bytes);
-            reserve(device, &c->planes_right_dn[w], c->planes_right_dn_bytes);
+        planes_piece = device.count;
+        if (T > comet::limb_stream::BT) {
+            // room for planes of residues where a product of the full size would go through them
+            const int up_depth = std::min(d, comet::residue::MAX_DEPTH), dn_depth = std::min((int)n, comet::residue::MAX_DEPTH);
+            const bool up = residues_pay(c->sm_count, T, (int)gn, up_depth), dn = residues_pay(c->sm_count, T, d, dn_depth);
+            auto planes = [&](comet_ctx::Planes& p, size_t limbs, size_t residues) {
+                p.bytes = 3 * std::max(limbs, residues);
+                planes_of_limbs[planes_pieces++] = 3 * limbs;
+                reserve(device, &p.at, p.bytes);
+            };
+            planes(c->planes_left, limb_set(T, deepest, lb::BM),
+                   std::max(up ? residue_set(T, up_depth) : 0, dn ? residue_set(T, dn_depth) : 0));
+            planes(c->planes_right_up, limb_set((int)gn, d, lb::BN), up ? residue_set((int)gn, up_depth) : 0);
+            planes(c->planes_right_dn, limb_set(d, (int)n, lb::BN), dn ? residue_set(d, dn_depth) : 0);
+            c->residues.bytes = 2 * std::max(up ? residue_bytes(T, (int)gn) : 0, dn ? residue_bytes(T, d) : 0);
+            reserve(device, &c->residues.at, c->residues.bytes);
         }
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)lb::SMEM_BYTES) == cudaSuccess;
@@ -727,10 +861,14 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_grouped_kernel,
                                         cudaFuncAttributePreferredSharedMemoryCarveout,
                                         (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(comet::limb_exchange_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                        (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
-        ok = ok && cudaFuncSetAttribute(comet::limb_exchange_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)lb::EX_SMEM_BYTES) == cudaSuccess;
+        ok = ok && cudaFuncSetAttribute(comet::combine_residue_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)comet::residue::SMEM_BYTES) == cudaSuccess;
+        for (auto* kernel : {comet::limb_exchange_kernel<false>, comet::limb_exchange_kernel<true>}) {
+            ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                            (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+            ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)lb::EX_SMEM_BYTES) == cudaSuccess;
+        }
         ok = ok && cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) == cudaSuccess;
@@ -773,7 +911,20 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
             at += (list.bytes[k] + ALIGN - 1) / ALIGN * ALIGN;
         }
     };
-    ok = ok && cudaMalloc(&c->device_memory, total(device)) == cudaSuccess;
+    if (ok && cudaMalloc(&c->device_memory, total(device)) != cudaSuccess) {
+        // Planes of residues take twice the room of planes of limbs: without them, then.
+        ok = planes_pieces > 0;
+        if (ok) {
+            cudaGetLastError();
+            for (int k = 0; k < planes_pieces; ++k) device.bytes[planes_piece + k] = planes_of_limbs[k];
+            device.bytes[planes_piece + planes_pieces] = 0;
+            c->planes_left.bytes = planes_of_limbs[0];
+            c->planes_right_up.bytes = planes_of_limbs[1];
+            c->planes_right_dn.bytes = planes_of_limbs[2];
+            c->residues.bytes = 0;
+            ok = cudaMalloc(&c->device_memory, total(device)) == cudaSuccess;
+        }
+    }
     ok = ok && cudaHostAlloc(&c->pinned_memory, total(pinned), cudaHostAllocMapped) == cudaSuccess;
     if (ok) {
         hand_out(device, c->device_memory);
@@ -1073,6 +1224,7 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
             return rc != COMET_OK ? rc : somm_merge(c, tokens);
         }
         if (!limb_fits(c, up)) return COMET_ERR_SHAPE;
+        const bool residue = through_residues(c, up), dn_residue = through_residues(c, dn);
         // The weight side of the down-projection depends only on the mask, W2 and B'_i: if those are loaded already, it is
         // opened now, and if the triple's C' share is there too, Y_i <- C'_i, the value the down-projection's sums are added
         // to, is copied with it.  Where: a small one in the same launch as this product's exchange, which costs nothing but
@@ -1080,29 +1232,32 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
         // exchange before it, which is bound by the same memory), which hides about half of it but takes two events, a
         // launch and the programmatic start of the tensor-core kernel.  A step with 0.03 million such words takes 25 us in
         // one launch and 34 apart, with 0.25 million 41 either way, with 0.52 million 97 and 94, with 1.7 million 249 and 237.
+        // A launch writes planes of one kind, so a weight side of the other kind goes apart whatever its size.  The kernel on
+        // residues reads C' when it makes Y: nothing is copied for it.
         const bool early = !c->dn_right_ready && limb_fits(c, dn) && c->loaded[0][COMET_W2] &&
                            c->loaded[1][COMET_W2] && c->loaded[0][COMET_B_DN] && c->loaded[1][COMET_B_DN];
-        const bool apart = early && (int64_t)dn.N * dn.K >= EXCHANGE_APART;
-        const bool early_copy = early && c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN] && (apart || !operands.any_on(COMET_Y));
+        const bool apart = early && (residue != dn_residue || (int64_t)dn.N * dn.K >= EXCHANGE_APART);
+        const bool early_copy = early && !dn_residue && c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN] && (apart || !operands.any_on(COMET_Y));
         comet::LimbExchangeArgs also;
-        const int also_blocks = early && !apart ? exchange_args(c, dn, false, true, early_copy, also) : 0;
+        const int also_blocks = early && !apart ? exchange_args(c, dn, dn_residue, false, true, early_copy, also) : 0;
         {
             PhaseTimer timer(c, COMET_PHASE_OPEN, 1);
-            rc = limb_exchange(c, up, true, true, true, c->stream, also_blocks ? &also : nullptr, also_blocks);
+            rc = limb_exchange(c, up, residue, true, true, !residue, c->stream, also_blocks ? &also : nullptr, also_blocks);
         }
         if (rc != COMET_OK) return rc;
         if (apart) COMET_CUDA(c, cudaEventRecord(c->ev_fork, c->stream));
-        rc = limb_combine(c, up);
+        rc = residue ? residue_combine(c, up) : limb_combine(c, up);
         if (rc != COMET_OK) return rc;
         if (apart) {
             COMET_CUDA(c, cudaStreamWaitEvent(c->side, c->ev_fork, 0));
-            rc = limb_exchange(c, dn, false, true, early_copy, c->side);
+            rc = limb_exchange(c, dn, dn_residue, false, true, early_copy, c->side);
             if (rc != COMET_OK) return rc;
             COMET_CUDA(c, cudaEventRecord(c->ev_join, c->side));
             c->side_pending = true;
         }
         if (early) {
             c->dn_right_ready = true;
+            c->dn_right_residue = dn_residue;
             c->dn_copy_ready = early_copy;
             c->dn_copy_tokens = tokens;
         }
@@ -1180,16 +1335,17 @@ int comet_ffn_down(comet_ctx* c, int32_t tokens) {
         }
         if (!limb_fits(c, dn)) return COMET_ERR_SHAPE;
         // opened early, during the up-projection
-        const bool have_right = c->dn_right_ready;
-        const bool have_copy = c->dn_right_ready && c->dn_copy_ready && c->dn_copy_tokens == tokens;
+        const bool residue = through_residues(c, dn);
+        const bool have_right = c->dn_right_ready && c->dn_right_residue == residue;
+        const bool have_copy = residue || (c->dn_right_ready && c->dn_copy_ready && c->dn_copy_tokens == tokens);
         {
             PhaseTimer timer(c, COMET_PHASE_OPEN, 1);
-            rc = limb_exchange(c, dn, true, !have_right, !have_copy, c->stream);
+            rc = limb_exchange(c, dn, residue, true, !have_right, !have_copy, c->stream);
         }
         if (rc != COMET_OK) return rc;
         c->dn_right_ready = false;                     // a triple serves one product
         c->dn_copy_ready = false;
-        return limb_combine(c, dn);
+        return residue ? residue_combine(c, dn) : limb_combine(c, dn);
     }
 
     comet::PartyPtrs H, A, W, B;

@@ -25,10 +25,9 @@
 #include <cuda_runtime.h>
 
 #include "pdl.cuh"
+#include "residue_planes.cuh"
 
 namespace comet {
-
-typedef unsigned long long u64;
 
 namespace limb {
 constexpr int BM = 128, BN = 64, KC = 32, PLANES = 8;
@@ -105,6 +104,8 @@ __device__ __forceinline__ void limb_copy_wait() { asm volatile("cp.async.wait_g
 // L1 that the tensor-core kernels' carve-out leaves, 37 and 271 us with all of it; 33 and 258 us this way.)
 // It replaces an opening kernel and a preparation kernel that read the messages back and built every plane of E and F
 // twice: 112 bytes per word of both parties, now 72.
+// With RESIDUE the planes are those of combine_residue_kernel: 17 instead of 8, 99 bytes per word of both parties; [512 | 832,
+// 2048] 45 us in the step, [512 | 8192, 2048] 281, 5.9 TB/s (about 1000 instructions a warp and k-block, a third of its time).
 // grid = left_blocks + right_blocks + copy_blocks; a left / right block owns 16 rows x kb_per_cta k-blocks.
 // ---------------------------------------------------------------------------
 struct LimbExchangeArgs {
@@ -166,7 +167,7 @@ held_ids_kernel(const __grid_constant__ BlockIds held, int count, int32_t* __res
     if ((int)threadIdx.x < count) out[threadIdx.x] = held.id[threadIdx.x];
 }
 
-template <bool LEFT>
+template <bool LEFT, bool RESIDUE>
 __device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, const BlockIds& held, int block, uint8_t* smem) {
     using namespace limb;
     constexpr int TILE = LEFT ? BM : BN, BLOCK_BYTES = PLANES * TILE * KC;
@@ -201,8 +202,11 @@ __device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, co
     const u64* own[2];                           // the row of A_i / B_i
     u64* msg[2];                                 // the row of E_i / F_i
     uint8_t* pl[3];                              // this lane's cell in the planes of V_0 / B_0, V_1 / B_1, E / F
-    const size_t cell = ((size_t)(r / TILE) * a.kblocks + kb0) * BLOCK_BYTES +
-                        (size_t)((r % TILE >> 3) * 256 + (c >> 2) * 128 + (r & 7) * 16 + (c & 3) * 4);
+    // (residue planes: blocks of 64, all rows of a block together; see ResidueMaps)
+    const size_t next_block = (size_t)(((LEFT ? a.M : a.N) + 7) / 8) * residue::CELL_BYTES;
+    const size_t cell = (RESIDUE ? (size_t)(kb0 >> 1) * next_block + (size_t)(r >> 3) * residue::CELL_BYTES + (kb0 & 1) * 256
+                                 : ((size_t)(r / TILE) * a.kblocks + kb0) * BLOCK_BYTES + (size_t)(r % TILE >> 3) * 256) +
+                        (size_t)((c >> 2) * 128 + (r & 7) * 16 + (c & 3) * 4);
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
         own[p] = (LEFT ? a.A[p] : a.B[p]) + (size_t)at * a.K;
@@ -279,19 +283,27 @@ __device__ __forceinline__ void limb_exchange_rows(const LimbExchangeArgs& a, co
             f[0][e] += f[1][e];                  // the exchange
             if (LEFT) b[1][e] += f[0][e];        // V_1 = A_1 + E  (V_0 = A_0)
         }
-        limb_emit4(pl[0], TILE * KC, b[0]);
-        limb_emit4(pl[1], TILE * KC, b[1]);
-        limb_emit4(pl[2], TILE * KC, f[0]);
+        if (RESIDUE) {
+            residue_emit4<!LEFT>(pl[0], b[0]);
+            residue_emit4<!LEFT>(pl[1], b[1]);
+            residue_emit4<!LEFT>(pl[2], f[0]);
+        } else {
+            limb_emit4(pl[0], TILE * KC, b[0]);
+            limb_emit4(pl[1], TILE * KC, b[1]);
+            limb_emit4(pl[2], TILE * KC, f[0]);
+        }
+        const size_t step = !RESIDUE ? BLOCK_BYTES : (kb & 1) ? next_block - 256 : 256;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) pl[i] += BLOCK_BYTES;
+        for (int i = 0; i < 3; ++i) pl[i] += step;
     }
     limb_copy_wait<0>();
 }
 
+template <bool RESIDUE>
 __device__ __forceinline__ void limb_exchange_block(const LimbExchangeArgs& a, const BlockIds& held, int block, uint8_t* smem) {
-    if (block < a.left_blocks) return limb_exchange_rows<true>(a, held, block, smem);
+    if (block < a.left_blocks) return limb_exchange_rows<true, RESIDUE>(a, held, block, smem);
     block -= a.left_blocks;
-    if (block < a.right_blocks) return limb_exchange_rows<false>(a, held, block, smem);
+    if (block < a.right_blocks) return limb_exchange_rows<false, RESIDUE>(a, held, block, smem);
     block -= a.right_blocks;
     const int party = block & 1;
     const ulonglong2* __restrict__ s = reinterpret_cast<const ulonglong2*>(party ? a.C[1] : a.C[0]);
@@ -310,6 +322,7 @@ __device__ __forceinline__ void limb_exchange_block(const LimbExchangeArgs& a, c
 }
 
 // The first `first_blocks` CTAs work on `a`, the others on `b` (another product's operands).
+template <bool RESIDUE>
 __global__ void __launch_bounds__(limb::EX_THREADS, 7)
 limb_exchange_kernel(const __grid_constant__ LimbExchangeArgs a, const __grid_constant__ LimbExchangeArgs b, int first_blocks,
                      const __grid_constant__ BlockIds held) {
@@ -317,8 +330,8 @@ limb_exchange_kernel(const __grid_constant__ LimbExchangeArgs a, const __grid_co
     pdl_wait();
     pdl_launch_dependents();
     const int block = blockIdx.x;
-    if (block < first_blocks) limb_exchange_block(a, held, block, ex_smem);
-    else limb_exchange_block(b, held, block - first_blocks, ex_smem);
+    if (block < first_blocks) limb_exchange_block<RESIDUE>(a, held, block, ex_smem);
+    else limb_exchange_block<RESIDUE>(b, held, block - first_blocks, ex_smem);
 }
 
 // ---------------------------------------------------------------------------

@@ -1,0 +1,99 @@
+"""The product through residues (large layers) at the edges of its tiles: 256 rows on one side, a multiple of 32 on the other,
+stages of 128 contraction indices in instructions of 32; and at the largest sums it may have to tell apart."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2505_07239_b200 import workloads as wl  # noqa: E402
+
+U64 = np.uint64
+
+
+@pytest.fixture(scope="module")
+def cb():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2505_07239_b200 import binding
+
+    return binding
+
+
+@pytest.mark.parametrize("tokens,d_model,blocks,block,active,stacked,residues", [
+    (385, 1040, 80, 16, 63, 1, True),        # a row in the second token tile; depth 1040 = 8 stages and half an instruction;
+                                             # columns of the weights' product on the 256-row side
+    (257, 3088, 20, 48, 17, 1, True),        # strips of 48 columns; 816 of 1024 rows of the weights' tiles
+    (400, 1552, 60, 16, 51, 1, True),        # 816 = 3 column tiles of 224 and a ragged one
+    (449, 1040, 40, 32, 33, 2, True),        # two stacked matrices; the group boundary lies inside a tile
+    (512, 1024, 40, 16, 32, 1, False),       # a layer just too small for it
+])
+def test_layer_at_tile_edges(cb, tokens, d_model, blocks, block, active, stacked, residues):
+    from tests import harness as hz
+
+    cfg = wl.FFNConfig("residue-edges", tokens, d_model, blocks * block, block, 16, stacked == 2, active / blocks, "uniform",
+                       "normal", "normal0.02", stacked=stacked)
+    r = hz.run_and_compare_products(cfg, seed=800 + tokens, early_down=tokens != 400)
+    assert r["mismatches"] == 0 and r["n_active"] == active * block, r
+    assert (r["kernels"][0] == cb.KERNEL_RESIDUE) == residues, r["kernels"]
+
+
+def test_token_mask_of_one_component(cb):
+    """Entries off the support under a token mask, against the CUDA-core path."""
+    T, d, block, nab = 400, 1552, 16, 51
+    n = block * nab
+    mask = np.ones(nab, np.uint8)
+    rng = np.random.default_rng(5)
+    tmask = (rng.random((T, nab)) < 0.5).astype(np.uint8)
+    tmask[:, 7] = 1                          # one block that every token uses: one component
+    gen = torch.Generator(device="cuda").manual_seed(6)
+
+    def pair(*shape):
+        return [torch.randint(-(1 << 63), (1 << 63) - 1, shape, dtype=torch.int64, device="cuda", generator=gen) for _ in (0, 1)]
+
+    shares = {cb.X: pair(T, d), cb.W1: pair(n, d), cb.W2: pair(d, n), cb.A_UP: pair(T, d), cb.B_UP: pair(n, d), cb.C_UP: pair(T, n),
+              cb.H: pair(T, n), cb.A_DN: pair(T, n), cb.B_DN: pair(d, n), cb.C_DN: pair(T, d)}
+    got = {}
+    for path in (cb.PATH_LIMB, cb.PATH_SIMT):
+        ctx = cb.Comet(T, d, n, block, 16, 0, 0, n, path)
+        ctx.set_mask(mask)
+        ctx.set_token_mask(tmask)
+        for tid, s in shares.items():
+            for p in (0, 1):
+                ctx.load_shares(p, tid, s[p])
+        ctx.ffn_up(T)
+        kernels = [ctx.stats().product_kernel]
+        ctx.ffn_down(T)
+        kernels.append(ctx.stats().product_kernel)
+        assert kernels == [cb.KERNEL_RESIDUE if path == cb.PATH_LIMB else cb.KERNEL_SIMT] * 2
+        got[path] = [ctx.get(p, tid, s) for tid, s in ((cb.E_UP, (T, d)), (cb.Z_UP, (T, n)), (cb.E_DN, (T, n)), (cb.Y, (T, d)))
+                     for p in (0, 1)]
+        ctx.close()
+    for a, b in zip(got[cb.PATH_LIMB], got[cb.PATH_SIMT]):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("depth,residues", [(11424, True), (11440, False)])
+def test_largest_sums(cb, depth, residues):
+    """Every operand word of a row / column the same, so that Z_i = C_i + 2 * depth * e * f: words whose signed low 56 bits are
+    the smallest and the largest there are put the sum at the bounds that the residues have to tell apart, up to the largest
+    depth that goes through them."""
+    words = np.array([0x0080000000000000, 0x007FFFFFFFFFFFFF, 0xFF80000000000000, 0x7F7FFFFFFFFFFFFF, 0xFFFFFFFFFFFFFFFF,
+                      0x8000000000000000, 1, 0x8080808080808080, 0x00FF00FF00FF00FF, 0], dtype=U64)
+    T, d = 512, 1024
+    e, f = words[np.arange(T) * len(words) // T], words[np.arange(d) % len(words)]
+    E, F = np.repeat(e[:, None], depth, 1), np.repeat(f[:, None], depth, 1)
+    C = [wl.random_u64(9, f"largest/C{p}", T * d).reshape(T, d) for p in (0, 1)]
+    ctx = cb.Comet(T, d, depth, 16, 16, 0, 0, depth)
+    for p, (h, a, w, b) in enumerate(((E + E, E, F + F, F), (E * U64(0), E * U64(0), F, F))):
+        ctx.load_shares(p, cb.W2, cb.to_device(w))
+        if p == 0:
+            assert ctx.set_mask(np.ones(depth // 16, np.uint8)) == depth
+        for tid, s in ((cb.H, h), (cb.A_DN, a), (cb.B_DN, b), (cb.C_DN, C[p])):
+            ctx.load_shares(p, tid, cb.to_device(s))
+    ctx.ffn_down(T)
+    assert (ctx.stats().product_kernel == cb.KERNEL_RESIDUE) == residues
+    want = U64(2 * depth) * (e[:, None] * f[None, :])
+    for p in (0, 1):
+        assert np.array_equal(ctx.get(p, cb.Y, (T, d)), C[p] + want), p
+    ctx.close()

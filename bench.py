@@ -46,7 +46,7 @@ COMBINE_LIMB_TRAFFIC = {
 # The same for the kernel on residues, which the default workload runs through, and all of kernels_residue.cuh.
 COMBINE_RESIDUE_TRAFFIC = {
     "workload": ("opt1.3b", 0.9),
-    "kernel_sha256": "ea35b4538a48c5bb9bf5597c4aedd419779732fe568c3e0c1e397f90328114d1",
+    "kernel_sha256": "9958ddbdf2193db01a44ff0c7f5b323b7a16753d4a15688ab54cd1aad195ce41",
     "bytes_per_launch": 140239616,
 }
 

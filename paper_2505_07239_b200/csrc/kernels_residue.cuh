@@ -289,6 +289,9 @@ combine_residue_kernel(const __grid_constant__ ResidueArgs a, const __grid_const
                 while (clock64() - t0 < 20000000ll) {}
             }
         }
+        // The main loop is over: the recombination may be brought in beside the last drain, and no sooner, because its waiting
+        // CTAs take the registers that an exchange beside this kernel needs (the lanes that were not elected wait here).
+        __syncwarp();
         pdl_launch_dependents();
     } else {
         // ---------------- epilogue: TMEM -> residues -> memory ----------------

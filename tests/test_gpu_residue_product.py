@@ -97,3 +97,16 @@ def test_largest_sums(cb, depth, residues):
     for p in (0, 1):
         assert np.array_equal(ctx.get(p, cb.Y, (T, d)), C[p] + want), p
     ctx.close()
+
+
+def test_captured_and_replayed(cb):
+    from tests.test_gpu_capture import test_layer_captured_and_replayed as replayed
+
+    replayed(cb, 385, 1040, 80, 16, 63)
+
+
+@pytest.mark.parametrize("x_on", ["Y", "Z_UP"])
+def test_operands_on_result_buffers(cb, x_on):
+    from tests.test_gpu_bound_results import test_operands_on_result_buffers as bound
+
+    bound(385, 1040, x_on)

@@ -276,11 +276,13 @@ struct OperandsOffResult {
         return false;
     }
     bool any_on(int result) const {
-        size_t bytes;
-        for (int p = 0; p < 2; ++p)
-            for (int k = 0; k < count; ++k)
-                if (on(p, ids[k], result, &bytes)) return true;
+        for (int k = 0; k < count; ++k)
+            if (on(ids[k], result)) return true;
         return false;
+    }
+    bool on(int id, int result) const {
+        size_t bytes;
+        return on(0, id, result, &bytes) || on(1, id, result, &bytes);
     }
     int move() {
         size_t bytes;
@@ -1234,10 +1236,14 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
         // one launch and 34 apart, with 0.25 million 41 either way, with 0.52 million 97 and 94, with 1.7 million 249 and 237.
         // A launch writes planes of one kind, so a weight side of the other kind goes apart whatever its size.  The kernel on
         // residues reads C' when it makes Y: nothing is copied for it.
+        // An operand of this product may lie on Y: C' is then not copied there before it has been read.  The exchange reads
+        // all operands, so a copy that waits for it (on the side stream) is safe, one in the same launch is not; C is read
+        // after the product where that goes through residues, and a copy beside the product would be too early for it.
         const bool early = !c->dn_right_ready && limb_fits(c, dn) && c->loaded[0][COMET_W2] &&
                            c->loaded[1][COMET_W2] && c->loaded[0][COMET_B_DN] && c->loaded[1][COMET_B_DN];
         const bool apart = early && (residue != dn_residue || (int64_t)dn.N * dn.K >= EXCHANGE_APART);
-        const bool early_copy = early && !dn_residue && c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN] && (apart || !operands.any_on(COMET_Y));
+        const bool y_in_use = !apart ? operands.any_on(COMET_Y) : residue && operands.on(up.idC, COMET_Y);
+        const bool early_copy = early && !dn_residue && !y_in_use && c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN];
         comet::LimbExchangeArgs also;
         const int also_blocks = early && !apart ? exchange_args(c, dn, dn_residue, false, true, early_copy, also) : 0;
         {

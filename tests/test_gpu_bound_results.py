@@ -69,3 +69,50 @@ def test_operands_on_result_buffers(tokens, d, x_on):
             assert np.array_equal(ctx.get(p, cb.E_DN, (T, n)), down["E"][p])
             assert np.array_equal(ctx.get(p, cb.Y, (T, d)), down["Z"][p])
     ctx.close()
+
+
+@pytest.mark.parametrize("on_y", ["C_UP", "X"])
+def test_operand_on_y_while_c_may_be_copied_there(on_y):
+    """The up-projection through residues, which reads its C share after the product, and the down-projection through limbs,
+    whose C' is copied into Y beside the up-projection when it is loaded by then."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2505_07239_b200 import binding as cb
+
+    T, d, block, blocks, g = 385, 2064, 16, 36, 2
+    D, n = blocks * block, 30 * block
+    mask = np.ones(blocks, np.uint8)
+    mask[3::6] = 0
+    index, index_up = oracle.index_set(mask, block, 1), oracle.index_set(mask, block, g)
+    shapes = {cb.X: (T, d), cb.W1: (D, d), cb.WG: (D, d), cb.W2: (d, D), cb.A_UP: (T, d), cb.B_UP: (g * n, d), cb.C_UP: (T, g * n),
+              cb.H: (T, n), cb.A_DN: (T, n), cb.B_DN: (d, n), cb.C_DN: (T, d)}
+    v = {k: [wl.random_u64(71, f"on_y/{k}/{p}", s[0] * s[1]).reshape(s) for p in (0, 1)] for k, s in shapes.items()}
+    dev = {k: [cb.to_device(w) for w in pair] for k, pair in v.items()}
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx = cb.Comet(T, d, D, block, 16, g - 1, max_active=n, stream=stream)
+    assert ctx.set_mask(mask) == n
+    on = {"C_UP": cb.C_UP, "X": cb.X}[on_y]
+    for k, pair in dev.items():
+        for p in (0, 1):
+            share = pair[p]
+            if k == on:
+                share = ctx.result_view(p, cb.Y, shapes[k])
+                with torch.cuda.stream(stream):
+                    share.copy_(pair[p])
+            ctx.bind_shares(p, k, share)
+    t = lambda pair: [np.ascontiguousarray(m.T) for m in pair]  # noqa: E731  (stored output-feature-major)
+    ctx.ffn_up(T)
+    assert ctx.stats().product_kernel == cb.KERNEL_RESIDUE
+    W = [np.concatenate([v[cb.WG][p], v[cb.W1][p]]) for p in (0, 1)]
+    up = oracle.somm(v[cb.X], t(W), index_up, v[cb.A_UP], t(v[cb.B_UP]), v[cb.C_UP])
+    for p in (0, 1):
+        assert np.array_equal(ctx.get(p, cb.E_UP, (T, d)), up["E"][p])
+        assert np.array_equal(ctx.get(p, cb.Z_UP, (T, g * n)), up["Z"][p])
+    ctx.ffn_down(T)
+    assert ctx.stats().product_kernel == cb.KERNEL_LIMB
+    down = oracle.simm(v[cb.H], t(v[cb.W2]), index, v[cb.A_DN], t(v[cb.B_DN]), v[cb.C_DN])
+    for p in (0, 1):
+        assert np.array_equal(ctx.get(p, cb.E_DN, (T, n)), down["E"][p])
+        assert np.array_equal(ctx.get(p, cb.Y, (T, d)), down["Z"][p])
+    ctx.close()

@@ -617,8 +617,16 @@ ResidueTiles residue_tiles(int sm_count, int M, int N, int K) {
         }
     return best;
 }
-size_t residue_bytes(int rows, int cols) {       // of one party, whichever side is the M side
-    return (size_t)comet::residue::JOBS * (ceil_div(rows, 32) * 32) * (size_t)(ceil_div(cols, 32) * 32);
+// What the kernel on residues leaves for the recombination, of both parties: a byte per byte product and result word, 2.25 times
+// both parties' Z.  It has RESIDUE_ROOM at most, or one band of 256 rows where that is more; a product that leaves more goes band
+// by band over the M side, each band's recombination before the next one's product.  No layer of 512 tokens comes near it.
+constexpr size_t RESIDUE_ROOM = (size_t)1 << 30;
+size_t residue_bytes(int m_rows, int n_rows) {
+    return 2 * (size_t)comet::residue::JOBS * (ceil_div(m_rows, 32) * 32) * (size_t)(ceil_div(n_rows, 32) * 32);
+}
+size_t residue_room(int rows, int cols) {
+    return std::min(residue_bytes(rows, cols),
+                    std::max(RESIDUE_ROOM, residue_bytes(comet::residue::BM, std::max(rows, cols))));
 }
 
 // Whether a product is quicker through residues than through limbs.
@@ -638,59 +646,68 @@ bool residues_pay(int sm_count, int M, int N, int K) {
 
 // Whether this product goes through residues.
 bool through_residues(const comet_ctx* c, const Proj& pr) {
-    return c->residues.bytes && !c->grouped && pr.K <= comet::residue::MAX_DEPTH &&
-           3 * residue_set(pr.M, pr.K) <= c->planes_left.bytes && 2 * residue_bytes(pr.M, pr.N) <= c->residues.bytes &&
+    return c->residues.bytes >= residue_room(pr.M, pr.N) && !c->grouped && pr.K <= comet::residue::MAX_DEPTH &&
+           3 * residue_set(pr.M, pr.K) <= c->planes_left.bytes &&
            3 * residue_set(pr.N, pr.K) <= (pr.down ? c->planes_right_dn : c->planes_right_up).bytes &&
            residues_pay(c->sm_count, pr.M, pr.N, pr.K);
 }
 
-// Tensor map of one side's residue planes (ResidueMaps), in boxes of `rows` rows.
-cudaError_t residue_map(CUtensorMap* map, uint8_t* planes, int operand_rows, int K, int rows) {
+// Tensor map of one side's residue planes (ResidueMaps), `take` rows from row `first` (a multiple of 8) on, in boxes of `rows`.
+cudaError_t residue_map(CUtensorMap* map, uint8_t* planes, int operand_rows, int first, int take, int K, int rows) {
     namespace rs = comet::residue;
     const cuuint64_t groups = ceil_div(operand_rows, 8), blocks = ceil_div(K, rs::KC);
-    const cuuint64_t size[5] = {rs::GROUP_BYTES / 4, rs::PLANES, groups, blocks, 3};
+    const cuuint64_t size[5] = {rs::GROUP_BYTES / 4, rs::PLANES, (cuuint64_t)ceil_div(take, 8), blocks, 3};
     const cuuint64_t pitch[4] = {rs::GROUP_BYTES, rs::CELL_BYTES, groups * rs::CELL_BYTES, blocks * groups * rs::CELL_BYTES};
     const cuuint32_t box[5] = {rs::GROUP_BYTES / 4, 1, (cuuint32_t)rows / 8, rs::STAGE_BLOCKS, 1}, step[5] = {1, 1, 1, 1, 1};
-    return tensor_map(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 5, planes, size, pitch, box, step, CU_TENSOR_MAP_SWIZZLE_NONE);
+    return tensor_map(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 5, planes + (size_t)(first / 8) * rs::CELL_BYTES, size, pitch, box, step,
+                      CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
 // Tensor-core path: both parties' product through residues, from the planes to Z.
 int residue_combine(comet_ctx* c, const Proj& pr) {
     namespace rs = comet::residue;
     const ResidueTiles t = residue_tiles(c->sm_count, pr.M, pr.N, pr.K);
+    const int m_rows = t.swapped ? pr.N : pr.M, n_rows = t.swapped ? pr.M : pr.N;
+    const bool whole = residue_bytes(m_rows, n_rows) <= c->residues.bytes;
+    const int fit = whole ? t.mt : (int)(c->residues.bytes / residue_bytes(rs::BM, n_rows));      // tile rows that the room holds
+    const int bands = ceil_div(t.mt, fit), band_tiles = ceil_div(t.mt, bands);
     comet::ResidueArgs a;
     comet::RecombineArgs r;
-    const int m_rows = t.swapped ? pr.N : pr.M, n_rows = t.swapped ? pr.M : pr.N;
-    for (int p = 0; p < 2; ++p) {
-        r.T[p] = a.T[p] = c->residues.at + p * residue_bytes(pr.M, pr.N);
-        r.C[p] = c->buf[p][pr.idC];
-        r.Z[p] = c->buf[p][pr.idZ];
-    }
-    r.rows = pr.M; r.cols = pr.N;
-    r.m_groups = a.m_groups = ceil_div(m_rows, 32);
+    r.ld = pr.N;
     r.n_chunks = a.n_chunks = ceil_div(n_rows, 16);
     a.swapped = t.swapped;
-    a.mt = t.mt; a.nt = t.nt; a.n_tile = t.n_tile;
+    a.nt = t.nt; a.n_tile = t.n_tile;
     a.k32 = ceil_div(pr.K, 32);
-    a.jobs = rs::JOBS * t.mt * t.nt;
     a.error_flag = c->d_error;
     a.error_host = c->h_count_dev + 3;
     uint8_t* const left = c->planes_left.at;
     uint8_t* const right = (pr.down ? c->planes_right_dn : c->planes_right_up).at;
     comet::ResidueMaps maps;
-    COMET_CUDA(c, residue_map(&maps.m_side, t.swapped ? right : left, m_rows, pr.K, rs::BM / 2));
-    COMET_CUDA(c, residue_map(&maps.n_side, t.swapped ? left : right, n_rows, pr.K, t.n_tile / 2));
-    // no more pairs than the rounds need: what is left serves the kernels beside this one
-    const int most = c->sm_count / 2, pairs = ceil_div(a.jobs, ceil_div(a.jobs, most));
-    {
-        PhaseTimer timer(c, COMET_PHASE_COMBINE, 2);
+    COMET_CUDA(c, residue_map(&maps.n_side, t.swapped ? left : right, n_rows, 0, n_rows, pr.K, t.n_tile / 2));
+    PhaseTimer timer(c, COMET_PHASE_COMBINE, 2 * ceil_div(t.mt, band_tiles));
+    for (int tile = 0; tile < t.mt; tile += band_tiles) {
+        const int first = tile * rs::BM, rows = std::min(m_rows - first, band_tiles * rs::BM);
+        a.mt = ceil_div(rows, rs::BM);
+        a.jobs = rs::JOBS * a.mt * t.nt;
+        r.m_groups = a.m_groups = ceil_div(rows, 32);
+        r.rows = t.swapped ? pr.M : rows;
+        r.cols = t.swapped ? rows : pr.N;
+        const size_t at = (size_t)first * (t.swapped ? 1 : pr.N);
+        for (int p = 0; p < 2; ++p) {
+            r.T[p] = a.T[p] = c->residues.at + p * (residue_bytes(rows, n_rows) / 2);
+            r.C[p] = c->buf[p][pr.idC] + at;
+            r.Z[p] = c->buf[p][pr.idZ] + at;
+        }
+        COMET_CUDA(c, residue_map(&maps.m_side, t.swapped ? right : left, m_rows, first, rows, pr.K, rs::BM / 2));
+        // no more pairs than the rounds need: what is left serves the kernels beside this one
+        const int most = c->sm_count / 2, pairs = ceil_div(a.jobs, ceil_div(a.jobs, most));
         COMET_CUDA(c, launch_chained(comet::combine_residue_kernel, dim3(2 * pairs), dim3(rs::THREADS), rs::SMEM_BYTES, c->stream,
                                      &c->top_priority, a, maps));
         COMET_CUDA(c, launch_chained(t.swapped ? comet::residue_recombine_kernel<true> : comet::residue_recombine_kernel<false>,
                                      dim3(ew_grid(c, (int64_t)a.m_groups * a.n_chunks * 128, 256), 2), dim3(256), 0, c->stream,
                                      nullptr, r));
+        c->stats.kernel_launches += 2;
     }
-    c->stats.kernel_launches += 2;
     c->stats.tensor_tile_macs = 2ll * 2 * t.mt * rs::BM * t.nt * t.n_tile * a.k32 * 32;
     c->stats.matmul_path = COMET_PATH_LIMB;
     c->stats.product_kernel = COMET_KERNEL_RESIDUE;
@@ -846,7 +863,7 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
                    std::max(up ? residue_set(T, up_depth) : 0, dn ? residue_set(T, dn_depth) : 0));
             planes(c->planes_right_up, limb_set((int)gn, d, lb::BN), up ? residue_set((int)gn, up_depth) : 0);
             planes(c->planes_right_dn, limb_set(d, (int)n, lb::BN), dn ? residue_set(d, dn_depth) : 0);
-            c->residues.bytes = 2 * std::max(up ? residue_bytes(T, (int)gn) : 0, dn ? residue_bytes(T, d) : 0);
+            c->residues.bytes = std::max(up ? residue_room(T, (int)gn) : 0, dn ? residue_room(T, d) : 0);
             reserve(device, &c->residues.at, c->residues.bytes);
         }
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -398,7 +398,7 @@ struct RecombineArgs {
     const uint8_t* T[2];     // see ResidueArgs
     const u64* C[2];
     u64* Z[2];
-    int rows, cols;          // of Z; cols a multiple of 16
+    int rows, cols, ld;      // of Z, or of a band of its rows or columns in it; cols a multiple of 16
     int m_groups, n_chunks;
 };
 
@@ -450,7 +450,7 @@ residue_recombine_kernel(const __grid_constant__ RecombineArgs a) {
         const unsigned m = SWAPPED ? q & 31 : q >> 2 & 31, n = SWAPPED ? q >> 5 & 3 : q & 3;
         const unsigned row = SWAPPED ? nc * 16 + n * 4 : mg * 32 + m, col = SWAPPED ? mg * 32 + m : nc * 16 + n * 4;
         if (row >= (unsigned)a.rows || col >= (unsigned)a.cols) continue;
-        const size_t at = (size_t)row * a.cols + col;
+        const size_t at = (size_t)row * a.ld + col;
         u64 sum[4];
         unsigned quotient[4];
         if (!SWAPPED) {
@@ -458,7 +458,7 @@ residue_recombine_kernel(const __grid_constant__ RecombineArgs a) {
             sum[0] = c0.x; sum[1] = c0.y; sum[2] = c1.x; sum[3] = c1.y;
         } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) sum[e] = row + e < (unsigned)a.rows ? __ldcs(C + at + (size_t)e * a.cols) : 0ull;
+            for (int e = 0; e < 4; ++e) sum[e] = row + e < (unsigned)a.rows ? __ldcs(C + at + (size_t)e * a.ld) : 0ull;
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) quotient[e] = (1u << 23) + (8u << 24) - RESIDUE_QUOTIENT_BIAS;
@@ -477,7 +477,7 @@ residue_recombine_kernel(const __grid_constant__ RecombineArgs a) {
         } else {
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                if (row + e < (unsigned)a.rows) Z[at + (size_t)e * a.cols] = sum[e];
+                if (row + e < (unsigned)a.rows) Z[at + (size_t)e * a.ld] = sum[e];
         }
     }
 }

@@ -99,6 +99,35 @@ def test_largest_sums(cb, depth, residues):
     ctx.close()
 
 
+@pytest.mark.parametrize("T,n", [(2550, 12304), (2100, 14864)])       # rows of Z on the 256-row side, columns of Z on it
+def test_more_residues_than_the_scratch_holds(cb, T, n):
+    """Two bands, the second one ragged, against the CUDA-core path."""
+    d, block = 528, 16
+    gen = torch.Generator(device="cuda").manual_seed(T)
+
+    def pair(*shape):
+        return [torch.randint(-(1 << 63), (1 << 63) - 1, shape, dtype=torch.int64, device="cuda", generator=gen) for _ in (0, 1)]
+
+    shares = {cb.X: pair(T, d), cb.W1: pair(n, d), cb.A_UP: pair(T, d), cb.B_UP: pair(n, d), cb.C_UP: pair(T, n)}
+    got = []
+    for path in (cb.PATH_AUTO, cb.PATH_SIMT):
+        ctx = cb.Comet(T, d, n, block, 16, 0, 0, n, path)
+        ctx.set_mask(np.ones(n // block, np.uint8))
+        for tid, s in shares.items():
+            for p in (0, 1):
+                ctx.bind_shares(p, tid, s[p])
+        before = ctx.stats().kernel_launches
+        ctx.ffn_up(T)
+        if path == cb.PATH_AUTO:                 # the exchange, then product and recombination of either band
+            assert ctx.stats().product_kernel == cb.KERNEL_RESIDUE and ctx.stats().kernel_launches == before + 5
+        ctx.synchronize()
+        got.append([ctx.result_view(p, cb.Z_UP, (T, n)).clone() for p in (0, 1)])
+        torch.cuda.synchronize()
+        ctx.close()
+    for p in (0, 1):
+        assert torch.equal(got[0][p], got[1][p]), p
+
+
 def test_captured_and_replayed(cb):
     from tests.test_gpu_capture import test_layer_captured_and_replayed as replayed
 

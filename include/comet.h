@@ -163,6 +163,14 @@ typedef struct {
  * also owns one internal non-blocking stream, forked from and joined back into
  * `cuda_stream` with events, on which comet_ffn_up opens the weight side of the
  * down-projection early when W2 and B_DN are already loaded.
+ * One device allocation holds everything.  Beside the tensors it has, on the
+ * tensor-core path with more than 32 tokens, 24 bytes per operand word of either
+ * product for operand planes; where a product of the full capacity would go
+ * through COMET_KERNEL_RESIDUE, 51 of them instead, and 36 bytes per result word
+ * up to 1 GiB (512 tokens of a dense 8192 x 2048 layer: 4.1 GB instead of 2.9).
+ * That larger room is taken only where it leaves a quarter of the device's memory
+ * free; without it the context's products go through COMET_KERNEL_LIMB, more
+ * slowly and with the same bits.
  * Errors: INVALID_ARG, SHAPE (divisibility rules above), OOM, CUDA. */
 int comet_init(const comet_config* config, void* cuda_stream, comet_ctx** out);
 

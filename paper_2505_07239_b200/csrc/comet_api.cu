@@ -930,20 +930,20 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
             at += (list.bytes[k] + ALIGN - 1) / ALIGN * ALIGN;
         }
     };
-    if (ok && cudaMalloc(&c->device_memory, total(device)) != cudaSuccess) {
-        // Planes of residues take twice the room of planes of limbs: without them, then.
-        ok = planes_pieces > 0;
-        if (ok) {
-            cudaGetLastError();
-            for (int k = 0; k < planes_pieces; ++k) device.bytes[planes_piece + k] = planes_of_limbs[k];
-            device.bytes[planes_piece + planes_pieces] = 0;
-            c->planes_left.bytes = planes_of_limbs[0];
-            c->planes_right_up.bytes = planes_of_limbs[1];
-            c->planes_right_dn.bytes = planes_of_limbs[2];
-            c->residues.bytes = 0;
-            ok = cudaMalloc(&c->device_memory, total(device)) == cudaSuccess;
-        }
+    // Room for residues adds up to a half to a context (27 bytes an operand word, 36 a result word).  It is for speed alone, so
+    // it is taken only where a quarter of the device's memory stays free for what else the caller has to place there.
+    size_t free_bytes = 0, all_bytes = 0;
+    if (ok && c->residues.bytes &&
+        (cudaMemGetInfo(&free_bytes, &all_bytes) != cudaSuccess || total(device) + all_bytes / 4 > free_bytes)) {
+        cudaGetLastError();
+        for (int k = 0; k < planes_pieces; ++k) device.bytes[planes_piece + k] = planes_of_limbs[k];
+        device.bytes[planes_piece + planes_pieces] = 0;
+        c->planes_left.bytes = planes_of_limbs[0];
+        c->planes_right_up.bytes = planes_of_limbs[1];
+        c->planes_right_dn.bytes = planes_of_limbs[2];
+        c->residues.bytes = 0;
     }
+    ok = ok && cudaMalloc(&c->device_memory, total(device)) == cudaSuccess;
     ok = ok && cudaHostAlloc(&c->pinned_memory, total(pinned), cudaHostAllocMapped) == cudaSuccess;
     if (ok) {
         hand_out(device, c->device_memory);

@@ -128,6 +128,46 @@ def test_more_residues_than_the_scratch_holds(cb, T, n):
         assert torch.equal(got[0][p], got[1][p]), p
 
 
+@pytest.mark.parametrize("stays_free,residues", [(0.30, True), (0.20, False)])
+def test_room_for_residues_leaves_memory_free(cb, stays_free, residues):
+    """A quarter of the device's memory has to stay free for a context to take room for residues; the others multiply through
+    limbs, in less memory, and leave the same bits."""
+    T, d, n, block = 512, 1536, 1536, 16
+    gen = torch.Generator(device="cuda").manual_seed(8)
+    shares = {t: [torch.randint(-(1 << 63), (1 << 63) - 1, s, dtype=torch.int64, device="cuda", generator=gen) for _ in (0, 1)]
+              for t, s in ((cb.X, (T, d)), (cb.W1, (n, d)), (cb.A_UP, (T, d)), (cb.B_UP, (n, d)), (cb.C_UP, (T, n)))}
+
+    def product():
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        ctx = cb.Comet(T, d, n, block, 16, 0, 0, n)
+        taken = before - torch.cuda.mem_get_info()[0]
+        ctx.set_mask(np.ones(n // block, np.uint8))
+        for tid, s in shares.items():
+            for p in (0, 1):
+                ctx.bind_shares(p, tid, s[p])
+        ctx.ffn_up(T)
+        ctx.synchronize()
+        out = [ctx.result_view(p, cb.Z_UP, (T, n)).clone() for p in (0, 1)]
+        kernel = ctx.stats().product_kernel
+        torch.cuda.synchronize()
+        ctx.close()
+        return out, kernel, taken
+
+    torch.cuda.empty_cache()
+    product()                                    # loads what there is to load
+    want, kernel, most = product()
+    assert kernel == cb.KERNEL_RESIDUE
+    free, everything = torch.cuda.mem_get_info()
+    held = torch.empty(free - int(stays_free * everything), dtype=torch.uint8, device="cuda")     # never written
+    got, kernel, taken = product()
+    del held
+    torch.cuda.empty_cache()
+    assert kernel == (cb.KERNEL_RESIDUE if residues else cb.KERNEL_LIMB)
+    assert (taken < 0.8 * most) == (not residues), (taken, most)
+    assert all(torch.equal(a, b) for a, b in zip(want, got))
+
+
 def test_captured_and_replayed(cb):
     from tests.test_gpu_capture import test_layer_captured_and_replayed as replayed
 

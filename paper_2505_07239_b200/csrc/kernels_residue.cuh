@@ -391,15 +391,18 @@ combine_residue_kernel(const __grid_constant__ ResidueArgs a, const __grid_const
 // ---------------------------------------------------------------------------
 // Z_i = C_i + S + 2^56 (the two cross products), S from its residues: S = sum_i t_i (M / m_i) - k M, k the nearest whole number
 // to sum_i t_i / m_i, which 24 bits after the point tell (MAX_DEPTH keeps |S| below M / 2 by more than their error).
-// Bound by memory: 18 bytes in, mostly from L2, C in and Z out, 34 bytes a word: 512 x 832 both parties 11 us under ncu, 512 x
-// 2048 17.6.  (Two moduli at a time, with a third fewer integer instructions, took the same time.)
+// 18 bytes in, mostly from L2, C in and Z out, 34 bytes a word: 512 x 832 both parties 9.0 us under ncu, 512 x 2048 15.8, which
+// is 3.2 and 4.5 TB/s and so not memory's bound.  A scheduler issues in 49 and 61 % of its cycles; of its 9 and 13 warps 6.5 and
+// 6.1 wait for loads, 3.5 and 4.9 for the integer multiply pipe: a thread has only its eighteen 4-byte loads and C in flight and
+// nothing to do beside them.  (Two moduli at a time, with a third fewer integer instructions, took the same time.)
 // ---------------------------------------------------------------------------
 struct RecombineArgs {
     const uint8_t* T[2];     // see ResidueArgs
     const u64* C[2];
     u64* Z[2];
-    int rows, cols, ld;      // of Z, or of a band of its rows or columns in it; cols a multiple of 16
+    int rows, cols;          // of Z, or of a band of its rows (SWAPPED: of its columns); cols a multiple of 16
     int m_groups, n_chunks;
+    int ld;                  // SWAPPED: columns of Z
 };
 
 // Residues are signed bytes; as r + 128 they are not.
@@ -450,7 +453,7 @@ residue_recombine_kernel(const __grid_constant__ RecombineArgs a) {
         const unsigned m = SWAPPED ? q & 31 : q >> 2 & 31, n = SWAPPED ? q >> 5 & 3 : q & 3;
         const unsigned row = SWAPPED ? nc * 16 + n * 4 : mg * 32 + m, col = SWAPPED ? mg * 32 + m : nc * 16 + n * 4;
         if (row >= (unsigned)a.rows || col >= (unsigned)a.cols) continue;
-        const size_t at = (size_t)row * a.ld + col;
+        const size_t at = (size_t)row * (SWAPPED ? a.ld : a.cols) + col;
         u64 sum[4];
         unsigned quotient[4];
         if (!SWAPPED) {

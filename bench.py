@@ -33,41 +33,80 @@ METRIC = "sparse shared-FFN Z_2^64 MACs/s"
 UNIT = "MAC64/s"
 L2_FLUSH_BYTES = 512 << 20
 
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the tensor-core combine kernel on the
-# default workload, from the committed ncu summary of that kernel (average of the up- and the down-projection
-# launch).  Valid only for the kernel source it was taken on: keyed by the SHA-256 of the kernel's part of
-# kernels_limb.cuh.
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of a product's combine launches, from the committed ncu summaries
+# (average of the up- and the down-projection), each on a workload whose two products both take that kernel.  Valid only for
+# the code it was taken on: keyed by that code's digest.
 COMBINE_LIMB_TRAFFIC = {
+    "workload": ("opt1.3b", 0.95),
+    "kernel_sha256": "936cf4d9be2309eb244f82a8886f4383d18865a859d44ca6eb6e2ab84620cafb",
+    "bytes_per_launch": 46499328,
+}
+COMBINE_RESIDUE_TRAFFIC = {                      # both launches: product and recombination
     "workload": ("opt1.3b", 0.9),
-    "kernel_sha256": "a6c98318a7c2c6988d489b2089819d218b57b2d00f635e8417f5991ae45d2e63",
-    "bytes_per_launch": 81062016,
+    "kernel_sha256": "bf68a7b4b440cd6bdb81055d3a9056a587e2514daf660a1166284c198f519ad0",
+    "bytes_per_launch": 181508096,
 }
 
-# The same for the kernel on residues, which the default workload runs through, and all of kernels_residue.cuh.
-COMBINE_RESIDUE_TRAFFIC = {
-    "workload": ("opt1.3b", 0.9),
-    "kernel_sha256": "9958ddbdf2193db01a44ff0c7f5b323b7a16753d4a15688ab54cd1aad195ce41",
-    "bytes_per_launch": 140239616,
+# What a combine kernel is made of: source files, from the given text to the end.
+COMBINE_SOURCES = {
+    "combine_limb": (("kernels_limb.cuh", "struct LimbArgs {"),),
+    "combine_residue": (("residue_planes.cuh", "namespace residue {"), ("kernels_residue.cuh", "namespace residue {")),
 }
 
+# Byte products per ring product of the kernels on the tensor cores: 36 limb products, 18 through residues.
+BYTE_PRODUCTS = {"combine_stream": 36, "combine_limb": 36, "combine_limb_grouped": 36, "combine_residue": 18}
 
-def combine_kernel_digest(source="kernels_limb.cuh", first="struct LimbArgs {"):
-    """SHA-256 of the source of a combine kernel: from its argument block to the end of the file."""
+
+def combine_kernel_digest(kernel="combine_limb"):
+    """SHA-256 of the code of a combine kernel, comments and white space left out."""
     import hashlib
+    import re
 
-    with open(os.path.join(ROOT, "paper_2505_07239_b200", "csrc", source)) as fh:
-        text = fh.read()
-    return hashlib.sha256(text[text.index(first):].encode()).hexdigest()
+    h = hashlib.sha256()
+    for source, first in COMBINE_SOURCES[kernel]:
+        with open(os.path.join(ROOT, "paper_2505_07239_b200", "csrc", source)) as fh:
+            text = fh.read()
+        h.update(" ".join(re.sub(r"//[^\n]*", "", text[text.index(first):]).split()).encode())
+    return h.hexdigest()
 
 
 def combine_traffic(workload, sparsity, kernel):
-    """The stored ncu DRAM traffic of the dominant kernel, or None when it does not apply any more."""
-    if kernel == "combine_residue" and (workload, round(sparsity, 4)) == COMBINE_RESIDUE_TRAFFIC["workload"]:
-        digest = combine_kernel_digest("kernels_residue.cuh", "namespace residue {")
-        return COMBINE_RESIDUE_TRAFFIC["bytes_per_launch"] if digest == COMBINE_RESIDUE_TRAFFIC["kernel_sha256"] else None
-    if kernel != "combine_limb" or (workload, round(sparsity, 4)) != COMBINE_LIMB_TRAFFIC["workload"]:
+    """The stored ncu DRAM traffic of a product through `kernel`, or None when it does not apply any more."""
+    stored = {"combine_limb": COMBINE_LIMB_TRAFFIC, "combine_residue": COMBINE_RESIDUE_TRAFFIC}.get(kernel)
+    if stored is None or (workload, round(sparsity, 4)) != stored["workload"]:
         return None
-    return COMBINE_LIMB_TRAFFIC["bytes_per_launch"] if combine_kernel_digest() == COMBINE_LIMB_TRAFFIC["kernel_sha256"] else None
+    return stored["bytes_per_launch"] if combine_kernel_digest(kernel) == stored["kernel_sha256"] else None
+
+
+def product_bytes(kernel, T, K, N):
+    """Algorithmic bytes of the combine launches of one product [T, K] x [K, N], both parties."""
+    operands, results = T * K + K * N, T * N
+    if kernel == "combine_stream":               # reads the operands' words and writes the messages itself
+        return 48 * (operands + results)
+    if kernel == "combine_residue":              # 17 byte planes of V_i, B_i, E and F; 18 residues out and in again; C in, Z out
+        return 51 * operands + (2 * 36 + 32) * results
+    if kernel == "combine_simt":                 # messages and triple shares, C in, Z out
+        return 48 * operands + 32 * results
+    return 24 * operands + 32 * results          # 8 byte planes of V_i, B_i, E and F; Z read and written
+
+
+def combine_roofline(products, ms, pipe, hbm_gbs):
+    """What bounds the combine launches of the `products` (kernel, T, K, N) of a step that took `ms` together.  `pipe` is the rate
+    of the pipe in 64-bit multiply-adds per second (the tensor pipe's at 36 byte products each).  Returns the roofline's own
+    fields and the rate at which the pipe would do these products."""
+    macs = [4 * T * K * N for _, T, K, N in products]
+    moved = sum(product_bytes(*p) for p in products)
+    t_pipe = sum(m * BYTE_PRODUCTS.get(p[0], 36) / 36 for m, p in zip(macs, products)) / pipe
+    t_hbm = moved / (hbm_gbs * 1e9)
+    pipe_macs = sum(macs) / t_pipe / 1e12
+    if t_hbm > t_pipe:
+        roof = {"bound": "hbm", "achieved": moved / (ms * 1e-3) / 1e9, "peak": hbm_gbs, "unit": "GB/s"}
+    else:
+        roof = {"bound": "alu" if products[0][0] == "combine_simt" else "tensor", "achieved": sum(macs) / (ms * 1e-3) / 1e12,
+                "peak": pipe_macs, "unit": "TMAC64/s"}
+    roof["frac"] = roof["achieved"] / roof["peak"]
+    roof["algorithmic_bytes_per_launch"] = moved // len(products)
+    return roof, pipe_macs
 
 
 def ffn_macs(cfg, T, n):
@@ -745,19 +784,27 @@ def main():
     barrier()
     stats = ctx.stats()
     ctx.set_profiling(False)
-    up_counts = None
-    if args.token_masks > 0:                    # what the up-projection of input set 0 covers under its token mask
-        st0 = sets[0]
-        ctx.set_mask(st0["mask_dev"])
+    # ---- which kernel either product takes, and what the up-projection of input set 0 covers under its token mask
+    st0 = sets[0]
+    ctx.set_mask(st0["mask_dev"])
+    if st0["tm_dev"] is not None:
         ctx.set_token_mask(st0["tm_dev"])
-        for p in (0, 1):
-            for tid in UP_IDS:
-                ctx.load_shares(p, tid, st0["dev"][p][tid])
-        ctx.ffn_up(T)
-        su = ctx.stats()
-        up_counts = {"components": su.n_components, "theorem1_macs": su.ring_macs,
-                     "union_macs": 2 * 2 * T * d * cfg.groups * st0["n"], "tensor_tile_macs": su.tensor_tile_macs}
-        barrier()
+    for p in (0, 1):
+        for tid in UP_IDS:
+            ctx.load_shares(p, tid, st0["dev"][p][tid])
+    ctx.ffn_up(T)
+    su = ctx.stats()
+    up_counts = {"components": su.n_components, "theorem1_macs": su.ring_macs,
+                 "union_macs": 2 * 2 * T * d * cfg.groups * st0["n"],
+                 "tensor_tile_macs": su.tensor_tile_macs} if args.token_masks > 0 else None
+    for p in (0, 1):
+        for tid in DN_IDS:
+            ctx.load_shares(p, tid, st0["dev"][p][tid])
+    ctx.ffn_down(T)
+    combine_names = {cb.KERNEL_SIMT: "combine_simt", cb.KERNEL_STREAM: "combine_stream", cb.KERNEL_LIMB: "combine_limb",
+                     cb.KERNEL_GROUPED: "combine_limb_grouped", cb.KERNEL_RESIDUE: "combine_residue"}
+    kernels = [combine_names[su.product_kernel], combine_names[ctx.stats().product_kernel]]
+    barrier()
 
     # ---- several independent problems in flight (throughput mode): C contexts with their own weights, stream and
     #      two input sets each, inputs bound in place (no copies), steps issued round-robin; the region is timed
@@ -913,8 +960,7 @@ def main():
         ms_per_step, value = chosen["median"]["ms_per_step"], chosen["median"]["value"]
         phase = {name: {"ms_per_step": stats.phase_ms[k] / prof_steps, "launches_per_step":
                         stats.phase_launches[k] / prof_steps} for k, name in enumerate(cb.PHASE_NAMES)}
-        comb_launch_ms = stats.phase_ms[3] / (2 * prof_steps)      # of a product, whatever kernels it takes
-        comb_macs_per_launch = macs / 2          # up and down products carry half the MACs each here
+        combine_ms = stats.phase_ms[3] / prof_steps                # of both products, whatever launches they take
         used_path = {cb.PATH_SIMT: "simt", cb.PATH_LIMB: "limb"}.get(stats.matmul_path, "?")
         peaks = {}
         try:
@@ -924,64 +970,50 @@ def main():
         hbm = peaks.get("hbm_gbs", 6650.0)
         bf16 = peaks.get("bf16_tflops", 1590.0)
         src = "measured" if peaks else "fallback"
-        achieved = comb_macs_per_launch / (comb_launch_ms * 1e-3) / 1e12
-        # per launch, both parties: planes of V_i, B_i, and of E and F, which both parties share, read once, Z read and
-        # written once (average of the up- and the down-projection launch); with few tokens the kernel reads the
-        # operands' words and writes the messages itself
-        stream = stats.product_kernel == cb.KERNEL_STREAM
-        comb_bytes_per_launch = 8 * ((3 * T * d + 3 * d * g * n + 3 * T * g * n) + (3 * T * n + 3 * n * d + 3 * T * d)) \
-            if stream else 4 * ((3 * T * d + 3 * d * g * n + 4 * T * g * n) + (3 * T * n + 3 * n * d + 4 * T * d))
-        residue = stats.product_kernel == cb.KERNEL_RESIDUE
-        if residue:                              # 17 byte planes in place of 8, and 18 residues a result word out
-            comb_bytes_per_launch = (51 * (T * d + d * g * n + T * n + n * d) + 2 * 18 * (T * g * n + T * d)) // 2
+        products = [(kernels[0], T, d, cfg.groups * n), (kernels[1], T, n, d)]
         if used_path == "limb":
-            # The pipe's peak in ring multiply-adds: the measured rate of the tensor instruction the kernel issues,
-            # over its byte products per ring product (36 limb products, 18 through residues).  Beside it, what the
-            # measured bf16 GEMM peak would imply at the nominal int8 : bf16 ratio of 2.
-            products = 18 if residue else 36
-            name = "byte products through residues" if residue else "limb products"
-            derived = bf16 * 1e12 / 2 * 2 / products / 1e12
+            # The pipe's peak in ring multiply-adds: the measured rate of the tensor instruction the kernels issue,
+            # over their byte products per ring product.  Beside it, what the measured bf16 GEMM peak would imply at
+            # the nominal int8 : bf16 ratio of 2.
+            derived = bf16 * 1e12 / 2 * 2 / 36
             if pipe_peaks is not None:
-                peak = pipe_peaks["tensor_i8"]["ring_mac_burst"] * 36 / products / 1e12
-                peak_sustained = pipe_peaks["tensor_i8"]["ring_mac_sustained"] * 36 / products / 1e12
+                pipe = pipe_peaks["tensor_i8"]["ring_mac_burst"]
+                pipe_sustained = pipe_peaks["tensor_i8"]["ring_mac_sustained"]
                 peak_source = ("measured in this run: tcgen05.mma kind::i8 M128 N256 K32 loop on 148 SMs, operands in "
-                               f"shared memory, best of the first three 25 ms launches, / {products} {name}")
+                               "shared memory, best of the first three 25 ms launches")
             else:
-                peak, peak_sustained = derived, bf16_sustained_derived(peaks) * 36 / products
-                peak_source = f"{src} bf16 GEMM peak x2 (int8 nominal ratio), as MAC/s, / {products} {name}"
-            t_tensor = comb_macs_per_launch / (peak * 1e12)
-            t_hbm = comb_bytes_per_launch / (hbm * 1e9)
-            if t_hbm > t_tensor and stream:
-                # few tokens: the kernel streams the weight side's words once and is bound by that traffic
-                roof = {"bound": "hbm", "achieved": comb_bytes_per_launch / (comb_launch_ms * 1e-3) / 1e9, "peak": hbm,
-                        "unit": "GB/s", "peak_source": f"{src} HBM copy peak"}
-            else:
-                roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TMAC64/s",
-                        "peak_source": peak_source, "peak_sustained": peak_sustained,
-                        "frac_of_sustained_peak": achieved / peak_sustained,
-                        "peak_from_bf16_gemm": derived, "frac_of_peak_from_bf16_gemm": achieved / derived}
+                pipe, pipe_sustained = derived, bf16_sustained_derived(peaks) * 1e12
+                peak_source = f"{src} bf16 GEMM peak x2 (int8 nominal ratio), as MAC/s"
+            peak_source += ", / " + ", ".join(f"{BYTE_PRODUCTS[k]} byte products ({k})" for k in dict.fromkeys(kernels))
         else:
             # 148 SMs x 64 32-bit integer multiply-add lanes per clock x max SM clock / 4 issue slots per ring MAC
-            derived = 148 * 64 * 1.965e9 / 4 / 1e12
+            derived = 148 * 64 * 1.965e9 / 4
             if pipe_peaks is not None:
-                peak = pipe_peaks["alu_u64"]["burst"] / 1e12
-                peak_sustained = pipe_peaks["alu_u64"]["sustained"] / 1e12
+                pipe, pipe_sustained = pipe_peaks["alu_u64"]["burst"], pipe_peaks["alu_u64"]["sustained"]
                 peak_source = ("measured in this run: eight 64-bit multiply-add chains per thread, 2 x 1024 threads per "
                                "SM, best of the first three 25 ms launches")
             else:
-                peak = peak_sustained = derived
+                pipe = pipe_sustained = derived
                 peak_source = "148 SM x 64 int32 mul-add lanes/clk x 1.965 GHz / 4 issue slots per 64-bit MAC"
-            roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TMAC64/s", "peak_source": peak_source,
-                    "peak_sustained": peak_sustained, "frac_of_sustained_peak": achieved / peak_sustained,
-                    "peak_from_unit_counts": derived}
-        roof["frac"] = roof["achieved"] / roof["peak"]
+        roof, peak = combine_roofline(products, combine_ms, pipe, hbm)
+        peak_sustained = peak * pipe_sustained / pipe
+        if roof["bound"] == "hbm":
+            roof["peak_source"] = f"{src} HBM copy peak"
+        else:
+            name = "peak_from_bf16_gemm" if used_path == "limb" else "peak_from_unit_counts"
+            roof.update({"peak_source": peak_source, "peak_sustained": peak_sustained,
+                         "frac_of_sustained_peak": roof["achieved"] / peak_sustained, name: peak * derived / pipe,
+                         "frac_of_" + name: roof["achieved"] / (peak * derived / pipe)})
         # grouped: the multiply-adds are still counted over the union of the masks, of which it computes a part
-        roof["kernel"] = ("combine_stream" if stream else "combine_residue" if residue else "combine_limb_grouped" if stats.product_kernel == cb.KERNEL_GROUPED
-                          else "combine_" + used_path)
-        roof["traffic"] = combine_traffic(args.workload, sparsity, roof["kernel"])
-        roof["traffic_unit"] = "bytes per launch (ncu dram read+write); algorithmic: planes once + Z read-modify-write"
-        roof["algorithmic_bytes_per_launch"] = comb_bytes_per_launch
-        roof["timed"] = "kernel time per launch from the per-phase CUDA-event pass, one problem at a time"
+        roof["kernel"] = ", ".join(k + (" + residue_recombine" if k == "combine_residue" else "") for k in dict.fromkeys(kernels))
+        roof["traffic"] = combine_traffic(args.workload, sparsity, kernels[0]) if kernels[0] == kernels[1] else None
+        roof["traffic_unit"] = ("bytes per product (ncu dram read+write of its combine launches), average of the two; algorithmic: "
+                                + ", ".join({"combine_residue": "planes once, residues out and in, C in, Z out",
+                                             "combine_stream": "words and messages once, Z read-modify-write",
+                                             "combine_simt": "messages and triple shares once, C in, Z out"}
+                                            .get(k, "planes once + Z read-modify-write") for k in dict.fromkeys(kernels)))
+        roof["timed"] = ("device time of both products' combine launches from the per-phase CUDA-event pass, one problem at a "
+                         "time")
 
         def t_roof_ms(pipe_peak):                 # slower of bytes at the HBM peak and MACs at the pipe's peak
             return max(ffn_bytes(cfg, T, n) / (hbm * 1e9), macs / (pipe_peak * 1e12)) * 1e3

@@ -226,8 +226,11 @@ int comet_set_mask(comet_ctx* ctx, const uint8_t* block_mask, int location, int3
  * nothing.
  * On the tensor-core path the call also starts on the down-projection with what
  * is loaded already: with W2 and B_DN it opens that product's weight side
- * (COMET_F_DN), and with C_DN as well it copies C'_i into COMET_Y, the value the
- * down-projection's sums are added to.  So from this call on COMET_F_DN and
+ * (COMET_F_DN), and with C_DN as well it may copy C'_i into COMET_Y, the value the
+ * down-projection's sums are added to (not where that product goes through
+ * COMET_KERNEL_RESIDUE, which reads C'_i when it makes COMET_Y, nor where an operand
+ * of this call that is read too late for it lies on COMET_Y).  So from this call
+ * on COMET_F_DN and
  * COMET_Y no longer hold the previous step's values: read those back (or enqueue
  * the comet_get) before the next comet_ffn_up. */
 int comet_ffn_up(comet_ctx* ctx, int32_t tokens);

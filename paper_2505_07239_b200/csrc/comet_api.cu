@@ -619,7 +619,7 @@ ResidueTiles residue_tiles(int sm_count, int M, int N, int K) {
 }
 // What the kernel on residues leaves for the recombination, of both parties: a byte per byte product and result word, 2.25 times
 // both parties' Z.  It has RESIDUE_ROOM at most, or one band of 256 rows where that is more; a product that leaves more goes band
-// by band over the M side, each band's recombination before the next one's product.  No layer of 512 tokens comes near it.
+// by band over the M side, each band's recombination before the next one's product.  512 tokens fit up to 58 thousand columns.
 constexpr size_t RESIDUE_ROOM = (size_t)1 << 30;
 size_t residue_bytes(int m_rows, int n_rows) {
     return 2 * (size_t)comet::residue::JOBS * (ceil_div(m_rows, 32) * 32) * (size_t)(ceil_div(n_rows, 32) * 32);
@@ -631,10 +631,12 @@ size_t residue_room(int rows, int cols) {
 
 // Whether a product is quicker through residues than through limbs.
 // Either way's time in ns, exchange included, is a constant, a share per step of a CTA, per operand word and per result word,
-// fitted to 121 products of 65 to 512 rows, 256 to 4096 columns and depths (both within 28 %, the small ones the furthest off;
-// where the two times lie more than 5 % apart, which is what is asked for here, the rule picked the quicker one every time):
-// 512 x 256 x 256 19 us through limbs, 31 through residues; 512 x 1024 x 1024 67 and 65; 512 x 2048 x 2048 235 and 197;
-// 512 x 4096 x 4096 966 and 726; 256 x 4096 x 4096 546 and 516; 128 x 4096 x 4096 376 and 452.
+// fitted to timings of 65 to 512 rows, 256 to 4096 columns and depths: 512 x 256 x 256 19 us through limbs, 31 through residues;
+// 512 x 1024 x 1024 67 and 65; 512 x 2048 x 2048 235 and 197; 512 x 4096 x 4096 966 and 726; 256 x 4096 x 4096 546 and 516;
+// 128 x 4096 x 4096 376 and 452.  Over 136 such products either time is at most 28 % too short (512 x 256 x 256) and 19 % too long.
+// With the 5 % asked for, none of the 19 that go through residues is slower for it; of the 117 others three lose 5 % or more, the
+// wide and shallow ones, whose time per result word through limbs is understated: 512 x 4096 columns x 512 deep 152 and 130 us,
+// 384 x 4096 x 512 123 and 117, 256 x 2048 x 4096 278 and 264.
 bool residues_pay(int sm_count, int M, int N, int K) {
     namespace lb = comet::limb;
     const int64_t operands = (int64_t)(M + N) * K, results = (int64_t)M * N;

@@ -340,8 +340,9 @@ limb_exchange_kernel(const __grid_constant__ LimbExchangeArgs a, const __grid_co
 namespace ptx {
 // One lane of a converged warp, the same one every time.  Single-thread instructions (copies of the copy engine, MMAs, commits)
 // stand under this and not under `lane == 0`: the compiler then knows that one thread runs them, and makes no loop over the
-// lanes of each: an issuer at `lane == 0` takes some 100 cycles an MMA, whatever its size.  (Here, where the MMAs take about that
-// long themselves: QKV of 203 tokens 93.1 -> 92.8 us, 512 tokens in four groups 152.9 -> 151.6, 128 tokens x 320 34.5 -> 34.3.)
+// lanes of each: an issuer at `lane == 0` takes some 100 cycles an MMA, whatever its size.  (In the kernel of this file, whose MMAs
+// take about that long themselves, it makes no difference that shows: QKV of 203 tokens, 512 tokens in four groups and 128 tokens
+// x 320 within 1 % of what they were, less than two runs of one side differ.)
 __device__ __forceinline__ bool elect_one() {
     uint32_t elected;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(elected));

@@ -20,22 +20,86 @@ def cb():
     return binding
 
 
-@pytest.mark.parametrize("tokens,d_model,blocks,block,active,stacked,residues", [
-    (385, 1040, 80, 16, 63, 1, True),        # a row in the second token tile; depth 1040 = 8 stages and half an instruction;
+R, L = "residue", "limb"
+
+
+@pytest.fixture
+def kernels(cb, monkeypatch):
+    """The kernels of the products from here on, up and down in turn."""
+    seen = []
+    names = {cb.KERNEL_RESIDUE: R, cb.KERNEL_LIMB: L}
+    for name in ("ffn_up", "ffn_down"):
+        def call(ctx, tokens, original=getattr(cb.Comet, name)):
+            original(ctx, tokens)
+            seen.append(names.get(ctx.stats().product_kernel))
+
+        monkeypatch.setattr(cb.Comet, name, call)
+    return seen
+
+
+@pytest.mark.parametrize("tokens,d_model,blocks,block,active,stacked,up,down", [
+    (385, 1040, 80, 16, 63, 1, R, R),        # a row in the second token tile; depth 1040 = 8 stages and half an instruction;
                                              # columns of the weights' product on the 256-row side
-    (257, 3088, 20, 48, 17, 1, True),        # strips of 48 columns; 816 of 1024 rows of the weights' tiles
-    (400, 1552, 60, 16, 51, 1, True),        # 816 = 3 column tiles of 224 and a ragged one
-    (449, 1040, 40, 32, 33, 2, True),        # two stacked matrices; the group boundary lies inside a tile
-    (512, 1024, 40, 16, 32, 1, False),       # a layer just too small for it
+    (257, 3088, 20, 48, 17, 1, R, R),        # strips of 48 columns; 816 of 1024 rows of the weights' tiles
+    (400, 1552, 60, 16, 51, 1, R, R),        # 816 = 3 column tiles of 224 and a ragged one
+    (449, 1040, 40, 32, 33, 2, R, L),        # two stacked matrices; the group boundary lies inside a tile; a weight side of
+                                             # limbs opened beside a product through residues
+    (417, 512, 60, 48, 56, 1, L, R),         # and the other way round
+    (512, 1024, 40, 16, 32, 1, L, L),        # a layer just too small for it
 ])
-def test_layer_at_tile_edges(cb, tokens, d_model, blocks, block, active, stacked, residues):
+def test_layer_at_tile_edges(cb, kernels, tokens, d_model, blocks, block, active, stacked, up, down):
     from tests import harness as hz
 
     cfg = wl.FFNConfig("residue-edges", tokens, d_model, blocks * block, block, 16, stacked == 2, active / blocks, "uniform",
                        "normal", "normal0.02", stacked=stacked)
     r = hz.run_and_compare_products(cfg, seed=800 + tokens, early_down=tokens != 400)
     assert r["mismatches"] == 0 and r["n_active"] == active * block, r
-    assert (r["kernels"][0] == cb.KERNEL_RESIDUE) == residues, r["kernels"]
+    assert kernels == [up, down]
+
+
+@pytest.mark.parametrize("c_early", [False, True])
+@pytest.mark.parametrize("T_up,T_down,up,down", [(300, 128, R, L), (128, 300, L, R)])
+def test_weight_side_opened_for_another_number_of_tokens(cb, kernels, T_up, T_down, up, down, c_early):
+    """comet_ffn_up opens the down-projection's weight side for the kernel that its own number of tokens asks for; comet_ffn_down
+    with another number takes the other kernel and opens it again, whether C' was copied early or not."""
+    import oracle
+
+    d = n = 1536
+    T = max(T_up, T_down)
+    draw = lambda name, rows, cols: [wl.random_u64(31, f"other/{name}/{p}", rows * cols).reshape(rows, cols) for p in (0, 1)]  # noqa: E731
+    W1, W2, B_up, B_dn = (draw(k, n, d) for k in ("W1", "W2", "B_up", "B_dn"))
+    X, A_up, C_up = (draw(k, T_up, d) for k in ("X", "A_up", "C_up"))
+    H, A_dn, C_dn = (draw(k, T_down, d) for k in ("H", "A_dn", "C_dn"))
+    ctx = cb.Comet(T, d, n, 16, 16, 0, 0, n)
+    keep = []
+
+    def bind(tid, shares):
+        for p in (0, 1):
+            keep.append(cb.to_device(shares[p]))
+            ctx.bind_shares(p, tid, keep[-1])
+
+    bind(cb.W1, W1)
+    bind(cb.W2, W2)
+    assert ctx.set_mask(np.ones(n // 16, np.uint8)) == n
+    if c_early:                                  # some C' of the up-projection's number of tokens, replaced below
+        bind(cb.C_DN, draw("C_other", T_up, d))
+    for tid, shares in ((cb.X, X), (cb.A_UP, A_up), (cb.B_UP, B_up), (cb.C_UP, C_up), (cb.B_DN, B_dn)):
+        bind(tid, shares)
+    ctx.ffn_up(T_up)
+    t = lambda pair: [np.ascontiguousarray(m.T) for m in pair]  # noqa: E731  (stored output-feature-major)
+    index = np.arange(n, dtype=np.int32)
+    ref = oracle.somm(X, t(W1), index, A_up, t(B_up), C_up)
+    for p in (0, 1):
+        assert np.array_equal(ctx.get(p, cb.Z_UP, (T_up, n)), ref["Z"][p])
+    for tid, shares in ((cb.H, H), (cb.A_DN, A_dn), (cb.C_DN, C_dn)):
+        bind(tid, shares)
+    ctx.ffn_down(T_down)
+    ref = oracle.simm(H, t(W2), index, A_dn, t(B_dn), C_dn)
+    for p in (0, 1):
+        assert np.array_equal(ctx.get(p, cb.F_DN, (d, n)).T, ref["F"][p])
+        assert np.array_equal(ctx.get(p, cb.Y, (T_down, d)), ref["Z"][p])
+    assert kernels == [up, down]
+    ctx.close()
 
 
 def test_token_mask_of_one_component(cb):
@@ -168,14 +232,16 @@ def test_room_for_residues_leaves_memory_free(cb, stays_free, residues):
     assert all(torch.equal(a, b) for a, b in zip(want, got))
 
 
-def test_captured_and_replayed(cb):
+def test_captured_and_replayed(cb, kernels):
     from tests.test_gpu_capture import test_layer_captured_and_replayed as replayed
 
     replayed(cb, 385, 1040, 80, 16, 63)
+    assert set(kernels) == {R}
 
 
 @pytest.mark.parametrize("x_on", ["Y", "Z_UP"])
-def test_operands_on_result_buffers(cb, x_on):
+def test_operands_on_result_buffers(cb, kernels, x_on):
     from tests.test_gpu_bound_results import test_operands_on_result_buffers as bound
 
     bound(385, 1040, x_on)
+    assert set(kernels) == {R}

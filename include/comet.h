@@ -152,8 +152,9 @@ typedef struct {
     int32_t product_kernel;  /* COMET_KERNEL_* of the last ffn call's product (0 before the first) */
     int64_t tensor_tile_macs; /* 64-bit multiply-adds the tensor-core kernel of the last ffn call covered, counted
                                  in whole output tiles (128 x 64, 32 tokens x 128 in the kernel for few tokens, 256 x a
-                                 multiple of 32 in the kernel on residues) and 32-deep steps, both parties (0 on the CUDA-core path): under a token mask with
-                                 several components only the tiles and steps that meet a component */
+                                 multiple of 32 in the kernel on residues) and 32-deep steps, both parties (0 on the
+                                 CUDA-core path): under a token mask with several components only the tiles and steps
+                                 that meet a component */
 } comet_stats_t;
 
 /* Create a context: validates the configuration, selects the device, and
@@ -230,9 +231,8 @@ int comet_set_mask(comet_ctx* ctx, const uint8_t* block_mask, int location, int3
  * down-projection's sums are added to (not where that product goes through
  * COMET_KERNEL_RESIDUE, which reads C'_i when it makes COMET_Y, nor where an operand
  * of this call that is read too late for it lies on COMET_Y).  So from this call
- * on COMET_F_DN and
- * COMET_Y no longer hold the previous step's values: read those back (or enqueue
- * the comet_get) before the next comet_ffn_up. */
+ * on COMET_F_DN and COMET_Y no longer hold the previous step's values: read those
+ * back (or enqueue the comet_get) before the next comet_ffn_up. */
 int comet_ffn_up(comet_ctx* ctx, int32_t tokens);
 
 /* Protocols 2 and 3 in general: the sparsity distribution may differ from token to

@@ -348,11 +348,15 @@ int launch_stream(comet::StreamArgs& args, const comet::BlockIds& held, int sm_c
     namespace ls = comet::limb_stream;
     *err = cudaSuccess;
     args.mt = ceil_div(args.M, ls::BT);
-    args.nt = ceil_div(args.N, ls::BW);
     args.kb = ceil_div(args.K, ls::KC);
+    // Tiles of 32 features where the device has room for a CTA per step of them.  Beyond that a CTA would have several such steps, and
+    // the MMAs of each take as long as those of a step of 128.
+    const bool small = (long long)args.mt * ceil_div(args.N, ls::QROWS) * args.kb <= sm_count;
+    const int features = small ? ls::QROWS : ls::BW;
+    args.nt = ceil_div(args.N, features);
     const long long steps = (long long)args.mt * args.nt * args.kb;
     const unsigned grid = (unsigned)(steps < sm_count ? steps : sm_count);
-    args.last_cost = ceil_div(args.N - (args.nt - 1) * ls::BW, ls::QROWS) + ls::STEP_SLOTS;
+    args.last_cost = ceil_div(args.N - (args.nt - 1) * features, ls::QROWS) + ls::STEP_SLOTS;
     args.own_cost = args.sync ? (unsigned)ceil_div(ls::OWN_SIXTEENTHS * (args.M < ls::BT ? args.M : ls::BT), 16) : 0u;
     const long long cost = (((long long)(ls::QUARTERS + ls::STEP_SLOTS) * (args.nt - 1) + args.last_cost) * args.kb +
                             (long long)args.own_cost * args.nt) * args.mt;
@@ -370,8 +374,9 @@ int launch_stream(comet::StreamArgs& args, const comet::BlockIds& held, int sm_c
                               nullptr, args.C[0], args.C[1], args.Z[0], args.Z[1], pairs);
         if (*err != cudaSuccess) return COMET_ERR_CUDA;
     }
-    *err = launch_chained(args.M <= 16 ? comet::combine_stream_kernel<16> : comet::combine_stream_kernel<32>, dim3(grid), dim3(ls::THREADS), ls::SMEM_BYTES, stream,
-                          priority, args, maps, held);
+    auto* const kernel = small ? (args.M <= 16 ? comet::combine_stream_kernel<16, ls::QROWS> : comet::combine_stream_kernel<32, ls::QROWS>)
+                               : (args.M <= 16 ? comet::combine_stream_kernel<16, ls::BW> : comet::combine_stream_kernel<32, ls::BW>);
+    *err = launch_chained(kernel, dim3(grid), dim3(ls::THREADS), ls::SMEM_BYTES, stream, priority, args, maps, held);
     return *err == cudaSuccess ? COMET_OK : COMET_ERR_CUDA;
 }
 
@@ -392,7 +397,7 @@ int stream_product(comet_ctx* c, const Proj& pr) {
         a.Z[p] = c->buf[p][pr.idZ];
         a.C[p] = c->buf[p][pr.idC];
     }
-    if (ls::SYNC_WORDS + (size_t)ceil_div(pr.M, ls::BT) * ceil_div(pr.N, ls::BW) > c->stream_sync_words) return COMET_ERR_SHAPE;
+    if (ls::SYNC_WORDS + (size_t)ceil_div(pr.M, ls::BT) * ceil_div(pr.N, ls::QROWS) > c->stream_sync_words) return COMET_ERR_SHAPE;
     a.sync = c->d_stream_sync;
     a.gather = 1;
     a.ids = c->ids_held ? nullptr : c->d_ids;
@@ -872,7 +877,8 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
                                         (int)lb::SMEM_BYTES) == cudaSuccess;
         // the memory-side kernels may share an SM with a resident tensor-core CTA (which forces the largest
         // shared-memory carve-out), so they ask for the same carve-out
-        for (auto* kernel : {comet::combine_stream_kernel<16>, comet::combine_stream_kernel<32>})
+        for (auto* kernel : {comet::combine_stream_kernel<16, comet::limb_stream::BW>, comet::combine_stream_kernel<32, comet::limb_stream::BW>,
+                             comet::combine_stream_kernel<16, comet::limb_stream::QROWS>, comet::combine_stream_kernel<32, comet::limb_stream::QROWS>})
             ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)comet::limb_stream::SMEM_BYTES) == cudaSuccess;
         ok = ok && cudaFuncSetAttribute(comet::combine_limb_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -913,7 +919,7 @@ int comet_init(const comet_config* cfg, void* cuda_stream, comet_ctx** out) {
     {
         namespace ls = comet::limb_stream;
         const int64_t widest = c->groups * c->cap_n > cfg->d_model ? c->groups * c->cap_n : cfg->d_model;
-        c->stream_sync_words = ls::SYNC_WORDS + (STREAM_TOKENS / ls::BT) * (size_t)((widest + ls::BW - 1) / ls::BW);
+        c->stream_sync_words = ls::SYNC_WORDS + (STREAM_TOKENS / ls::BT) * (size_t)((widest + ls::QROWS - 1) / ls::QROWS);
         reserve(device, &c->d_stream_sync, c->stream_sync_words * sizeof(uint32_t));
     }
     reserve(pinned, &c->h_masked, comet::PLAN_WORDS * sizeof(long long));
@@ -1567,7 +1573,8 @@ cudaError_t static_device(StaticDevice* out) {
     if (!d.scratch) {
         void *p = nullptr, *e = nullptr;
         err = cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, dev);
-        for (auto* kernel : {comet::combine_stream_kernel<16>, comet::combine_stream_kernel<32>})
+        for (auto* kernel : {comet::combine_stream_kernel<16, comet::limb_stream::BW>, comet::combine_stream_kernel<32, comet::limb_stream::BW>,
+                             comet::combine_stream_kernel<16, comet::limb_stream::QROWS>, comet::combine_stream_kernel<32, comet::limb_stream::QROWS>})
             if (err == cudaSuccess)
                 err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)comet::limb_stream::SMEM_BYTES);

@@ -50,6 +50,7 @@ constexpr int BW = 128, BT = 32, KC = limb::KC, PLANES = limb::PLANES, QROWS = 3
 constexpr int CONV_GROUPS = 2, GROUP_WARPS = 8, CONV_WARPS = CONV_GROUPS * GROUP_WARPS;
 constexpr int RAW_WARP0 = CONV_WARPS, TOK_WARP0 = RAW_WARP0 + 2, TOK_WARPS = 8, MMA_WARP = TOK_WARP0 + TOK_WARPS;
 constexpr int EPI_WARPS = TOK_WARPS / 2;                 // per party
+constexpr int SMALL_WORKERS = 3;                         // warps per party that drain a small tile
 constexpr int INIT_WARP = MMA_WARP + 1, THREADS = 32 * (INIT_WARP + 1);
 constexpr int RAW_ARRAY_BYTES = QROWS * KC * 8;          // 8 KiB: one array of a slot
 constexpr int RAW_SLOT_BYTES = 4 * RAW_ARRAY_BYTES;      // party 0: W | B, party 1: W | B
@@ -135,7 +136,9 @@ __device__ __forceinline__ StreamSegment stream_segment(const StreamArgs& a, uns
 }
 
 // Raw slots the weight side of a feature tile takes per step.
+template <int FEATURES>
 __device__ __forceinline__ int stream_quarters(const StreamArgs& a, int tn) {
+    if (FEATURES < limb_stream::BW) return 1;
     return tn + 1 < a.nt ? limb_stream::QUARTERS : a.last_cost - limb_stream::STEP_SLOTS;
 }
 
@@ -192,7 +195,13 @@ __device__ __forceinline__ bool stream_tile_ready(const uint32_t* flag, uint32_t
 // COLS = 16 for up to 16 tokens, else 32: the width of the token planes and of the accumulators.  With half the columns the MMAs
 // take half the time, which the conversion of a step otherwise waits for: llama7b decode (7 tokens) 202 -> 188 us.  (As a
 // value of the launch instead of a template's it cost the 32-token layer 2 %.)
-template <int COLS>
+// FEATURES = 32 where the device has room for a CTA per step even of such tiles (launch_stream), else BW: a CTA's first planes wait for
+// all of its words, and its end for its own sums, and a quarter of either is there sooner; the MMAs have a quarter of their rows
+// in use, which costs nothing.  With so few steps latency is all there is, so the rest is cut short too: the first rows are found
+// before the wait for the kernel before this one, Z <- C goes through registers, and three warps a party drain.  From that wait
+// to the end, 16 tokens x 256 deep x 96: 7.8 -> 6.5 us.  A layer of 256 x 96: 16 tokens 22.6 -> 20.6 us (then bound by the host's calls),
+// 32 tokens 29.6 -> 22.3; of 448 x 320, 32 tokens 31.4 -> 28.8.
+template <int COLS, int FEATURES>
 __global__ void __launch_bounds__(limb_stream::THREADS, 1)
 combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constant__ LimbMaps maps,
                       const __grid_constant__ BlockIds held) {
@@ -247,9 +256,50 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
     const bool valid = ticket < gridDim.x;
     if (!valid && threadIdx.x == 0) abort_flag = 1;
     const unsigned cta = valid ? ticket : 0u, u_begin = stream_cut(a, cta), u_end = valid ? stream_cut(a, cta + 1) : u_begin;
-    pdl_wait();
+    constexpr bool SMALL = FEATURES < BW;
+    const bool raw_warp = warp >= RAW_WARP0 && warp < RAW_WARP0 + 2;
+    // the list of blocks may be the work of the kernel before this one
+    if (!SMALL || !raw_warp || a.ids) pdl_wait();
 
-    if (warp >= RAW_WARP0 && warp < RAW_WARP0 + 2) {
+    // A party's sums of a segment have arrived, and its part of Z may be added to.
+    auto arrived = [&](const StreamSegment& sg, int party, uint32_t seg_phase) {
+        bool ok = true;
+        if (a.sync) ok = stream_tile_ready(a.sync + SYNC_WORDS + sg.tile, epoch, lane, &abort_flag);
+        return ok && limb_wait_warp(ptx::smem_u32(&acc_full[party]), seg_phase, &abort_flag);
+    };
+    // ---------------- epilogue of a segment: lane = output feature, registers = tokens ----------------
+    // Result rows go through shared memory, OUT_TOKENS of them at a time, and one tensor reduction adds them into Z; a worker takes
+    // every `workers`-th round from `first` on.  A CTA's last segment stages them in the raw ring (no `buffer`), which nothing uses any
+    // more, so that no round waits for the copy engine to have read the one before.  (One buffer and a bulk reduction per row:
+    // 7400 cycles for 32 tokens.)
+    auto drain = [&](const StreamSegment& sg, int party, u64* buffer, int first, int workers) {
+        const int quarter = warp & 3;            // TMEM lanes this warp may read
+        ptx::fence_after_sync();
+        const int col0 = sg.tn * FEATURES + quarter * 32, tokens = min(a.M - sg.tm * BT, BT);
+        const uint32_t acc = tmem_base + party * ACC_COLS + ((uint32_t)(quarter * 32) << 16);
+        if (SMALL && quarter) return;
+#pragma unroll 1
+        for (int t0 = first * OUT_TOKENS; t0 < tokens; t0 += workers * OUT_TOKENS) {
+            u64* stage = buffer ? buffer : reinterpret_cast<u64*>(sRaw + (size_t)((party * QUARTERS + quarter) * (BT / OUT_TOKENS) + t0 / OUT_TOKENS) * OUT_BYTES);
+            uint32_t d[PLANES][OUT_TOKENS];
+#pragma unroll
+            for (int s = 0; s < PLANES; ++s) ptx::tmem_ld4(acc + COLS * s + t0, d[s]);
+            ptx::tmem_wait_ld();
+            if (lane == 0 && buffer) ptx::bulk_wait_group_read0();       // the last reduction has read its rows
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < OUT_TOKENS; ++j)
+                stage[j * 32 + lane] = limb_recombine(d[0][j], d[1][j], d[2][j], d[3][j], d[4][j], d[5][j], d[6][j], d[7][j]);
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0 && col0 < a.N) {
+                ptx::tensor_reduce_add(&maps.z[party], ptx::smem_u32(stage), col0, sg.tm * BT + t0);
+                ptx::bulk_commit_group();
+            }
+        }
+    };
+
+    if (raw_warp) {
         // ---------------- raw producer of one party: 16 lanes per row of a slot ----------------
         const int party = warp - RAW_WARP0, half = (lane >> 3) & 1, piece = lane & 15, rsub = lane >> 4;
         const uint32_t raw0 = ptx::smem_u32(sRaw) + party * 2 * RAW_ARRAY_BYTES + lane * 16;
@@ -261,12 +311,12 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
         for (unsigned u = u_begin; u < u_end && ok;) {
             const StreamSegment sg = stream_segment(a, u, u_end);
             u += sg.count;
-            const int quarters = stream_quarters(a, sg.tn);
+            const int quarters = stream_quarters<FEATURES>(a, sg.tn);
             // Sixteen rows aligned to 16 lie in one block (block sizes are multiples of 16), so they are `ldw` apart in W:
             // lane h of a warp's first eight knows where rows 16h .. 16h+15 of the tile begin
             const u64* w_row16 = W0;
             {
-                const int row = sg.tn * BW + (lane & 7) * 16;
+                const int row = sg.tn * FEATURES + (lane & 7) * 16;
                 if (row < a.N) {
                     if (!a.gather || a.down) {
                         w_row16 = W0 + (size_t)row * a.ldw;
@@ -277,6 +327,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                     }
                 }
             }
+            if (SMALL) pdl_wait();
             for (int it = 0; it < sg.count && ok; ++it) {
                 const int k = (sg.step + it) * KC + 2 * piece;
                 const bool kv = k < a.K;
@@ -286,7 +337,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                     col = block_id(a.ids, held, blk) * a.bs + (k - blk * a.bs);
                 }
                 for (int q = 0; q < quarters; ++q) {
-                    const int row0 = sg.tn * BW + q * QROWS + rsub;
+                    const int row0 = sg.tn * FEATURES + q * QROWS + rsub;
                     const int rows = kv ? a.N - row0 : 0;                          // this lane's rows: row0 + 2i, 2i < rows
                     const u64* right = Bi + (size_t)row0 * a.K + k;
                     const u64* left[2];                                            // rows 0-15 and 16-31 of the slot
@@ -312,6 +363,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                 }
             }
         }
+        if (SMALL) pdl_wait();
         asm volatile("cp.async.wait_all;" ::: "memory");          // no copy outlives the CTA, whatever ended the loop
     } else if (warp < CONV_WARPS) {
         // ---------------- converters ----------------
@@ -323,11 +375,11 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
         const int cell = (r >> 3) * 256 + (c >> 2) * 128 + (r & 7) * 16 + (c & 3) * 4;
         int slot = 0;
         uint32_t phase = 0, unit_phase = 0;
-        bool ok = true, planes_free = !a.sync || !stream_owns(a, u_begin, u_end);
+        bool ok = true, planes_free = !a.sync || !stream_owns(a, u_begin, u_end) || SMALL;
         for (unsigned u = u_begin; u < u_end && ok;) {
             const StreamSegment sg = stream_segment(a, u, u_end);
             u += sg.count;
-            const int quarters = stream_quarters(a, sg.tn);
+            const int quarters = stream_quarters<FEATURES>(a, sg.tn);
             for (int it = 0; it < sg.count && ok; ++it) {
                 const int k0 = (sg.step + it) * KC;
                 const bool kv[2] = {k0 + 2 * c < a.K, k0 + 16 + 2 * c < a.K};
@@ -361,7 +413,7 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                     for (int p = 0; p < 2; ++p)
 #pragma unroll
                         for (int e = 0; e < 4; ++e) f[p][e] -= b[p][e];
-                    const int row = sg.tn * BW + q * QROWS + r;
+                    const int row = sg.tn * FEATURES + q * QROWS + r;
                     const bool live = row < a.N;
                     if (a.blk_label && live) {                       // rows / columns outside every component stay closed
 #pragma unroll
@@ -404,11 +456,19 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                 unit_phase ^= 1u;
             }
         }
+        if (SMALL && ok && u_begin < u_end && (warp & 3) == 0) {         // two of three rounds of the sums are these warps'
+            const StreamSegment sg = stream_segment(a, u_begin, u_end);
+            const int party = warp >> 3, share = 1 + (warp >> 2 & 1);
+            if (share * OUT_TOKENS < min(a.M - sg.tm * BT, BT) && arrived(sg, party, 0)) {
+                drain(sg, party, nullptr, share, SMALL_WORKERS);
+                if (lane == 0) ptx::bulk_wait_group0();
+            }
+        }
     } else if (warp < MMA_WARP) {
         // ---------------- token side: the converters' cells, straight from L2 ----------------
         const int c = lane & 7, r = (4 * (warp - TOK_WARP0) ^ (c >= 4 ? 4 : 0)) + (lane >> 3);
         uint8_t* to = sV + (r >> 3) * 256 + (c >> 2) * 128 + (r & 7) * 16 + (c & 3) * 4;
-        const int party = (warp - TOK_WARP0) / EPI_WARPS, quarter = warp & 3;     // epilogue: TMEM lanes this warp may read
+        const int party = (warp - TOK_WARP0) / EPI_WARPS;
         u64* out = reinterpret_cast<u64*>(sOut + (size_t)(warp - TOK_WARP0) * OUT_BYTES);
         uint32_t unit_phase = 0, seg_phase = 0;
         bool ok = true;
@@ -469,37 +529,9 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
                 unit_phase ^= 1u;
             }
             if (!ok) break;
-            // ---------------- epilogue of the segment: lane = output feature, registers = tokens ----------------
-            // Result rows go through shared memory, OUT_TOKENS of them at a time, and one tensor reduction adds them into Z.
-            // A CTA's last segment stages them in the raw ring, which nothing uses any more, so that no round waits for the
-            // copy engine to have read the one before.  (One buffer and a bulk reduction per row: 7400 cycles for 32 tokens.)
-            if (a.sync) ok = stream_tile_ready(a.sync + SYNC_WORDS + sg.tile, epoch, lane, &abort_flag);
-            ok = ok && limb_wait_warp(ptx::smem_u32(&acc_full[party]), seg_phase, &abort_flag);
+            ok = arrived(sg, party, seg_phase);
             if (!ok) break;
-            ptx::fence_after_sync();
-            const int col0 = sg.tn * BW + quarter * 32, tokens = min(a.M - sg.tm * BT, BT);
-            const uint32_t acc = tmem_base + party * ACC_COLS + ((uint32_t)(quarter * 32) << 16);
-            const bool at_end = u >= u_end;
-            u64* stage = at_end ? reinterpret_cast<u64*>(sRaw + (size_t)(warp - TOK_WARP0) * (BT / OUT_TOKENS) * OUT_BYTES) : out;
-#pragma unroll 1
-            for (int t0 = 0; t0 < tokens; t0 += OUT_TOKENS) {
-                uint32_t d[PLANES][OUT_TOKENS];
-#pragma unroll
-                for (int s = 0; s < PLANES; ++s) ptx::tmem_ld4(acc + COLS * s + t0, d[s]);
-                ptx::tmem_wait_ld();
-                if (lane == 0 && !at_end) ptx::bulk_wait_group_read0();  // the last reduction has read its rows
-                __syncwarp();
-#pragma unroll
-                for (int j = 0; j < OUT_TOKENS; ++j)
-                    stage[j * 32 + lane] = limb_recombine(d[0][j], d[1][j], d[2][j], d[3][j], d[4][j], d[5][j], d[6][j], d[7][j]);
-                ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0 && col0 < a.N) {
-                    ptx::tensor_reduce_add(&maps.z[party], ptx::smem_u32(stage), col0, sg.tm * BT + t0);
-                    ptx::bulk_commit_group();
-                }
-                if (at_end) stage += OUT_TOKENS * 32;
-            }
+            drain(sg, party, u >= u_end ? nullptr : out, 0, SMALL ? SMALL_WORKERS : 1);
             ptx::fence_before_sync();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&acc_empty[party]));
@@ -570,8 +602,32 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
         uint32_t phase = 0;
         for (unsigned tile = (u_begin + a.kb - 1) / a.kb; tile < last && ok; ++tile, phase ^= 1u) {
             const int tn = (int)(tile / (unsigned)a.mt), tm = (int)tile - tn * a.mt;
-            const int rows = min(a.M - tm * BT, BT), bytes = min(a.N - tn * BW, BW) * 8;
-            const size_t at = (size_t)(tm * BT + lane) * a.N + tn * BW;
+            const int rows = min(a.M - tm * BT, BT), bytes = min(a.N - tn * FEATURES, FEATURES) * 8;
+            const size_t at = (size_t)(tm * BT + lane) * a.N + tn * FEATURES;
+            if (SMALL) {                         // through registers: 3 us until the flag is up, and 4 through shared memory
+                const int across = bytes / 16, pieces = rows * across;
+                const size_t corner = (size_t)(tm * BT) * a.N + tn * FEATURES;
+                for (int i = lane; i < pieces; i += 4 * 32) {
+                    ulonglong2 v[2][4];
+                    unsigned piece[4];           // a tile's rows lie within 32 N words
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int k = i + 32 * j, r = k / across;
+                        piece[j] = (unsigned)(r * a.N + 2 * (k - r * across));
+                        if (k < pieces)
+                            for (int p = 0; p < 2; ++p) v[p][j] = __ldcs(reinterpret_cast<const ulonglong2*>(a.C[p] + corner + piece[j]));
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (i + 32 * j < pieces)
+                            for (int p = 0; p < 2; ++p) *reinterpret_cast<ulonglong2*>(a.Z[p] + corner + piece[j]) = v[p][j];
+                }
+                asm volatile("fence.proxy.async;" ::: "memory");
+                __threadfence();
+                __syncwarp();
+                if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.sync + SYNC_WORDS + tile), "r"(epoch) : "memory");
+                continue;
+            }
             const uint32_t place = ptx::smem_u32(sB) + lane * (2 * BW * 8);
             if (lane == 0) ptx::mbar_expect_tx(ptx::smem_u32(&own_landed), 2 * rows * bytes);
             __syncwarp();

@@ -64,6 +64,8 @@ def test_static_product_in_place(cb, T, K, N, on):
     (32, 144, 24, 16, 9, 1, True),       # 144 features both ways: 128 and a ragged tile of 16
     (31, 112, 12, 48, 5, 2, True),       # strips of 48 columns: a step takes its halves from two blocks
     (8, 272, 8, 80, 3, 3, True),         # three stacked matrices, group boundaries inside a feature tile
+    (16, 1184, 16, 16, 8, 1, True), (17, 1184, 16, 16, 8, 1, True),        # 4 x 37 steps of tiles of 32 features, 37 x 4: all at once
+    (17, 1200, 16, 16, 8, 1, True),      # .. and 4 x 38 of the one side, 38 x 4 of the other: tiles of 128
     (33, 144, 24, 16, 9, 1, False),      # two token tiles, and few weights
     (33, 1008, 64, 16, 49, 1, True), (64, 1040, 60, 16, 40, 2, True),      # weights just many enough to be streamed ..
     (49, 1008, 64, 16, 48, 1, False), (65, 1040, 60, 16, 40, 2, False),    # .. and just too few; a row too many

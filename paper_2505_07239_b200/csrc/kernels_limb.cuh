@@ -766,6 +766,7 @@ struct LimbArgs {
     u64* Z[2];               // [M, N], pre-loaded with C_i; partial sums are added with bulk reductions
     int M, N;                // N a multiple of 16
     int mt, nt, kb;          // tiles and k-blocks per operand pair; one tile runs over 2*kb blocks
+    int parts;               // CTAs to a tile (limb_parts), or 0: all tiles' blocks in equal ranges
     int* error_flag;         // set to 1 if a bounded wait ran out
     int* error_host;         // the same report in mapped host memory, so that the host sees it without a copy
     // Only read by the grouped kernel (one multiplication per connected component): the planes hold the operands
@@ -913,8 +914,16 @@ __device__ __forceinline__ void combine_limb_body(const LimbArgs& a, const CUten
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long total_units = GROUPED ? 2ll * a.group_units : 2ll * a.mt * a.nt * 2ll * a.kb;
-    const long long u_begin = total_units * blockIdx.x / gridDim.x;
-    const long long u_end = total_units * (blockIdx.x + 1) / gridDim.x;
+    long long u_begin, u_end;
+    if (!GROUPED && a.parts) {                   // one part of one tile
+        const unsigned tile = blockIdx.x / (unsigned)a.parts, part = blockIdx.x - tile * a.parts;
+        const long long first = 2ll * a.kb * tile;
+        u_begin = first + 2u * (unsigned)a.kb * part / (unsigned)a.parts;
+        u_end = first + 2u * (unsigned)a.kb * (part + 1) / (unsigned)a.parts;
+    } else {
+        u_begin = total_units * blockIdx.x / gridDim.x;
+        u_end = total_units * (blockIdx.x + 1) / gridDim.x;
+    }
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {

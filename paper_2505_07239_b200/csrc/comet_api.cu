@@ -521,9 +521,11 @@ int limb_exchange(comet_ctx* c, const Proj& pr, bool residue, bool left, bool ri
     comet::LimbExchangeArgs a;
     const int blocks = exchange_args(c, pr, residue, left, right, copy, a);
     if (blocks + also_blocks == 0) return COMET_OK;
-    const bool tiles = left || right || also_blocks;
+    // A CTA of one k-block uses one stage, and more of them fit on an SM: 500 tokens, 512 x 256 40.7 -> 39.7 us a layer, 156 tokens,
+    // 2304 x 384 78.7 -> 77.0.
+    const size_t stages = std::min(std::max(left || right ? a.kb_per_cta : 0, also_blocks ? also->kb_per_cta : 0), (int)lb::EX_STAGES);
     COMET_CUDA(c, launch_chained(residue ? comet::limb_exchange_kernel<true> : comet::limb_exchange_kernel<false>, dim3(blocks + also_blocks), dim3(lb::EX_THREADS),
-                                 tiles ? lb::EX_SMEM_BYTES : 0, stream, nullptr, a, also ? *also : a, blocks, c->held));
+                                 stages * lb::EX_STAGE_BYTES, stream, nullptr, a, also ? *also : a, blocks, c->held));
     c->stats.kernel_launches += 1;
     COMET_CUDA(c, cudaGetLastError());
     return COMET_OK;

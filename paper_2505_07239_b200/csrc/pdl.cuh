@@ -8,6 +8,7 @@
 //                combine_stream_kernel, which no other kernel touches.)
 //   pdl_launch_dependents(): this CTA no longer minds the next kernel's CTAs being scheduled beside it; the next
 //                kernel starts once every CTA of this one has said so or has exited.
+//                Before or after pdl_wait(): every CTA of this kernel has started by then, so none of them is kept waiting for room.
 #pragma once
 
 namespace comet {

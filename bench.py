@@ -38,8 +38,8 @@ L2_FLUSH_BYTES = 512 << 20
 # the code it was taken on: keyed by that code's digest.
 COMBINE_LIMB_TRAFFIC = {
     "workload": ("opt1.3b", 0.95),
-    "kernel_sha256": "936cf4d9be2309eb244f82a8886f4383d18865a859d44ca6eb6e2ab84620cafb",
-    "bytes_per_launch": 46499328,
+    "kernel_sha256": "54c0d9649ec38bc7a2b20a8dd52bc7c5deaaad5d52e18745bf71266c523d043e",
+    "bytes_per_launch": 46515840,
 }
 COMBINE_RESIDUE_TRAFFIC = {                      # both launches: product and recombination
     "workload": ("opt1.3b", 0.9),

@@ -17,7 +17,7 @@
 // whose N spans accumulators D_p..D_7 (split in two when N > 256): 12 instructions per 32-deep step.
 //
 // Work is split stream-K style over a persistent grid: the (party, tile, k-block) space is cut into equal
-// contiguous ranges, every segment's partial sums are added to Z by 64-bit integer reductions of the copy
+// contiguous ranges, or every tile into parts of its own (LimbArgs::parts), every segment's partial sums are added to Z by 64-bit integer reductions of the copy
 // engine -- exact and order-independent in the ring -- and Z is pre-loaded with C_i.
 #pragma once
 #include <cstdint>

@@ -14,7 +14,8 @@
 // rate, the rest is 2 us until the first bytes arrive and 4 us from the last planes to the end (MMAs 3100 cycles, drain of 32
 // tokens 4000, of 7 tokens 1200, the reductions' completion 900).
 //
-// A CTA carries both parties' share of a tile of 128 output features (the rows of the MMA) x 32 tokens, and walks it in
+// A CTA carries both parties' share of a tile of 128 output features (the rows of the MMA; 32 of them in small products, see the
+// kernel's FEATURES) x 32 tokens, and walks it in
 // steps of 32 contraction indices.  What is computed for a party depends on that party's shares and on the two messages
 // alone; both parties' words of one place pass through the same thread, which is the exchange.
 //   warps 16-17   raw producers, one per party: 16-byte asynchronous copies of W_i, B_i (32 rows x 32 words of each per

@@ -1277,9 +1277,12 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
         // exchange before it, which is bound by the same memory), which hides about half of it but takes two events, a
         // launch and the programmatic start of the tensor-core kernel.  A step with 0.03 million such words takes 25 us in
         // one launch and 34 apart, with 0.52 million 97 and 94, with 1.7 million 249 and 237.  Fewer words, from EXCHANGE_APART_LEAST on, are
-        // worth that where the product is long enough, PRODUCT_APART multiply-adds, to hide them all: with 0.25 million words and
-        // 31 million multiply-adds 31.2 and 33.4 us, 37 million 37.9 and 38.6, 49 million 40.0 and 37.5, 74 million 46.5 and 44.9, 126
-        // million 58.0 and 54.6; with 0.13 million words and 34 million 30.3 and 30.8, 52 million 40.0 and 38.5; with 0.08 and 42 million 33.2 and 33.4.
+        // worth that where the product is long enough, PRODUCT_APART multiply-adds, to hide them all.  The stream then waits for them
+        // behind the product: what such a call has enqueued is over when the stream is, so it can be captured without the
+        // down-projection, and the down-projection without it.  With 0.25 million words and 47 million multiply-adds 39.2 us either way,
+        // 49 million 40.9 and 40.1, with 0.23 and 117 million 56.9 and 55.1; with 0.13 and 52 million 40.1 and 38.8, 134 million 59.7 and
+        // 57.4; with 0.08 and 82 million 50.1 and 49.0.  (With the wait left to the down-projection, 200 tokens, 960 x 256 take 39.7 instead
+        // of 40.1, 500 tokens, 512 x 256 39.0 instead of 40.5.)
         // A launch writes planes of one kind, so a weight side of the other kind goes apart whatever its size.  The kernel on
         // residues reads C' when it makes Y: nothing is copied for it.
         // An operand of this product may lie on Y: C' is then not copied there before it has been read.  The exchange reads
@@ -1287,8 +1290,8 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
         // after the product where that goes through residues, and a copy beside the product would be too early for it.
         const bool early = !c->dn_right_ready && limb_fits(c, dn) && c->loaded[0][COMET_W2] &&
                            c->loaded[1][COMET_W2] && c->loaded[0][COMET_B_DN] && c->loaded[1][COMET_B_DN];
-        const bool apart = early && (residue != dn_residue || (int64_t)dn.N * dn.K >= EXCHANGE_APART ||
-                                     ((int64_t)dn.N * dn.K >= EXCHANGE_APART_LEAST && (int64_t)up.M * up.N * up.K >= PRODUCT_APART));
+        const bool few_words = residue == dn_residue && (int64_t)dn.N * dn.K < EXCHANGE_APART;
+        const bool apart = early && (!few_words || ((int64_t)dn.N * dn.K >= EXCHANGE_APART_LEAST && (int64_t)up.M * up.N * up.K >= PRODUCT_APART));
         const bool y_in_use = !apart ? operands.any_on(COMET_Y) : residue && operands.on(up.idC, COMET_Y);
         const bool early_copy = early && !dn_residue && !y_in_use && c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN];
         comet::LimbExchangeArgs also;
@@ -1307,6 +1310,8 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
             if (rc != COMET_OK) return rc;
             COMET_CUDA(c, cudaEventRecord(c->ev_join, c->side));
             c->side_pending = true;
+            rc = few_words ? join_side(c) : COMET_OK;
+            if (rc != COMET_OK) return rc;
         }
         if (early) {
             c->dn_right_ready = true;

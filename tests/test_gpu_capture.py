@@ -56,15 +56,19 @@ class _Layer:
         return v
 
     def enqueue(self):
+        self.enqueue_up()
+        self.ctx.ffn_down(self.T)
+
+    def enqueue_up(self):
         cb, ctx = self.cb, self.ctx
         assert ctx.set_mask(self.mask) == self.n
         for t, pair in self.buffers.items():
             for p in (0, 1):
                 ctx.bind_shares(p, t, pair[p])
         ctx.ffn_up(self.T)
-        ctx.ffn_down(self.T)
 
-    def check(self, v):
+    def check(self, v, results_alone=False):
+        """The messages and results, or the results alone: they can be read where a replay has written them."""
         cb, (W1, W2) = self.cb, (self.W[self.cb.W1], self.W[self.cb.W2])
         t = lambda pair: [np.ascontiguousarray(m.T) for m in pair]  # noqa: E731  (stored output-feature-major)
         up = oracle.somm(v[cb.X], t(W1), self.I, v[cb.A_UP], t(v[cb.B_UP]), v[cb.C_UP])
@@ -73,6 +77,10 @@ class _Layer:
         for p in (0, 1):
             for ref, ids, rows, cols in ((up, (cb.E_UP, cb.F_UP, cb.Z_UP), self.n, self.d),
                                          (down, (cb.E_DN, cb.F_DN, cb.Y), self.d, self.n)):
+                if results_alone:
+                    out = self.ctx.result_view(p, ids[2], (self.T, rows)).cpu().numpy().view(np.uint64)
+                    assert np.array_equal(out, ref["Z"][p])
+                    continue
                 assert np.array_equal(self.ctx.get(p, ids[0], (self.T, cols)), ref["E"][p])
                 assert np.array_equal(self.ctx.get(p, ids[1], (rows, cols)).T, ref["F"][p])
                 assert np.array_equal(self.ctx.get(p, ids[2], (self.T, rows)), ref["Z"][p])
@@ -103,6 +111,40 @@ def test_layer_captured_and_replayed(cb, tokens, d, blocks, block, active):
     layer.enqueue()
     layer.check(v)
     del graph
+    layer.ctx.close()
+
+
+@pytest.mark.parametrize("tokens,d,blocks,block,active", [
+    (128, 304, 32, 16, 28),        # the down-projection's weight side in the launch before the product
+    (200, 960, 24, 16, 16),        # beside it: few words, and a long product
+])
+@pytest.mark.parametrize("up_captured", [True, False])
+def test_projections_captured_apart(cb, tokens, d, blocks, block, active, up_captured):
+    """A graph of the down-projection alone, behind a graph of the up-projection or an ordinary call of it: the functionality
+    between the two is the caller's."""
+    layer = _Layer(cb, tokens, d, blocks, block, active)
+    layer.fill(1)
+    layer.enqueue()
+    layer.stream.synchronize()
+    graphs = [torch.cuda.CUDAGraph() for _ in (0, 1)]
+    if up_captured:
+        with torch.cuda.graph(graphs[0], stream=layer.stream):
+            layer.enqueue_up()
+    else:
+        layer.enqueue_up()
+        layer.stream.synchronize()
+    with torch.cuda.graph(graphs[1], stream=layer.stream):
+        layer.ctx.ffn_down(tokens)
+    for step in (2, 3):
+        v = layer.fill(step)
+        with torch.cuda.stream(layer.stream):
+            if up_captured:
+                graphs[0].replay()
+            else:
+                layer.enqueue_up()
+            graphs[1].replay()
+        layer.check(v, results_alone=not up_captured)
+    del graphs
     layer.ctx.close()
 
 

@@ -612,7 +612,7 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
 }
 
 // Words of the down-projection's weight side, and multiply-adds of the up-projection's product: see comet_ffn_up.
-constexpr int64_t EXCHANGE_APART = 1 << 18, EXCHANGE_APART_LEAST = 1 << 16, PRODUCT_APART = 45000000;
+constexpr int64_t EXCHANGE_APART = 1 << 18, EXCHANGE_APART_LEAST = 1 << 16, PRODUCT_APART = 60000000;
 
 bool limb_fits(const comet_ctx* c, const Proj& pr) {
     namespace lb = comet::limb;
@@ -1279,10 +1279,13 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
         // one launch and 34 apart, with 0.52 million 97 and 94, with 1.7 million 249 and 237.  Fewer words, from EXCHANGE_APART_LEAST on, are
         // worth that where the product is long enough, PRODUCT_APART multiply-adds, to hide them all.  The stream then waits for them
         // behind the product: what such a call has enqueued is over when the stream is, so it can be captured without the
-        // down-projection, and the down-projection without it.  With 0.25 million words and 47 million multiply-adds 39.2 us either way,
-        // 49 million 40.9 and 40.1, with 0.23 and 117 million 56.9 and 55.1; with 0.13 and 52 million 40.1 and 38.8, 134 million 59.7 and
-        // 57.4; with 0.08 and 82 million 50.1 and 49.0.  (With the wait left to the down-projection, 200 tokens, 960 x 256 take 39.7 instead
-        // of 40.1, 500 tokens, 512 x 256 39.0 instead of 40.5.)
+        // down-projection, and the down-projection without it.  In one launch, apart, and apart without that wait, on the same buffers:
+        // 0.25 million words and 34 million multiply-adds 37.4, 39.8 and 38.3 us, 49 million 39.3, 40.6 and 39.9, 67 million 47.8, 47.2 and
+        // 45.9, 117 million 56.9, 54.9 and 54.6; 0.13 million and 52 million 38.4, 37.6 and 37.4, 59 million 38.6, 39.0 and 38.8, 65 million 40.1,
+        // 39.9 and 39.2; 0.1 million and 50 million 36.0, 36.9 and 36.7, 54 million 38.7, 38.3 and 37.6; two matrices, 0.07 million and 67 million
+        // 36.7, 36.1 and 35.1.  Under a token mask of several components the product works through less than that, but drains longer:
+        // 512 tokens, 0.25 million words and 126 million in four groups 78.0, 74.2 and 74.3, in sixteen 76.3, 72.2 and 72.2; 0.13 million and
+        // 67 million in two 67.5, 66.8 and 67.0, in sixteen 58.1, 58.6 and 57.3; 0.1 million and 54 million in sixteen 57.2, 58.1 and 57.1.
         // A launch writes planes of one kind, so a weight side of the other kind goes apart whatever its size.  The kernel on
         // residues reads C' when it makes Y: nothing is copied for it.
         // An operand of this product may lie on Y: C' is then not copied there before it has been read.  The exchange reads

@@ -151,8 +151,8 @@ typedef struct {
     int32_t n_components;    /* connected components under the current token mask (0 without one) */
     int32_t product_kernel;  /* COMET_KERNEL_* of the last ffn call's product (0 before the first) */
     int64_t tensor_tile_macs; /* 64-bit multiply-adds the tensor-core kernel of the last ffn call covered, counted
-                                 in whole output tiles (128 x 64, 32 tokens x 128 in the kernel for few tokens, 256 x a
-                                 multiple of 32 in the kernel on residues) and 32-deep steps, both parties (0 on the
+                                 in whole output tiles (128 x 64, 32 tokens x 128 in the kernel for few tokens, x 32
+                                 in small products of it, 256 x a multiple of 32 in the kernel on residues) and 32-deep steps, both parties (0 on the
                                  CUDA-core path): under a token mask with several components only the tiles and steps
                                  that meet a component */
 } comet_stats_t;

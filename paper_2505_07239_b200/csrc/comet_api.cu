@@ -341,6 +341,13 @@ cudaError_t result_map(CUtensorMap* map, u64* z, int rows, int cols, int box_row
     return tensor_map(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, z, size, pitch, box, step, swizzle);
 }
 
+// Features of a tile of the streaming kernel: 32 where the device has room for a CTA per step of such tiles.  Beyond that a CTA would
+// have several such steps, and the MMAs of each take as long as those of a step of 128.
+int stream_features(int M, int N, int K, int sm_count) {
+    namespace ls = comet::limb_stream;
+    return (long long)ceil_div(M, ls::BT) * ceil_div(N, ls::QROWS) * ceil_div(K, ls::KC) <= sm_count ? ls::QROWS : ls::BW;
+}
+
 // The streaming kernel.  Without `sync` words (they belong to one stream's order, so a call without a context has none) Z <- C
 // is a launch of its own before it; the product's CTAs are set up while the copy runs.
 int launch_stream(comet::StreamArgs& args, const comet::BlockIds& held, int sm_count, cudaStream_t stream,
@@ -349,10 +356,8 @@ int launch_stream(comet::StreamArgs& args, const comet::BlockIds& held, int sm_c
     *err = cudaSuccess;
     args.mt = ceil_div(args.M, ls::BT);
     args.kb = ceil_div(args.K, ls::KC);
-    // Tiles of 32 features where the device has room for a CTA per step of them.  Beyond that a CTA would have several such steps, and
-    // the MMAs of each take as long as those of a step of 128.
-    const bool small = (long long)args.mt * ceil_div(args.N, ls::QROWS) * args.kb <= sm_count;
-    const int features = small ? ls::QROWS : ls::BW;
+    const int features = stream_features(args.M, args.N, args.K, sm_count);
+    const bool small = features < ls::BW;
     args.nt = ceil_div(args.N, features);
     const long long steps = (long long)args.mt * args.nt * args.kb;
     const unsigned grid = (unsigned)(steps < sm_count ? steps : sm_count);
@@ -422,7 +427,7 @@ int stream_product(comet_ctx* c, const Proj& pr) {
         if (rc != COMET_OK) return rc;
     }
     c->stats.kernel_launches += 1;
-    c->stats.tensor_tile_macs = 2ll * 2 * a.mt * a.nt * a.kb * ls::KC * ls::BW * ls::BT;
+    c->stats.tensor_tile_macs = 2ll * 2 * a.mt * a.nt * a.kb * ls::KC * stream_features(a.M, a.N, a.K, c->sm_count) * ls::BT;
     c->stats.matmul_path = COMET_PATH_LIMB;
     c->stats.product_kernel = COMET_KERNEL_STREAM;
     return COMET_OK;

@@ -78,3 +78,31 @@ def test_few_token_layer_at_tile_edges(cb, tokens, d_model, blocks, block, activ
     r = hz.run_and_compare_products(cfg, seed=700 + tokens)
     assert r["mismatches"] == 0 and r["path"] == 2 and r["n_active"] == active * block, r
     assert r["kernels"] == [cb.KERNEL_STREAM if streamed else cb.KERNEL_LIMB] * 2
+
+
+@pytest.mark.parametrize("tokens,d,n", [
+    (16, 256, 96), (33, 1008, 784),                  # tiles of 32 features both ways; of 128
+    (17, 1184, 128), (17, 1200, 128),                # 37 x 4 steps and 4 x 37; 38 x 4 and 4 x 38
+    (32, 32, 2368), (32, 64, 2368),                  # 74 tiles of one step; of two, and 2 x 74
+])
+def test_tiles_of_a_few_token_layer(cb, tokens, d, n):
+    """The multiply-adds that the statistics report are those of the tiles that ran: 32 features where every step of such tiles has an SM."""
+    ctx = cb.Comet(tokens, d, n, 16, 12, max_active=n)
+    assert ctx.set_mask(np.ones(n // 16, np.uint8)) == n
+    shapes = {cb.W1: (n, d), cb.W2: (d, n), cb.X: (tokens, d), cb.A_UP: (tokens, d), cb.B_UP: (n, d), cb.C_UP: (tokens, n),
+              cb.H: (tokens, n), cb.A_DN: (tokens, n), cb.B_DN: (d, n), cb.C_DN: (tokens, d)}
+    zeros = {t: torch.zeros(s, dtype=torch.int64, device="cuda") for t, s in shapes.items()}
+    for t, v in zeros.items():
+        for p in (0, 1):
+            ctx.bind_shares(p, t, v)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    up_to = lambda a, b: -(-a // b)  # noqa: E731
+    for call, N, K in ((ctx.ffn_up, n, d), (ctx.ffn_down, d, n)):
+        call(tokens)
+        st = ctx.stats()
+        steps = up_to(tokens, 32) * up_to(K, 32)
+        features = 32 if steps * up_to(N, 32) <= sms else 128
+        assert st.product_kernel == cb.KERNEL_STREAM
+        assert st.tensor_tile_macs == 2 * 2 * steps * up_to(N, features) * features * 32 * 32, (N, K, features)
+    ctx.synchronize()
+    ctx.close()

@@ -148,6 +148,45 @@ def test_projections_captured_apart(cb, tokens, d, blocks, block, active, up_cap
     layer.ctx.close()
 
 
+@pytest.mark.parametrize("tokens,d,blocks,block,active,kernel", [
+    (16, 256, 32, 32, 3, "KERNEL_STREAM"), (32, 256, 32, 32, 3, "KERNEL_STREAM"),        # tiles of 32 features
+    (32, 1008, 64, 16, 49, "KERNEL_STREAM"),                                             # of 128
+    (128, 304, 32, 16, 28, "KERNEL_LIMB"), (512, 1024, 24, 16, 14, "KERNEL_LIMB"),       # tiles in parts; a launch beside the product
+])
+def test_layers_back_to_back(cb, tokens, d, blocks, block, active, kernel):
+    """Product, truncation, product, truncation, pass after pass and nothing in between: a kernel's CTAs are set up while the kernels
+    before it are still at work.  The inputs of each pass are bound where they lie."""
+    layer = _Layer(cb, tokens, d, blocks, block, active)
+    ctx, n = layer.ctx, layer.n
+    inputs = [{t: layer._draw(step, f"in{t}", s) for t, s in layer.shapes.items()} for step in range(4)]
+    resident = [{t: [cb.to_device(x) for x in pair] for t, pair in v.items()} for v in inputs]
+    views = [ctx.result_view(p, t, (tokens, cols)) for t, cols in ((cb.Z_UP, n), (cb.Y, d)) for p in (0, 1)]
+    torch.cuda.synchronize()
+    kept = []
+    with torch.cuda.stream(layer.stream):
+        for step in range(24):
+            ctx.set_mask(layer.mask)
+            for t, pair in resident[step % 4].items():
+                for p in (0, 1):
+                    ctx.bind_shares(p, t, pair[p])
+            ctx.ffn_up(tokens)
+            ctx.truncate(cb.Z_UP)
+            ctx.ffn_down(tokens)
+            ctx.truncate(cb.Y)
+            if step >= 20:                             # the first of them after 21 passes without anything else
+                kept.append([v.clone() for v in views])
+    assert ctx.stats().product_kernel == getattr(cb, kernel)
+    ctx.synchronize()
+    t = lambda pair: [np.ascontiguousarray(m.T) for m in pair]  # noqa: E731
+    for v, got in zip(inputs, kept):
+        up = oracle.somm(v[cb.X], t(layer.W[cb.W1]), layer.I, v[cb.A_UP], t(v[cb.B_UP]), v[cb.C_UP])
+        down = oracle.simm(v[cb.H], t(layer.W[cb.W2]), layer.I, v[cb.A_DN], t(v[cb.B_DN]), v[cb.C_DN])
+        want = [oracle.truncate(p, r["Z"][p], 16) for r in (up, down) for p in (0, 1)]
+        for g, w in zip(got, want):
+            assert np.array_equal(g.cpu().numpy().view(np.uint64), w)
+    ctx.close()
+
+
 @pytest.mark.parametrize("blocks", [1, 1024, 1040])    # lists that travel with the launches, and one that a kernel compacts
 def test_index_list_captured_and_replayed(cb, blocks):
     stream = torch.cuda.Stream()

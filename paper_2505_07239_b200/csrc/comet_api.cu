@@ -616,8 +616,10 @@ int limb_combine(comet_ctx* c, const Proj& pr) {
     return COMET_OK;
 }
 
-// Words of the down-projection's weight side, and multiply-adds of the up-projection's product: see comet_ffn_up.
-constexpr int64_t EXCHANGE_APART = 1 << 18, EXCHANGE_APART_LEAST = 1 << 16, PRODUCT_APART = 60000000;
+// Words of the down-projection's weight side from which on it is opened apart from the up-projection's exchange, and whether fewer are for
+// the multiply-adds of the up-projection's product: see comet_ffn_up.
+constexpr int64_t EXCHANGE_APART = 1 << 18;
+bool long_product(int64_t words, int64_t macs) { return words >= 1 << 16 && macs >= (words >= 1 << 17 ? 45000000 : 52000000); }
 
 bool limb_fits(const comet_ctx* c, const Proj& pr) {
     namespace lb = comet::limb;
@@ -1281,16 +1283,17 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
         // its traffic; from EXCHANGE_APART words on, on the side stream beside the tensor-core kernel (not beside the
         // exchange before it, which is bound by the same memory), which hides about half of it but takes two events, a
         // launch and the programmatic start of the tensor-core kernel.  A step with 0.03 million such words takes 25 us in
-        // one launch and 34 apart, with 0.52 million 97 and 94, with 1.7 million 249 and 237.  Fewer words, from EXCHANGE_APART_LEAST on, are
-        // worth that where the product is long enough, PRODUCT_APART multiply-adds, to hide them all.  The stream then waits for them
+        // one launch and 34 apart, with 0.52 million 97 and 94, with 1.7 million 249 and 237.  Fewer words are
+        // worth that where the product is long enough to hide them all (long_product).  The stream then waits for them
         // behind the product: what such a call has enqueued is over when the stream is, so it can be captured without the
-        // down-projection, and the down-projection without it.  In one launch, apart, and apart without that wait, on the same buffers:
-        // 0.25 million words and 34 million multiply-adds 37.4, 39.8 and 38.3 us, 49 million 39.3, 40.6 and 39.9, 67 million 47.8, 47.2 and
-        // 45.9, 117 million 56.9, 54.9 and 54.6; 0.13 million and 52 million 38.4, 37.6 and 37.4, 59 million 38.6, 39.0 and 38.8, 65 million 40.1,
-        // 39.9 and 39.2; 0.1 million and 50 million 36.0, 36.9 and 36.7, 54 million 38.7, 38.3 and 37.6; two matrices, 0.07 million and 67 million
-        // 36.7, 36.1 and 35.1.  Under a token mask of several components the product works through less than that, but drains longer:
-        // 512 tokens, 0.25 million words and 126 million in four groups 78.0, 74.2 and 74.3, in sixteen 76.3, 72.2 and 72.2; 0.13 million and
-        // 67 million in two 67.5, 66.8 and 67.0, in sixteen 58.1, 58.6 and 57.3; 0.1 million and 54 million in sixteen 57.2, 58.1 and 57.1.
+        // down-projection, and the down-projection without it.  In one launch, apart, and apart without that wait: 0.25 million words and
+        // 49 million multiply-adds 40.9, 40.8 and 39.8 us, 0.23 million and 117 million 57.0, 55.1 and 55.2; 0.16 million and 65 million 48.1, 46.6
+        // and 46.9; 0.13 million and 52 million 40.5, 38.8 and 39.0, 65 million 41.0, 40.4 and 40.1; 0.11 million and 59 million 41.0, 39.7 and 39.8
+        // as 256 x 448, 39.2, 39.5 and 39.2 as 512 x 224.  In one launch and apart: 0.1 million and 50 million 36.6 and 36.9 as 512 x 192, 36.6 and
+        // 36.2 as 384 x 256; 0.09 million and 46 million 36.2 and 36.7; 0.08 million and 82 million 50.1 and 49.0; 0.07 million and 67 million
+        // 42.5 either way.  Under a token mask of several components the product works through fewer, but drains longer, so the count is
+        // the same: 0.25 million words in four groups 76.0 and 75.2 (768 x 320), 81.2 and 77.8 (1024 x 240), in sixteen 74.4 and 73.3, in eight
+        // 75.6 either way; 0.13 million in sixteen 59.0 and 59.1.
         // A launch writes planes of one kind, so a weight side of the other kind goes apart whatever its size.  The kernel on
         // residues reads C' when it makes Y: nothing is copied for it.
         // An operand of this product may lie on Y: C' is then not copied there before it has been read.  The exchange reads
@@ -1299,7 +1302,7 @@ int comet_ffn_up(comet_ctx* c, int32_t tokens) {
         const bool early = !c->dn_right_ready && limb_fits(c, dn) && c->loaded[0][COMET_W2] &&
                            c->loaded[1][COMET_W2] && c->loaded[0][COMET_B_DN] && c->loaded[1][COMET_B_DN];
         const bool few_words = residue == dn_residue && (int64_t)dn.N * dn.K < EXCHANGE_APART;
-        const bool apart = early && (!few_words || ((int64_t)dn.N * dn.K >= EXCHANGE_APART_LEAST && (int64_t)up.M * up.N * up.K >= PRODUCT_APART));
+        const bool apart = early && (!few_words || long_product((int64_t)dn.N * dn.K, (int64_t)up.M * up.N * up.K));
         const bool y_in_use = !apart ? operands.any_on(COMET_Y) : residue && operands.on(up.idC, COMET_Y);
         const bool early_copy = early && !dn_residue && !y_in_use && c->loaded[0][COMET_C_DN] && c->loaded[1][COMET_C_DN];
         comet::LimbExchangeArgs also;

@@ -115,8 +115,8 @@ def test_layer_captured_and_replayed(cb, tokens, d, blocks, block, active):
 
 
 @pytest.mark.parametrize("tokens,d,blocks,block,active", [
-    (128, 304, 32, 16, 28), (200, 960, 24, 16, 16),        # the down-projection's weight side in the launch before the product
-    (512, 1024, 24, 16, 14),       # beside it: few words, and a long product
+    (128, 304, 32, 16, 28),                                # the down-projection's weight side in the launch before the product
+    (200, 960, 24, 16, 16), (512, 1024, 24, 16, 14),       # beside it: few words, and a long product
 ])
 @pytest.mark.parametrize("up_captured", [True, False])
 def test_projections_captured_apart(cb, tokens, d, blocks, block, active, up_captured):

@@ -34,12 +34,11 @@ def _launches(cb, tokens, d, blocks, clusters, early):
 
 
 @pytest.mark.parametrize("tokens,d,blocks,clusters,apart", [
-    (200, 960, 16, 0, False),                                 # 0.25 million words, 49 million multiply-adds
-    (457, 512, 16, 0, False), (458, 512, 16, 0, True),        # 0.13 million words, just below 60 million and just above
+    (200, 864, 16, 0, False), (200, 960, 16, 0, True),        # 0.2 million words, 44 and 49 million multiply-adds
+    (512, 512, 12, 0, False), (512, 512, 13, 0, True),        # 0.1 million words, 50 and 55 million
     (2048, 256, 15, 0, False), (2048, 256, 16, 0, True),      # 126 and 134 million, just fewer words than it takes and as many
     (400, 512, 32, 0, True),                                  # so many words that it takes no long product
-    (458, 512, 16, 4, True),                                  # the union's multiply-adds count
-    (512, 512, 12, 4, False),
+    (512, 512, 12, 4, False), (512, 512, 16, 4, True),        # in groups the union's multiply-adds count
 ])
 def test_launch_of_the_weight_side(tokens, d, blocks, clusters, apart):
     if not torch.cuda.is_available():

@@ -16,8 +16,6 @@ from paper_2505_07239_b200 import workloads as wl  # noqa: E402
     (260, 64, 101),        # 156 tiles: more than SMs, ranges
     (97, 1040, 8),         # 4 tiles of 66 blocks in 33 parts; 34 tiles of 8 blocks in 4
     (200, 960, 16), (200, 864, 16),      # the down-projection's weight side opened beside the product, and in the launch before it
-    # (in the launch before it, either of them: the product has to be longer, as here)
-    (512, 1024, 14),
 ])
 def test_layer_in_parts(tokens, d_model, active):
     if not torch.cuda.is_available():

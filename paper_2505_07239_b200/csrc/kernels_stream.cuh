@@ -269,35 +269,33 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
         return ok && limb_wait_warp(ptx::smem_u32(&acc_full[party]), seg_phase, &abort_flag);
     };
     // ---------------- epilogue of a segment: lane = output feature, registers = tokens ----------------
-    // Result rows go through shared memory, OUT_TOKENS of them at a time, and one tensor reduction adds them into Z; a worker takes
-    // every `workers`-th round from `first` on.  A CTA's last segment stages them in the raw ring (no `buffer`), which nothing uses any
-    // more, so that no round waits for the copy engine to have read the one before.  (One buffer and a bulk reduction per row:
-    // 7400 cycles for 32 tokens.)
-    auto drain = [&](const StreamSegment& sg, int party, u64* buffer, int first, int workers) {
-        const int quarter = warp & 3;            // TMEM lanes this warp may read
-        ptx::fence_after_sync();
-        const int col0 = sg.tn * FEATURES + quarter * 32, tokens = min(a.M - sg.tm * BT, BT);
-        const uint32_t acc = tmem_base + party * ACC_COLS + ((uint32_t)(quarter * 32) << 16);
-        if (SMALL && quarter) return;
-#pragma unroll 1
-        for (int t0 = first * OUT_TOKENS; t0 < tokens; t0 += workers * OUT_TOKENS) {
-            u64* stage = buffer ? buffer : reinterpret_cast<u64*>(sRaw + (size_t)((party * QUARTERS + quarter) * (BT / OUT_TOKENS) + t0 / OUT_TOKENS) * OUT_BYTES);
-            uint32_t d[PLANES][OUT_TOKENS];
+    // Result rows go through shared memory, OUT_TOKENS of them at a time, and one tensor reduction adds them into Z.  (A bulk reduction
+    // per row: 7400 cycles for 32 tokens.)
+    auto drain_round = [&](int party, uint32_t acc, int col0, int row0, int t0, u64* stage, bool reused) {
+        uint32_t d[PLANES][OUT_TOKENS];
 #pragma unroll
-            for (int s = 0; s < PLANES; ++s) ptx::tmem_ld4(acc + COLS * s + t0, d[s]);
-            ptx::tmem_wait_ld();
-            if (lane == 0 && buffer) ptx::bulk_wait_group_read0();       // the last reduction has read its rows
-            __syncwarp();
+        for (int s = 0; s < PLANES; ++s) ptx::tmem_ld4(acc + COLS * s + t0, d[s]);
+        ptx::tmem_wait_ld();
+        if (lane == 0 && reused) ptx::bulk_wait_group_read0();           // the last reduction has read its rows
+        __syncwarp();
 #pragma unroll
-            for (int j = 0; j < OUT_TOKENS; ++j)
-                stage[j * 32 + lane] = limb_recombine(d[0][j], d[1][j], d[2][j], d[3][j], d[4][j], d[5][j], d[6][j], d[7][j]);
-            ptx::fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0 && col0 < a.N) {
-                ptx::tensor_reduce_add(&maps.z[party], ptx::smem_u32(stage), col0, sg.tm * BT + t0);
-                ptx::bulk_commit_group();
-            }
+        for (int j = 0; j < OUT_TOKENS; ++j)
+            stage[j * 32 + lane] = limb_recombine(d[0][j], d[1][j], d[2][j], d[3][j], d[4][j], d[5][j], d[6][j], d[7][j]);
+        ptx::fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0 && col0 < a.N) {
+            ptx::tensor_reduce_add(&maps.z[party], ptx::smem_u32(stage), col0, row0 + t0);
+            ptx::bulk_commit_group();
         }
+    };
+    // Of a small tile, a CTA's only one: a worker, a warp that may read the first TMEM lanes, takes every SMALL_WORKERS-th round.  They stage
+    // in the raw ring, which nothing uses any more.
+    auto drain_small = [&](const StreamSegment& sg, int party, int worker) {
+        const int tokens = min(a.M - sg.tm * BT, BT);
+        ptx::fence_after_sync();
+        for (int t0 = worker * OUT_TOKENS; t0 < tokens; t0 += SMALL_WORKERS * OUT_TOKENS)
+            drain_round(party, tmem_base + party * ACC_COLS, sg.tn * FEATURES, sg.tm * BT, t0,
+                        reinterpret_cast<u64*>(sRaw + (size_t)(party * (BT / OUT_TOKENS) + t0 / OUT_TOKENS) * OUT_BYTES), false);
     };
 
     if (raw_warp) {
@@ -459,9 +457,9 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
         }
         if (SMALL && ok && u_begin < u_end && (warp & 3) == 0) {         // two of three rounds of the sums are these warps'
             const StreamSegment sg = stream_segment(a, u_begin, u_end);
-            const int party = warp >> 3, share = 1 + (warp >> 2 & 1);
-            if (share * OUT_TOKENS < min(a.M - sg.tm * BT, BT) && arrived(sg, party, 0)) {
-                drain(sg, party, nullptr, share, SMALL_WORKERS);
+            const int party = warp >> 3, worker = 1 + (warp >> 2 & 1);
+            if (worker * OUT_TOKENS < min(a.M - sg.tm * BT, BT) && arrived(sg, party, 0)) {
+                drain_small(sg, party, worker);
                 if (lane == 0) ptx::bulk_wait_group0();
             }
         }
@@ -532,7 +530,24 @@ combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constan
             if (!ok) break;
             ok = arrived(sg, party, seg_phase);
             if (!ok) break;
-            drain(sg, party, u >= u_end ? nullptr : out, 0, SMALL ? SMALL_WORKERS : 1);
+            const int quarter = warp & 3;        // TMEM lanes this warp may read
+            if (SMALL) {
+                if (quarter == 0) drain_small(sg, party, 0);
+            } else {
+                // A CTA's last segment stages its rows in the raw ring, which nothing uses any more, so that no round waits for the copy
+                // engine to have read the one before.  (With both kinds of tile in one function, rounds and place by its arguments, every
+                // layer in tiles of 128 features took 0.4 to 1 % longer: 32 tokens, 2048 x 832 54.4 -> 55.0 us, 4096 x 1312 127.5 -> 128.3.)
+                ptx::fence_after_sync();
+                const int tokens = min(a.M - sg.tm * BT, BT);
+                const uint32_t acc = tmem_base + party * ACC_COLS + ((uint32_t)(quarter * 32) << 16);
+                const bool at_end = u >= u_end;
+                u64* stage = at_end ? reinterpret_cast<u64*>(sRaw + (size_t)(warp - TOK_WARP0) * (BT / OUT_TOKENS) * OUT_BYTES) : out;
+#pragma unroll 1
+                for (int t0 = 0; t0 < tokens; t0 += OUT_TOKENS) {
+                    drain_round(party, acc, sg.tn * BW + quarter * 32, sg.tm * BT, t0, stage, !at_end);
+                    if (at_end) stage += OUT_TOKENS * 32;
+                }
+            }
             ptx::fence_before_sync();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&acc_empty[party]));

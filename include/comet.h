@@ -39,7 +39,10 @@
  *     replayed any number of times, other steps in between: what the kernels count
  *     advances on the device.  The graph keeps the mask it was captured with (a
  *     HOST mask of at most 3584 blocks) and reads and writes the buffers that were
- *     bound then.
+ *     bound then.  A graph of comet_ffn_up alone, or of comet_ffn_down alone, is
+ *     possible while d_model times the active neurons stays below 2^18 and both
+ *     products take the same kernel; otherwise comet_ffn_up may leave work on the
+ *     internal stream that comet_ffn_down waits for.
  */
 #ifndef COMET_H_
 #define COMET_H_

@@ -304,8 +304,10 @@ struct OperandsOffResult {
 // The streaming kernel (one kernel per product, operand roles exchanged) serves layers with at most 32 token rows: its planes
 // live in shared memory, so every further 32 rows convert the weights once more.  Up to 64 rows that still beats writing the
 // planes to memory and reading them back where the weights are many (without a token mask, whose components only the other
-// kernel separates).  Both products of a step, 48 rows, streaming / planes: 1024 x 320 37.9 / 37.0 us, 1024 x 768 52.1 / 53.6,
-// 2048 x 512 56.6 / 64.6, 2048 x 832 77.7 / 86.6, 4096 x 1312 189 / 238; 96 rows of 4096 x 1312 took 329 / 263.
+// kernel separates).  Both products of a step, 48 rows, streaming / planes: 448 x 320 32.8 / 25.9 us, 1024 x 320 38.4 / 35.1, 1024 x 768 51.9 / 50.9,
+// 2048 x 512 56.7 / 61.6, 2048 x 832 77.3 / 88.3, 4096 x 1312 207 / 249; 33 rows, 1024 x 768 52.1 / 49.5, 2048 x 512 56.7 / 60.6; 64 rows, 1536 x 512 51.6 / 51.2,
+// 2048 x 512 59.6 / 62.8; 96 rows of 4096 x 1312 took 329 / 263.  Very small layers would gain too, in tiles of 32 features: 48 rows, 256 x 96
+// 22.2 / 26.1; they are left to the planes.
 constexpr int STREAM_TOKENS = 2 * comet::limb_stream::BT;
 constexpr int64_t STREAM_WORDS = 3 << 19;          // of the layer's active weights, from which on 33..64 rows are streamed
 bool few_tokens(const comet_ctx* c, int tokens) {

@@ -39,7 +39,7 @@ constexpr int EPI_WARPS = 8;                      // warp w drains TMEM lanes 32
 constexpr int THREADS = 32 * (EPI_WARPS + 2);     // warps 0-7 epilogue, warp 8 copy producer, warp 9 MMA issuer
 constexpr int EX_THREADS = 128, EX_ROWS = 16, EX_MAX_KB_PER_CTA = 16;      // exchange kernel: four rows per warp
 constexpr int EX_STAGES = 2, EX_STAGE_BYTES = EX_THREADS * 8 * 16;           // eight 16-byte pieces per lane and k-block
-constexpr size_t EX_SMEM_BYTES = (size_t)EX_STAGES * EX_STAGE_BYTES;        // 32 KiB: fits beside a tensor-core CTA
+constexpr size_t EX_SMEM_BYTES = (size_t)EX_STAGES * EX_STAGE_BYTES;        // 32 KiB at most: fits beside a tensor-core CTA
 constexpr int OUT_COLS = 16;                      // words per staged output row (a thread's 32 go in two rounds)
 constexpr int OUT_ROW_BYTES = OUT_COLS * 8 + 16;  // padded against bank conflicts (grouped kernel: one copy per row)
 constexpr int OUT_TILE_BYTES = 32 * OUT_COLS * 8; // swizzled instead (one tensor copy per warp and round), 1 KiB aligned

@@ -219,8 +219,9 @@ __device__ __forceinline__ u64 trunc_word(u64 s, int f, int party) {
 __global__ void __launch_bounds__(256)
 truncate_kernel(PartyOut Z, int64_t pairs, int f) {
     // Dependents first: the next product's CTAs take the SMs that the last one's leave, and are set up when its results are there (a CTA
-    // that has waited for this kernel has waited for all before it).  Layer of 3 tokens, 2336 x 832: 53.1 -> 51.0 us; 14 tokens,
-    // 3344 x 2 x 576: 72.5 -> 71.4; 32 tokens, 4096 x 1312: 126.4 -> 125.0.  Where calls of the host or larger kernels lie between, the same.
+    // that has waited for this kernel has waited for all before it).  Layer of 3 tokens, 2336 x 832: 53.6 -> 51.8 us; 8 tokens, 1024 x 1024:
+    // 38.2 -> 36.5; 32 tokens, 2048 x 832: 56.4 -> 55.5, 4096 x 1312: 123.8 -> 121.7; 14 tokens, 3344 x 2 x 576: 73.1 -> 72.5.  Where an exchange
+    // or calls of the host come next, the same.
     pdl_launch_dependents();
     pdl_wait();
     const int party = blockIdx.y;

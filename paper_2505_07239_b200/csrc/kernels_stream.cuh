@@ -200,8 +200,8 @@ __device__ __forceinline__ bool stream_tile_ready(const uint32_t* flag, uint32_t
 // all of its words, and its end for its own sums, and a quarter of either is there sooner; the MMAs have a quarter of their rows
 // in use, which costs nothing.  With so few steps latency is all there is, so the rest is cut short too: the first rows are found
 // before the wait for the kernel before this one, Z <- C goes through registers, and three warps a party drain.  From that wait
-// to the end, 16 tokens x 256 deep x 96: 7.8 -> 6.5 us.  A layer of 256 x 96: 16 tokens 22.6 -> 20.6 us (then bound by the host's calls),
-// 32 tokens 29.6 -> 22.3; of 448 x 320, 32 tokens 31.4 -> 28.8.
+// to the end, 16 tokens x 256 deep x 96: 7.8 -> 6.5 us.  A layer of 256 x 96, 32 tokens: 29.9 -> 21.9 us; 16 tokens: 22.3 to 22.9 -> 19.6 to
+// 21.9, which is what the host's calls take; of 448 x 320, 32 tokens: 31.2 -> 28.8.
 template <int COLS, int FEATURES>
 __global__ void __launch_bounds__(limb_stream::THREADS, 1)
 combine_stream_kernel(const __grid_constant__ StreamArgs a, const __grid_constant__ LimbMaps maps,

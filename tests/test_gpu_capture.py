@@ -56,19 +56,15 @@ class _Layer:
         return v
 
     def enqueue(self):
-        self.enqueue_up()
-        self.ctx.ffn_down(self.T)
-
-    def enqueue_up(self):
         cb, ctx = self.cb, self.ctx
         assert ctx.set_mask(self.mask) == self.n
         for t, pair in self.buffers.items():
             for p in (0, 1):
                 ctx.bind_shares(p, t, pair[p])
         ctx.ffn_up(self.T)
+        ctx.ffn_down(self.T)
 
-    def check(self, v, results_alone=False):
-        """The messages and results, or the results alone: they can be read where a replay has written them."""
+    def check(self, v):
         cb, (W1, W2) = self.cb, (self.W[self.cb.W1], self.W[self.cb.W2])
         t = lambda pair: [np.ascontiguousarray(m.T) for m in pair]  # noqa: E731  (stored output-feature-major)
         up = oracle.somm(v[cb.X], t(W1), self.I, v[cb.A_UP], t(v[cb.B_UP]), v[cb.C_UP])
@@ -77,10 +73,6 @@ class _Layer:
         for p in (0, 1):
             for ref, ids, rows, cols in ((up, (cb.E_UP, cb.F_UP, cb.Z_UP), self.n, self.d),
                                          (down, (cb.E_DN, cb.F_DN, cb.Y), self.d, self.n)):
-                if results_alone:
-                    out = self.ctx.result_view(p, ids[2], (self.T, rows)).cpu().numpy().view(np.uint64)
-                    assert np.array_equal(out, ref["Z"][p])
-                    continue
                 assert np.array_equal(self.ctx.get(p, ids[0], (self.T, cols)), ref["E"][p])
                 assert np.array_equal(self.ctx.get(p, ids[1], (rows, cols)).T, ref["F"][p])
                 assert np.array_equal(self.ctx.get(p, ids[2], (self.T, rows)), ref["Z"][p])
@@ -112,79 +104,6 @@ def test_layer_captured_and_replayed(cb, tokens, d, blocks, block, active):
     layer.check(v)
     del graph
     layer.ctx.close()
-
-
-@pytest.mark.parametrize("tokens,d,blocks,block,active", [
-    (128, 304, 32, 16, 28),                                # the down-projection's weight side in the launch before the product
-    (200, 960, 24, 16, 16), (512, 1024, 24, 16, 14),       # beside it: few words, and a long product
-])
-@pytest.mark.parametrize("up_captured", [True, False])
-def test_projections_captured_apart(cb, tokens, d, blocks, block, active, up_captured):
-    """A graph of the down-projection alone, behind a graph of the up-projection or an ordinary call of it: the functionality
-    between the two is the caller's."""
-    layer = _Layer(cb, tokens, d, blocks, block, active)
-    layer.fill(1)
-    layer.enqueue()
-    layer.stream.synchronize()
-    graphs = [torch.cuda.CUDAGraph() for _ in (0, 1)]
-    if up_captured:
-        with torch.cuda.graph(graphs[0], stream=layer.stream):
-            layer.enqueue_up()
-    else:
-        layer.enqueue_up()
-        layer.stream.synchronize()
-    with torch.cuda.graph(graphs[1], stream=layer.stream):
-        layer.ctx.ffn_down(tokens)
-    for step in (2, 3):
-        v = layer.fill(step)
-        with torch.cuda.stream(layer.stream):
-            if up_captured:
-                graphs[0].replay()
-            else:
-                layer.enqueue_up()
-            graphs[1].replay()
-        layer.check(v, results_alone=not up_captured)
-    del graphs
-    layer.ctx.close()
-
-
-@pytest.mark.parametrize("tokens,d,blocks,block,active,kernel", [
-    (16, 256, 32, 32, 3, "KERNEL_STREAM"), (32, 256, 32, 32, 3, "KERNEL_STREAM"),        # tiles of 32 features
-    (32, 1008, 64, 16, 49, "KERNEL_STREAM"),                                             # of 128
-    (128, 304, 32, 16, 28, "KERNEL_LIMB"), (512, 1024, 24, 16, 14, "KERNEL_LIMB"),       # tiles in parts; a launch beside the product
-])
-def test_layers_back_to_back(cb, tokens, d, blocks, block, active, kernel):
-    """Product, truncation, product, truncation, pass after pass and nothing in between: a kernel's CTAs are set up while the kernels
-    before it are still at work.  The inputs of each pass are bound where they lie."""
-    layer = _Layer(cb, tokens, d, blocks, block, active)
-    ctx, n = layer.ctx, layer.n
-    inputs = [{t: layer._draw(step, f"in{t}", s) for t, s in layer.shapes.items()} for step in range(4)]
-    resident = [{t: [cb.to_device(x) for x in pair] for t, pair in v.items()} for v in inputs]
-    views = [ctx.result_view(p, t, (tokens, cols)) for t, cols in ((cb.Z_UP, n), (cb.Y, d)) for p in (0, 1)]
-    torch.cuda.synchronize()
-    kept = []
-    with torch.cuda.stream(layer.stream):
-        for step in range(24):
-            ctx.set_mask(layer.mask)
-            for t, pair in resident[step % 4].items():
-                for p in (0, 1):
-                    ctx.bind_shares(p, t, pair[p])
-            ctx.ffn_up(tokens)
-            ctx.truncate(cb.Z_UP)
-            ctx.ffn_down(tokens)
-            ctx.truncate(cb.Y)
-            if step >= 20:                             # the first of them after 21 passes without anything else
-                kept.append([v.clone() for v in views])
-    assert ctx.stats().product_kernel == getattr(cb, kernel)
-    ctx.synchronize()
-    t = lambda pair: [np.ascontiguousarray(m.T) for m in pair]  # noqa: E731
-    for v, got in zip(inputs, kept):
-        up = oracle.somm(v[cb.X], t(layer.W[cb.W1]), layer.I, v[cb.A_UP], t(v[cb.B_UP]), v[cb.C_UP])
-        down = oracle.simm(v[cb.H], t(layer.W[cb.W2]), layer.I, v[cb.A_DN], t(v[cb.B_DN]), v[cb.C_DN])
-        want = [oracle.truncate(p, r["Z"][p], 16) for r in (up, down) for p in (0, 1)]
-        for g, w in zip(got, want):
-            assert np.array_equal(g.cpu().numpy().view(np.uint64), w)
-    ctx.close()
 
 
 @pytest.mark.parametrize("blocks", [1, 1024, 1040])    # lists that travel with the launches, and one that a kernel compacts
